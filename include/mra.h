@@ -176,7 +176,8 @@ typedef struct {
                          three l_z, term), each one set of stage-1, 2 and 3 MMAs; 0 otherwise */
 } mra_apply_stats;
 
-#define MRA_KERNEL_F64 0        /* FP64 destination-stationary kernel */
+#define MRA_KERNEL_F64 0        /* FP64: source-stationary in parity components where every record
+                                   lies within |l|_inf <= 1, else destination-stationary */
 #define MRA_KERNEL_SPLIT_DEST 1 /* split-BF16 destination-stationary tensor-core kernel */
 #define MRA_KERNEL_SPLIT_SRC 2  /* split-BF16 source-stationary tensor-core kernel */
 

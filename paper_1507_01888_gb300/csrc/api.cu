@@ -102,6 +102,7 @@ void free_operator(Operator *op) {
   cudaFree(op->d_t);
   cudaFree(op->d_R);
   cudaFree(op->d_N);
+  cudaFree(op->d_W);
   cudaFree(op->d_D);
   cudaFree(op->d_level_off);
   cudaFree(op->d_Rsplit);
@@ -284,9 +285,9 @@ int mra_release_memory(void) {
 int mra_debug_status(int *line, void *stream) {
   if (!line) return fail(MRA_ERR_ARG, "mra_debug_status: NULL line");
   cudaStream_t s = (cudaStream_t)stream;
-  const int a = debug_line_apply(s), b = debug_line_split(s), c = debug_line_src(s);
-  if (a < 0 || b < 0 || c < 0) return fail(MRA_ERR_CUDA, "mra_debug_status: reading the check words failed");
-  *line = a ? a : (b ? b : c);
+  const int a = debug_line_apply(s), b = debug_line_split(s), c = debug_line_src(s), d = debug_line_f64(s);
+  if (a < 0 || b < 0 || c < 0 || d < 0) return fail(MRA_ERR_CUDA, "mra_debug_status: reading the check words failed");
+  *line = a ? a : (b ? b : (c ? c : d));
   return MRA_OK;
 }
 
@@ -377,6 +378,7 @@ int mra_operator_create(int kernel, double mu, int M, double fit_eps, double r_l
   if (e != cudaSuccess) return bail(fail(MRA_ERR_CUDA, "operator blocks: %s", cudaGetErrorString(e)));
   {
     int rc = split_blocks_build(*op, s);  // BF16 pieces of every block for the tensor-core path
+    if (rc == MRA_OK) rc = f64_parity_build(*op, s);  // and their parity components for the FP64 path
     if (rc != MRA_OK) return bail(rc);
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return bail(fail(MRA_ERR_CUDA, "split blocks: %s", cudaGetErrorString(e)));
@@ -427,6 +429,8 @@ int mra_operator_refit(mra_operator *h, double mu, int *blocks_reused, void *str
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(d_gl);
     if (e != cudaSuccess) return fail(MRA_ERR_CUDA, "operator blocks: %s", cudaGetErrorString(e));
+    const int rcp = f64_parity_build(*op, s);
+    if (rcp != MRA_OK) return rcp;
   }
   const int rc2 = split_blocks_build(*op, s, true);  // the c_m-scaled pieces change with c_m
   if (rc2 != MRA_OK) return rc2;

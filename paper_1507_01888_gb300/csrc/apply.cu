@@ -419,7 +419,7 @@ __global__ void func_offsets_kernel(int64_t n, const int *dest_func, int nfunc, 
 }
 
 // ---------------------------------------------------------------- FP64 gather-apply
-// One CTA per destination box.  For each of its records (source b, l, mask)
+// Records beyond |l|_inf = 1 (the others run in apply_f64.cu).  One CTA per destination box.  For each of its records (source b, l, mask)
 // and each kept term m:  t1 = s x_1 Rx, t2 = t1 x_2 Ry, t3 = t2 x_3 Rz,
 // acc += c_m t3 (Sec. 2.3), acc held in registers across all records.
 // PT accumulators per thread: k^3 <= 256 PT (PT = 16 up to k = 16, 32 for the non-standard
@@ -735,6 +735,21 @@ bool apply_uses_src_path(const Operator &op, const mra_apply_opts &o) {
   int dmax = 0;
   for (int n = op.min_level; n <= op.max_level; ++n) dmax = std::max(dmax, records_disp(op, o, n));
   return src_path_supported(op.k, dmax);
+}
+
+// Whether an FP64 apply runs the source-stationary kernel of apply_f64.cu: every record within
+// |l|_inf <= 1 (wider ones are gathered per destination by apply_f64_kernel).
+static bool apply_uses_f64_sym(const Operator &op, const mra_apply_opts &o) {
+  if (o.precision != MRA_PREC_FP64) return false;
+  int dmax = 0;
+  for (int n = op.min_level; n <= op.max_level; ++n) dmax = std::max(dmax, records_disp(op, o, n));
+  return dmax <= 1;
+}
+
+size_t graph_partial_bytes(const Operator &op, const mra_apply_opts &o, int64_t P) {
+  if (P <= 0) return 0;
+  if (apply_uses_src_path(op, o)) return (size_t)P * op.k * op.k * op.k * sizeof(float);
+  return apply_uses_f64_sym(op, o) ? f64_partial_bytes(op.k, P) : 0;
 }
 
 size_t apply_workspace_bytes(const Operator &op, const mra_apply_opts &o, int64_t n_in) {
@@ -1053,7 +1068,10 @@ int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts 
   wk.fx = fx;
   if (stats)
     stats->kernel = o.precision == MRA_PREC_FP64 ? MRA_KERNEL_F64 : src_path ? MRA_KERNEL_SPLIT_SRC : MRA_KERNEL_SPLIT_DEST;
-  if (o.precision == MRA_PREC_FP64) {
+  if (apply_uses_f64_sym(op, o)) {
+    rc = apply_f64_run(op, in, out, wk, s);
+    if (rc != MRA_OK) return rc;
+  } else if (o.precision == MRA_PREC_FP64) {
     if (ev0) MRA_CUDA_TRY(cudaEventRecord(ev0, s));
     size_t smem = (size_t)(3 * k3 + 3 * k * k) * sizeof(double);
     auto kern = k3 <= 16 * F64_THREADS ? apply_f64_kernel<16> : apply_f64_kernel<32>;
@@ -1070,7 +1088,7 @@ int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts 
     // recorded, else from the library's memory pool for this call
     int dap[MRA_MAX_LEVEL + 1];
     for (int n = 0; n <= MRA_MAX_LEVEL; ++n) dap[n] = records_disp(op, o, n);
-    float *partial = fx ? fx->partial : nullptr;
+    float *partial = fx ? (float *)fx->partial : nullptr;
     if (!fx) MRA_CUDA_TRY(pool_malloc((void **)&partial, (size_t)P * k3 * sizeof(float), s));
     if (!partial) return fail(MRA_ERR_ARG, "mra_apply: no partial-sum buffer for the recorded apply");
     int64_t passes = 0;

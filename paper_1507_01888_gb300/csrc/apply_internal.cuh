@@ -14,7 +14,7 @@ struct FixedSizes {
   int64_t P = 0, nd = 0;
   int *status = nullptr;                  // device word
   const int64_t *d_in_offsets = nullptr;  // device copy of the batched input offsets (nfunc + 1)
-  float *partial = nullptr;               // the source-stationary kernel's partial sums (P k^3 floats)
+  void *partial = nullptr;                // the source-stationary kernels' partial sums (graph_partial_bytes)
 };
 
 // The sorted work list handed from the screen/sort stage to an apply kernel.
@@ -61,6 +61,13 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
 // whether an apply with these options runs the source-stationary kernel (its partial sums need
 // P k^3 floats besides the workspace)
 bool apply_uses_src_path(const Operator &op, const mra_apply_opts &o);
+// FP64 source-stationary apply of records with |l|_inf <= 1 (apply_f64.cu): its parity tables (made
+// again when the blocks change), its partial buffer, and the run
+int f64_parity_build(Operator &op, cudaStream_t s);
+size_t f64_partial_bytes(int k, int64_t P);
+int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &out, const ApplyWork &wk, cudaStream_t s);
+// bytes of partial sums that a recorded apply with P records owns (0: its kernel needs none)
+size_t graph_partial_bytes(const Operator &op, const mra_apply_opts &o, int64_t P);
 // test hook of the failure path (one-shot), and the fixed-size mode's status from a kernel error word
 bool take_injected_stall();
 void split_fixed_err(const int *err, int *status, cudaStream_t s);

@@ -20,7 +20,7 @@ struct ApplyGraph {
   cudaStream_t cap = nullptr;
   int *d_status = nullptr;
   int64_t *d_in_offsets = nullptr;
-  float *d_partial = nullptr;
+  void *d_partial = nullptr;
   FixedSizes fx;
   int64_t n_out = 0;
   long long kernels = 0;
@@ -84,8 +84,8 @@ int mra_apply_graph_create(const mra_operator *h, int nfunc, const mra_tree_view
   g->fx.d_in_offsets = g->d_in_offsets;
   g->n_out = out->n;
   const Operator *op = reinterpret_cast<const Operator *>(h);
-  if (apply_uses_src_path(*op, *o) && st.pairs > 0) {  // the recorded apply's partial sums, owned by the graph
-    e = cudaMalloc((void **)&g->d_partial, (size_t)st.pairs * op->k * op->k * op->k * sizeof(float));
+  if (const size_t pb = graph_partial_bytes(*op, *o, st.pairs)) {  // the recorded apply's partial sums, owned by the graph
+    e = cudaMalloc(&g->d_partial, pb);
     if (e != cudaSuccess) return bail(MRA_ERR_CUDA, "partial-sum buffer", e);
     g->fx.partial = g->d_partial;
   }

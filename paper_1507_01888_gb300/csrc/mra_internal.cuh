@@ -71,6 +71,7 @@ static inline int debug_take_line(cudaStream_t) { return 0; }
 int debug_line_apply(cudaStream_t s);
 int debug_line_split(cudaStream_t s);
 int debug_line_src(cudaStream_t s);
+int debug_line_f64(cudaStream_t s);
 
 // ---------------------------------------------------------------- keys
 __host__ __device__ inline uint64_t make_key(int n, int64_t x, int64_t y, int64_t z) {
@@ -100,6 +101,7 @@ struct Operator {
   double *d_c = nullptr, *d_t = nullptr;  // device fit
   double *d_R = nullptr;                  // device blocks, n_blocks * k*k
   double *d_N = nullptr;                  // device block norms, n_blocks
+  double *d_W = nullptr;                  // parity components of the |l| <= 1 blocks (apply_f64.cu)
   int *d_D = nullptr;                     // device copy of D (20 entries, by absolute level)
   int64_t *d_level_off = nullptr;         // device copy (20 entries, by absolute level; -1 = absent)
   // split-precision copies of the blocks for the tensor-core path (lazily built)

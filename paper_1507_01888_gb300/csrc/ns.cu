@@ -776,6 +776,10 @@ extern "C" int mra_operator_ns_create(const mra_operator *h, int max_disp, mra_o
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return bail(fail(MRA_ERR_CUDA, "mra_operator_ns_create: %s", cudaGetErrorString(e)));
+  {  // parity components of the blocks, for the FP64 path
+    int rc = f64_parity_build(*ns, s);
+    if (rc != MRA_OK) return bail(rc);
+  }
   if (ns->k <= MRA_MAX_K) {  // BF16 pieces of the 2k blocks for the tensor-core path
     int rc = split_blocks_build(*ns, s);
     if (rc != MRA_OK) return bail(rc);
