@@ -3,9 +3,11 @@
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <cub/cub.cuh>
@@ -516,12 +518,24 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
       out->n = total;
       return fail(MRA_ERR_CAPACITY, "mra_project: %lld boxes needed, cap %lld", (long long)total, (long long)out->cap);
     }
-    std::vector<uint64_t> keys(total);
+    std::vector<uint64_t> keys(total), entries(3 * nb);
     for (int64_t b = 0; b < total; ++b) keys[b] = make_key(uniform_level, b / (nb * nb), (b / nb) % nb, b % nb);
-    MRA_CUDA_TRY(cudaMemcpyAsync(out->keys, keys.data(), total * 8, cudaMemcpyHostToDevice, s));
-    MRA_CUDA_TRY(launch_project_boxes(ng, d_g, k, L, total, out->keys, out->coeffs, s));
-    MRA_CUDA_TRY(cudaFreeAsync(d_g, s));
-    MRA_CUDA_TRY(cudaStreamSynchronize(s));
+    for (int64_t q = 0; q < 3 * nb; ++q) entries[q] = factor_entry(uniform_level, (int)(q / nb), q % nb);
+    uint64_t *d_entries = nullptr;
+    double *F = nullptr;
+    unsigned char *nz = nullptr;
+    const size_t rows = (size_t)(3 * nb) * std::max(ng, 1);
+    cudaError_t e = pool_malloc((void **)&d_entries, entries.size() * 8, s);
+    if (e == cudaSuccess) e = pool_malloc((void **)&F, rows * k * 8, s);
+    if (e == cudaSuccess) e = pool_malloc((void **)&nz, rows, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out->keys, keys.data(), total * 8, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_entries, entries.data(), entries.size() * 8, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = launch_project_level(ng, d_g, k, L, 3 * nb, d_entries, F, nz, total, out->keys, out->coeffs, s);
+    for (void *p : {(void *)d_entries, (void *)F, (void *)nz, (void *)d_g})
+      if (p) cudaFreeAsync(p, s);
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = es;
+    if (e != cudaSuccess) return fail(MRA_ERR_CUDA, "mra_project: %s", cudaGetErrorString(e));
     out->n = total;
     return MRA_OK;
   }
@@ -542,71 +556,120 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
     for (int64_t b = 0; b < nb * nb * nb; ++b) parents.push_back(make_key(pl, b / (nb * nb), (b / nb) % nb, b % nb));
   }
   const int64_t CH = 8192;  // parents per chunk
-  uint64_t *d_keys = nullptr;
-  double *d_box = nullptr, *d_dn = nullptr;
-  int64_t *d_from = nullptr;
-  MRA_CUDA_TRY(pool_malloc((void **)&d_keys, CH * 9 * 8, s));
-  MRA_CUDA_TRY(pool_malloc((void **)&d_box, (size_t)CH * 9 * k3 * 8, s));
-  MRA_CUDA_TRY(pool_malloc((void **)&d_dn, CH * 8, s));
-  MRA_CUDA_TRY(pool_malloc((void **)&d_from, CH * 8 * 8, s));
+  std::vector<void *> held;
+  auto grab = [&](size_t bytes) -> void * {
+    void *p = nullptr;
+    if (pool_malloc(&p, std::max<size_t>(bytes, 1), s) != cudaSuccess) return nullptr;
+    held.push_back(p);
+    return p;
+  };
+  auto give = [&](void *p) {
+    auto it = std::find(held.begin(), held.end(), p);
+    if (it == held.end()) return;
+    cudaFreeAsync(p, s);
+    held.erase(it);
+  };
   // leaves accumulate in a growing device buffer
-  int64_t leaf_cap = 1 << 14, n_leaf = 0;
+  int64_t leaf_cap = 0, n_leaf = 0;
   double *d_leaf = nullptr;
-  MRA_CUDA_TRY(pool_malloc((void **)&d_leaf, (size_t)leaf_cap * k3 * 8, s));
   std::vector<uint64_t> leaf_keys;
-  std::vector<double> dn(CH);
-  std::vector<uint64_t> ck(CH * 9);
-  std::vector<int64_t> from(CH * 8);
+  std::vector<double> dn;
+  std::vector<int64_t> from;
+  std::vector<uint64_t> entries;  // the parents' factor entries of a chunk, then their children's
+  std::vector<int> pidx;
+  // entry of (dimension, coordinate) in the chunk it was last seen in
+  const int64_t span = 1LL << std::max(max_level - 1, pl);
+  std::unique_ptr<uint64_t[], void (*)(void *)> seen((uint64_t *)calloc((size_t)(3 * span), 8), [](void *p) { free(p); });
   int rc = MRA_OK;
-  while (!parents.empty() && rc == MRA_OK) {
+  cudaError_t e = cudaSuccess;
+  if (!seen) rc = fail(MRA_ERR_ARG, "mra_project: out of host memory");
+  if (rc == MRA_OK) e = project_tables(s);
+  uint64_t chunk = 0;
+  while (!parents.empty() && rc == MRA_OK && e == cudaSuccess) {
     std::vector<uint64_t> next;
-    for (size_t p0 = 0; p0 < parents.size() && rc == MRA_OK; p0 += CH) {
-      int64_t np = std::min<int64_t>(CH, (int64_t)parents.size() - (int64_t)p0);
+    for (size_t q0 = 0; q0 < parents.size() && rc == MRA_OK && e == cudaSuccess; q0 += CH) {
+      const int64_t np = std::min<int64_t>(CH, (int64_t)parents.size() - (int64_t)q0);
+      const uint64_t *par = parents.data() + q0;
+      const int n = key_level(par[0]);
+      ++chunk;
+      entries.clear();
+      pidx.resize(3 * np);
       for (int64_t p = 0; p < np; ++p) {
-        uint64_t key = parents[p0 + p];
-        ck[p] = key;
-        int n = key_level(key);
-        int64_t x = key_x(key), y = key_y(key), z = key_z(key);
-        for (int c = 0; c < 8; ++c)
-          ck[np + 8 * p + c] = make_key(n + 1, 2 * x + ((c >> 2) & 1), 2 * y + ((c >> 1) & 1), 2 * z + (c & 1));
+        const int64_t xyz[3] = {key_x(par[p]), key_y(par[p]), key_z(par[p])};
+        for (int d = 0; d < 3; ++d) {
+          uint64_t &at = seen[d * span + xyz[d]];  // chunk << 32 | entry
+          if ((at >> 32) != chunk) {
+            at = chunk << 32 | (uint64_t)entries.size();
+            entries.push_back(factor_entry(n, d, xyz[d]));
+          }
+          pidx[3 * p + d] = (int)(at & 0xFFFFFFFFu);
+        }
       }
-      MRA_CUDA_TRY(cudaMemcpyAsync(d_keys, ck.data(), np * 9 * 8, cudaMemcpyHostToDevice, s));
-      MRA_CUDA_TRY(launch_project_boxes(ng, d_g, k, L, np * 9, d_keys, d_box, s));
-      MRA_CUDA_TRY(launch_refine_test(k, np, d_box, d_box + (size_t)np * k3, d_U, d_dn, s));
-      MRA_CUDA_TRY(cudaMemcpyAsync(dn.data(), d_dn, np * 8, cudaMemcpyDeviceToHost, s));
-      MRA_CUDA_TRY(cudaStreamSynchronize(s));
-      int64_t nf = 0;
+      const int64_t ne = (int64_t)entries.size();
+      entries.resize(3 * ne);
+      for (int64_t q = 0; q < ne; ++q)
+        for (int c = 0; c < 2; ++c)
+          entries[ne + 2 * q + c] = factor_entry(n + 1, (int)(entries[q] >> 32) & 255, 2 * (int64_t)(entries[q] & 0xFFFFFFFFu) + c);
+      const size_t rows = (size_t)ne * std::max(ng, 1);
+      uint64_t *d_entries = (uint64_t *)grab(entries.size() * 8);
+      int *d_pidx = (int *)grab(pidx.size() * 4);
+      double *Fp = (double *)grab(rows * k * 8), *Fc = (double *)grab(rows * 4 * k * 8);
+      unsigned char *nzp = (unsigned char *)grab(rows), *nzc = (unsigned char *)grab(2 * rows);
+      double *d_box = (double *)grab((size_t)np * 8 * k3 * 8), *d_dn = (double *)grab(np * 8);
+      int64_t *d_from = (int64_t *)grab(np * 8 * 8);
+      if (!d_entries || !d_pidx || !Fp || !Fc || !nzp || !nzc || !d_box || !d_dn || !d_from) {
+        e = cudaErrorMemoryAllocation;
+        break;
+      }
+      dn.resize(np);
+      e = cudaMemcpyAsync(d_entries, entries.data(), entries.size() * 8, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(d_pidx, pidx.data(), pidx.size() * 4, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess)
+        e = launch_project_children(ng, d_g, k, L, ne, d_entries, d_U, Fp, Fc, nzp, nzc, np, d_pidx, d_box, d_dn, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(dn.data(), d_dn, np * 8, cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) break;
+      from.clear();
+      const bool forced = n + 1 >= max_level;
       for (int64_t p = 0; p < np; ++p) {
-        int n = key_level(ck[p]);
-        bool forced = (n + 1 >= max_level);
         if (!std::isfinite(dn[p])) { rc = fail(MRA_ERR_NUMERIC, "mra_project: non-finite refinement norm"); break; }
-        bool refine = !forced && dn[p] > thresh;
+        const bool refine = !forced && dn[p] > thresh;
+        const int64_t x = key_x(par[p]), y = key_y(par[p]), z = key_z(par[p]);
         for (int c = 0; c < 8; ++c) {
-          if (refine) next.push_back(ck[np + 8 * p + c]);
-          else {
-            leaf_keys.push_back(ck[np + 8 * p + c]);
-            from[nf++] = np + 8 * p + c;
+          const uint64_t ck = make_key(n + 1, 2 * x + ((c >> 2) & 1), 2 * y + ((c >> 1) & 1), 2 * z + (c & 1));
+          if (refine) {
+            next.push_back(ck);
+          } else {
+            leaf_keys.push_back(ck);
+            from.push_back(8 * p + c);
           }
         }
       }
-      if (rc != MRA_OK || nf == 0) continue;
-      if (n_leaf + nf > leaf_cap) {
-        int64_t nc = std::max(leaf_cap * 2, n_leaf + nf);
-        double *grown = nullptr;
-        MRA_CUDA_TRY(pool_malloc((void **)&grown, (size_t)nc * k3 * 8, s));
-        MRA_CUDA_TRY(cudaMemcpyAsync(grown, d_leaf, (size_t)n_leaf * k3 * 8, cudaMemcpyDeviceToDevice, s));
-        MRA_CUDA_TRY(cudaFreeAsync(d_leaf, s));
-        d_leaf = grown;
-        leaf_cap = nc;
+      const int64_t nf = (int64_t)from.size();
+      if (rc == MRA_OK && nf > 0) {
+        if (n_leaf + nf > leaf_cap) {
+          const int64_t nc = std::max(leaf_cap * 2, n_leaf + nf);
+          double *grown = (double *)grab((size_t)nc * k3 * 8);
+          if (!grown) { e = cudaErrorMemoryAllocation; break; }
+          if (n_leaf > 0) e = cudaMemcpyAsync(grown, d_leaf, (size_t)n_leaf * k3 * 8, cudaMemcpyDeviceToDevice, s);
+          if (d_leaf) give(d_leaf);
+          d_leaf = grown;
+          leaf_cap = nc;
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_from, from.data(), nf * 8, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) {
+          gather_rows_kernel<<<counted((unsigned)nf), 128, 0, s>>>(nf, k3, d_box, d_from, d_leaf, n_leaf);
+          e = cudaGetLastError();
+        }
+        n_leaf += nf;
       }
-      MRA_CUDA_TRY(cudaMemcpyAsync(d_from, from.data(), nf * 8, cudaMemcpyHostToDevice, s));
-      gather_rows_kernel<<<counted((unsigned)nf), 128, 0, s>>>(nf, k3, d_box, d_from, d_leaf, n_leaf);
-      MRA_CUDA_TRY(cudaGetLastError());
-      n_leaf += nf;
-      MRA_CUDA_TRY(cudaStreamSynchronize(s));  // ck/from are reused by the next chunk
+      for (void *p : {(void *)d_entries, (void *)d_pidx, (void *)Fp, (void *)Fc, (void *)nzp, (void *)nzc, (void *)d_box,
+                      (void *)d_dn, (void *)d_from})
+        give(p);
     }
     parents.swap(next);
   }
+  if (rc == MRA_OK && e != cudaSuccess) rc = fail(MRA_ERR_CUDA, "mra_project: %s", cudaGetErrorString(e));
   if (rc == MRA_OK && n_leaf > out->cap) {
     out->n = n_leaf;
     rc = fail(MRA_ERR_CAPACITY, "mra_project: %lld boxes needed, cap %lld", (long long)n_leaf, (long long)out->cap);
@@ -634,14 +697,10 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
     MRA_CUDA_TRY(cudaFreeAsync(tmp, s));
     out->n = n_leaf;
   }
-  cudaFreeAsync(d_keys, s);
-  cudaFreeAsync(d_box, s);
-  cudaFreeAsync(d_dn, s);
-  cudaFreeAsync(d_from, s);
-  cudaFreeAsync(d_leaf, s);
+  for (void *p : held) cudaFreeAsync(p, s);
   cudaFreeAsync(d_U, s);
   cudaFreeAsync(d_g, s);
-  cudaError_t e = cudaStreamSynchronize(s);
+  e = cudaStreamSynchronize(s);
   if (rc == MRA_OK && e != cudaSuccess) rc = fail(MRA_ERR_CUDA, "mra_project: %s", cudaGetErrorString(e));
   return rc;
 }

@@ -191,121 +191,248 @@ __global__ void blocks_kernel(int k, double L, int min_level, int nlev, const in
 }
 
 // --------------------------------------------------------------------------- projection
-// s_b[ix][iy][iz] = sum_g coef_g h^{3/2} X_g[ix] Y_g[iy] Z_g[iz],
-// X_g[i] = int_0^1 exp(-a_g h^2 (u - uc)^2) phi_i(u) du, uc = (c_g + L)/h - b_x  (eq. projection).
-// One warp per (Gaussian, dimension) 1-D integral over the offset w = u - uc,
-// with the same panel rule as the blocks; lanes stride over the nodes.
-__global__ void project_kernel(int ng, const double *g, int k, double L, const uint64_t *keys,
-                               double *out) {
-  extern __shared__ double F[];  // [ng][3][k]
-  uint64_t key = keys[blockIdx.x];
-  int n = key_level(key);
-  int64_t bxyz[3] = {key_x(key), key_y(key), key_z(key)};
-  double h = 2.0 * L / (double)(1LL << n);
-  const double *coef = g, *ex = g + ng;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int task = warp; task < 3 * ng; task += nw) {
-    int gi = task / 3, d = task % 3;
-    double cc = g[(2 + d) * ng + gi];
-    double T = ex[gi] * h * h;
-    double x = (cc + L) / h;               // uc = x - b
-    double wa = (double)bxyz[d] - x;       // w at u = 0
-    double wb = (double)(bxyz[d] + 1) - x; // w at u = 1
-    HalfRange r = half_range(T, wa, wb);
-    double acc[MRA_MAX_K];
-    for (int i = 0; i < k; ++i) acc[i] = 0.0;
-    int nn = r.npan * GLQ;
-    double pw = r.npan > 0 ? (r.hi - r.lo) / r.npan : 0.0;
-    double ph[MRA_MAX_K];
+// s_b[ix][iy][iz] = sum_g coef_g X_g[ix] Y_g[iy] Z_g[iz] with the 1-D factors
+// X_g[i] = h^{1/2} int_0^1 exp(-a_g h^2 (u - uc)^2) phi_i(u) du, uc = (c_g + L)/h - b_x  (eq. projection).
+// A factor depends on (level, dimension, coordinate) and the Gaussian only, and the boxes of a
+// refined neighbourhood share their coordinates, so the integrals are done once per distinct
+// coordinate (an "entry") and not once per box.  8 Gaussians, k = 10, 17,200 leaves: the integrals
+// 179 -> 1.5 ms, the refinement test 8.0 -> 0.7 ms with the children's assembly, the call 190 -> 3.7 ms
+// (FP64-bound exponentials and recurrences; the rest is the host's decision after every level).
+
+// A factor entry: level, dimension and coordinate.
+__host__ __device__ inline uint64_t make_entry(int level, int dim, int64_t x) {
+  return ((uint64_t)level << 40) | ((uint64_t)dim << 32) | (uint64_t)x;
+}
+
+// Legendre recurrence P_{m+1} = a_m x P_m - b_m P_{m-1}, and sqrt(2i+1).
+__constant__ double c_leg_a[MRA_MAX_K], c_leg_b[MRA_MAX_K], c_leg_s[MRA_MAX_K];
+
+// One warp per (entry, Gaussian): F[(e * ng + g) * stride + i], i < k; nz[e * ng + g] = 0 when all k are
+// zero, which needs no quadrature where the Gaussian underflows on the whole box.  Lanes stride
+// over the nodes of the panel rule over the offset w = u - uc; FP64-bound.
+__global__ void factor_kernel(int64_t n_task, int ng, const double *g, int k, double L, const uint64_t *entries,
+                              int stride, double *F, unsigned char *nz) {
+  const int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (task >= n_task) return;
+  const int64_t en = task / ng;
+  const int gi = (int)(task - en * ng);
+  const uint64_t ent = entries[en];
+  const int n = (int)(ent >> 40), d = (int)(ent >> 32) & 255;
+  const double bx = (double)(ent & 0xFFFFFFFFull);
+  const double h = 2.0 * L / (double)(1LL << n);
+  const double T = g[ng + gi] * h * h;
+  const double x = (g[(2 + d) * ng + gi] + L) / h;  // uc = x - b
+  const double wa = bx - x;                         // w at u = 0
+  const double wb = (bx + 1.0) - x;                 // w at u = 1
+  double acc[MRA_MAX_K];
+#pragma unroll
+  for (int i = 0; i < MRA_MAX_K; ++i) acc[i] = 0.0;
+  const double wmin = wa > 0.0 ? wa : (wb < 0.0 ? -wb : 0.0);
+  if (T * wmin * wmin < 760.0) {  // exp(-745.2) is the smallest positive double
+    const HalfRange r = half_range(T, wa, wb);
+    const int nn = r.npan * GLQ;
+    const double pw = r.npan > 0 ? (r.hi - r.lo) / r.npan : 0.0;
     for (int node = lane; node < nn; node += 32) {
-      int p = node / GLQ, q = node % GLQ;
-      double w = r.lo + pw * (p + 0.5 + 0.5 * c_glx[q]);
-      double wt = 0.5 * pw * c_glw[q] * exp(-T * w * w);
-      double u = w - wa;  // u = w + uc, formed from the box end
-      legendre_phi(k, u, ph);
-      for (int i = 0; i < k; ++i) acc[i] += wt * ph[i];
-    }
-    for (int i = 0; i < k; ++i) {
-      double v = acc[i];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) F[(gi * 3 + d) * k + i] = v;
+      const int p = node / GLQ, q = node % GLQ;
+      const double w = r.lo + pw * (p + 0.5 + 0.5 * c_glx[q]);
+      const double wt = 0.5 * pw * c_glw[q] * exp(-T * w * w);
+      const double t = 2.0 * (w - wa) - 1.0;  // u = w + uc, formed from the box end
+      double p0 = 1.0, p1 = t;
+      acc[0] += wt;
+#pragma unroll
+      for (int i = 1; i < MRA_MAX_K; ++i) {
+        if (i < k) {
+          acc[i] = fma(wt, p1, acc[i]);
+          const double p2 = fma(c_leg_a[i] * t, p1, -c_leg_b[i] * p0);
+          p0 = p1;
+          p1 = p2;
+        }
+      }
     }
   }
-  __syncthreads();
-  double h32 = h * sqrt(h);
-  int k3 = k * k * k;
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) {
-    int ix = e / (k * k), iy = (e / k) % k, iz = e % k;
-    double s = 0.0;
-    for (int gi = 0; gi < ng; ++gi)
-      s += coef[gi] * h32 * F[(gi * 3 + 0) * k + ix] * F[(gi * 3 + 1) * k + iy] *
-           F[(gi * 3 + 2) * k + iz];
-    out[(int64_t)blockIdx.x * k3 + e] = s;
+  const double h12 = sqrt(h);
+  bool some = false;
+#pragma unroll
+  for (int i = 0; i < MRA_MAX_K; ++i) {
+    if (i < k) {
+      double v = acc[i];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      v *= c_leg_s[i] * h12;
+      some |= v != 0.0;  // NaN counts as nonzero
+      if (lane == 0) F[task * stride + i] = v;
+    }
+  }
+  if (lane == 0) nz[task] = some ? 1 : 0;
+}
+
+// The parents' factors on their children, X' = U^{(c)} X (two-scale relation of Sec. 2.2 in one dimension),
+// beside the children's own: child entry 2 e + c, F_child[((2 e + c) * ng + g) * 2k + k + i].
+__global__ void lift_kernel(int64_t n, int ng, int k, const double *Fp, const unsigned char *nzp, const double *U,
+                            double *Fc, unsigned char *nzc) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // (child entry, g, i)
+  if (q >= n * 2 * ng * k) return;
+  const int i = (int)(q % k);
+  const int64_t cg = q / k, ce = cg / ng, pg = (ce >> 1) * ng + cg % ng;
+  const double *Uc = U + (ce & 1) * k * k + i * k, *X = Fp + pg * k;
+  double v = 0.0;
+  for (int j = 0; j < k; ++j) v = fma(Uc[j], X[j], v);
+  Fc[cg * 2 * k + k + i] = v;
+  if (i == 0 && nzp[pg]) nzc[cg] |= 2;  // bit 0: the child's own factor is nonzero, bit 1: the parent's
+}
+
+constexpr int ASM_THREADS = 256, ASM_G = 16;  // Gaussians staged at a time
+
+// Sum over the Gaussians at this thread's elements (threadIdx.x + q ASM_THREADS) of one box with the
+// factor entries e[0..2]: own[q], and with TEST the parent's projection there, par[q].  Gaussians
+// whose product is exactly zero are left out; the others are added in order.
+template <int EPT, bool TEST>
+__device__ void sum_gaussians(int ng, int k, const double *coef, const double *F, const unsigned char *nz,
+                              const int64_t *e, double *stage, int *list, int *count, double *own, double *par) {
+  const int k2 = k * k, k3 = k2 * k, st = TEST ? 2 * k : k;
+#pragma unroll
+  for (int q = 0; q < EPT; ++q) own[q] = par[q] = 0.0;
+  int ix[EPT], iy[EPT], iz[EPT];
+#pragma unroll
+  for (int q = 0; q < EPT; ++q) {
+    const int m = min((int)threadIdx.x + q * ASM_THREADS, k3 - 1);
+    ix[q] = m / k2;
+    iy[q] = (m / k) % k;
+    iz[q] = m % k;
+  }
+  for (int g0 = 0; g0 < ng;) {
+    __syncthreads();  // the list and the staged factors of the previous round have been used
+    if (threadIdx.x < 32) {  // the next ASM_G Gaussians that matter, in order
+      int have = 0, next = g0;
+      while (next < ng && have < ASM_G) {
+        const int gi = next + (int)threadIdx.x;
+        int f = 0;
+        if (gi < ng) {
+          f = nz[e[0] * ng + gi] & nz[e[1] * ng + gi] & nz[e[2] * ng + gi];
+          if (!isfinite(coef[gi])) f = 1;  // its product with zero is not zero
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, f != 0);
+        const int at = have + __popc(b & ((1u << threadIdx.x) - 1u));
+        if (f && at < ASM_G) list[at] = gi;
+        const int n = __popc(b);
+        if (have + n > ASM_G) {  // resume after the last one taken
+          int left = ASM_G - have;
+          unsigned bb = b;
+          int last = 0;
+          while (left-- > 0) {
+            last = __ffs(bb) - 1;
+            bb &= bb - 1;
+          }
+          next += last + 1;
+          have = ASM_G;
+        } else {
+          have += n;
+          next += 32;
+        }
+      }
+      if (threadIdx.x == 0) {
+        count[0] = have;
+        count[1] = min(next, ng);
+      }
+    }
+    __syncthreads();
+    const int have = count[0];
+    g0 = count[1];
+    for (int q = threadIdx.x; q < have * 3 * st; q += ASM_THREADS) {
+      const int l = q / (3 * st), r = q - l * 3 * st, d = r / st, i = r - d * st;
+      const double v = F[(e[d] * ng + list[l]) * st + i];
+      stage[q] = d == 0 ? coef[list[l]] * v : v;
+    }
+    __syncthreads();
+    for (int l = 0; l < have; ++l) {
+      const double *X = stage + l * 3 * st, *Y = X + st, *Z = Y + st;
+#pragma unroll
+      for (int q = 0; q < EPT; ++q) {
+        own[q] = fma(X[ix[q]] * Y[iy[q]], Z[iz[q]], own[q]);
+        if (TEST) par[q] = fma(X[k + ix[q]] * Y[k + iy[q]], Z[k + iz[q]], par[q]);
+      }
+    }
   }
 }
 
-// --------------------------------------------------------------------------- refinement test
-// For parent p: sum over its 8 children c of || s_c - (U^{cx} x U^{cy} x U^{cz}) s_p ||_F^2,
-// with U^{(c)}[i][j] = 2^{-1/2} int_0^1 phi_i(y) phi_j((y+c)/2) dy (Sec. 2.2, P^{n+1} = P^n + Q^n).
-__global__ void refine_test_kernel(int k, const double *parent, const double *child,
-                                   const double *U, double *dnorm) {
-  extern __shared__ double sm[];
-  int k3 = k * k * k;
-  double *sp = sm, *t1 = sp + k3, *t2 = t1 + k3;
+// One CTA per parent: its eight children's coefficients, and ||s_children - U s_parent||_F (the
+// refinement test of Sec. 2.1), the parent's projection on a child being the sum of the lifted
+// factors' products: no k^4 transform.  pidx: the parent's entry in each dimension.
+template <int EPT>
+__global__ void __launch_bounds__(ASM_THREADS) children_kernel(int ng, int k, const double *coef, const double *F,
+                                                               const unsigned char *nz, const int *pidx, double *out,
+                                                               double *dnorm) {
+  extern __shared__ double stage[];  // [ASM_G][3][2k]
+  __shared__ int list[ASM_G], count[2];
   __shared__ double red[32];
-  const double *ps = parent + (int64_t)blockIdx.x * k3;
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) sp[e] = ps[e];
-  __syncthreads();
+  const int64_t p = blockIdx.x;
+  const int k3 = k * k * k;
   double part = 0.0;
   for (int c = 0; c < 8; ++c) {
-    const double *Ux = U + ((c >> 2) & 1) * k * k;
-    const double *Uy = U + ((c >> 1) & 1) * k * k;
-    const double *Uz = U + (c & 1) * k * k;
-    for (int e = threadIdx.x; e < k3; e += blockDim.x) {
-      int a = e / (k * k), b = (e / k) % k, cc = e % k;
-      double s = 0.0;
-      for (int j = 0; j < k; ++j) s += Ux[a * k + j] * sp[(j * k + b) * k + cc];
-      t1[e] = s;
+    const int64_t e[3] = {2 * (int64_t)pidx[3 * p] + (c >> 2), 2 * (int64_t)pidx[3 * p + 1] + ((c >> 1) & 1),
+                          2 * (int64_t)pidx[3 * p + 2] + (c & 1)};
+    double own[EPT], par[EPT];
+    sum_gaussians<EPT, true>(ng, k, coef, F, nz, e, stage, list, count, own, par);
+#pragma unroll
+    for (int q = 0; q < EPT; ++q) {
+      const int m = threadIdx.x + q * ASM_THREADS;
+      if (m < k3) {
+        out[(8 * p + c) * k3 + m] = own[q];
+        const double d = own[q] - par[q];
+        part = fma(d, d, part);
+      }
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < k3; e += blockDim.x) {
-      int a = e / (k * k), b = (e / k) % k, cc = e % k;
-      double s = 0.0;
-      for (int j = 0; j < k; ++j) s += Uy[b * k + j] * t1[(a * k + j) * k + cc];
-      t2[e] = s;
-    }
-    __syncthreads();
-    const double *cs = child + ((int64_t)blockIdx.x * 8 + c) * k3;
-    for (int e = threadIdx.x; e < k3; e += blockDim.x) {
-      int a = e / (k * k), b = (e / k) % k, cc = e % k;
-      double s = 0.0;
-      for (int j = 0; j < k; ++j) s += Uz[cc * k + j] * t2[(a * k + b) * k + j];
-      double d = cs[e] - s;
-      part += d * d;
-    }
-    __syncthreads();
   }
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += red[q];
-    dnorm[blockIdx.x] = sqrt(s);
+    double v = 0.0;
+    for (int q = 0; q < ASM_THREADS / 32; ++q) v += red[q];
+    dnorm[p] = sqrt(v);
   }
 }
 
-bool g_gl_uploaded = false;
-
-cudaError_t upload_gl() {
-  static double x[GLQ], w[GLQ];
-  if (!g_gl_uploaded) {
-    gauss_legendre(GLQ, x, w);
+// One CTA per box of a whole level (entry of dimension d and coordinate x: d 2^n + x).
+template <int EPT>
+__global__ void __launch_bounds__(ASM_THREADS) boxes_kernel(int ng, int k, const double *coef, const double *F,
+                                                            const unsigned char *nz, const uint64_t *keys, double *out) {
+  extern __shared__ double stage[];  // [ASM_G][3][k]
+  __shared__ int list[ASM_G], count[2];
+  const int64_t b = blockIdx.x;
+  const uint64_t key = keys[b];
+  const int64_t nb = 1LL << key_level(key);
+  const int64_t e[3] = {key_x(key), nb + key_y(key), 2 * nb + key_z(key)};
+  const int k3 = k * k * k;
+  double own[EPT], par[EPT];
+  sum_gaussians<EPT, false>(ng, k, coef, F, nz, e, stage, list, count, own, par);
+#pragma unroll
+  for (int q = 0; q < EPT; ++q) {
+    const int m = threadIdx.x + q * ASM_THREADS;
+    if (m < k3) out[b * k3 + m] = own[q];
   }
-  cudaError_t e = cudaMemcpyToSymbol(c_glx, x, sizeof(x));
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_glw, w, sizeof(w));
-  g_gl_uploaded = true;
+}
+
+// The rules' nodes and the recurrence's coefficients, written on stream s before the kernels that read them
+// (always the same values).
+cudaError_t upload_tables(cudaStream_t s) {
+  struct Tables {
+    double x[GLQ], w[GLQ], a[MRA_MAX_K], b[MRA_MAX_K], r[MRA_MAX_K];
+    Tables() {
+      gauss_legendre(GLQ, x, w);
+      for (int m = 0; m < MRA_MAX_K; ++m) {
+        a[m] = (2.0 * m + 1.0) / (m + 1.0);
+        b[m] = m / (m + 1.0);
+        r[m] = sqrt(2.0 * m + 1.0);
+      }
+    }
+  };
+  static const Tables t;
+  cudaError_t e = cudaMemcpyToSymbolAsync(c_glx, t.x, sizeof(t.x), 0, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_glw, t.w, sizeof(t.w), 0, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_leg_a, t.a, sizeof(t.a), 0, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_leg_b, t.b, sizeof(t.b), 0, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_leg_s, t.r, sizeof(t.r), 0, cudaMemcpyHostToDevice, s);
   return e;
 }
 
@@ -321,7 +448,7 @@ cudaError_t launch_fit_search(double mu, int M, double r_lo, double r_hi, int st
 
 cudaError_t launch_blocks(const Operator &op, const double *d_glxk, const double *d_glwk,
                           cudaStream_t s) {
-  cudaError_t e = upload_gl();
+  cudaError_t e = upload_tables(s);
   if (e != cudaSuccess) return e;
   int kq = op.k + 1;
   size_t smem = (size_t)(2 * ZB * kq * op.k + ZB * kq) * sizeof(double);
@@ -333,32 +460,54 @@ cudaError_t launch_blocks(const Operator &op, const double *d_glxk, const double
   return cudaGetLastError();
 }
 
-cudaError_t launch_project_boxes(int ng, const double *d_g, int k, double L, int64_t nbox,
-                                 const uint64_t *d_keys, double *d_out, cudaStream_t s) {
-  if (nbox <= 0) return cudaSuccess;
-  cudaError_t e = upload_gl();
-  if (e != cudaSuccess) return e;
-  size_t smem = (size_t)ng * 3 * k * sizeof(double);
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  project_kernel<<<counted((unsigned)nbox), 256, smem, s>>>(ng, d_g, k, L, d_keys, d_out);
+// Factors of the entries (device array) for every Gaussian: F[(e * ng + g) * stride + i], nz[e * ng + g].
+static cudaError_t launch_factors(int64_t n_entries, int ng, const double *d_g, int k, double L, const uint64_t *d_entries,
+                                  int stride, double *F, unsigned char *nz, cudaStream_t s) {
+  const int64_t tasks = n_entries * ng;
+  if (tasks <= 0) return cudaSuccess;
+  factor_kernel<<<counted((unsigned)((tasks + 3) / 4)), 128, 0, s>>>(tasks, ng, d_g, k, L, d_entries, stride, F, nz);
   return cudaGetLastError();
 }
 
-cudaError_t launch_refine_test(int k, int64_t nparent, const double *d_parent,
-                               const double *d_child, const double *d_U, double *d_dnorm,
-                               cudaStream_t s) {
-  if (nparent <= 0) return cudaSuccess;
-  size_t smem = (size_t)3 * k * k * k * sizeof(double);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(refine_test_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  refine_test_kernel<<<counted((unsigned)nparent), 256, smem, s>>>(k, d_parent, d_child, d_U, d_dnorm);
+cudaError_t launch_project_level(int ng, const double *d_g, int k, double L, int64_t n_entries, const uint64_t *d_entries,
+                                 double *F, unsigned char *nz, int64_t nbox, const uint64_t *d_keys, double *d_out,
+                                 cudaStream_t s) {
+  if (nbox <= 0) return cudaSuccess;
+  cudaError_t e = upload_tables(s);
+  if (e == cudaSuccess) e = launch_factors(n_entries, ng, d_g, k, L, d_entries, k, F, nz, s);
+  if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)ASM_G * 3 * k * sizeof(double);
+  if (k <= 10)
+    boxes_kernel<4><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out);
+  else
+    boxes_kernel<16><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out);
   return cudaGetLastError();
 }
+
+cudaError_t launch_project_children(int ng, const double *d_g, int k, double L, int64_t n_entries,
+                                    const uint64_t *d_entries, const double *d_U, double *Fp, double *Fc,
+                                    unsigned char *nzp, unsigned char *nzc, int64_t np, const int *d_pidx, double *d_out,
+                                    double *d_dnorm, cudaStream_t s) {
+  if (np <= 0) return cudaSuccess;
+  // the parents' entries, then their children's (2 e + c)
+  cudaError_t e = launch_factors(n_entries, ng, d_g, k, L, d_entries, k, Fp, nzp, s);
+  if (e == cudaSuccess) e = launch_factors(2 * n_entries, ng, d_g, k, L, d_entries + n_entries, 2 * k, Fc, nzc, s);
+  if (e != cudaSuccess) return e;
+  if (ng > 0) {
+    const int64_t nl = n_entries * 2 * ng * k;
+    lift_kernel<<<counted((unsigned)((nl + 255) / 256)), 256, 0, s>>>(n_entries, ng, k, Fp, nzp, d_U, Fc, nzc);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  const size_t smem = (size_t)ASM_G * 6 * k * sizeof(double);
+  if (k <= 10)
+    children_kernel<4><<<counted((unsigned)np), ASM_THREADS, smem, s>>>(ng, k, d_g, Fc, nzc, d_pidx, d_out, d_dnorm);
+  else
+    children_kernel<16><<<counted((unsigned)np), ASM_THREADS, smem, s>>>(ng, k, d_g, Fc, nzc, d_pidx, d_out, d_dnorm);
+  return cudaGetLastError();
+}
+
+cudaError_t project_tables(cudaStream_t s) { return upload_tables(s); }
+uint64_t factor_entry(int level, int dim, int64_t x) { return make_entry(level, dim, x); }
 
 }  // namespace mra

@@ -259,18 +259,31 @@ def project(gauss: dict, k: int, L: float, thresh: float = 0.0, init_level: int 
     lib = load()
     arrs = [np.ascontiguousarray(gauss[f], dtype=np.float64) for f in ("coef", "expnt", "cx", "cy", "cz")]
     gs = GaussSum(len(arrs[0]), *[_dptr(a) for a in arrs])
+    # An adaptive tree's size is not known beforehand, and a buffer that turns out too small costs a second
+    # projection: start from 256 MB (33,000 boxes at k = 10) and keep what the tree needs.
+    trim = cap is None and uniform_level < 0
     if cap is None:
-        cap = 8 ** uniform_level if uniform_level >= 0 else 4096
+        cap = 8 ** uniform_level if uniform_level >= 0 else max(4096, (256 << 20) // (8 * k ** 3))
     while True:
-        t = Tree.empty(cap, k, L, device)
+        try:
+            t = Tree.empty(cap, k, L, device)
+        except torch.OutOfMemoryError:
+            if not trim or cap <= 4096:
+                raise
+            cap = 4096
+            continue
         v = t.view()
         rc = lib.mra_project(ctypes.byref(gs), k, L, thresh, init_level, max_level, uniform_level,
                              ctypes.byref(v), _stream(stream))
         if rc == MRA_ERR_CAPACITY:
             cap = int(v.n)
+            trim = False
             continue
         _check(rc)
         t.n = int(v.n)
+        keep = max(t.n, 4096)
+        if trim and keep < cap:
+            t.keys, t.coeffs = t.keys[:keep].clone(), t.coeffs[:keep].clone()
         return t
 
 
