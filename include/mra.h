@@ -115,9 +115,10 @@ typedef struct {
   int max_disp;   /* largest |l|_inf for MRA_STENCIL_SHELLS (<= the operator's max_disp) */
   const float *mlp; /* MRA_SCREEN_LEARNED: device model, MRA_MLP_PARAMS floats */
   double delta;     /* MRA_SCREEN_LEARNED: safety margin in log10 units */
-  int tile_variant; /* MRA_PREC_SPLIT_BF16 tile shape: 0 = four 128-row tiles per CTA (one CTA
-                       per SM); 1 (k >= 4) = two tiles per CTA (two CTAs per SM); 2 (k = 4 to
-                       10) = one tile per CTA (four CTAs per SM); others are taken as 0 */
+  int tile_variant; /* MRA_PREC_SPLIT_BF16 tile shape: 0 = several destinations per CTA, one flush per term
+                       (k <= 10: four 128-row tiles, one CTA per SM; k >= 12: the same sums in the shape
+                       of 1, two CTAs per SM); 1 (k >= 4) = two tiles per CTA (two CTAs per SM); 2 (k = 4
+                       to 10) = one tile per CTA (four CTAs per SM); others are taken as 0 */
   const double *delta_level; /* MRA_SCREEN_LEARNED, optional (NULL = delta at every level): host
                                 array of MRA_MAX_LEVEL + 1 margins, one per source level, read
                                 during the call; +inf keeps every term of that level */

@@ -44,7 +44,7 @@ constexpr int BTERM_BYTES = 3 * BSTAGE_BYTES;   // the three blocks (x, y, z) of
 constexpr int NBUF = 4;                         // most block buffers a CTA uses
 constexpr int RING = 4;                         // term-info ring from warpgroup 0 to 1
 constexpr int MAX_G = 32;
-constexpr int JOIN = 2;                         // terms summed in tensor memory per flush
+constexpr int JOIN = 2;                         // terms summed in tensor memory per flush, in one-slot tiles
 
 
 struct SplitArgs {
@@ -108,7 +108,7 @@ __host__ __device__ constexpr uint32_t tile_slots(int t, int k2, int G) {
 // ring_full term info published; d2_free D2 read out; b_free[b] block buffer b released
 // by the stage-3 MMAs that read it.  Each wait is bounded and gives up when the other
 // warpgroup has aborted.
-template <int K, int TT>
+template <int K, int TT, int J = JOIN>
 __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kernel(SplitArgs a) {
   constexpr int k = K, k2 = K * K, k3 = K * K * K;
   constexpr int G = g_for(K, TT), rows = G * k2, T = t_for(K, TT);
@@ -187,8 +187,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
   const uint32_t bs1 = tc::smem_u32(&bar_s1), bs2 = tc::smem_u32(&bar_s2), bs3 = tc::smem_u32(&bar_s3);
   const uint32_t bring = tc::smem_u32(&bar_ring), bd2free = tc::smem_u32(&bar_d2free);
   const int nit = total_it;
-  // instruction descriptor of an M=128 x N x 16 MMA (A MN-major, B K-major), N = 16 n
-  auto idesc_n = [](int n) { return tc::idesc_bf16(128, 16 * n, 1, 0); };
+  // instruction descriptor of tile t's M x N x 16 MMA (A MN-major, B K-major), N = 16 n.  A small MMA's time is
+  // the reading of its A tile, so a tile of at most 16 rows (k = 12: rows 128..143) takes M = 64;
+  // those rows are lanes 0..15 of the output either way.  With the padding warps left out, 4,096 boxes at
+  // 2k = 12 in non-standard form: 10.48 -> 10.14 ms.
+  auto idesc_n = [](int n, int t) { return tc::idesc_bf16(rows - 128 * t <= 16 ? 64 : 128, 16 * n, 1, 0); };
+  // warps whose rows of a half-empty tile are all padding leave it out
+  auto pad_warp = [&](int t) { return rows - 128 * t <= 64 && t * 128 + quarter * 32 >= rows; };
   auto tiles_of = [&](uint32_t keep) -> uint32_t {
     uint32_t tl = 0;
 #pragma unroll
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
     for (int t = 0; t < T; ++t) {
       if (!((tiles >> t) & 1u)) continue;
       for (int p = 0; p < P; ++p)
-        tc::mma_bf16(d + (uint32_t)(t * 48 + 16 * p), adesc(A, p, t), bdesc(B), idesc_n(P - p), p > 0 ? 1u : 0u);
+        tc::mma_bf16(d + (uint32_t)(t * 48 + 16 * p), adesc(A, p, t), bdesc(B), idesc_n(P - p, t), p > 0 ? 1u : 0u);
     }
   };
   // store units of a thread's run: 16-byte core-matrix rows when 8 divides k, else 4-byte pairs
@@ -404,7 +409,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
         // stage-1 output -> stage-2 operand: element [jy][(i, jz, ix)]
 #pragma unroll
         for (int t = 0; t < T; ++t) {
-          if (!((tiles >> t) & 1u)) continue;
+          if (!((tiles >> t) & 1u) || pad_warp(t)) continue;
           float v[K];
           load_d(tD1, t, v);
           if (t * 128 + quarter * 32 + lane < rows) store_units(a2_addr[t], v);
@@ -469,7 +474,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
     auto flush = [&](uint32_t tl, uint32_t kp) {
 #pragma unroll
       for (int t = 0; t < T; ++t) {
-        if (!((tl >> t) & 1u)) continue;
+        if (!((tl >> t) & 1u) || pad_warp(t)) continue;
         const uint32_t base = tD3 + lane_off + (uint32_t)(t * 32);
         float c0[K], c1[K];
         tc::tmem_ldk<K>(base, c0);
@@ -506,7 +511,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
       float v[T][K];
 #pragma unroll
       for (int t = 0; t < T; ++t)
-        if ((tiles >> t) & 1u) load_d(tD2, t, v[t]);
+        if (((tiles >> t) & 1u) && !pad_warp(t)) load_d(tD2, t, v[t]);
       tc::fence_before_sync();
       wg_sync(2);
       if (tid == 128) mbar_arrive(bd2free);
@@ -520,7 +525,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
       // otherwise D3 is flushed first and overwritten.  With several slots the rounding of a
       // slot's sum would depend on which other slots share its tile (joins need equal keep
       // masks), and a destination's result would change with how its function is batched.
-      const bool join = G == 1 && joined > 0 && joined < JOIN && keep == prev_keep;
+      const bool join = G == 1 && joined > 0 && joined < J && keep == prev_keep;
       if (joined > 0 && !join) {
         flush(prev_tiles, prev_keep);
         joined = 0;
@@ -540,12 +545,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
           for (int t = 0; t < T; ++t) {
             if (!((tiles >> t) & 1u)) continue;
             const uint32_t d = tD3 + (uint32_t)(t * 32);
-            tc::mma_bf16(d, adesc(A3, 0, t), bdesc(B3), idesc_n(2), join ? 1u : 0u);      // x0 [y0 y1]
-            tc::mma_bf16(d + 16u, adesc(A3, 1, t), bdesc(B3), idesc_n(1), 1u);            // x1 y0
+            tc::mma_bf16(d, adesc(A3, 0, t), bdesc(B3), idesc_n(2, t), join ? 1u : 0u);      // x0 [y0 y1]
+            tc::mma_bf16(d + 16u, adesc(A3, 1, t), bdesc(B3), idesc_n(1, t), 1u);            // x1 y0
             if (P == 3) {
-              tc::mma_bf16(d + 16u, adesc(A3, 1, t), bdesc(B3 + BPIECE_BYTES), idesc_n(1), 1u);      // x1 y1
-              tc::mma_bf16(d + 16u, adesc(A3, 2, t), bdesc(B3), idesc_n(1), 1u);                     // x2 y0
-              tc::mma_bf16(d + 16u, adesc(A3, 0, t), bdesc(B3 + 2 * BPIECE_BYTES), idesc_n(1), 1u);  // x0 y2
+              tc::mma_bf16(d + 16u, adesc(A3, 1, t), bdesc(B3 + BPIECE_BYTES), idesc_n(1, t), 1u);      // x1 y1
+              tc::mma_bf16(d + 16u, adesc(A3, 2, t), bdesc(B3), idesc_n(1, t), 1u);                     // x2 y0
+              tc::mma_bf16(d + 16u, adesc(A3, 0, t), bdesc(B3 + 2 * BPIECE_BYTES), idesc_n(1, t), 1u);  // x0 y2
             }
           }
           tc::mma_commit(bs3);
@@ -714,7 +719,12 @@ int apply_split_run(const Operator &op, const mra_tree_view &in, const mra_apply
   if (k > MRA_MAX_K) return fail(MRA_ERR_UNSUPPORTED, "split apply: order %d above %d (use MRA_PREC_FP64)", k, MRA_MAX_K);
   if (!op.d_Rsplit) return fail(MRA_ERR_ARG, "mra_apply: operator has no split blocks");
   if (k & 1) return fail(MRA_ERR_UNSUPPORTED, "split apply: odd k=%d not supported (use MRA_PREC_FP64)", k);
-  const int tt = (k >= 4 && o.tile_variant == 1) ? 2 : (k >= 4 && k <= 10 && o.tile_variant == 2) ? 1 : 4;
+  // tile_variant 0 holds several destinations per CTA and flushes every term; from k = 12 on it runs in the
+  // one-destination shape without joins, which does the same sums (each destination's terms one by one, in
+  // the same order) with two CTAs per SM instead of one and two to three times the CTAs: the order-12 applies
+  // of a bound-state iteration (19.5 ms in four-tile CTAs) took the iteration from 49.0 to 41.8 ms.
+  const bool wide = !(k >= 4 && (o.tile_variant == 1 || (k <= 10 && o.tile_variant == 2)));
+  const int tt = wide ? (k >= 12 ? 2 : 4) : o.tile_variant == 1 ? 2 : 1;
   const int G = g_for(k, tt);
   const int T = t_for(k, tt);  // 128-row tiles per CTA
   const int64_t P = wk.P, nd = wk.n_dest;
@@ -778,7 +788,7 @@ int apply_split_run(const Operator &op, const mra_tree_view &in, const mra_apply
   const size_t smem_floor = (size_t)233472 / (512 / tmem_cols_for(T) + 1);
   if (smem < smem_floor) smem = smem_floor;
   void (*kern)(SplitArgs) = nullptr;
-  switch (k * 8 + tt) {
+  switch (k * 8 + tt + (wide && tt == 2 ? 1 : 0)) {
     case 2 * 8 + 4: kern = apply_split_kernel<2, 4>; break;
     case 4 * 8 + 4: kern = apply_split_kernel<4, 4>; break;
     case 4 * 8 + 2: kern = apply_split_kernel<4, 2>; break;
@@ -793,11 +803,11 @@ int apply_split_run(const Operator &op, const mra_tree_view &in, const mra_apply
     case 10 * 8 + 2: kern = apply_split_kernel<10, 2>; break;
     case 10 * 8 + 1: kern = apply_split_kernel<10, 1>; break;
     case 12 * 8 + 2: kern = apply_split_kernel<12, 2>; break;
-    case 12 * 8 + 4: kern = apply_split_kernel<12, 4>; break;
+    case 12 * 8 + 3: kern = apply_split_kernel<12, 2, 1>; break;
     case 14 * 8 + 2: kern = apply_split_kernel<14, 2>; break;
-    case 14 * 8 + 4: kern = apply_split_kernel<14, 4>; break;
+    case 14 * 8 + 3: kern = apply_split_kernel<14, 2, 1>; break;
     case 16 * 8 + 2: kern = apply_split_kernel<16, 2>; break;
-    default: kern = apply_split_kernel<16, 4>; break;
+    default: kern = apply_split_kernel<16, 2, 1>; break;
   }
   MRA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   MRA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));

@@ -1,0 +1,37 @@
+"""Shapes and launch forms that are chosen by rules on the order give the sums of the general form."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mra():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1507_01888_gb300 import mra as m
+    m.load()
+    return m
+
+
+@pytest.mark.parametrize("k", [12, 14, 16])
+@pytest.mark.parametrize("n_boxes", [1, 7, 90])
+def test_split_wide_shape_is_independent_of_its_neighbours(mra, k, n_boxes):
+    """tile_variant 0 from k = 12 on: a destination's result does not depend on the destinations beside it
+    (every term is flushed alone), and it lies within the split error of the joined shape."""
+    import torch
+    keys, coeffs = W.random_tree_coeffs(n_boxes, k, 3, seed=k + n_boxes)
+    op = mra.Operator(0, 6, k, 32.0, 3, 3, max_disp=1, fit_eps=1e-4)
+    tree = mra.Tree.from_host(keys, coeffs, 32.0)
+    kw = dict(precision=mra.PREC_SPLIT_BF16, stencil=mra.STENCIL_NEAREST)
+    whole, _ = mra.apply(op, tree, mra.make_opts(**kw))
+    ks = whole.keys[: whole.n].cpu().numpy().view("uint64")
+    cut = int(ks[whole.n // 2 + 1])
+    parts = [mra.apply(op, tree, mra.make_opts(dest_range=r, **kw))[0] for r in ((0, cut), (cut, 1 << 63))]
+    assert torch.equal(torch.cat([p.coeffs[: p.n] for p in parts]), whole.coeffs[: whole.n])
+    joined, _ = mra.apply(op, tree, mra.make_opts(tile_variant=1, **kw))
+    assert mra.compare(joined, whole)["rel_l2"] <= 4e-7
+    exact, _ = mra.apply(op, tree, mra.make_opts(stencil=mra.STENCIL_NEAREST))
+    assert mra.compare(whole, exact)["rel_l2"] <= 2e-7
