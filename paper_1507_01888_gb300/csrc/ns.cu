@@ -85,6 +85,19 @@ __global__ void scatter_dense_kernel(int64_t n_rows, const uint64_t *keys, const
   for (int e = threadIdx.x; e < rowlen; e += blockDim.x) dense[d * rowlen + e] = rows[r * rowlen + e];
 }
 
+// The same for rows of several whole levels, n0 first, back to back.
+__global__ void scatter_levels_kernel(int64_t n_rows, const uint64_t *keys, const double *rows, int rowlen, int n0,
+                                      double *dense) {
+  const int64_t r = blockIdx.x;
+  if (r >= n_rows) return;
+  const uint64_t key = keys[r];
+  const int n = key_level(key);
+  const int64_t nb = 1LL << n;
+  int64_t d = (key_x(key) * nb + key_y(key)) * nb + key_z(key);
+  for (int m = n0; m < n; ++m) d += 1LL << (3 * m);
+  for (int e = threadIdx.x; e < rowlen; e += blockDim.x) dense[d * rowlen + e] = rows[r * rowlen + e];
+}
+
 // ---------------------------------------------------------------- two-scale transforms
 // One CTA per box of level n: S = the children (dense level n+1) as a (2k)^3 tensor, written
 // out, and s = (Ubar^T)^{x3} S.  Shared memory: S (2k)^3, a k (2k)^2, b k^2 (2k) doubles.
@@ -263,23 +276,46 @@ __global__ void halo_kernel(int64_t ni, const uint64_t *ikeys, int D, uint64_t *
   out[e] = (x < 0 || x >= nb || y < 0 || y >= nb || z < 0 || z >= nb) ? ~0ull : make_key(n, x, y, z);
 }
 
-// Every node p of R_n: refined when it lies in the sources' halo (every box an unscreened apply
-// of the level would reach); its output rows of the level's two applies, if any.
-// The halo's count *nh is read on the device (its last key may be the largest key, which no
-// node has).
-__global__ void reach_kernel(int64_t nr, const uint64_t *rkeys, const uint64_t *hkeys, const int64_t *nh,
-                             const uint64_t *ykeys, int64_t ny, const uint64_t *zkeys, int64_t nz, int64_t *yi,
-                             int64_t *zi, int *refine, int *leaf) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nr) return;
-  yi[p] = find_sorted(ykeys, ny, rkeys[p]);
-  zi[p] = find_sorted(zkeys, nz, rkeys[p]);
-  const bool in = find_sorted(hkeys, *nh, rkeys[p]) >= 0;
-  refine[p] = in ? 1 : 0;
-  leaf[p] = in ? 0 : 1;
+// Children of the halo boxes (all levels; entry 8 j + c): a child that lies in the next level's halo is
+// refined there (its rank in the whole halo list goes to dst), the others are leaves of the result
+// (their keys to leaf_key, the largest key elsewhere).  *found counts the refined children.
+__global__ void halo_children_kernel(int64_t nh, const uint64_t *hkeys, const int64_t *off, int nmax, int64_t *dst,
+                                     uint64_t *leaf_key, int *id, unsigned long long *found) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  bool in = false;
+  if (e < 8 * nh) {
+    const uint64_t k = hkeys[e >> 3];
+    const int n = key_level(k), c = (int)(e & 7);
+    const uint64_t ck = make_key(n + 1, 2 * key_x(k) + (c >> 2), 2 * key_y(k) + ((c >> 1) & 1), 2 * key_z(k) + (c & 1));
+    int64_t p = -1;
+    if (n + 1 < nmax) p = find_sorted(hkeys + off[n + 1], off[n + 2] - off[n + 1], ck);
+    in = p >= 0;
+    dst[e] = in ? off[n + 1] + p : -1;
+    leaf_key[e] = in ? ~0ull : ck;
+    id[e] = (int)e;
+  }
+  const unsigned b = __ballot_sync(0xffffffffu, in);
+  if ((threadIdx.x & 31) == 0 && b) atomicAdd(found, (unsigned long long)__popc(b));
 }
 
-// Every target row of an apply must be a node of R_n.
+// Leaf i in key order: its place in the output, kept at its child entry as -2 - i, and its key.
+__global__ void leaf_places_kernel(int64_t n_leaf, const uint64_t *sorted, const int *id, int64_t *dst, uint64_t *okeys) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_leaf) return;
+  dst[id[i]] = -2 - i;
+  okeys[i] = sorted[i];
+}
+
+// The output rows of the two applies at every halo box (-1: a screened apply wrote none).
+__global__ void halo_rows_kernel(int64_t nh, const uint64_t *hkeys, const uint64_t *ykeys, int64_t ny,
+                                 const uint64_t *zkeys, int64_t nz, int64_t *yi, int64_t *zi) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= nh) return;
+  yi[j] = find_sorted(ykeys, ny, hkeys[j]);
+  zi[j] = find_sorted(zkeys, nz, hkeys[j]);
+}
+
+// Every target row of an apply must lie in the sources' halo.
 __global__ void targets_in_kernel(int64_t nt, const uint64_t *tkeys, const uint64_t *rkeys, int64_t nr, int *err) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nt) return;
@@ -297,23 +333,21 @@ __global__ void emit_leaves_kernel(int64_t nr, int k3, const uint64_t *rkeys, co
   for (int e = threadIdx.x; e < k3; e += blockDim.x) ocoeffs[o * k3 + e] = r[p * k3 + e];
 }
 
-// One CTA per reached node p: its children get (Ubar)^{x3} (r_p - Z_p) + Y_p (absent rows as
-// zero), written at 8 ref_pos[p] + child in the unsorted level-(n+1) arrays.
-__global__ void sum_down_tree_kernel(int k, int64_t nr, const uint64_t *rkeys, const double *r, const int *refine,
-                                     const int *ref_pos, const int64_t *yi, const double *Y, const int64_t *zi,
-                                     const double *Z, const double *Ub, uint64_t *ckeys, double *cr) {
+// One CTA per halo box of one level (j0 + blockIdx.x): its children get (Ubar)^{x3} (r - Z) + Y (absent rows
+// as zero), written to the next level's r where the child is refined there, else to the result.
+__global__ void sum_down_tree_kernel(int k, int64_t j0, double *r, const int64_t *yi, const double *Y,
+                                     const int64_t *zi, const double *Z, const int64_t *dst, const double *Ub,
+                                     double *out) {
   extern __shared__ double sh[];
-  const int64_t p = blockIdx.x;
-  if (p >= nr || !refine[p]) return;
+  __shared__ double *to[8];
+  const int64_t p = j0 + blockIdx.x;
   const int kk = 2 * k, k2 = k * k, k3 = k2 * k, kk3 = kk * kk * kk;
   double *d = sh, *a = d + k3, *b = a + kk * k2;
-  const int64_t y = yi[p], z = zi[p], base = 8 * (int64_t)ref_pos[p];
+  const int64_t y = yi[p], z = zi[p];
   for (int e = threadIdx.x; e < k3; e += blockDim.x) d[e] = r[p * k3 + e] - (z >= 0 ? Z[z * k3 + e] : 0.0);
-  const uint64_t key = rkeys[p];
   if (threadIdx.x < 8) {
-    const int cx = threadIdx.x >> 2, cy = (threadIdx.x >> 1) & 1, cz = threadIdx.x & 1;
-    ckeys[base + threadIdx.x] =
-        make_key(key_level(key) + 1, 2 * key_x(key) + cx, 2 * key_y(key) + cy, 2 * key_z(key) + cz);
+    const int64_t t = dst[8 * p + threadIdx.x];
+    to[threadIdx.x] = t >= 0 ? r + t * k3 : out + (-2 - t) * k3;
   }
   __syncthreads();
   for (int e = threadIdx.x; e < kk * k2; e += blockDim.x) {
@@ -335,7 +369,7 @@ __global__ void sum_down_tree_kernel(int k, int64_t nr, const uint64_t *rkeys, c
     double v = y >= 0 ? Y[y * kk3 + e] : 0.0;
     for (int l = 0; l < k; ++l) v += Ub[Lq * k + l] * b[(I * kk + J) * k + l];
     const int child = ((I / k) << 2) | ((J / k) << 1) | (Lq / k);
-    cr[(base + child) * k3 + ((I % k) * k + J % k) * k + Lq % k] = v;
+    to[child][((I % k) * k + J % k) * k + Lq % k] = v;
   }
 }
 
@@ -614,12 +648,12 @@ mra_apply_opts coarse_opts(const mra_apply_opts &o, int n0) {
   return c;
 }
 
-// Workspace of mra_apply_ns: dense s^n, S^n (n0 <= n < N), r ping-pong, Y, Z (level N-1
-// sizes), Ubar, an error word, one level's keys, the per-level apply outputs (keys +
-// coefficients of Y and of Z / the coarse r), and the largest per-level apply workspace.
+// Workspace of mra_apply_ns: dense s^n, S^n (n0 <= n < N, back to back), r ping-pong, Y, Z (all
+// levels), Ubar, an error word, the levels' keys, the applies' outputs (keys +
+// coefficients of Y and of Z / the coarse r), and the largest apply's workspace.
 struct NsLayout {
-  std::vector<size_t> s, S;
-  size_t rA, rB, Yd, Zd, Ub, err, keys, yk, yc, zk, zc, apply, total;
+  std::vector<int64_t> first;  // first box of level n among all levels' (n0 <= n <= N)
+  size_t s, S, rA, rB, Yd, Zd, Ub, err, keys, yk, yc, zk, zc, apply, total;
   size_t apply_bytes;
 };
 
@@ -633,15 +667,13 @@ NsLayout ns_layout(const Operator &op, const Operator &ns, int N, int n0, const 
     off = al(off + (bytes ? bytes : 1));
     return at;
   };
-  L.s.assign(N + 1, 0);
-  L.S.assign(N + 1, 0);
-  for (int n = n0; n < N; ++n) {
-    L.s[n] = take(boxes(n) * k3 * 8);
-    L.S[n] = take(boxes(n) * kk3 * 8);
-  }
-  const int64_t nt = boxes(N - 1);
-  L.rA = take(nt * k3 * 8);
-  L.rB = take(nt * k3 * 8);
+  L.first.assign(N + 1, 0);
+  for (int n = n0; n < N; ++n) L.first[n + 1] = L.first[n] + boxes(n);
+  const int64_t nt = L.first[N];
+  L.s = take(nt * k3 * 8);
+  L.S = take(nt * kk3 * 8);
+  L.rA = take(boxes(N - 1) * k3 * 8);
+  L.rB = take(boxes(N - 1) * k3 * 8);
   L.Yd = take(nt * kk3 * 8);
   L.Zd = take(nt * k3 * 8);
   L.Ub = take((size_t)kk * k * 8);
@@ -652,10 +684,8 @@ NsLayout ns_layout(const Operator &op, const Operator &ns, int N, int n0, const 
   L.zk = take(nt * 8);
   L.zc = take(nt * k3 * 8);
   size_t ab = apply_workspace_bytes(op, coarse_opts(o, n0), boxes(n0));
-  for (int n = n0; n < N; ++n) {
-    ab = std::max(ab, apply_workspace_bytes(op, level_opts(o), boxes(n)));
-    ab = std::max(ab, apply_workspace_bytes(ns, level_opts(o), boxes(n)));
-  }
+  ab = std::max(ab, apply_workspace_bytes(op, level_opts(o), nt));
+  ab = std::max(ab, apply_workspace_bytes(ns, level_opts(o), nt));
   L.apply_bytes = ab;
   L.apply = take(ab);
   L.total = off;
@@ -847,10 +877,13 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
   const size_t sh_d = (size_t)(k3 + kk * k * k + kk * kk * k) * 8;
   MRA_CUDA_TRY(cudaFuncSetAttribute(compress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_c));
   MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
+  double *s_all = (double *)(w + Lw.s), *S_all = (double *)(w + Lw.S);
   for (int n = N - 1; n >= n0; --n) {
-    const double *fine = n == N - 1 ? in->coeffs : (const double *)(w + Lw.s[n + 1]);
-    compress_kernel<<<counted((unsigned)boxes(n)), 256, sh_c, s>>>(k, n, fine, Ub, (double *)(w + Lw.S[n]),
-                                                          (double *)(w + Lw.s[n]));
+    const double *fine = n == N - 1 ? in->coeffs : s_all + Lw.first[n + 1] * k3;
+    compress_kernel<<<counted((unsigned)boxes(n)), 256, sh_c, s>>>(k, n, fine, Ub, S_all + Lw.first[n] * kk3,
+                                                                   s_all + Lw.first[n] * k3);
+    MRA_CUDA_TRY(cudaGetLastError());
+    level_keys_kernel<<<counted((unsigned)((boxes(n) + 255) / 256)), 256, 0, s>>>(n, boxes(n), keys + Lw.first[n]);
     MRA_CUDA_TRY(cudaGetLastError());
   }
 
@@ -873,42 +906,47 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
     }
   };
   void *aws = w + Lw.apply;
-  // one apply on every box of level n: its output rows scattered into a zeroed dense array
-  auto level_apply = [&](const Operator &opx, int n, const double *coeffs, const mra_apply_opts &oo,
-                         uint64_t *okeys, double *ocoeffs, double *dense) -> int {
-    const int64_t nbx = boxes(n);
+  // one apply on every box of the levels [a, b); *dense: its rows in the boxes' order, which is its own output
+  // when every box has a row (both are in key order), else scattered into the zeroed array
+  auto levels_apply = [&](const Operator &opx, int a, int b, double *coeffs, const mra_apply_opts &oo,
+                          uint64_t *okeys, double *ocoeffs, double *zeroed, double **dense) -> int {
+    const int64_t nbx = Lw.first[b] - Lw.first[a];
     const int rowlen = opx.k * opx.k * opx.k;
-    level_keys_kernel<<<counted((unsigned)((nbx + 255) / 256)), 256, 0, s>>>(n, nbx, keys);
-    MRA_CUDA_TRY(cudaGetLastError());
-    mra_tree_view vin{nbx, nbx, keys, const_cast<double *>(coeffs), opx.k, opx.L};
+    mra_tree_view vin{nbx, nbx, keys + Lw.first[a], coeffs, opx.k, opx.L};
     mra_tree_view vout{0, nbx, okeys, ocoeffs, opx.k, opx.L};
     mra_apply_stats st{};
     int rc2 = apply_run(opx, vin, oo, vout, aws, Lw.apply_bytes, &st, s);
     if (rc2 != MRA_OK) return rc2;
     add_stats(st);
-    MRA_CUDA_TRY(cudaMemsetAsync(dense, 0, (size_t)nbx * rowlen * 8, s));
+    *dense = ocoeffs;
+    if (vout.n == nbx) return MRA_OK;
+    *dense = zeroed;
+    MRA_CUDA_TRY(cudaMemsetAsync(zeroed, 0, (size_t)nbx * rowlen * 8, s));
     if (vout.n > 0) {
-      scatter_dense_kernel<<<counted((unsigned)vout.n), 128, 0, s>>>(vout.n, okeys, ocoeffs, rowlen, dense);
+      scatter_levels_kernel<<<counted((unsigned)vout.n), 128, 0, s>>>(vout.n, okeys, ocoeffs, rowlen, a, zeroed);
       MRA_CUDA_TRY(cudaGetLastError());
     }
     return MRA_OK;
   };
   uint64_t *yk = (uint64_t *)(w + Lw.yk), *zk = (uint64_t *)(w + Lw.zk);
   double *yc = (double *)(w + Lw.yc), *zc = (double *)(w + Lw.zc);
-  double *Yd = (double *)(w + Lw.Yd), *Zd = (double *)(w + Lw.Zd);
   double *rcur = (double *)(w + Lw.rA), *rnext = (double *)(w + Lw.rB);
 
   // ---- coarsest level: T^{n0} with every displacement
-  rc = level_apply(*op, n0, (const double *)(w + Lw.s[n0]), coarse_opts(*o, n0), zk, zc, rcur);
+  double *r0 = nullptr, *Y = nullptr, *Z = nullptr;
+  rc = levels_apply(*op, n0, n0 + 1, s_all, coarse_opts(*o, n0), zk, zc, (double *)(w + Lw.Zd), &r0);
   if (rc != MRA_OK) return rc;
-  // ---- levels n0 .. N-1
+  MRA_CUDA_TRY(cudaMemcpyAsync(rcur, r0, (size_t)boxes(n0) * k3 * 8, cudaMemcpyDeviceToDevice, s));
+  // ---- levels n0 .. N-1: their applies do not depend on one another, so all levels in one apply each (level by
+  // level the coarse levels left most SMs idle and every apply paid its launches and synchronisations)
+  rc = levels_apply(*ns, n0, N, S_all, level_opts(*o), yk, yc, (double *)(w + Lw.Yd), &Y);
+  if (rc != MRA_OK) return rc;
+  rc = levels_apply(*op, n0, N, s_all, level_opts(*o), zk, zc, (double *)(w + Lw.Zd), &Z);
+  if (rc != MRA_OK) return rc;
   for (int n = n0; n < N; ++n) {
-    rc = level_apply(*ns, n, (const double *)(w + Lw.S[n]), level_opts(*o), yk, yc, Yd);
-    if (rc != MRA_OK) return rc;
-    rc = level_apply(*op, n, (const double *)(w + Lw.s[n]), level_opts(*o), zk, zc, Zd);
-    if (rc != MRA_OK) return rc;
     double *fine = n == N - 1 ? out->coeffs : rnext;
-    sum_down_kernel<<<counted((unsigned)boxes(n)), 256, sh_d, s>>>(k, n, rcur, Zd, Yd, Ub, fine);
+    sum_down_kernel<<<counted((unsigned)boxes(n)), 256, sh_d, s>>>(k, n, rcur, Z + Lw.first[n] * k3, Y + Lw.first[n] * kk3, Ub,
+                                                                   fine);
     MRA_CUDA_TRY(cudaGetLastError());
     std::swap(rcur, rnext);
   }
@@ -933,6 +971,11 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
 // rows of screened applies as zero); the other nodes, and every node of the deepest leaf
 // level, are the result's leaves.  The halo keeps every later level's targets inside the
 // result: a target's parent lies in the previous level's halo.
+// The tree depends on the keys alone and the levels' applies on one another's results not at all, so
+// the structure is made first (two sorts over all levels) and then three applies run: the
+// coarsest level's, and T2k and T over the sources of all levels at once.  Level by level, each
+// with two applies of few boxes, the launches, their synchronisations and the idle SMs took longer than
+// the kernels' work.
 extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns, const mra_tree_view *in, int n0,
                                  const mra_apply_opts *o, mra_tree_view *out, mra_apply_stats *stats, void *stream) {
   const Operator *op = reinterpret_cast<const Operator *>(h);
@@ -1012,7 +1055,7 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
   // ---- interior nodes of every level: the leaves' ancestors, sorted and unique, all levels in
   // one sort (keys order by level first, so each level is one range)
   std::vector<uint64_t *> Ik(Nmax + 1, nullptr);
-  std::vector<int64_t> In(Nmax + 1, 0);
+  std::vector<int64_t> In(Nmax + 1, 0), off_int(21, 0);
   {
     const int nlev = std::max(Nmax - n0, 1);
     if (n_leaf * nlev >= (int64_t)INT32_MAX) return fail(MRA_ERR_ARG, "mra_apply_ns_tree: too many leaves x levels");
@@ -1034,7 +1077,7 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
     MRA_CUDA_TRY(cub::DeviceSelect::Unique(tmp, tt, anc_s, anc, d_nsel, (int)na, s));
     level_offsets_kernel<<<counted(1), 32, 0, s>>>(anc, d_nsel, d_off);
     MRA_CUDA_TRY(cudaGetLastError());
-    std::vector<int64_t> off(21);
+    std::vector<int64_t> &off = off_int;
     MRA_CUDA_TRY(cudaMemcpyAsync(off.data(), d_off, 21 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MRA_CUDA_TRY(cudaStreamSynchronize(s));
     for (int n = n0; n < Nmax; ++n) {
@@ -1046,39 +1089,109 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
   }
   if (In[n0] != boxes(n0)) return fail(MRA_ERR_ARG, "mra_apply_ns_tree: level %d is not complete", n0);
 
-  // ---- compress, from the deepest interior level up
+  const int64_t n_int = off_int[Nmax] - off_int[n0];
+
+  // ---- the halo of every level's sources, sorted and unique, all levels in one sort: the boxes that are
+  // refined.  It fixes the whole result tree: the children of the halo boxes are the next level's halo
+  // boxes and the result's leaves, so every size and place is known before any apply runs.
+  const int64_t w3 = (int64_t)(2 * D + 1) * (2 * D + 1) * (2 * D + 1);
+  const int64_t nh_all = n_int * w3;
+  std::vector<int64_t> hoff(21, 0);
+  NS_ALLOC(d_hoff, int64_t, 21);
+  uint64_t *hk = nullptr;
+  {
+    NS_ALLOC(hal, uint64_t, nh_all);
+    NS_ALLOC(hal_s, uint64_t, nh_all);
+    NS_ALLOC(d_nh, int64_t, 1);
+    size_t t1 = 0, t2 = 0;
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, t1, hal, hal_s, nh_all, 0, 64, s));
+    MRA_CUDA_TRY(cub::DeviceSelect::Unique(nullptr, t2, hal_s, hal, d_nh, nh_all, s));
+    const size_t tb = std::max(t1, t2);
+    NS_ALLOC(tmph, unsigned char, tb);
+    halo_kernel<<<counted((unsigned)((nh_all + 255) / 256)), 256, 0, s>>>(n_int, Ik[n0], D, hal);
+    MRA_CUDA_TRY(cudaGetLastError());
+    size_t tt = tb;
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(tmph, tt, hal, hal_s, nh_all, 0, 64, s));
+    tt = tb;
+    MRA_CUDA_TRY(cub::DeviceSelect::Unique(tmph, tt, hal_s, hal, d_nh, nh_all, s));
+    level_offsets_kernel<<<counted(1), 32, 0, s>>>(hal, d_nh, d_hoff);
+    MRA_CUDA_TRY(cudaGetLastError());
+    MRA_CUDA_TRY(cudaMemcpyAsync(hoff.data(), d_hoff, 21 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    MRA_CUDA_TRY(cudaStreamSynchronize(s));
+    drop(hal_s);
+    drop(tmph);
+    hk = hal;
+  }
+  const int64_t nh = hoff[Nmax];  // halo boxes, levels n0 .. Nmax-1
+  if (hoff[n0 + 1] - hoff[n0] != boxes(n0))
+    return fail(MRA_ERR_NUMERIC, "mra_apply_ns_tree: the halo of level %d is not the whole level", n0);
+  if (8 * nh >= (int64_t)INT32_MAX) return fail(MRA_ERR_ARG, "mra_apply_ns_tree: too many result boxes");
+  const int64_t nout = 8 * nh - (nh - boxes(n0));
+  mra_apply_stats acc{};
+  acc.n_in = n_leaf;
+  acc.n_out = nout;
+  if (nout > out->cap) {
+    out->L = op->L;
+    out->n = nout;
+    if (stats) *stats = acc;
+    return fail(MRA_ERR_CAPACITY, "mra_apply_ns_tree: %lld result leaves, capacity %lld", (long long)nout,
+                (long long)out->cap);
+  }
+  NS_ALLOC(dst, int64_t, 8 * nh);
+  {
+    NS_ALLOC(lk, uint64_t, 8 * nh);
+    NS_ALLOC(lks, uint64_t, 8 * nh);
+    NS_ALLOC(id, int, 8 * nh);
+    NS_ALLOC(ids, int, 8 * nh);
+    size_t tb = 0;
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, lk, lks, id, ids, (int)(8 * nh), 0, 64, s));
+    NS_ALLOC(tmp, unsigned char, tb);
+    NS_ALLOC(found, unsigned long long, 1);
+    MRA_CUDA_TRY(cudaMemsetAsync(found, 0, 8, s));
+    halo_children_kernel<<<counted((unsigned)((8 * nh + 255) / 256)), 256, 0, s>>>(nh, hk, d_hoff, Nmax, dst, lk, id, found);
+    MRA_CUDA_TRY(cudaGetLastError());
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp, tb, lk, lks, id, ids, (int)(8 * nh), 0, 64, s));
+    unsigned long long hfound = 0;
+    MRA_CUDA_TRY(cudaMemcpyAsync(&hfound, found, 8, cudaMemcpyDeviceToHost, s));
+    MRA_CUDA_TRY(cudaStreamSynchronize(s));
+    if ((int64_t)hfound != nh - boxes(n0))  // every halo box is a child of one of the level above
+      return fail(MRA_ERR_NUMERIC, "mra_apply_ns_tree: a halo box lies outside the result tree");
+    leaf_places_kernel<<<counted((unsigned)((nout + 255) / 256)), 256, 0, s>>>(nout, lks, ids, dst, out->keys);
+    MRA_CUDA_TRY(cudaGetLastError());
+    for (void *p : {(void *)lk, (void *)lks, (void *)id, (void *)ids, (void *)tmp, (void *)found}) drop(p);
+  }
+
+  // ---- compress, from the deepest interior level up; all levels' S and s back to back in key order
   const size_t sh_c = (size_t)(kk * kk * kk + k * kk * kk + k * k * kk) * 8;
   const size_t sh_d = (size_t)(k3 + kk * k * k + kk * kk * k) * 8;
+  const int kk3 = kk * kk * kk;
   MRA_CUDA_TRY(cudaFuncSetAttribute(compress_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_c));
   MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
-  std::vector<double *> Sn(Nmax + 1, nullptr), sn(Nmax + 1, nullptr);
+  NS_ALLOC(S_all, double, n_int * kk3);
+  NS_ALLOC(s_all, double, n_int * k3);
+  auto first = [&](int n) { return off_int[n] - off_int[n0]; };
   for (int n = Nmax - 1; n >= n0; --n) {
-    NS_ALLOC(S, double, In[n] * kk * kk * kk);
-    NS_ALLOC(sv, double, In[n] * k3);
-    Sn[n] = S;
-    sn[n] = sv;
     const bool deeper = n + 1 < Nmax;
-    compress_tree_kernel<<<counted((unsigned)In[n]), 256, sh_c, s>>>(k, n, Ik[n], In[n], in->keys, in->coeffs, n_leaf,
-                                                            deeper ? Ik[n + 1] : nullptr, deeper ? sn[n + 1] : nullptr,
-                                                            deeper ? In[n + 1] : 0, Ub, S, sv, d_int);
+    compress_tree_kernel<<<counted((unsigned)In[n]), 256, sh_c, s>>>(
+        k, n, Ik[n], In[n], in->keys, in->coeffs, n_leaf, deeper ? Ik[n + 1] : nullptr,
+        deeper ? s_all + first(n + 1) * k3 : nullptr, deeper ? In[n + 1] : 0, Ub, S_all + first(n) * kk3,
+        s_all + first(n) * k3, d_int);
     MRA_CUDA_TRY(cudaGetLastError());
   }
   MRA_CUDA_TRY(cudaMemcpyAsync(hint, d_int, sizeof(int), cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
   if (hint[0]) return fail(MRA_ERR_ARG, "mra_apply_ns_tree: the leaves are not a complete octree");
 
-  mra_apply_stats acc{};
-  // one library apply on the given boxes of one level; its output allocated here
-  auto run_apply = [&](const Operator &opx, int64_t nsrc, uint64_t *skeys, double *scoeffs,
-                       const mra_apply_opts &oo, int64_t cap, uint64_t **okeys, double **ocoeffs,
-                       int64_t *nout) -> int {
-    const size_t wb = apply_workspace_bytes(opx, oo, nsrc);
+  // one library apply of opx on the interior boxes [b0, b1) (their coefficients at coeffs): its rows appended
+  // at okeys/ocoeffs + *nout_rows
+  auto run_apply = [&](const Operator &opx, int64_t b0, int64_t b1, double *coeffs, const mra_apply_opts &oo, int64_t rows_cap,
+                       uint64_t *okeys, double *ocoeffs, int64_t *nout_rows) -> int {
+    const int64_t rl = (int64_t)opx.k * opx.k * opx.k;
+    const size_t wb = apply_workspace_bytes(opx, oo, b1 - b0);
     void *ws = dalloc(wb);
-    *okeys = (uint64_t *)dalloc((size_t)cap * 8);
-    *ocoeffs = (double *)dalloc((size_t)cap * opx.k * opx.k * opx.k * 8);
-    if (!ws || !*okeys || !*ocoeffs) return fail(MRA_ERR_CUDA, "mra_apply_ns_tree: out of device memory");
-    mra_tree_view vin{nsrc, nsrc, skeys, scoeffs, opx.k, opx.L};
-    mra_tree_view vout{0, cap, *okeys, *ocoeffs, opx.k, opx.L};
+    if (!ws) return fail(MRA_ERR_CUDA, "mra_apply_ns_tree: out of device memory");
+    mra_tree_view vin{b1 - b0, b1 - b0, Ik[n0] + b0, coeffs + b0 * rl, opx.k, opx.L};
+    mra_tree_view vout{0, rows_cap - *nout_rows, okeys + *nout_rows, ocoeffs + *nout_rows * rl, opx.k, opx.L};
     mra_apply_stats st{};
     const int rc2 = apply_run(opx, vin, oo, vout, ws, wb, &st, s);
     drop(ws);
@@ -1097,144 +1210,69 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
       acc.level_sources[q] += st.level_sources[q];
       acc.level_terms_kept[q] += st.level_terms_kept[q];
     }
-    *nout = vout.n;
+    *nout_rows += vout.n;
+    return MRA_OK;
+  };
+  // the applies of the levels are independent: all levels in one apply (levels in groups only where the
+  // record bound of one apply would pass 2^31)
+  auto run_levels = [&](const Operator &opx, double *coeffs, uint64_t *okeys, double *ocoeffs, int64_t *rows) -> int {
+    for (int n = n0; n < Nmax;) {
+      int m = n + 1;
+      while (m < Nmax && (first(m + 1) - first(n)) * w3 < (int64_t)INT32_MAX) ++m;
+      const int rc2 = run_apply(opx, first(n), first(m), coeffs, level_opts(*o), nh, okeys, ocoeffs, rows);
+      if (rc2 != MRA_OK) return rc2;
+      n = m;
+    }
     return MRA_OK;
   };
 
   // ---- coarsest level: every box, T^{n0} with every displacement
-  int64_t nR = boxes(n0);
-  uint64_t *Rk = Ik[n0];
-  NS_ALLOC(r0, double, nR * k3);
-  double *R = r0;
+  NS_ALLOC(r, double, nh * k3);
   {
-    uint64_t *ok;
-    double *oc;
+    NS_ALLOC(ok, uint64_t, boxes(n0));
+    NS_ALLOC(oc, double, boxes(n0) * k3);
     int64_t no = 0;
-    int rc = run_apply(*op, nR, Rk, sn[n0], coarse_opts(*o, n0), nR, &ok, &oc, &no);
+    const int rc = run_apply(*op, 0, boxes(n0), s_all, coarse_opts(*o, n0), boxes(n0), ok, oc, &no);
     if (rc != MRA_OK) return rc;
-    MRA_CUDA_TRY(cudaMemsetAsync(R, 0, (size_t)nR * k3 * 8, s));
+    MRA_CUDA_TRY(cudaMemsetAsync(r, 0, (size_t)boxes(n0) * k3 * 8, s));
     if (no > 0) {
-      scatter_dense_kernel<<<counted((unsigned)no), 128, 0, s>>>(no, ok, oc, k3, R);  // level n0 is complete: dense order
+      scatter_dense_kernel<<<counted((unsigned)no), 128, 0, s>>>(no, ok, oc, k3, r);  // level n0 is complete: dense order
       MRA_CUDA_TRY(cudaGetLastError());
     }
     drop(ok);
     drop(oc);
   }
-  int64_t nout = 0;
-  const int64_t cap = out->cap;
-  const int64_t w3 = (int64_t)(2 * D + 1) * (2 * D + 1) * (2 * D + 1);
+  // ---- T2k^n S^n and T^n s^n of every level
+  NS_ALLOC(yk, uint64_t, nh);
+  NS_ALLOC(yc, double, nh * kk3);
+  NS_ALLOC(zk, uint64_t, nh);
+  NS_ALLOC(zc, double, nh * k3);
+  int64_t ny = 0, nz = 0;
+  int rc = run_levels(*ns, S_all, yk, yc, &ny);
+  if (rc != MRA_OK) return rc;
+  rc = run_levels(*op, s_all, zk, zc, &nz);
+  if (rc != MRA_OK) return rc;
+  MRA_CUDA_TRY(cudaMemsetAsync(d_int, 0, sizeof(int), s));
+  if (ny > 0) targets_in_kernel<<<counted((unsigned)((ny + 255) / 256)), 256, 0, s>>>(ny, yk, hk, nh, d_int);
+  if (nz > 0) targets_in_kernel<<<counted((unsigned)((nz + 255) / 256)), 256, 0, s>>>(nz, zk, hk, nh, d_int);
+  MRA_CUDA_TRY(cudaGetLastError());
+  // ---- down the levels
+  NS_ALLOC(yi, int64_t, nh);
+  NS_ALLOC(zi, int64_t, nh);
+  halo_rows_kernel<<<counted((unsigned)((nh + 255) / 256)), 256, 0, s>>>(nh, hk, yk, ny, zk, nz, yi, zi);
+  MRA_CUDA_TRY(cudaGetLastError());
   for (int n = n0; n < Nmax; ++n) {
-    const int64_t tcap = std::min<int64_t>(boxes(n), In[n] * w3);
-    uint64_t *yk, *zk;
-    double *yc, *zc;
-    int64_t ny = 0, nz = 0;
-    int rc = run_apply(*ns, In[n], Ik[n], Sn[n], level_opts(*o), tcap, &yk, &yc, &ny);
-    if (rc != MRA_OK) return rc;
-    rc = run_apply(*op, In[n], Ik[n], sn[n], level_opts(*o), tcap, &zk, &zc, &nz);
-    if (rc != MRA_OK) return rc;
-    MRA_CUDA_TRY(cudaMemsetAsync(d_int, 0, sizeof(int), s));
-    if (ny > 0) targets_in_kernel<<<counted((unsigned)((ny + 255) / 256)), 256, 0, s>>>(ny, yk, Rk, nR, d_int);
-    if (nz > 0) targets_in_kernel<<<counted((unsigned)((nz + 255) / 256)), 256, 0, s>>>(nz, zk, Rk, nR, d_int);
+    const int64_t j0 = hoff[n], nj = hoff[n + 1] - hoff[n];
+    if (nj == 0) continue;
+    sum_down_tree_kernel<<<counted((unsigned)nj), 256, sh_d, s>>>(k, j0, r, yi, yc, zi, zc, dst, Ub, out->coeffs);
     MRA_CUDA_TRY(cudaGetLastError());
-    // the halo of the level's sources, sorted and unique
-    const int64_t nh_all = In[n] * w3;
-    NS_ALLOC(hal, uint64_t, nh_all);
-    NS_ALLOC(hal_s, uint64_t, nh_all);
-    NS_ALLOC(hk, uint64_t, nh_all);
-    NS_ALLOC(d_nh, int64_t, 1);
-    MRA_CUDA_TRY(cudaMemsetAsync(d_nh, 0, 8, s));
-    if (nh_all > 0) {
-      halo_kernel<<<counted((unsigned)((nh_all + 255) / 256)), 256, 0, s>>>(In[n], Ik[n], D, hal);
-      MRA_CUDA_TRY(cudaGetLastError());
-      size_t t1 = 0, t2 = 0;
-      MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, t1, hal, hal_s, (int)nh_all, 0, 64, s));
-      MRA_CUDA_TRY(cub::DeviceSelect::Unique(nullptr, t2, hal_s, hk, d_nh, (int)nh_all, s));
-      NS_ALLOC(tmph, unsigned char, std::max(t1, t2));
-      MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(tmph, t1, hal, hal_s, (int)nh_all, 0, 64, s));
-      MRA_CUDA_TRY(cub::DeviceSelect::Unique(tmph, t2, hal_s, hk, d_nh, (int)nh_all, s));
-      drop(tmph);
-    }
-    NS_ALLOC(yi, int64_t, nR);
-    NS_ALLOC(zi, int64_t, nR);
-    NS_ALLOC(refine, int, nR + 1);
-    NS_ALLOC(leaf, int, nR + 1);
-    NS_ALLOC(ref_pos, int, nR + 1);
-    NS_ALLOC(leaf_pos, int, nR + 1);
-    if (nR > 0) {
-      reach_kernel<<<counted((unsigned)((nR + 255) / 256)), 256, 0, s>>>(nR, Rk, hk, d_nh, yk, ny, zk, nz, yi, zi, refine, leaf);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    MRA_CUDA_TRY(cudaMemsetAsync(refine + nR, 0, sizeof(int), s));
-    MRA_CUDA_TRY(cudaMemsetAsync(leaf + nR, 0, sizeof(int), s));
-    size_t tb = 0;
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, refine, ref_pos, (int)(nR + 1), s));
-    NS_ALLOC(tmp, unsigned char, tb);
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp, tb, refine, ref_pos, (int)(nR + 1), s));
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp, tb, leaf, leaf_pos, (int)(nR + 1), s));
-    int hcount[2] = {0, 0};
-    MRA_CUDA_TRY(cudaMemcpyAsync(&hcount[0], ref_pos + nR, sizeof(int), cudaMemcpyDeviceToHost, s));
-    MRA_CUDA_TRY(cudaMemcpyAsync(&hint[0], d_int, sizeof(int), cudaMemcpyDeviceToHost, s));
-    MRA_CUDA_TRY(cudaStreamSynchronize(s));
-    if (hint[0]) return fail(MRA_ERR_NUMERIC, "mra_apply_ns_tree: a level-%d apply reached a box outside the result tree", n);
-    const int64_t nref = hcount[0], nleaf_here = nR - nref;
-    if (nleaf_here > 0 && nR > 0) {
-      emit_leaves_kernel<<<counted((unsigned)nR), 128, 0, s>>>(nR, k3, Rk, R, leaf, leaf_pos, nout, cap, out->keys, out->coeffs);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    nout += nleaf_here;
-    // children of the reached nodes, then in key order
-    const int64_t nC = 8 * nref;
-    NS_ALLOC(cku, uint64_t, nC);
-    NS_ALLOC(cru, double, nC * k3);
-    if (nref > 0) {
-      sum_down_tree_kernel<<<counted((unsigned)nR), 256, sh_d, s>>>(k, nR, Rk, R, refine, ref_pos, yi, yc, zi, zc, Ub, cku, cru);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    NS_ALLOC(cks, uint64_t, nC);
-    NS_ALLOC(crs, double, nC * k3);
-    NS_ALLOC(idx, int, nC);
-    NS_ALLOC(idx_s, int, nC);
-    if (nC > 0) {
-      iota_ns_kernel<<<counted((unsigned)((nC + 255) / 256)), 256, 0, s>>>(nC, idx);
-      MRA_CUDA_TRY(cudaGetLastError());
-      size_t ts = 0;
-      MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, ts, cku, cks, idx, idx_s, (int)nC, 0, 64, s));
-      NS_ALLOC(tmp2, unsigned char, ts);
-      MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp2, ts, cku, cks, idx, idx_s, (int)nC, 0, 64, s));
-      gather_rows_ns_kernel<<<counted((unsigned)nC), 128, 0, s>>>(nC, k3, idx_s, cru, crs);
-      MRA_CUDA_TRY(cudaGetLastError());
-      drop(tmp2);
-    }
-    for (void *p : {(void *)yk, (void *)yc, (void *)zk, (void *)zc, (void *)yi, (void *)zi, (void *)refine,
-                    (void *)leaf, (void *)ref_pos, (void *)leaf_pos, (void *)tmp, (void *)cku, (void *)cru,
-                    (void *)idx, (void *)idx_s, (void *)hal, (void *)hal_s, (void *)hk, (void *)d_nh})
-      drop(p);
-    if (Rk != Ik[n0]) drop(Rk);
-    drop(R);
-    Rk = cks;
-    R = crs;
-    nR = nC;
   }
-  // the deepest level: every node is a result leaf
-  if (nR > 0 && nout < cap) {
-    const int64_t ncopy = std::min<int64_t>(nR, cap - nout);
-    MRA_CUDA_TRY(cudaMemcpyAsync(out->keys + nout, Rk, (size_t)ncopy * 8, cudaMemcpyDeviceToDevice, s));
-    MRA_CUDA_TRY(cudaMemcpyAsync(out->coeffs + nout * k3, R, (size_t)ncopy * k3 * 8, cudaMemcpyDeviceToDevice, s));
-  }
-  nout += nR;
+  MRA_CUDA_TRY(cudaMemcpyAsync(hint, d_int, sizeof(int), cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
-  if (stats) {
-    acc.n_in = n_leaf;
-    acc.n_out = nout;
-    *stats = acc;
-  }
+  if (hint[0]) return fail(MRA_ERR_NUMERIC, "mra_apply_ns_tree: an apply reached a box outside the result tree");
   out->L = op->L;
-  if (nout > cap) {
-    out->n = nout;
-    return fail(MRA_ERR_CAPACITY, "mra_apply_ns_tree: %lld result leaves, capacity %lld", (long long)nout,
-                (long long)cap);
-  }
   out->n = nout;
+  if (stats) *stats = acc;
   return MRA_OK;
 #undef NS_ALLOC
 }
