@@ -23,6 +23,7 @@
 #include <cub/cub.cuh>
 
 #include "apply_internal.cuh"
+#include "twoscale.cuh"
 
 namespace mra {
 
@@ -99,15 +100,32 @@ __global__ void scatter_levels_kernel(int64_t n_rows, const uint64_t *keys, cons
 }
 
 // ---------------------------------------------------------------- two-scale transforms
+// Threads of the kernels that transform one box per CTA.  A level often has fewer boxes than the chip has
+// room for, so a launch lasts as long as one box does: 512 threads instead of 256.
+constexpr int BOX_THREADS = 512;
+// Shared memory of the transforms: U (k^2) and the buffers up (S 8 k^3, a 4 k^3) and down (7 k^3) need.
+size_t up_smem(int k) { return (size_t)(k * k + 12 * k * k * k) * 8; }
+size_t down_smem(int k) { return (size_t)(k * k + 7 * k * k * k) * 8; }
+
+// S (shared, complete, overwritten) filtered to the parent's coefficients, written to s_out.
+__device__ __forceinline__ void filter_box(int k, const double *U, double *S, double *a, double *s_out) {
+  const int k3 = k * k * k;
+  twoscale::up_first(k, U, S, a);
+  double *b = S, *sv = S + 2 * k3;
+  twoscale::up_rest(k, U, a, b, sv);
+  for (int e = threadIdx.x; e < k3; e += blockDim.x) s_out[e] = sv[e];
+}
+
 // One CTA per box of level n: S = the children (dense level n+1) as a (2k)^3 tensor, written
-// out, and s = (Ubar^T)^{x3} S.  Shared memory: S (2k)^3, a k (2k)^2, b k^2 (2k) doubles.
+// out, and s = (Ubar^T)^{x3} S.
 __global__ void compress_kernel(int k, int n, const double *fine, const double *Ub, double *S_out,
                                 double *s_out) {
   extern __shared__ double sh[];
   const int kk = 2 * k, k3 = k * k * k, kk3 = kk * kk * kk;
-  double *S = sh, *a = S + kk3, *b = a + k * kk * kk;
+  double *U = sh, *S = U + k * k, *a = S + kk3;
   const int64_t box = blockIdx.x, nb = 1LL << n, nf = 2 * nb;
   const int64_t x = box / (nb * nb), y = (box / nb) % nb, z = box % nb;
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) U[e] = Ub[e];
   for (int e = threadIdx.x; e < kk3; e += blockDim.x) {
     const int I = e / (kk * kk), J = (e / kk) % kk, Lq = e % kk;
     const int64_t child = ((2 * x + I / k) * nf + 2 * y + J / k) * nf + 2 * z + Lq / k;
@@ -116,60 +134,25 @@ __global__ void compress_kernel(int k, int n, const double *fine, const double *
     S_out[box * kk3 + e] = v;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < k * kk * kk; e += blockDim.x) {  // a[i][J][L] = sum_I Ub[I][i] S[I][J][L]
-    const int i = e / (kk * kk), q = e % (kk * kk);
-    double v = 0.0;
-    for (int I = 0; I < kk; ++I) v += Ub[I * k + i] * S[I * kk * kk + q];
-    a[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < k * k * kk; e += blockDim.x) {  // b[i][j][L] = sum_J Ub[J][j] a[i][J][L]
-    const int i = e / (k * kk), j = (e / kk) % k, Lq = e % kk;
-    double v = 0.0;
-    for (int J = 0; J < kk; ++J) v += Ub[J * k + j] * a[(i * kk + J) * kk + Lq];
-    b[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) {  // s[i][j][l] = sum_L Ub[L][l] b[i][j][L]
-    const int q = e / k, l = e % k;
-    double v = 0.0;
-    for (int Lq = 0; Lq < kk; ++Lq) v += Ub[Lq * k + l] * b[q * kk + Lq];
-    s_out[box * k3 + e] = v;
-  }
+  filter_box(k, U, S, a, s_out + box * k3);
 }
 
 // One CTA per box of level n: r^{n+1}(children) = (Ubar)^{x3} (r_b - Z_b) + Y_b, into the
-// dense level n+1 array.  Shared memory: d k^3, a (2k) k^2, b (2k)^2 k doubles.
+// dense level n+1 array.
 __global__ void sum_down_kernel(int k, int n, const double *r, const double *Z, const double *Y,
                                 const double *Ub, double *fine) {
   extern __shared__ double sh[];
-  const int kk = 2 * k, k2 = k * k, k3 = k2 * k, kk3 = kk * kk * kk;
-  double *d = sh, *a = d + k3, *b = a + kk * k2;
+  const int kk = 2 * k, k3 = k * k * k, kk3 = kk * kk * kk;
+  double *U = sh, *d = U + k * k, *a = d + k3, *b = a + 2 * k3;
   const int64_t box = blockIdx.x, nb = 1LL << n, nf = 2 * nb;
   const int64_t x = box / (nb * nb), y = (box / nb) % nb, z = box % nb;
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) U[e] = Ub[e];
   for (int e = threadIdx.x; e < k3; e += blockDim.x) d[e] = r[box * k3 + e] - Z[box * k3 + e];
   __syncthreads();
-  for (int e = threadIdx.x; e < kk * k2; e += blockDim.x) {  // a[I][j][l] = sum_i Ub[I][i] d[i][j][l]
-    const int I = e / k2, q = e % k2;
-    double v = 0.0;
-    for (int i = 0; i < k; ++i) v += Ub[I * k + i] * d[i * k2 + q];
-    a[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kk * kk * k; e += blockDim.x) {  // b[I][J][l] = sum_j Ub[J][j] a[I][j][l]
-    const int I = e / (kk * k), J = (e / k) % kk, l = e % k;
-    double v = 0.0;
-    for (int j = 0; j < k; ++j) v += Ub[J * k + j] * a[(I * k + j) * k + l];
-    b[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kk3; e += blockDim.x) {  // + sum_l Ub[L][l] b[I][J][l] + Y
-    const int I = e / (kk * kk), J = (e / kk) % kk, Lq = e % kk;
-    double v = Y[box * kk3 + e];
-    for (int l = 0; l < k; ++l) v += Ub[Lq * k + l] * b[(I * kk + J) * k + l];
+  twoscale::down(k, U, d, a, b, [&](int I, int J, int Lq, double v) {
     const int64_t child = ((2 * x + I / k) * nf + 2 * y + J / k) * nf + 2 * z + Lq / k;
-    fine[child * k3 + ((I % k) * k + J % k) * k + Lq % k] = v;
-  }
+    fine[child * k3 + ((I % k) * k + J % k) * k + Lq % k] = Y[box * kk3 + (I * kk + J) * kk + Lq] + v;
+  });
 }
 
 // ---------------------------------------------------------------- adaptive trees
@@ -214,9 +197,10 @@ __global__ void compress_tree_kernel(int k, int n, const uint64_t *ikeys, int64_
   extern __shared__ double sh[];
   __shared__ const double *src[8];
   const int kk = 2 * k, k3 = k * k * k, kk3 = kk * kk * kk;
-  double *S = sh, *a = S + kk3, *b = a + k * kk * kk;
+  double *U = sh, *S = U + k * k, *a = S + kk3;
   const int64_t box = blockIdx.x;
   if (box >= n_int) return;
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) U[e] = Ub[e];
   const uint64_t key = ikeys[box];
   if (threadIdx.x < 8) {
     const int cx = threadIdx.x >> 2, cy = (threadIdx.x >> 1) & 1, cz = threadIdx.x & 1;
@@ -241,26 +225,7 @@ __global__ void compress_tree_kernel(int k, int n, const uint64_t *ikeys, int64_
     S_out[box * kk3 + e] = v;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < k * kk * kk; e += blockDim.x) {
-    const int i = e / (kk * kk), q = e % (kk * kk);
-    double v = 0.0;
-    for (int I = 0; I < kk; ++I) v += Ub[I * k + i] * S[I * kk * kk + q];
-    a[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < k * k * kk; e += blockDim.x) {
-    const int i = e / (k * kk), j = (e / kk) % k, Lq = e % kk;
-    double v = 0.0;
-    for (int J = 0; J < kk; ++J) v += Ub[J * k + j] * a[(i * kk + J) * kk + Lq];
-    b[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) {
-    const int q = e / k, l = e % k;
-    double v = 0.0;
-    for (int Lq = 0; Lq < kk; ++Lq) v += Ub[Lq * k + l] * b[q * kk + Lq];
-    s_out[box * k3 + e] = v;
-  }
+  filter_box(k, U, S, a, s_out + box * k3);
 }
 
 // The halo of the level's sources: every in-cell box within |l|_inf <= D of one (others: the
@@ -322,17 +287,6 @@ __global__ void targets_in_kernel(int64_t nt, const uint64_t *tkeys, const uint6
   if (find_sorted(rkeys, nr, tkeys[i]) < 0) atomicExch(err, 3);
 }
 
-// Result leaves of this level: nodes of R_n that no apply reached, appended at out + base.
-__global__ void emit_leaves_kernel(int64_t nr, int k3, const uint64_t *rkeys, const double *r, const int *leaf,
-                                   const int *leaf_pos, int64_t base, int64_t cap, uint64_t *okeys, double *ocoeffs) {
-  const int64_t p = blockIdx.x;
-  if (p >= nr || !leaf[p]) return;
-  const int64_t o = base + leaf_pos[p];
-  if (o >= cap) return;
-  if (threadIdx.x == 0) okeys[o] = rkeys[p];
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) ocoeffs[o * k3 + e] = r[p * k3 + e];
-}
-
 // One CTA per halo box of one level (j0 + blockIdx.x): its children get (Ubar)^{x3} (r - Z) + Y (absent rows
 // as zero), written to the next level's r where the child is refined there, else to the result.
 __global__ void sum_down_tree_kernel(int k, int64_t j0, double *r, const int64_t *yi, const double *Y,
@@ -341,48 +295,20 @@ __global__ void sum_down_tree_kernel(int k, int64_t j0, double *r, const int64_t
   extern __shared__ double sh[];
   __shared__ double *to[8];
   const int64_t p = j0 + blockIdx.x;
-  const int kk = 2 * k, k2 = k * k, k3 = k2 * k, kk3 = kk * kk * kk;
-  double *d = sh, *a = d + k3, *b = a + kk * k2;
+  const int kk = 2 * k, k3 = k * k * k, kk3 = kk * kk * kk;
+  double *U = sh, *d = U + k * k, *a = d + k3, *b = a + 2 * k3;
   const int64_t y = yi[p], z = zi[p];
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) U[e] = Ub[e];
   for (int e = threadIdx.x; e < k3; e += blockDim.x) d[e] = r[p * k3 + e] - (z >= 0 ? Z[z * k3 + e] : 0.0);
   if (threadIdx.x < 8) {
     const int64_t t = dst[8 * p + threadIdx.x];
     to[threadIdx.x] = t >= 0 ? r + t * k3 : out + (-2 - t) * k3;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kk * k2; e += blockDim.x) {
-    const int I = e / k2, q = e % k2;
-    double v = 0.0;
-    for (int i = 0; i < k; ++i) v += Ub[I * k + i] * d[i * k2 + q];
-    a[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kk * kk * k; e += blockDim.x) {
-    const int I = e / (kk * k), J = (e / k) % kk, l = e % k;
-    double v = 0.0;
-    for (int j = 0; j < k; ++j) v += Ub[J * k + j] * a[(I * k + j) * k + l];
-    b[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kk3; e += blockDim.x) {
-    const int I = e / (kk * kk), J = (e / kk) % kk, Lq = e % kk;
-    double v = y >= 0 ? Y[y * kk3 + e] : 0.0;
-    for (int l = 0; l < k; ++l) v += Ub[Lq * k + l] * b[(I * kk + J) * k + l];
+  twoscale::down(k, U, d, a, b, [&](int I, int J, int Lq, double v) {
     const int child = ((I / k) << 2) | ((J / k) << 1) | (Lq / k);
-    to[child][((I % k) * k + J % k) * k + Lq % k] = v;
-  }
-}
-
-__global__ void gather_rows_ns_kernel(int64_t n, int rowlen, const int *perm, const double *src, double *dst) {
-  const int64_t i = blockIdx.x;
-  if (i >= n) return;
-  const int64_t from = perm[i];
-  for (int e = threadIdx.x; e < rowlen; e += blockDim.x) dst[i * rowlen + e] = src[from * rowlen + e];
-}
-
-__global__ void iota_ns_kernel(int64_t n, int *v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] = (int)i;
+    to[child][((I % k) * k + J % k) * k + Lq % k] = (y >= 0 ? Y[y * kk3 + (I * kk + J) * kk + Lq] : 0.0) + v;
+  });
 }
 
 // ---------------------------------------------------------------- reconstruct
@@ -429,211 +355,264 @@ __global__ void level_offsets_kernel(const uint64_t *keys, const int64_t *n, int
   off[l] = a;
 }
 
-// Input boxes of level n in [lo, hi): tops join the level's boxes (appended after `base`
-// passed-down boxes, at their rank pos[b] - pos0 among the level's tops), the others add their
-// coefficients to the passed-down box of the same key.
-__global__ void tops_kernel(int64_t lo, int64_t hi, int n, const int *top, const uint64_t *keys, const double *coeffs,
-                            int k3, const int *pos, int pos0, int64_t base, uint64_t *rkeys, double *rv) {
-  const int64_t b = lo + blockIdx.x;
-  if (b >= hi || top[b] != n) return;
-  const int64_t o = base + (pos[b] - pos0);
-  if (threadIdx.x == 0) rkeys[o] = keys[b];
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) rv[o * k3 + e] = coeffs[b * k3 + e];
+// Keys strictly increasing and no level above 19 (*bad otherwise); off[l] = first position of level l, l <= 20.
+__global__ void leaf_offsets_kernel(int64_t n, const uint64_t *keys, int64_t *off, int64_t *bad) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i > n) return;
+  const int lv = i < n ? min(key_level(keys[i]), 21) : 21;
+  const int pv = i > 0 ? min(key_level(keys[i - 1]), 21) : -1;
+  if (i < n && (lv > MRA_MAX_LEVEL || (i > 0 && keys[i] <= keys[i - 1])))
+    atomicMax((unsigned long long *)bad, lv > MRA_MAX_LEVEL ? 2ull : 1ull);
+  for (int l = pv + 1; l <= min(lv, 20); ++l) off[l] = i;
 }
-// flag[b] = 1 for the input boxes that are tops (no input box above them), flag[n] = 0
-__global__ void top_flags_kernel(int64_t n, const uint64_t *keys, const int *top, int *flag) {
+
+// Input boxes that are tops (no input box above them): all of them and those that are interior too.
+__global__ void count_tops_kernel(int64_t n, const uint64_t *keys, const int *top, const uint64_t *ikeys,
+                                  const int64_t *ni, unsigned long long *count) {
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b > n) return;
-  flag[b] = b < n && top[b] == key_level(keys[b]) ? 1 : 0;
+  bool t = false, in = false;
+  if (b < n) {
+    t = top[b] == key_level(keys[b]);
+    if (t) in = find_sorted(ikeys, *ni, keys[b]) >= 0;
+  }
+  const unsigned bt = __ballot_sync(0xffffffffu, t), bi = __ballot_sync(0xffffffffu, in);
+  if ((threadIdx.x & 31) == 0) {
+    if (bt) atomicAdd(count, (unsigned long long)__popc(bt));
+    if (bi) atomicAdd(count + 1, (unsigned long long)__popc(bi));
+  }
 }
-// the level's interior boxes found among its boxes must be all of them (a consistent tree)
-__global__ void inner_count_check_kernel(const int *ipos, int64_t nr, int64_t ni, int *err) {
-  if (ipos[nr] != ni) atomicExch(err, 2);
-}
-__global__ void add_inputs_kernel(int64_t lo, int64_t hi, int n, const int *top, const uint64_t *keys,
-                                  const double *coeffs, int k3, const uint64_t *rkeys, int64_t nr, double *rv,
-                                  int *err) {
-  const int64_t b = lo + blockIdx.x;
-  if (b >= hi || top[b] == n) return;
-  __shared__ int64_t p;
-  if (threadIdx.x == 0) p = find_sorted(rkeys, nr, keys[b]);
-  __syncthreads();
-  if (p < 0) {
-    if (threadIdx.x == 0) atomicExch(err, 1);
+
+// The nodes of the result by entry: 8 j + c, child c of interior box j, then 8 ni + b, input box b.  A child
+// that is interior is passed on (dst = its rank), the other children and the tops that are not interior are
+// leaves (their keys in leaf_key, the largest key elsewhere).  own: the input box at the child, or -1;
+// start[j], iown[j]: interior box j is a top, the input box at it.
+__global__ void recon_nodes_kernel(int64_t ni, const uint64_t *ikeys, int64_t n_in, const uint64_t *keys, const int *top,
+                                   int64_t *dst, int64_t *own, int64_t *iown, unsigned char *start, uint64_t *leaf_key,
+                                   int *id) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 8 * ni + n_in) return;
+  id[e] = (int)e;
+  if (e >= 8 * ni) {
+    const int64_t b = e - 8 * ni;
+    const bool leaf = top[b] == key_level(keys[b]) && find_sorted(ikeys, ni, keys[b]) < 0;
+    leaf_key[e] = leaf ? keys[b] : ~0ull;
+    dst[e] = -1;
     return;
   }
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) rv[p * k3 + e] += coeffs[b * k3 + e];
+  const int64_t j = e >> 3;
+  const uint64_t k = ikeys[j];
+  const int n = key_level(k), c = (int)(e & 7);
+  const uint64_t ck = make_key(n + 1, 2 * key_x(k) + (c >> 2), 2 * key_y(k) + ((c >> 1) & 1), 2 * key_z(k) + (c & 1));
+  const int64_t p = find_sorted(ikeys, ni, ck);
+  dst[e] = p >= 0 ? p : -1;
+  own[e] = p >= 0 ? -1 : find_sorted(keys, n_in, ck);
+  leaf_key[e] = p >= 0 ? ~0ull : ck;
+  if (c == 0) {
+    const int64_t b = find_sorted(keys, n_in, k);
+    iown[j] = b;
+    start[j] = b >= 0 && top[b] == n;
+  }
 }
 
-// Is box p of the level interior (passes down) or a leaf of the result?
-__global__ void classify_kernel(int64_t nr, const uint64_t *rkeys, const uint64_t *ikeys, int64_t ni, int *inner,
-                                int *leaf) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nr) return;
-  const bool in = find_sorted(ikeys, ni, rkeys[p]) >= 0;
-  inner[p] = in ? 1 : 0;
-  leaf[p] = in ? 0 : 1;
+// The tops that are leaves, copied to their places.
+__global__ void copy_tops_kernel(int64_t n_in, int64_t base, int k3, const int64_t *dst, const double *coeffs, double *out) {
+  const int64_t b = blockIdx.x, t = dst[base + b];
+  if (t == -1) return;
+  double *o = out + (-2 - t) * k3;
+  for (int e = threadIdx.x; e < k3; e += blockDim.x) o[e] = coeffs[b * k3 + e];
 }
 
-// One CTA per interior box: its eight children get Ubar^{x3} s (two-scale relation).
-__global__ void pass_down_kernel(int k, int64_t nr, const uint64_t *rkeys, const double *rv, const int *inner,
-                                 const int *pos, int64_t ninner, const double *Ub, uint64_t *ckeys, double *cv,
-                                 int *err) {
+// One CTA per interior box of one level (j0 + blockIdx.x): what it was passed plus its own input coefficients,
+// to its eight children by the two-scale relation; a leaf child adds its own input coefficients.
+__global__ void pass_down_kernel(int k, int64_t j0, double *r, const int64_t *iown, const unsigned char *start,
+                                 const int64_t *dst, const int64_t *own, const double *coeffs, const double *Ub,
+                                 double *out) {
   extern __shared__ double sh[];
-  const int64_t p = blockIdx.x;
-  if (p >= nr || !inner[p]) return;
-  if (pos[p] >= ninner) {  // more interior boxes than the level has room for: inconsistent tree
-    if (threadIdx.x == 0) atomicExch(err, 2);
-    return;
+  __shared__ double *to[8];
+  __shared__ const double *add[8];
+  const int64_t p = j0 + blockIdx.x;
+  const int k3 = k * k * k;
+  double *U = sh, *d = U + k * k, *a = d + k3, *b = a + 2 * k3;
+  const int64_t in = iown[p];
+  const bool first = start[p];
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) U[e] = Ub[e];
+  for (int e = threadIdx.x; e < k3; e += blockDim.x) {
+    double v = first ? 0.0 : r[p * k3 + e];
+    if (in >= 0) v = first ? coeffs[in * k3 + e] : v + coeffs[in * k3 + e];
+    d[e] = v;
   }
-  const int kk = 2 * k, k2 = k * k, k3 = k2 * k, kk3 = kk * kk * kk;
-  double *d = sh, *a = d + k3, *b = a + kk * k2;
-  const int64_t base = 8 * (int64_t)pos[p];
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) d[e] = rv[p * k3 + e];
-  const uint64_t key = rkeys[p];
   if (threadIdx.x < 8) {
-    const int cx = threadIdx.x >> 2, cy = (threadIdx.x >> 1) & 1, cz = threadIdx.x & 1;
-    ckeys[base + threadIdx.x] =
-        make_key(key_level(key) + 1, 2 * key_x(key) + cx, 2 * key_y(key) + cy, 2 * key_z(key) + cz);
+    const int64_t t = dst[8 * p + threadIdx.x], o = own[8 * p + threadIdx.x];
+    to[threadIdx.x] = t >= 0 ? r + t * k3 : out + (-2 - t) * k3;
+    add[threadIdx.x] = o >= 0 ? coeffs + o * k3 : nullptr;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kk * k2; e += blockDim.x) {
-    const int I = e / k2, q = e % k2;
-    double v = 0.0;
-    for (int i = 0; i < k; ++i) v += Ub[I * k + i] * d[i * k2 + q];
-    a[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kk * kk * k; e += blockDim.x) {
-    const int I = e / (kk * k), J = (e / k) % kk, l = e % k;
-    double v = 0.0;
-    for (int j = 0; j < k; ++j) v += Ub[J * k + j] * a[(I * k + j) * k + l];
-    b[e] = v;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kk3; e += blockDim.x) {
-    const int I = e / (kk * kk), J = (e / kk) % kk, Lq = e % kk;
-    double v = 0.0;
-    for (int l = 0; l < k; ++l) v += Ub[Lq * k + l] * b[(I * kk + J) * k + l];
-    const int child = ((I / k) << 2) | ((J / k) << 1) | (Lq / k);
-    cv[(base + child) * k3 + ((I % k) * k + J % k) * k + Lq % k] = v;
-  }
+  twoscale::down(k, U, d, a, b, [&](int I, int J, int Lq, double v) {
+    const int child = ((I / k) << 2) | ((J / k) << 1) | (Lq / k), e = ((I % k) * k + J % k) * k + Lq % k;
+    const double *w = add[child];
+    to[child][e] = w ? v + w[e] : v;
+  });
 }
 
 // ---------------------------------------------------------------- truncate
-// One CTA per leaf of level n (sorted keys): a leaf with even (x, y, z) whose seven siblings
-// are leaves too forms S from the eight, s = (Ubar^T)^{x3} S and the detail
-// d = S - Ubar^{x3} s; if ||d||_F <= thresh the eight are marked gone, the parent (key, s) is
-// appended at an atomic slot of the level above and ||d||^2 is kept at the first child's slot.
-// Shared memory: the filter's two intermediates (4k^3, 2k^3) and s (k^3), the unfilter's
-// intermediates reusing the filter's; S itself (8k^3) is staged too when s_smem is set, and
-// read from the children's rows otherwise (k > 12, where it does not fit).
-__global__ void truncate_level_kernel(int k, int n, int64_t nl, const uint64_t *keys, const double *v, double thresh,
-                                      const double *Ub, int *gone, double *d2, uint64_t *pkeys, double *pv,
-                                      int *pcount, int s_smem) {
+// Boxes that could hold a merged parent: a box all of whose eight children are leaves or merged parents
+// holds the leaf at its low corner.  So leaf i proposes its ancestors as long as it is their low corner,
+// each box at most once; *count and the per-level counts of what is written to cand.
+__global__ void corner_parents_kernel(int64_t n, const uint64_t *keys, uint64_t *cand, unsigned long long *count,
+                                      unsigned long long *level_count) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const uint64_t k = keys[i];
+  const int lv = key_level(k);
+  int64_t x = key_x(k), y = key_y(k), z = key_z(k);
+  for (int m = lv - 1; m >= 0 && !((x | y | z) & 1); --m) {
+    x >>= 1;
+    y >>= 1;
+    z >>= 1;
+    cand[atomicAdd(count, 1ull)] = make_key(m, x, y, z);
+    atomicAdd(level_count + m, 1ull);
+  }
+}
+
+// Child c of candidate j (entry 8 j + c): the leaf there, or -2 - (candidate there), or -1.
+__global__ void merge_children_kernel(int64_t nc, const uint64_t *cand, int64_t n_in, const uint64_t *keys, int64_t *child) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 8 * nc) return;
+  const uint64_t k = cand[e >> 3];
+  const int n = key_level(k), c = (int)(e & 7);
+  const uint64_t ck = make_key(n + 1, 2 * key_x(k) + (c >> 2), 2 * key_y(k) + ((c >> 1) & 1), 2 * key_z(k) + (c & 1));
+  int64_t p = find_sorted(keys, n_in, ck);
+  if (p < 0) {
+    p = find_sorted(cand, nc, ck);
+    p = p >= 0 ? -2 - p : -1;
+  }
+  child[e] = p;
+}
+
+// One CTA per candidate of one level (j0 + blockIdx.x): if its eight children are leaves or merged, S from the
+// eight, s = (Ubar^T)^{x3} S and the detail d = S - Ubar^{x3} s; if ||d||_F <= thresh the eight are gone
+// (gone: leaves, then candidates), the candidate holds s (pv) and ||d||^2 is kept.  Shared memory: U,
+// S (8 k^3) and 4 k^3 with s_smem, else 7 k^3 and S read from the children's rows (k > 12, where S does not fit).
+__global__ void truncate_level_kernel(int k, int64_t j0, int64_t n_in, const int64_t *child, const double *coeffs,
+                                      double thresh, const double *Ub, int *gone, int *merged, double *d2, double *pv,
+                                      int s_smem) {
   extern __shared__ double sh[];
-  __shared__ int64_t idx[8];
+  __shared__ const double *src[8];
   __shared__ int all;
-  __shared__ double red[8];
-  const int64_t i = blockIdx.x;
-  if (i >= nl) return;
-  const uint64_t key = keys[i];
-  const int64_t x = key_x(key), y = key_y(key), z = key_z(key);
-  if ((x & 1) || (y & 1) || (z & 1)) return;
+  __shared__ double red[BOX_THREADS / 32];
+  const int64_t j = j0 + blockIdx.x;
   const int kk = 2 * k, k3 = k * k * k, kk3 = kk * kk * kk;
-  double *a = sh, *b = a + k * kk * kk, *sv = b + k * k * kk, *S = sv + k3;
-  double *c = b, *e = a;  // the unfilter's intermediates (kk k^2 and kk^2 k) once a and b are consumed
   if (threadIdx.x == 0) all = 1;
   __syncthreads();
   if (threadIdx.x < 8) {
-    const int cx = threadIdx.x >> 2, cy = (threadIdx.x >> 1) & 1, cz = threadIdx.x & 1;
-    idx[threadIdx.x] = find_sorted(keys, nl, make_key(n, x + cx, y + cy, z + cz));
-    if (idx[threadIdx.x] < 0) atomicExch(&all, 0);
+    const int64_t c = child[8 * j + threadIdx.x];
+    const bool there = c >= 0 || (c <= -2 && merged[-2 - c]);
+    src[threadIdx.x] = c >= 0 ? coeffs + c * k3 : (there ? pv + (-2 - c) * k3 : nullptr);
+    if (!there) all = 0;
   }
   __syncthreads();
   if (!all) return;
   // S[(I, J, L)] = child (I/k, J/k, L/k)'s coefficient (I%k, J%k, L%k)
-  auto s_at = [&](int q) {
-    const int I = q / (kk * kk), J = (q / kk) % kk, Lq = q % kk;
-    const int64_t src = idx[((I / k) << 2) | ((J / k) << 1) | (Lq / k)];
-    return v[src * k3 + ((I % k) * k + J % k) * k + Lq % k];
+  auto s_at = [&](int I, int J, int Lq) {
+    return src[((I / k) << 2) | ((J / k) << 1) | (Lq / k)][((I % k) * k + J % k) * k + Lq % k];
   };
+  double *U = sh, *S = U + k * k, *a, *b, *sv, *c;  // b also serves the way down (2 k^3), as does a (4 k^3)
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) U[e] = Ub[e];
   if (s_smem) {
-    for (int q = threadIdx.x; q < kk3; q += blockDim.x) S[q] = s_at(q);
+    a = S + kk3;
+    b = S;
+    sv = S + 2 * k3;
+    c = S + 3 * k3;
+    for (int q = threadIdx.x; q < kk3; q += blockDim.x) S[q] = s_at(q / (kk * kk), (q / kk) % kk, q % kk);
+    __syncthreads();
+    twoscale::up_first(k, U, S, a);
+  } else {
+    a = S;
+    b = a + 4 * k3;
+    sv = b + 2 * k3;
+    c = b;
+    __syncthreads();
+    for (int q = threadIdx.x; q < k * kk * kk; q += blockDim.x) {
+      const int jx = q / (kk * kk), J = (q / kk) % kk, Lq = q % kk;
+      double t = 0.0;
+      for (int i = jx; i >= 0; --i) {
+        const double x0 = s_at(i, J, Lq), x1 = s_at(k + i, J, Lq);
+        t = fma(U[i * k + jx], ((jx - i) & 1) ? x0 - x1 : x0 + x1, t);
+      }
+      a[q] = t;
+    }
     __syncthreads();
   }
-  for (int q = threadIdx.x; q < k * kk * kk; q += blockDim.x) {  // filter
-    const int ii = q / (kk * kk), r = q % (kk * kk);
-    double t = 0.0;
-    for (int I = 0; I < kk; ++I) t += Ub[I * k + ii] * (s_smem ? S[I * kk * kk + r] : s_at(I * kk * kk + r));
-    a[q] = t;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < k * k * kk; q += blockDim.x) {
-    const int ii = q / (k * kk), j = (q / kk) % k, Lq = q % kk;
-    double t = 0.0;
-    for (int J = 0; J < kk; ++J) t += Ub[J * k + j] * a[(ii * kk + J) * kk + Lq];
-    b[q] = t;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < k3; q += blockDim.x) {
-    const int r = q / k, l = q % k;
-    double t = 0.0;
-    for (int Lq = 0; Lq < kk; ++Lq) t += Ub[Lq * k + l] * b[r * kk + Lq];
-    sv[q] = t;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < kk * k * k; q += blockDim.x) {  // unfilter of s
-    const int I = q / (k * k), r = q % (k * k);
-    double t = 0.0;
-    for (int ii = 0; ii < k; ++ii) t += Ub[I * k + ii] * sv[ii * k * k + r];
-    c[q] = t;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < kk * kk * k; q += blockDim.x) {
-    const int I = q / (kk * k), J = (q / k) % kk, l = q % k;
-    double t = 0.0;
-    for (int j = 0; j < k; ++j) t += Ub[J * k + j] * c[(I * k + j) * k + l];
-    e[q] = t;
-  }
-  __syncthreads();
+  twoscale::up_rest(k, U, a, b, sv);
   double part = 0.0;
-  for (int q = threadIdx.x; q < kk3; q += blockDim.x) {
-    const int I = q / (kk * kk), J = (q / kk) % kk, Lq = q % kk;
-    double t = 0.0;
-    for (int l = 0; l < k; ++l) t += Ub[Lq * k + l] * e[(I * kk + J) * k + l];
-    const double dd = (s_smem ? S[q] : s_at(q)) - t;
-    part += dd * dd;
-  }
+  twoscale::down(k, U, sv, c, a, [&](int I, int J, int Lq, double v) {
+    const double dd = s_at(I, J, Lq) - v;
+    part = fma(dd, dd, part);
+  });
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
-  __shared__ int slot;
+  __shared__ int merge;
   if (threadIdx.x == 0) {
     double tot = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-    const bool merge = sqrt(tot) <= thresh;
-    slot = -1;
+    merge = sqrt(tot) <= thresh;
     if (merge) {
-      for (int cc = 0; cc < 8; ++cc) gone[idx[cc]] = 1;
-      d2[i] = tot;
-      slot = atomicAdd(pcount, 1);
-      pkeys[slot] = make_key(n - 1, x >> 1, y >> 1, z >> 1);
+      merged[j] = 1;
+      d2[j] = tot;
     }
   }
   __syncthreads();
-  if (slot >= 0)
-    for (int q = threadIdx.x; q < k3; q += blockDim.x) pv[(int64_t)slot * k3 + q] = sv[q];
+  if (!merge) return;
+  if (threadIdx.x < 8) {
+    const int64_t q = child[8 * j + threadIdx.x];
+    gone[q >= 0 ? q : n_in + (-2 - q)] = 1;
+  }
+  for (int q = threadIdx.x; q < k3; q += blockDim.x) pv[j * k3 + q] = sv[q];
 }
 
-__global__ void keep_flags_kernel(int64_t n, const uint64_t *keys, const int *gone, int *keep) {
+// Survivors, entries as gone's (leaves, then candidates), one more entry of zero.
+__global__ void keep_flags_kernel(int64_t n_in, int64_t nc, const int *gone, const int *merged, int *keep) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) keep[i] = gone[i] || keys[i] == ~0ull ? 0 : 1;  // the largest key pads the level
+  if (i > n_in + nc) return;
+  keep[i] = i < n_in + nc && !gone[i] && (i < n_in || merged[i - n_in]) ? 1 : 0;
 }
-// the level's survivor count and merged squared detail into per-level slots
-__global__ void level_totals_kernel(const int *kpos, int64_t nl, const double *dsum, int n, int *cnt, double *d2l) {
-  cnt[n] = kpos[nl];
-  d2l[n] = *dsum;
+
+// One CTA per entry: a survivor to its place among all survivors in key order, its rank among its own kind
+// plus the survivors of the other kind with smaller keys (pos: exclusive sum of keep).
+__global__ void emit_kept_kernel(int64_t n_in, int64_t nc, int k3, const uint64_t *keys, const double *coeffs,
+                                 const uint64_t *cand, const double *pv, const int *keep, const int *pos, int64_t cap,
+                                 uint64_t *okeys, double *ocoeffs) {
+  const int64_t i = blockIdx.x;
+  if (!keep[i]) return;
+  const bool leaf = i < n_in;
+  const uint64_t key = leaf ? keys[i] : cand[i - n_in];
+  const uint64_t *other = leaf ? cand : keys;
+  int64_t lo = 0, hi = leaf ? nc : n_in;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (other[mid] < key) lo = mid + 1; else hi = mid;
+  }
+  const int64_t o = leaf ? (int64_t)pos[i] + pos[n_in + lo] - pos[n_in] : (int64_t)pos[i] - pos[n_in] + pos[lo];
+  if (o >= cap) return;
+  const double *v = leaf ? coeffs + i * k3 : pv + (i - n_in) * k3;
+  if (threadIdx.x == 0) okeys[o] = key;
+  for (int e = threadIdx.x; e < k3; e += blockDim.x) ocoeffs[o * k3 + e] = v[e];
+}
+
+// Sum of v in a fixed order, one CTA.
+__global__ void sum_kernel(int64_t n, const double *v, double *out) {
+  __shared__ double red[32];
+  double t = 0.0;
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) t += v[i];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double w = 0.0;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) w += red[q];
+    *out = w;
+  }
 }
 
 inline size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -873,14 +852,13 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
   if (herr) return fail(MRA_ERR_ARG, "mra_apply_ns: the input is not every box of level %d in key order", N);
 
   // ---- compress: S^n and s^n for n = N-1 .. n0
-  const size_t sh_c = (size_t)(kk3 + k * kk * kk + k * k * kk) * 8;
-  const size_t sh_d = (size_t)(k3 + kk * k * k + kk * kk * k) * 8;
+  const size_t sh_c = up_smem(k), sh_d = down_smem(k);
   MRA_CUDA_TRY(cudaFuncSetAttribute(compress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_c));
   MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
   double *s_all = (double *)(w + Lw.s), *S_all = (double *)(w + Lw.S);
   for (int n = N - 1; n >= n0; --n) {
     const double *fine = n == N - 1 ? in->coeffs : s_all + Lw.first[n + 1] * k3;
-    compress_kernel<<<counted((unsigned)boxes(n)), 256, sh_c, s>>>(k, n, fine, Ub, S_all + Lw.first[n] * kk3,
+    compress_kernel<<<counted((unsigned)boxes(n)), BOX_THREADS, sh_c, s>>>(k, n, fine, Ub, S_all + Lw.first[n] * kk3,
                                                                    s_all + Lw.first[n] * k3);
     MRA_CUDA_TRY(cudaGetLastError());
     level_keys_kernel<<<counted((unsigned)((boxes(n) + 255) / 256)), 256, 0, s>>>(n, boxes(n), keys + Lw.first[n]);
@@ -945,7 +923,7 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
   if (rc != MRA_OK) return rc;
   for (int n = n0; n < N; ++n) {
     double *fine = n == N - 1 ? out->coeffs : rnext;
-    sum_down_kernel<<<counted((unsigned)boxes(n)), 256, sh_d, s>>>(k, n, rcur, Z + Lw.first[n] * k3, Y + Lw.first[n] * kk3, Ub,
+    sum_down_kernel<<<counted((unsigned)boxes(n)), BOX_THREADS, sh_d, s>>>(k, n, rcur, Z + Lw.first[n] * k3, Y + Lw.first[n] * kk3, Ub,
                                                                    fine);
     MRA_CUDA_TRY(cudaGetLastError());
     std::swap(rcur, rnext);
@@ -1162,8 +1140,7 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
   }
 
   // ---- compress, from the deepest interior level up; all levels' S and s back to back in key order
-  const size_t sh_c = (size_t)(kk * kk * kk + k * kk * kk + k * k * kk) * 8;
-  const size_t sh_d = (size_t)(k3 + kk * k * k + kk * kk * k) * 8;
+  const size_t sh_c = up_smem(k), sh_d = down_smem(k);
   const int kk3 = kk * kk * kk;
   MRA_CUDA_TRY(cudaFuncSetAttribute(compress_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_c));
   MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
@@ -1172,7 +1149,7 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
   auto first = [&](int n) { return off_int[n] - off_int[n0]; };
   for (int n = Nmax - 1; n >= n0; --n) {
     const bool deeper = n + 1 < Nmax;
-    compress_tree_kernel<<<counted((unsigned)In[n]), 256, sh_c, s>>>(
+    compress_tree_kernel<<<counted((unsigned)In[n]), BOX_THREADS, sh_c, s>>>(
         k, n, Ik[n], In[n], in->keys, in->coeffs, n_leaf, deeper ? Ik[n + 1] : nullptr,
         deeper ? s_all + first(n + 1) * k3 : nullptr, deeper ? In[n + 1] : 0, Ub, S_all + first(n) * kk3,
         s_all + first(n) * k3, d_int);
@@ -1264,7 +1241,7 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
   for (int n = n0; n < Nmax; ++n) {
     const int64_t j0 = hoff[n], nj = hoff[n + 1] - hoff[n];
     if (nj == 0) continue;
-    sum_down_tree_kernel<<<counted((unsigned)nj), 256, sh_d, s>>>(k, j0, r, yi, yc, zi, zc, dst, Ub, out->coeffs);
+    sum_down_tree_kernel<<<counted((unsigned)nj), BOX_THREADS, sh_d, s>>>(k, j0, r, yi, yc, zi, zc, dst, Ub, out->coeffs);
     MRA_CUDA_TRY(cudaGetLastError());
   }
   MRA_CUDA_TRY(cudaMemcpyAsync(hint, d_int, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1321,166 +1298,98 @@ extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void
   if (!var) return fail(MRA_ERR_CUDA, "mra_reconstruct: out of device memory (%s)", #var);
 
   // order and the level ranges of the sorted input
-  std::vector<uint64_t> hk(n_in);
-  MRA_CUDA_TRY(cudaMemcpyAsync(hk.data(), in->keys, (size_t)n_in * 8, cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaStreamSynchronize(s));
-  std::vector<int64_t> lo(21, n_in), hi(21, n_in);
-  for (int64_t i = 0; i < n_in; ++i) {
-    if (i > 0 && hk[i] <= hk[i - 1]) return fail(MRA_ERR_ARG, "mra_reconstruct: keys must be sorted and unique");
-    const int lv = key_level(hk[i]);
-    if (lv > 19) return fail(MRA_ERR_ARG, "mra_reconstruct: level %d above 19", lv);
-  }
-  for (int n = 0; n <= 20; ++n) {
-    lo[n] = std::lower_bound(hk.begin(), hk.end(), (uint64_t)n << 57) - hk.begin();
-    hi[n] = n < 20 ? std::lower_bound(hk.begin(), hk.end(), (uint64_t)(n + 1) << 57) - hk.begin() : n_in;
-  }
-  const int nmin = key_level(hk.front()), nmax = key_level(hk.back());
-  RC_ALLOC(Ub, double, kk * k);
-  std::vector<double> U(2 * k * k), Ubh(2 * k * k);
-  two_scale(k, U.data());
-  for (int c = 0; c < 2; ++c)
-    for (int i = 0; i < k; ++i)
-      for (int j = 0; j < k; ++j) Ubh[(c * k + i) * k + j] = U[c * k * k + i * k + j];
-  MRA_CUDA_TRY(cudaMemcpyAsync(Ub, Ubh.data(), Ubh.size() * 8, cudaMemcpyHostToDevice, s));
+  RC_ALLOC(d_off, int64_t, 22);
+  MRA_CUDA_TRY(cudaMemsetAsync(d_off, 0, 22 * 8, s));
+  leaf_offsets_kernel<<<counted((unsigned)((n_in + 256) / 256)), 256, 0, s>>>(n_in, in->keys, d_off, d_off + 21);
+  MRA_CUDA_TRY(cudaGetLastError());
   RC_ALLOC(top, int, n_in);
   top_level_kernel<<<counted((unsigned)((n_in + 255) / 256)), 256, 0, s>>>(n_in, in->keys, top);
   MRA_CUDA_TRY(cudaGetLastError());
-  RC_ALLOC(d_err, int, 1);
-  MRA_CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), s));
-  // Every size of the level loop is known in advance, so the loop runs without a host
-  // synchronisation: the interior boxes of all levels (one sort), the tops of all levels
-  // (one scan), one copy to the host.  A level's boxes are the 8 children of the previous
-  // level's interior boxes and its tops; its interior boxes are exactly the interior keys of
-  // the level (checked on the device), the others are leaves of the result.
+  RC_ALLOC(Ub, double, kk * k);
+  std::vector<double> U(2 * k * k);
+  two_scale(k, U.data());  // [c][i][j]: the rows (c, i) of Ubar in order
+  MRA_CUDA_TRY(cudaMemcpyAsync(Ub, U.data(), U.size() * 8, cudaMemcpyHostToDevice, s));
+  int64_t off[22];
+  MRA_CUDA_TRY(cudaMemcpyAsync(off, d_off, 22 * 8, cudaMemcpyDeviceToHost, s));
+  MRA_CUDA_TRY(cudaStreamSynchronize(s));
+  if (off[21] == 2) return fail(MRA_ERR_ARG, "mra_reconstruct: level above %d", MRA_MAX_LEVEL);
+  if (off[21]) return fail(MRA_ERR_ARG, "mra_reconstruct: keys must be sorted and unique");
+  int nmin = 0, nmax = MRA_MAX_LEVEL;
+  while (off[nmin + 1] == 0) ++nmin;
+  while (off[nmax] == n_in) --nmax;
+  // The result's tree depends on the keys alone: the interior boxes of all levels (one sort), their children and
+  // the tops that stay leaves (one sort for the leaves' order).  Then each level is one kernel that
+  // passes its interior boxes' sums down into the next level's or to the leaves' places.
   const int nlev = std::max(nmax - nmin, 1);
   if (n_in * nlev >= (int64_t)INT32_MAX) return fail(MRA_ERR_ARG, "mra_reconstruct: too many boxes x levels");
   const int64_t na = n_in * nlev;
   RC_ALLOC(anc, uint64_t, na);
   RC_ALLOC(iall, uint64_t, na);
-  RC_ALLOC(d_nsel, int64_t, 1);
-  RC_ALLOC(d_ioff, int64_t, 21);
-  RC_ALLOC(tflag, int, n_in + 1);
-  RC_ALLOC(tpos, int, n_in + 1);
+  RC_ALLOC(d_info, int64_t, 24);  // offsets of the interior levels, then tops, interior tops, interior boxes
+  MRA_CUDA_TRY(cudaMemsetAsync(d_info, 0, 24 * 8, s));
+  int64_t *d_ni = d_info + 23;
   interior_all_kernel<<<counted((unsigned)((na + 255) / 256)), 256, 0, s>>>(n_in, in->keys, top, nmin, nlev, anc);
   MRA_CUDA_TRY(cudaGetLastError());
-  top_flags_kernel<<<counted((unsigned)((n_in + 256) / 256)), 256, 0, s>>>(n_in, in->keys, top, tflag);
-  MRA_CUDA_TRY(cudaGetLastError());
   {
-    size_t tb = 0, t2 = 0, t3 = 0;
+    size_t tb = 0, t2 = 0;
     MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, tb, anc, iall, (int)na, 0, 64, s));
-    MRA_CUDA_TRY(cub::DeviceSelect::Unique(nullptr, t2, iall, anc, d_nsel, (int)na, s));
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, t3, tflag, tpos, (int)(n_in + 1), s));
-    tb = std::max(tb, std::max(t2, t3));
+    MRA_CUDA_TRY(cub::DeviceSelect::Unique(nullptr, t2, iall, anc, d_ni, (int)na, s));
+    tb = std::max(tb, t2);
     RC_ALLOC(tmp, unsigned char, tb);
     size_t tt = tb;
     MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(tmp, tt, anc, iall, (int)na, 0, 64, s));
     tt = tb;
-    MRA_CUDA_TRY(cub::DeviceSelect::Unique(tmp, tt, iall, anc, d_nsel, (int)na, s));
-    tt = tb;
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp, tt, tflag, tpos, (int)(n_in + 1), s));
+    MRA_CUDA_TRY(cub::DeviceSelect::Unique(tmp, tt, iall, anc, d_ni, (int)na, s));
     drop(tmp);
   }
-  uint64_t *ik_all = anc;  // the unique interior keys, in key order (so level by level)
-  level_offsets_kernel<<<counted(1), 32, 0, s>>>(ik_all, d_nsel, d_ioff);
+  const uint64_t *ik = anc;  // the unique interior keys, in key order (so level by level)
+  level_offsets_kernel<<<counted(1), 32, 0, s>>>(ik, d_ni, d_info);
   MRA_CUDA_TRY(cudaGetLastError());
-  std::vector<int64_t> ioff(21);
-  std::vector<int> tposh(n_in + 1);
-  MRA_CUDA_TRY(cudaMemcpyAsync(ioff.data(), d_ioff, 21 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaMemcpyAsync(tposh.data(), tpos, (size_t)(n_in + 1) * sizeof(int), cudaMemcpyDeviceToHost, s));
+  count_tops_kernel<<<counted((unsigned)((n_in + 255) / 256)), 256, 0, s>>>(n_in, in->keys, top, ik, d_info + 20,
+                                                                            (unsigned long long *)(d_info + 21));
+  MRA_CUDA_TRY(cudaGetLastError());
+  int64_t info[24];
+  MRA_CUDA_TRY(cudaMemcpyAsync(info, d_info, 24 * 8, cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
   drop(iall);
-  const size_t sh_d = (size_t)(k3 + kk * k * k + kk * kk * k) * 8;
-  MRA_CUDA_TRY(cudaFuncSetAttribute(pass_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
-  uint64_t *Ck = nullptr;  // boxes passed down to the current level (unsorted) and their values
-  double *Cv = nullptr;
-  int64_t nC = 0, nout = 0;
-  const int64_t cap = out->cap;
-  for (int n = nmin; n <= nmax; ++n) {
-    const int64_t ni = ioff[n + 1] - ioff[n];  // interior boxes of level n
-    const uint64_t *ik = ik_all + ioff[n];
-    // the level's boxes: passed down, then the tops of this level; in key order
-    const int64_t nl = hi[n] - lo[n];
-    const int ntop = tposh[hi[n]] - tposh[lo[n]];
-    const int64_t nr = nC + ntop;
-    RC_ALLOC(uk, uint64_t, nr);
-    RC_ALLOC(uv, double, nr * k3);
-    if (nC > 0) {
-      MRA_CUDA_TRY(cudaMemcpyAsync(uk, Ck, (size_t)nC * 8, cudaMemcpyDeviceToDevice, s));
-      MRA_CUDA_TRY(cudaMemcpyAsync(uv, Cv, (size_t)nC * k3 * 8, cudaMemcpyDeviceToDevice, s));
-    }
-    if (ntop > 0) {
-      tops_kernel<<<counted((unsigned)nl), 128, 0, s>>>(lo[n], hi[n], n, top, in->keys, in->coeffs, k3, tpos,
-                                                        tposh[lo[n]], nC, uk, uv);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    RC_ALLOC(rk, uint64_t, nr);
-    RC_ALLOC(rv, double, nr * k3);
-    RC_ALLOC(idx, int, nr);
-    RC_ALLOC(idx_s, int, nr);
-    if (nr > 0) {
-      iota_ns_kernel<<<counted((unsigned)((nr + 255) / 256)), 256, 0, s>>>(nr, idx);
-      MRA_CUDA_TRY(cudaGetLastError());
-      size_t tsp = 0;
-      MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tsp, uk, rk, idx, idx_s, (int)nr, 0, 64, s));
-      RC_ALLOC(tmp4, unsigned char, tsp);
-      MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp4, tsp, uk, rk, idx, idx_s, (int)nr, 0, 64, s));
-      gather_rows_ns_kernel<<<counted((unsigned)nr), 128, 0, s>>>(nr, k3, idx_s, uv, rv);
-      MRA_CUDA_TRY(cudaGetLastError());
-      drop(tmp4);
-    }
-    if (nl > 0) {  // input boxes below a top add their coefficients
-      add_inputs_kernel<<<counted((unsigned)nl), 128, 0, s>>>(lo[n], hi[n], n, top, in->keys, in->coeffs, k3, rk, nr, rv, d_err);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    // leaves out, interior boxes passed down
-    RC_ALLOC(inner, int, nr + 1);
-    RC_ALLOC(leaf, int, nr + 1);
-    RC_ALLOC(ipos, int, nr + 1);
-    RC_ALLOC(lpos, int, nr + 1);
-    MRA_CUDA_TRY(cudaMemsetAsync(inner + nr, 0, sizeof(int), s));
-    MRA_CUDA_TRY(cudaMemsetAsync(leaf + nr, 0, sizeof(int), s));
-    if (nr > 0) {
-      classify_kernel<<<counted((unsigned)((nr + 255) / 256)), 256, 0, s>>>(nr, rk, ik, ni, inner, leaf);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    size_t tsc = 0;
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tsc, inner, ipos, (int)(nr + 1), s));
-    RC_ALLOC(tmp5, unsigned char, tsc);
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp5, tsc, inner, ipos, (int)(nr + 1), s));
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp5, tsc, leaf, lpos, (int)(nr + 1), s));
-    inner_count_check_kernel<<<counted(1), 1, 0, s>>>(ipos, nr, ni, d_err);
-    MRA_CUDA_TRY(cudaGetLastError());
-    if (nr - ni > 0) {
-      emit_leaves_kernel<<<counted((unsigned)nr), 128, 0, s>>>(nr, k3, rk, rv, leaf, lpos, nout, cap, out->keys, out->coeffs);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    nout += std::max<int64_t>(nr - ni, 0);
-    const int64_t nnext = 8 * ni;
-    RC_ALLOC(nk, uint64_t, nnext);
-    RC_ALLOC(nv, double, nnext * k3);
-    if (ni > 0 && nr > 0) {
-      pass_down_kernel<<<counted((unsigned)nr), 256, sh_d, s>>>(k, nr, rk, rv, inner, ipos, ni, Ub, nk, nv, d_err);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    for (void *p : {(void *)uk, (void *)uv, (void *)rk, (void *)rv, (void *)idx, (void *)idx_s, (void *)inner,
-                    (void *)leaf, (void *)ipos, (void *)lpos, (void *)tmp5})
-      drop(p);
-    if (Ck) drop(Ck);
-    if (Cv) drop(Cv);
-    Ck = nk;
-    Cv = nv;
-    nC = nnext;
-  }
-  int herr = 0;
-  MRA_CUDA_TRY(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaStreamSynchronize(s));
-  if (herr == 1) return fail(MRA_ERR_NUMERIC, "mra_reconstruct: an input box has no place in the result");
-  if (herr) return fail(MRA_ERR_NUMERIC, "mra_reconstruct: the interior boxes of a level are inconsistent");
-  if (nC != 0) return fail(MRA_ERR_NUMERIC, "mra_reconstruct: boxes passed below the deepest level");
-  if (nout > cap) {
+  const int64_t ni = info[20], ntop = info[21], itop = info[22];
+  const int64_t nout = 8 * ni - (ni - itop) + (ntop - itop);
+  if (nout > out->cap) {
     out->n = nout;
-    return fail(MRA_ERR_CAPACITY, "mra_reconstruct: %lld leaves, capacity %lld", (long long)nout, (long long)cap);
+    return fail(MRA_ERR_CAPACITY, "mra_reconstruct: %lld leaves, capacity %lld", (long long)nout, (long long)out->cap);
   }
+  const int64_t nn = 8 * ni + n_in;
+  if (nn >= (int64_t)INT32_MAX) return fail(MRA_ERR_ARG, "mra_reconstruct: too many boxes in the result");
+  RC_ALLOC(dst, int64_t, nn);
+  RC_ALLOC(own, int64_t, 8 * ni);
+  RC_ALLOC(iown, int64_t, ni);
+  RC_ALLOC(start, unsigned char, ni);
+  RC_ALLOC(lk, uint64_t, nn);
+  RC_ALLOC(lks, uint64_t, nn);
+  RC_ALLOC(id, int, nn);
+  RC_ALLOC(ids, int, nn);
+  size_t tb = 0;
+  MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, lk, lks, id, ids, (int)nn, 0, 64, s));
+  RC_ALLOC(tmp, unsigned char, tb);
+  recon_nodes_kernel<<<counted((unsigned)((nn + 255) / 256)), 256, 0, s>>>(ni, ik, n_in, in->keys, top, dst, own, iown, start,
+                                                                           lk, id);
+  MRA_CUDA_TRY(cudaGetLastError());
+  MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp, tb, lk, lks, id, ids, (int)nn, 0, 64, s));
+  leaf_places_kernel<<<counted((unsigned)((nout + 255) / 256)), 256, 0, s>>>(nout, lks, ids, dst, out->keys);
+  MRA_CUDA_TRY(cudaGetLastError());
+  copy_tops_kernel<<<counted((unsigned)n_in), 128, 0, s>>>(n_in, 8 * ni, k3, dst, in->coeffs, out->coeffs);
+  MRA_CUDA_TRY(cudaGetLastError());
+  const size_t sh_d = down_smem(k);
+  MRA_CUDA_TRY(cudaFuncSetAttribute(pass_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
+  RC_ALLOC(r, double, ni * k3);
+  for (int n = nmin; n < nmax; ++n) {
+    const int64_t nj = info[n + 1] - info[n];
+    if (nj == 0) continue;
+    pass_down_kernel<<<counted((unsigned)nj), BOX_THREADS, sh_d, s>>>(k, info[n], r, iown, start, dst, own, in->coeffs, Ub,
+                                                              out->coeffs);
+    MRA_CUDA_TRY(cudaGetLastError());
+  }
+  MRA_CUDA_TRY(cudaStreamSynchronize(s));
   out->n = nout;
   return MRA_OK;
 #undef RC_ALLOC
@@ -1524,134 +1433,84 @@ extern "C" int mra_truncate(const mra_tree_view *in, double thresh, mra_tree_vie
   type *var = (type *)dalloc((size_t)(count) * sizeof(type));                                   \
   if (!var) return fail(MRA_ERR_CUDA, "mra_truncate: out of device memory (%s)", #var);
 
-  std::vector<uint64_t> hk(n_in);
-  MRA_CUDA_TRY(cudaMemcpyAsync(hk.data(), in->keys, (size_t)n_in * 8, cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaStreamSynchronize(s));
-  for (int64_t i = 1; i < n_in; ++i)
-    if (hk[i] <= hk[i - 1]) return fail(MRA_ERR_ARG, "mra_truncate: keys must be sorted and unique");
-  if (key_level(hk.back()) > 19) return fail(MRA_ERR_ARG, "mra_truncate: level above 19");
-  std::vector<int64_t> lo(21), hi(21);
-  for (int n = 0; n <= 20; ++n) {
-    lo[n] = std::lower_bound(hk.begin(), hk.end(), (uint64_t)n << 57) - hk.begin();
-    hi[n] = n < 20 ? std::lower_bound(hk.begin(), hk.end(), (uint64_t)(n + 1) << 57) - hk.begin() : n_in;
-  }
   TR_ALLOC(Ub, double, kk * k);
-  std::vector<double> U(2 * k * k), Ubh(2 * k * k);
-  two_scale(k, U.data());
-  for (int c = 0; c < 2; ++c)
-    for (int i = 0; i < k; ++i)
-      for (int j = 0; j < k; ++j) Ubh[(c * k + i) * k + j] = U[c * k * k + i * k + j];
-  MRA_CUDA_TRY(cudaMemcpyAsync(Ub, Ubh.data(), Ubh.size() * 8, cudaMemcpyHostToDevice, s));
-  // S stays in shared memory up to k = 12 (120 k^3 bytes); above, only the filter's pieces (56 k^3)
-  const int s_smem = k <= 12 ? 1 : 0;
-  const size_t sh = (size_t)(k * kk * kk + k * k * kk + k3 + (s_smem ? kk * kk * kk : 0)) * 8;
-  MRA_CUDA_TRY(cudaFuncSetAttribute(truncate_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-  TR_ALLOC(pcount, int, 1);
-  TR_ALLOC(d_cnt, int, 20);
-  TR_ALLOC(d_d2l, double, 20);
-  MRA_CUDA_TRY(cudaMemsetAsync(d_cnt, 0, 20 * sizeof(int), s));
-  MRA_CUDA_TRY(cudaMemsetAsync(d_d2l, 0, 20 * sizeof(double), s));
-  // The level loop runs without a host synchronisation.  The parents merged from level n+1
-  // are at most an eighth of that level's leaves, so every array is sized by that bound; the
-  // merged parents are written at atomic slots of an array prefilled with the largest key,
-  // which sorts after every real key, is never a leaf of a sibling group and is not kept.
-  // The survivors of each level stay on the device until the counts are read at the end.
-  std::vector<uint64_t *> keep_k(20, nullptr);
-  std::vector<double *> keep_v(20, nullptr);
-  uint64_t *mk = nullptr;  // parents merged from the level below (unsorted, padded)
-  double *mv = nullptr;
-  int64_t nm = 0;  // bound on their number
-  const int top = key_level(hk.back());
-  for (int n = top; n >= 0; --n) {
-    // this level's leaves: the input's, then the merged parents, in key order
-    const int64_t ni = hi[n] - lo[n], nl = ni + nm;
-    if (nl == 0) continue;
-    TR_ALLOC(uk, uint64_t, nl);
-    TR_ALLOC(uv, double, nl * k3);
-    if (ni > 0) {
-      MRA_CUDA_TRY(cudaMemcpyAsync(uk, in->keys + lo[n], (size_t)ni * 8, cudaMemcpyDeviceToDevice, s));
-      MRA_CUDA_TRY(cudaMemcpyAsync(uv, in->coeffs + lo[n] * k3, (size_t)ni * k3 * 8, cudaMemcpyDeviceToDevice, s));
-    }
-    if (nm > 0) {
-      MRA_CUDA_TRY(cudaMemcpyAsync(uk + ni, mk, (size_t)nm * 8, cudaMemcpyDeviceToDevice, s));
-      MRA_CUDA_TRY(cudaMemcpyAsync(uv + ni * k3, mv, (size_t)nm * k3 * 8, cudaMemcpyDeviceToDevice, s));
-    }
-    TR_ALLOC(lk, uint64_t, nl);
-    TR_ALLOC(lv, double, nl * k3);
-    TR_ALLOC(idx, int, nl);
-    TR_ALLOC(idx_s, int, nl);
-    iota_ns_kernel<<<counted((unsigned)((nl + 255) / 256)), 256, 0, s>>>(nl, idx);
-    MRA_CUDA_TRY(cudaGetLastError());
-    size_t tsp = 0;
-    MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tsp, uk, lk, idx, idx_s, (int)nl, 0, 64, s));
-    TR_ALLOC(tmp, unsigned char, tsp);
-    MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp, tsp, uk, lk, idx, idx_s, (int)nl, 0, 64, s));
-    gather_rows_ns_kernel<<<counted((unsigned)nl), 128, 0, s>>>(nl, k3, idx_s, uv, lv);
-    MRA_CUDA_TRY(cudaGetLastError());
-    // merges into level n-1
-    TR_ALLOC(gone, int, nl + 1);
-    TR_ALLOC(d2, double, nl);
-    MRA_CUDA_TRY(cudaMemsetAsync(gone, 0, (size_t)(nl + 1) * sizeof(int), s));
-    MRA_CUDA_TRY(cudaMemsetAsync(d2, 0, (size_t)nl * 8, s));
-    MRA_CUDA_TRY(cudaMemsetAsync(pcount, 0, sizeof(int), s));
-    const int64_t np_max = n > 0 ? nl / 8 : 0;
-    TR_ALLOC(pk, uint64_t, np_max + 1);
-    TR_ALLOC(pv, double, (np_max + 1) * k3);
-    MRA_CUDA_TRY(cudaMemsetAsync(pk, 0xFF, (size_t)(np_max + 1) * 8, s));
-    if (n > 0) {
-      truncate_level_kernel<<<counted((unsigned)nl), 256, sh, s>>>(k, n, nl, lk, lv, thresh, Ub, gone, d2, pk, pv, pcount,
-                                                                   s_smem);
-      MRA_CUDA_TRY(cudaGetLastError());
-    }
-    // survivors, compacted in key order
-    TR_ALLOC(keep, int, nl + 1);
-    TR_ALLOC(kpos, int, nl + 1);
-    keep_flags_kernel<<<counted((unsigned)((nl + 255) / 256)), 256, 0, s>>>(nl, lk, gone, keep);
-    MRA_CUDA_TRY(cudaGetLastError());
-    MRA_CUDA_TRY(cudaMemsetAsync(keep + nl, 0, sizeof(int), s));
-    size_t tsc = 0;
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tsc, keep, kpos, (int)(nl + 1), s));
-    size_t tsr = 0;
-    double *dsum = nullptr;
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(nullptr, tsr, d2, dsum, (int)nl, s));
-    TR_ALLOC(tmp2, unsigned char, std::max(tsc, tsr));
-    TR_ALLOC(dsum_d, double, 1);
-    MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp2, tsc, keep, kpos, (int)(nl + 1), s));
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(tmp2, tsr, d2, dsum_d, (int)nl, s));
-    level_totals_kernel<<<counted(1), 1, 0, s>>>(kpos, nl, dsum_d, n, d_cnt, d_d2l);
-    MRA_CUDA_TRY(cudaGetLastError());
-    TR_ALLOC(kk_, uint64_t, nl);
-    TR_ALLOC(kv, double, nl * k3);
-    emit_leaves_kernel<<<counted((unsigned)nl), 128, 0, s>>>(nl, k3, lk, lv, keep, kpos, 0, nl, kk_, kv);
-    MRA_CUDA_TRY(cudaGetLastError());
-    keep_k[n] = kk_;
-    keep_v[n] = kv;
-    mk = pk;
-    mv = pv;
-    nm = np_max;
-  }
-  std::vector<int> keep_n(20);
-  std::vector<double> d2l(20);
-  MRA_CUDA_TRY(cudaMemcpyAsync(keep_n.data(), d_cnt, 20 * sizeof(int), cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaMemcpyAsync(d2l.data(), d_d2l, 20 * sizeof(double), cudaMemcpyDeviceToHost, s));
+  std::vector<double> U(2 * k * k);
+  two_scale(k, U.data());  // [c][i][j]: the rows (c, i) of Ubar in order
+  MRA_CUDA_TRY(cudaMemcpyAsync(Ub, U.data(), U.size() * 8, cudaMemcpyHostToDevice, s));
+  // The boxes where a merge is possible are known from the keys (their low corner is a leaf's); sorted once,
+  // they are worked through from the deepest level up, one kernel per level.
+  TR_ALLOC(d_info, int64_t, 44);  // leaf level offsets [0..20], bad [21], candidates [22], per level [23..42]
+  MRA_CUDA_TRY(cudaMemsetAsync(d_info, 0, 44 * 8, s));
+  leaf_offsets_kernel<<<counted((unsigned)((n_in + 256) / 256)), 256, 0, s>>>(n_in, in->keys, d_info, d_info + 21);
+  MRA_CUDA_TRY(cudaGetLastError());
+  int64_t info[44];
+  MRA_CUDA_TRY(cudaMemcpyAsync(info, d_info, 22 * 8, cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
+  if (info[21] == 2) return fail(MRA_ERR_ARG, "mra_truncate: level above 19");
+  if (info[21]) return fail(MRA_ERR_ARG, "mra_truncate: keys must be sorted and unique");
+  // a level-l leaf proposes at most l boxes
+  int64_t nc_max = 0;
+  for (int l = 0; l < 20; ++l) nc_max += l * (info[l + 1] - info[l]);
+  TR_ALLOC(cand0, uint64_t, nc_max);
+  corner_parents_kernel<<<counted((unsigned)((n_in + 255) / 256)), 256, 0, s>>>(
+      n_in, in->keys, cand0, (unsigned long long *)(d_info + 22), (unsigned long long *)(d_info + 23));
+  MRA_CUDA_TRY(cudaGetLastError());
+  MRA_CUDA_TRY(cudaMemcpyAsync(info, d_info, 44 * 8, cudaMemcpyDeviceToHost, s));
+  MRA_CUDA_TRY(cudaStreamSynchronize(s));
+  const int64_t nc = info[22];
+  if (n_in + nc >= (int64_t)INT32_MAX) return fail(MRA_ERR_ARG, "mra_truncate: too many boxes");
+  TR_ALLOC(cand, uint64_t, nc);
+  TR_ALLOC(child, int64_t, 8 * nc);
+  TR_ALLOC(flags, int, n_in + 2 * nc);  // gone (leaves, candidates), merged
+  TR_ALLOC(d2, double, nc + 1);
+  TR_ALLOC(pv, double, nc * k3);
+  int *gone = flags, *merged = flags + n_in + nc;
+  MRA_CUDA_TRY(cudaMemsetAsync(flags, 0, (size_t)(n_in + 2 * nc) * sizeof(int), s));
+  MRA_CUDA_TRY(cudaMemsetAsync(d2, 0, (size_t)(nc + 1) * 8, s));
+  if (nc > 0) {
+    size_t tb = 0;
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(nullptr, tb, cand0, cand, (int)nc, 0, 62, s));
+    TR_ALLOC(tmp, unsigned char, tb);
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortKeys(tmp, tb, cand0, cand, (int)nc, 0, 62, s));
+    merge_children_kernel<<<counted((unsigned)((8 * nc + 255) / 256)), 256, 0, s>>>(nc, cand, n_in, in->keys, child);
+    MRA_CUDA_TRY(cudaGetLastError());
+    // S stays in shared memory up to k = 12 (96 k^3 bytes); above, only the filter's pieces (56 k^3)
+    const int s_smem = k <= 12 ? 1 : 0;
+    const size_t sh = s_smem ? up_smem(k) : down_smem(k);
+    MRA_CUDA_TRY(cudaFuncSetAttribute(truncate_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
+    int64_t end = nc;
+    for (int n = 19; n >= 0; --n) {
+      const int64_t here = info[23 + n];
+      if (here == 0) continue;
+      truncate_level_kernel<<<counted((unsigned)here), BOX_THREADS, sh, s>>>(k, end - here, n_in, child, in->coeffs, thresh, Ub,
+                                                                     gone, merged, d2, pv, s_smem);
+      MRA_CUDA_TRY(cudaGetLastError());
+      end -= here;
+    }
+  }
+  // survivors in key order
+  const int64_t ne = n_in + nc;
+  TR_ALLOC(keep, int, ne + 1);
+  TR_ALLOC(pos, int, ne + 1);
+  keep_flags_kernel<<<counted((unsigned)((ne + 256) / 256)), 256, 0, s>>>(n_in, nc, gone, merged, keep);
+  MRA_CUDA_TRY(cudaGetLastError());
+  size_t tsc = 0;
+  MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tsc, keep, pos, (int)(ne + 1), s));
+  TR_ALLOC(tmp2, unsigned char, tsc);
+  MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp2, tsc, keep, pos, (int)(ne + 1), s));
+  sum_kernel<<<counted(1), 1024, 0, s>>>(nc, d2, d2 + nc);
+  MRA_CUDA_TRY(cudaGetLastError());
+  emit_kept_kernel<<<counted((unsigned)ne), 128, 0, s>>>(n_in, nc, k3, in->keys, in->coeffs, cand, pv, keep, pos, out->cap,
+                                                         out->keys, out->coeffs);
+  MRA_CUDA_TRY(cudaGetLastError());
+  int nout = 0;
   double e2 = 0.0;
-  for (int n = top; n >= 0; --n) e2 += d2l[n];
-  int64_t nout = 0;
-  for (int n = 0; n < 20; ++n) nout += keep_n[n];
-  if (nout > out->cap) {
-    out->n = nout;
-    return fail(MRA_ERR_CAPACITY, "mra_truncate: %lld leaves, capacity %lld", (long long)nout, (long long)out->cap);
-  }
-  int64_t o = 0;
-  for (int n = 0; n < 20; ++n) {
-    if (keep_n[n] == 0) continue;
-    MRA_CUDA_TRY(cudaMemcpyAsync(out->keys + o, keep_k[n], (size_t)keep_n[n] * 8, cudaMemcpyDeviceToDevice, s));
-    MRA_CUDA_TRY(cudaMemcpyAsync(out->coeffs + o * k3, keep_v[n], (size_t)keep_n[n] * k3 * 8, cudaMemcpyDeviceToDevice, s));
-    o += keep_n[n];
-  }
+  MRA_CUDA_TRY(cudaMemcpyAsync(&nout, pos + ne, sizeof(int), cudaMemcpyDeviceToHost, s));
+  MRA_CUDA_TRY(cudaMemcpyAsync(&e2, d2 + nc, 8, cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
   out->n = nout;
+  if (nout > out->cap)
+    return fail(MRA_ERR_CAPACITY, "mra_truncate: %d leaves, capacity %lld", nout, (long long)out->cap);
   if (err2) *err2 = e2;
   return MRA_OK;
 #undef TR_ALLOC
