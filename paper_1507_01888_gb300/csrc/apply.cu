@@ -24,11 +24,6 @@ namespace mra {
 
 namespace {
 
-__global__ void iota_kernel(int64_t n, int *p) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = (int)i;
-}
-
 __global__ void square_kernel(int64_t n, const double *a, double *b) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) b[i] = a[i] * a[i];
@@ -109,9 +104,11 @@ struct ScreenArgs {
   int lfilter;
   float ltau_hi, ltau_lo;
   // several functions in one apply: boxes [fn_off[f], fn_off[f+1]) belong to function f,
-  // and records sort on (f, level, x, y, z) packed as f<<53 | n<<48 | x<<32 | y<<16 | z
+  // and records sort on (f, level, x, y, z)
   int nfunc;
   const int64_t *fn_off;
+  int nb, lb, lev0;           // destination sort keys: see sort_key
+  int *rec_idx;               // 0, 1, 2, ... (the sort's values)
 };
 
 // Margin (in log2) of the screen's FP32 filter.  The five FP32 logs of a bound are each within
@@ -128,13 +125,16 @@ __global__ void screen_log_tables_kernel(int64_t n_blocks, int M, const double *
   }
 }
 
-// Sort key of a destination box of function f in a batched apply (levels <= 15).
-__device__ __forceinline__ uint64_t batched_key(int f, int n, int64_t x, int64_t y, int64_t z) {
-  return ((uint64_t)f << 53) | ((uint64_t)n << 48) | ((uint64_t)x << 32) | ((uint64_t)y << 16) | (uint64_t)z;
+// Sort key of a destination box: (function, level - lev0, x, y, z) in as few bits as the operator's levels
+// need (nb per coordinate, lb for the level), so that the radix sort makes fewer passes: 9 bits instead of
+// 62 for whole trees of level 3 (two passes of eight bits for eight), 43 for levels 2 to 13.
+__device__ __forceinline__ uint64_t sort_key(int nb, int lb, int lev0, int f, int n, int64_t x, int64_t y, int64_t z) {
+  return ((((((uint64_t)f << lb) | (uint64_t)(n - lev0)) << nb | (uint64_t)x) << nb | (uint64_t)y) << nb) | (uint64_t)z;
 }
-__device__ __forceinline__ uint64_t public_key(uint64_t bk) {
-  return make_key((int)((bk >> 48) & 31), (int64_t)((bk >> 32) & 0xFFFF), (int64_t)((bk >> 16) & 0xFFFF),
-                  (int64_t)(bk & 0xFFFF));
+__device__ __forceinline__ uint64_t public_key(uint64_t k, int nb, int lb, int lev0) {
+  const uint64_t m = (1ull << nb) - 1;
+  return make_key((int)((k >> (3 * nb)) & ((1ull << lb) - 1)) + lev0, (int64_t)((k >> (2 * nb)) & m),
+                  (int64_t)((k >> nb) & m), (int64_t)(k & m));
 }
 
 // PASS 0 screens and counts (LEARNED: with the learned screen), PASS 1 writes the records.
@@ -198,8 +198,8 @@ __global__ void __launch_bounds__(256, LEARNED ? 1 : 2) screen_kernel(ScreenArgs
             if (!(m0 | m1)) continue;
             if (lane == 0) {
               const int64_t wp = MRA_IDX(wpos, a.rec_cap);
-              a.rec_key[wp] = a.nfunc > 1 ? batched_key(func, n, x + lx, y + ly, z + lz)
-                                          : make_key(n, x + lx, y + ly, z + lz);
+              a.rec_key[wp] = sort_key(a.nb, a.lb, a.lev0, func, n, x + lx, y + ly, z + lz);
+              a.rec_idx[wp] = (int)wp;
               a.rec_src[wp] = (int)b;
               a.rec_l[wp] = (lx + 128) | ((ly + 128) << 8) | ((lz + 128) << 16);
               a.rec_mask[2 * wp] = m0;
@@ -391,13 +391,13 @@ __global__ void head_flags_kernel(int64_t P, const uint64_t *skey, int *head) {
 
 __global__ void segments_kernel(int64_t P, const uint64_t *skey, const int *head,
                                 const int *dest_id /*inclusive scan*/, uint64_t *dest_key,
-                                int64_t *seg, int64_t *n_dest, int batched, int *dest_func) {
+                                int64_t *seg, int64_t *n_dest, int batched, int *dest_func, int nb, int lb, int lev0) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= P) return;
   if (head[i]) {
     int64_t d = dest_id[i] - 1;
-    dest_key[d] = batched ? public_key(skey[i]) : skey[i];
-    if (batched) dest_func[d] = (int)(skey[i] >> 53);
+    dest_key[d] = public_key(skey[i], nb, lb, lev0);
+    if (batched) dest_func[d] = (int)(skey[i] >> (3 * nb + lb));
     seg[d] = i;
   }
   if (i == P - 1) {
@@ -544,21 +544,101 @@ __global__ void compare_kernel(int64_t nt, const uint64_t *tk, const double *tc,
   }
 }
 
-// Per source level: boxes and kept triples (a shared-memory histogram per CTA, then one
-// integer atomic per level: the sums are exact whatever the order).
-__global__ void level_counts_kernel(int64_t n, const uint64_t *keys, const int64_t *kept, int64_t *lev) {
-  __shared__ unsigned long long hb[MRA_MAX_LEVEL + 1], ht[MRA_MAX_LEVEL + 1];
-  if (threadIdx.x <= MRA_MAX_LEVEL) hb[threadIdx.x] = ht[threadIdx.x] = 0ull;
-  __syncthreads();
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
-    const int l = key_level(keys[b]);
-    atomicAdd(&hb[l], 1ull);
-    atomicAdd(&ht[l], (unsigned long long)kept[b]);
+// The screen's totals, read by the host in one copy.
+struct ScreenTotals {
+  int64_t records;            // records of the last box's end
+  int64_t err;                // the screen's error word
+  int64_t kept, screened, truncated, learned;
+  double skipped, lbound;
+  int64_t lev_boxes[MRA_MAX_LEVEL + 1], lev_kept[MRA_MAX_LEVEL + 1];
+  unsigned int ticket;        // CTAs done
+};
+constexpr int TOTAL_CTAS = 128;  // most CTAs of screen_totals_kernel
+
+// All totals over the boxes in one pass: integer sums by atomics (exact in any order; a warp adds per level it
+// holds), the two FP64 sums per CTA into part[2 blockIdx], added in CTA order by the last CTA to finish.
+// *t is zero before the launch.  With stats = 0 only the record count and the error word.
+__global__ void screen_totals_kernel(int64_t n, const uint64_t *keys, const int64_t *cnt, const int64_t *off, const int *err,
+                                     const int64_t *kept, const int64_t *screened, const int *trunc,
+                                     const int64_t *learned, const double *skipped, const double *lbound, int stats,
+                                     double *part, ScreenTotals *t) {
+  __shared__ double rd[2][32];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    t->records = off[n - 1] + cnt[n - 1];
+    t->err = *err;
+  }
+  if (!stats) return;
+  auto add = [](int64_t *p, int64_t v) { atomicAdd((unsigned long long *)p, (unsigned long long)v); };
+  auto sum = [](int64_t v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  int64_t sk = 0, sc = 0, tr = 0, ln = 0;
+  double a = 0.0, b = 0.0;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride) {
+    const int64_t i = i0 + threadIdx.x;
+    int lev = -1;
+    int64_t kp = 0;
+    if (i < n) {
+      lev = key_level(keys[i]);
+      kp = kept[i];
+      sk += kp;
+      sc += screened[i];
+      tr += trunc[i];
+      ln += learned[i];
+      a += skipped[i];
+      b += lbound[i];
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, lev >= 0);
+    while (todo) {  // the levels this warp holds: one or two, the boxes being in key order
+      const int l = __shfl_sync(0xffffffffu, lev, __ffs(todo) - 1);
+      const unsigned mine = __ballot_sync(0xffffffffu, lev == l);
+      const int64_t k = sum(lev == l ? kp : 0);
+      if (lane == 0) {
+        add(&t->lev_boxes[l], __popc(mine));
+        add(&t->lev_kept[l], k);
+      }
+      todo &= ~mine;
+    }
+  }
+  sk = sum(sk);
+  sc = sum(sc);
+  tr = sum(tr);
+  ln = sum(ln);
+  a = warp_sum(a);
+  b = warp_sum(b);
+  if (lane == 0) {
+    add(&t->kept, sk);
+    add(&t->screened, sc);
+    add(&t->truncated, tr);
+    add(&t->learned, ln);
+    rd[0][warp] = a;
+    rd[1][warp] = b;
   }
   __syncthreads();
-  if (threadIdx.x <= MRA_MAX_LEVEL) {
-    if (hb[threadIdx.x]) atomicAdd((unsigned long long *)&lev[threadIdx.x], hb[threadIdx.x]);
-    if (ht[threadIdx.x]) atomicAdd((unsigned long long *)&lev[MRA_MAX_LEVEL + 1 + threadIdx.x], ht[threadIdx.x]);
+  if (threadIdx.x == 0) {
+    a = b = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      a += rd[0][w];
+      b += rd[1][w];
+    }
+    part[2 * blockIdx.x] = a;
+    part[2 * blockIdx.x + 1] = b;
+    __threadfence();
+    last = atomicAdd(&t->ticket, 1u) == gridDim.x - 1;
+    if (last) {
+      __threadfence();
+      a = b = 0.0;
+      for (int c = 0; c < (int)gridDim.x; ++c) {
+        a += __ldcg(part + 2 * c);
+        b += __ldcg(part + 2 * c + 1);
+      }
+      t->skipped = a;
+      t->lbound = b;
+    }
   }
 }
 
@@ -661,7 +741,7 @@ int64_t apply_max_records(const Operator &op, const mra_apply_opts &o, int64_t n
 //   CUB temp storage (max over scan / sort / reduce needs)
 struct Layout {
   size_t snorm, dstop, cnt, off, kept, screened, skipped, trunc, learned, lbound, bmask, ltab;
-  size_t rkey, rsrc, rl, rmask, skey, pin, pout, head, did, dkey, seg, ndest, dfunc, fnoff, lev, split, tmp;
+  size_t rkey, rsrc, rl, rmask, skey, pin, pout, head, did, dkey, seg, ndest, dfunc, fnoff, tot, split, tmp;
   size_t split_bytes, tmp_bytes, total;
 };
 
@@ -701,19 +781,17 @@ static Layout make_layout(int64_t n_in, int64_t P, int dmax, int64_t n_tab, bool
   L.ndest = take(8);
   L.dfunc = take(np * 4);
   L.fnoff = take((MRA_MAX_FUNCS + 1) * 8);
-  L.lev = take(2 * (MRA_MAX_LEVEL + 1) * 8);
+  L.tot = take(sizeof(ScreenTotals) + 2 * TOTAL_CTAS * sizeof(double));
   L.split_bytes = src_path ? std::max(split_workspace_bytes(np), src_workspace_bytes(nb)) : split_workspace_bytes(np);
   L.split = take(L.split_bytes);
   // CUB temporary storage: the largest of the calls below
-  size_t a = 0, b = 0, c = 0, d = 0, e = 0;
+  size_t a = 0, b = 0, c = 0;
   cub::DeviceScan::ExclusiveSum(nullptr, a, (int64_t *)nullptr, (int64_t *)nullptr, (int)nb);
   cub::DeviceScan::InclusiveSum(nullptr, b, (int *)nullptr, (int *)nullptr, (int)np);
   cub::DeviceRadixSort::SortPairs(nullptr, c, (uint64_t *)nullptr, (uint64_t *)nullptr,
                                   (int *)nullptr, (int *)nullptr, (int)np);
-  cub::DeviceReduce::Sum(nullptr, d, (double *)nullptr, (double *)nullptr, (int)nb);
-  cub::DeviceReduce::Sum(nullptr, e, (int64_t *)nullptr, (int64_t *)nullptr, (int)nb);
   size_t t = a;
-  for (size_t v : {b, c, d, e}) t = v > t ? v : t;
+  for (size_t v : {b, c}) t = v > t ? v : t;
   L.tmp_bytes = t;
   L.tmp = take(t);
   L.total = o;
@@ -771,7 +849,7 @@ struct WsPtrs {
   int64_t *seg, *ndest;
   int *dfunc;
   int64_t *fnoff;
-  int64_t *lev;  // per level: source boxes, kept triples
+  void *tot;  // ScreenTotals and its CTAs' partial sums
   void *tmp;
   size_t tmpb;
 };
@@ -805,10 +883,27 @@ static WsPtrs carve(const Layout &L, void *ws) {
   p.ndest = (int64_t *)(w + L.ndest);
   p.dfunc = (int *)(w + L.dfunc);
   p.fnoff = (int64_t *)(w + L.fnoff);
-  p.lev = (int64_t *)(w + L.lev);
+  p.tot = w + L.tot;
   p.tmp = w + L.tmp;
   p.tmpb = L.tmp_bytes;
   return p;
+}
+
+// Bits of the destination sort keys (sort_key) of an operator's levels and nfunc functions.
+struct KeyBits {
+  int nb, lb, bits;
+};
+static KeyBits key_bits(const Operator &op, int nfunc) {
+  auto need = [](uint64_t v) {  // bits that hold 0 .. v
+    int b = 0;
+    while (v >> b) ++b;
+    return b;
+  };
+  KeyBits k;
+  k.nb = nfunc > 1 ? std::min(op.max_level, 15) : op.max_level;  // coordinates below 2^level
+  k.lb = need((uint64_t)(op.max_level - op.min_level));
+  k.bits = std::max(1, 3 * k.nb + k.lb + need((uint64_t)(nfunc - 1)));
+  return k;
 }
 
 // Source norms, norm (and learned) screen, record counts, scan and record emission.
@@ -877,6 +972,11 @@ static int screen_run(const Operator &op, const mra_tree_view &in, const mra_app
   a.box_mask = w.bmask;
   a.nfunc = nfunc;
   a.fn_off = w.fnoff;
+  const KeyBits kb = key_bits(op, nfunc);
+  a.nb = kb.nb;
+  a.lb = kb.lb;
+  a.lev0 = op.min_level;
+  a.rec_idx = w.pin;
   const size_t ssm = a.mlp ? (size_t)MLP_NALL * sizeof(float) : 0;
   if (a.mlp)
     screen_kernel<0, true><<<counted(gboxes), 32 * wpb, ssm, s>>>(a);
@@ -896,59 +996,39 @@ static int screen_run(const Operator &op, const mra_tree_view &in, const mra_app
     *P_out = fx->P;
     return MRA_OK;
   }
-  // statistics reduced on the device (deterministic), read with the record count
-  int64_t *red_i = w.seg;  // seg is free until the segments pass
-  double *red_d = (double *)(w.seg + 4);
-  if (stats) {
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(tmp, tmpb, w.bkept, red_i + 0, (int)n_in, s));
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(tmp, tmpb, w.bscr, red_i + 1, (int)n_in, s));
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(tmp, tmpb, w.btrunc, (int *)(red_i + 2), (int)n_in, s));
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(tmp, tmpb, w.blearned, red_i + 3, (int)n_in, s));
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(tmp, tmpb, w.bskip, red_d, (int)n_in, s));
-    MRA_CUDA_TRY(cub::DeviceReduce::Sum(tmp, tmpb, w.blbound, red_d + 1, (int)n_in, s));
-    MRA_CUDA_TRY(cudaMemsetAsync(w.lev, 0, 2 * (MRA_MAX_LEVEL + 1) * sizeof(int64_t), s));
-    level_counts_kernel<<<counted((unsigned)std::min<int64_t>((n_in + 255) / 256, 1024)), 256, 0, s>>>(
-        n_in, in.keys, w.bkept, w.lev);
-    MRA_CUDA_TRY(cudaGetLastError());
-  }
-  int64_t h_last[2] = {0, 0};
-  int h_err = 0;
-  int64_t hs[4] = {0, 0, 0, 0};
-  double hd[2] = {0.0, 0.0};
-  int64_t hl[2 * (MRA_MAX_LEVEL + 1)] = {};
-  MRA_CUDA_TRY(cudaMemcpyAsync(&h_last[0], w.off + n_in - 1, 8, cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaMemcpyAsync(&h_last[1], w.cnt + n_in - 1, 8, cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaMemcpyAsync(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-  if (stats) {
-    MRA_CUDA_TRY(cudaMemcpyAsync(hs, red_i, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    MRA_CUDA_TRY(cudaMemcpyAsync(hd, red_d, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    MRA_CUDA_TRY(cudaMemcpyAsync(hl, w.lev, sizeof(hl), cudaMemcpyDeviceToHost, s));
-  }
+  // the record count, the error word and the statistics in one kernel and one copy
+  ScreenTotals *tot = (ScreenTotals *)w.tot;
+  MRA_CUDA_TRY(cudaMemsetAsync(tot, 0, sizeof(ScreenTotals), s));
+  const unsigned gt = stats ? (unsigned)std::min<int64_t>((n_in + 255) / 256, TOTAL_CTAS) : 1u;
+  screen_totals_kernel<<<counted(gt), 256, 0, s>>>(n_in, in.keys, w.cnt, w.off, d_err, w.bkept, w.bscr, w.btrunc, w.blearned,
+                                                   w.bskip, w.blbound, stats ? 1 : 0, (double *)(tot + 1), tot);
+  MRA_CUDA_TRY(cudaGetLastError());
+  ScreenTotals h{};
+  MRA_CUDA_TRY(cudaMemcpyAsync(&h, tot, sizeof(h), cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
+  const int64_t h_err = h.err;
   if (h_err == 3)
     return fail(MRA_ERR_UNSUPPORTED, "mra_apply_batched: levels above 15 are not supported");
   if (h_err)
     return fail(MRA_ERR_ARG, "mra_apply: an input box lies on a level the operator does not cover "
                 "(levels %d..%d)", op.min_level, op.max_level);
-  const int64_t P = h_last[0] + h_last[1];
+  const int64_t P = h.records;
   if (P > Pmax) return fail(MRA_ERR_CAPACITY, "mra_apply: internal record bound exceeded");
   if (stats) {
-    int ntr = 0;
-    memcpy(&ntr, &hs[2], sizeof(int));
     *stats = mra_apply_stats{};
     stats->n_in = n_in;
-    stats->terms_kept = hs[0];
-    stats->terms_screened = hs[1] - hs[3];  // the norm screen's drops; the model's are below
-    stats->sources_truncated = ntr;
-    stats->skipped_bound = hd[0];
+    stats->terms_kept = h.kept;
+    stats->terms_screened = h.screened - h.learned;  // the norm screen's drops; the model's are below
+    stats->sources_truncated = h.truncated;
+    stats->skipped_bound = h.skipped;
     stats->pairs = P;
-    stats->terms_issued = hs[0];
-    stats->terms_learned_skipped = hs[3];
-    stats->learned_skipped_bound = hd[1];
-    stats->algo_flops = (double)hs[0] * (6.0 * op.k * op.k * op.k * op.k + (double)op.k * op.k * op.k);
+    stats->terms_issued = h.kept;
+    stats->terms_learned_skipped = h.learned;
+    stats->learned_skipped_bound = h.lbound;
+    stats->algo_flops = (double)h.kept * (6.0 * op.k * op.k * op.k * op.k + (double)op.k * op.k * op.k);
     for (int n = 0; n <= MRA_MAX_LEVEL; ++n) {
-      stats->level_sources[n] = hl[n];
-      stats->level_terms_kept[n] = hl[MRA_MAX_LEVEL + 1 + n];
+      stats->level_sources[n] = h.lev_boxes[n];
+      stats->level_terms_kept[n] = h.lev_kept[n];
     }
   }
   if (P > 0) {
@@ -999,15 +1079,15 @@ int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts 
     return MRA_OK;
   }
   // sort record indices on the destination key
+  const KeyBits kb = key_bits(op, nfunc);
   {
     unsigned g = (unsigned)((P + 255) / 256);
-    iota_kernel<<<counted(g), 256, 0, s>>>(P, pin);
-    MRA_CUDA_TRY(cudaGetLastError());
-    MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmpb, rkey, skey, pin, pout, (int)P, 0, 64, s));
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmpb, rkey, skey, pin, pout, (int)P, 0, kb.bits, s));
     head_flags_kernel<<<counted(g), 256, 0, s>>>(P, skey, head);
     MRA_CUDA_TRY(cudaGetLastError());
     MRA_CUDA_TRY(cub::DeviceScan::InclusiveSum(tmp, tmpb, head, did, (int)P, s));
-    segments_kernel<<<counted(g), 256, 0, s>>>(P, skey, head, did, dkey, seg, ndest, nfunc > 1, W.dfunc);
+    segments_kernel<<<counted(g), 256, 0, s>>>(P, skey, head, did, dkey, seg, ndest, nfunc > 1, W.dfunc, kb.nb,
+                                                 kb.lb, op.min_level);
     MRA_CUDA_TRY(cudaGetLastError());
   }
   int64_t nd = 0;
@@ -1051,7 +1131,6 @@ int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts 
   wk.seg = seg;
   wk.perm = pout;
   wk.did = did;
-  wk.skey = skey;
   wk.rec_src = rsrc;
   wk.rec_l = rl;
   wk.rec_mask = rmask;

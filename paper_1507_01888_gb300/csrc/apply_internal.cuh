@@ -26,7 +26,6 @@ struct ApplyWork {
   const int64_t *seg;
   const int *perm;
   const int *did;             // 1-based destination index of each dest-sorted record
-  const uint64_t *skey;       // dest-sorted destination keys (one per record)
   const int *rec_src;
   const int *rec_l;
   const uint64_t *rec_mask;

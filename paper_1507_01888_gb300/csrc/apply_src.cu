@@ -701,10 +701,10 @@ __global__ void src_key_kernel(int64_t n, int G, const uint64_t *keys, const int
   sval[b] = (int)b;
 }
 
-// One thread: per level the first sorted position and the tile numbering; the tile count.
+// One warp: per level the first sorted position and the tile numbering; the tile count.  A lane searches the
+// bounds of its level, all lanes at once (one lane doing the 40 searches in turn took 27 us).
 __global__ void src_tiles_kernel(int64_t n, int G, const uint64_t *skey, int *lev_first, int *tile_base,
                                  int *n_tiles) {
-  if (threadIdx.x != 0) return;
   auto lower = [&](uint64_t v) {
     int64_t lo = 0, hi = n;
     while (lo < hi) {
@@ -713,21 +713,23 @@ __global__ void src_tiles_kernel(int64_t n, int G, const uint64_t *skey, int *le
     }
     return (int)lo;
   };
-  const int n_active = lower(~0ull);
-  int tiles = 0;
-  if (G == 1) {
-    lev_first[0] = 0;
-    tile_base[0] = 0;
-    tiles = n_active;
-  } else {
-    for (int l = 0; l <= MRA_MAX_LEVEL; ++l) {
-      const int f = lower((uint64_t)l << 32), e = min(lower((uint64_t)(l + 1) << 32), n_active);
-      lev_first[l] = f;
-      tile_base[l] = tiles;
-      tiles += (e - f + G - 1) / G;
-    }
+  static_assert(MRA_MAX_LEVEL + 2 <= 32, "a lane per level");
+  const int l = threadIdx.x;
+  // lanes 0 .. MRA_MAX_LEVEL + 1: the first position of their level; the last lane: the active sources
+  const int f = lower(l == 31 ? ~0ull : (uint64_t)min(l, MRA_MAX_LEVEL + 1) << 32);
+  const int n_active = __shfl_sync(0xffffffffu, f, 31);
+  const int e = min(__shfl_down_sync(0xffffffffu, f, 1), n_active);
+  const int mine = G == 1 ? (l == 0 ? n_active : 0) : (l <= MRA_MAX_LEVEL ? max(e - f + G - 1, 0) / G : 0);
+  int sum = mine;  // inclusive over the levels
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, sum, o);
+    if (l >= o) sum += v;
   }
-  *n_tiles = tiles;
+  if (l <= MRA_MAX_LEVEL) {
+    lev_first[l] = G == 1 ? 0 : f;
+    tile_base[l] = G == 1 ? 0 : sum - mine;
+  }
+  if (l == 31) *n_tiles = sum;
 }
 
 __global__ void src_scatter_kernel(int64_t n, int G, const uint64_t *skey, const int *sval, const int *lev_first,
@@ -926,11 +928,13 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
     split_fixed_err(err, wk.fx->status, s);
     return MRA_OK;
   }
+  char host[4 * (MRA_MAX_LEVEL + 2) * 4];  // the scratch with the error word and the pass counter, in one copy
+  MRA_CUDA_TRY(cudaMemcpyAsync(host, small, sizeof(host), cudaMemcpyDeviceToHost, s));
+  MRA_CUDA_TRY(cudaStreamSynchronize(s));
   int herr = 0;
   unsigned long long hpass = 0;
-  MRA_CUDA_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaMemcpyAsync(&hpass, pass_ctr, sizeof(hpass), cudaMemcpyDeviceToHost, s));
-  MRA_CUDA_TRY(cudaStreamSynchronize(s));
+  memcpy(&herr, host + ((char *)err - (char *)small), sizeof(herr));
+  memcpy(&hpass, host + ((char *)pass_ctr - (char *)small), sizeof(hpass));
   if (passes) *passes = (int64_t)hpass;
   if (herr == 1) return fail(MRA_ERR_TIMEOUT, "split apply: a tensor-core completion wait gave up");
   if (herr) return fail(MRA_ERR_ARG, "split apply: inconsistent work list (%d)", herr);
