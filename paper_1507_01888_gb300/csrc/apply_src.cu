@@ -34,6 +34,8 @@
 // issued by a ninth warp (plain sums) or by a thread of warpgroup 1 (compensated sums), so the
 // two warpgroups work on consecutive terms.  The kernel is persistent: CTAs take
 // tiles from a device counter until none are left; tiles come heaviest first.
+#include <type_traits>
+
 #include <cub/cub.cuh>
 
 #include "apply_internal.cuh"
@@ -47,8 +49,7 @@ namespace {
 using namespace split;
 
 constexpr int SRC_THREADS = 256;
-constexpr int SRC_NB = 6;                          // block buffers (terms whose blocks are in shared memory)
-constexpr int SRC_MAX_AHEAD = SRC_NB - 2;          // the block copies run up to this many terms ahead
+constexpr int SRC_MAX_NB = 6;                      // block buffers (terms whose blocks are in shared memory) at most
 constexpr int SRC_MAX_JOIN = 8;                    // most terms summed in tensor memory per flush
 constexpr int SRC_RING = 4;                        // term-info ring from warpgroup 0 to 1
 constexpr int SRC_MAX_G = 8;                       // sources per tile
@@ -65,6 +66,10 @@ constexpr int FLAG_GROUP_END = 1, FLAG_TERM = 2, FLAG_JOIN = 4;
 __host__ __device__ constexpr int src_g(int k) {
   return (128 / (k * k)) > SRC_MAX_G ? SRC_MAX_G : 128 / (k * k);
 }
+
+// Block buffers of order k: at k = 4 four, since the record tables of its eight sources per tile (25 KB) would leave
+// room for one CTA per SM only.  The block copies run up to two fewer terms ahead.
+__host__ __device__ constexpr int src_nb(int k) { return k == 4 ? 4 : SRC_MAX_NB; }
 
 struct SrcArgs {
   int k, M, P;
@@ -88,7 +93,7 @@ struct SrcArgs {
   int join;                     // terms summed in D3 by the stage-3 MMAs before one flush
   int join_all;                 // 1: join in tiles of several sources too (else those flush every term)
   int compensated;              // record sums: 1 = FP32 sum + Kahan correction, 0 = plain FP32 sum
-  int ahead;                    // block copies run this many terms ahead (1 .. SRC_MAX_AHEAD)
+  int ahead;                    // block copies run this many terms ahead (1 .. src_nb - 2)
   int64_t n_src, n_rec, n_blocks;
 };
 
@@ -98,26 +103,27 @@ struct SrcArgs {
 template <int K, bool PLAIN>
 __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) apply_src_kernel(SrcArgs a) {
   constexpr int k2 = K * K, k3 = K * K * K;
-  constexpr int G = src_g(K), rows = G * k2;
+  constexpr int G = src_g(K), rows = G * k2, SRC_NB = src_nb(K);
   extern __shared__ __align__(1024) unsigned char smem[];
   const int P = a.P;
   unsigned char *A1 = smem;                    // [P] tiles: stage-1 operand (the tile's sources)
   unsigned char *A2 = A1 + 3 * TILE_BYTES;     // [P] tiles: stage-2 operand
-  unsigned char *A3 = A2 + 3 * TILE_BYTES;     // [P] tiles: stage-3 operand
-  unsigned char *Bt = A3 + 3 * TILE_BYTES;     // [SRC_NB][BIT_BYTES]: the blocks of a term
+  unsigned char *A3 = A2 + 3 * TILE_BYTES;     // [2][P] tiles: stage-3 operand of even and odd terms
+  unsigned char *Bt = A3 + 6 * TILE_BYTES;     // [SRC_NB][BIT_BYTES]: the blocks of a term
   // per-tile record table: record index and kept-term mask of (group, slot, lz in window)
   int *grp_rec = (int *)(Bt + SRC_NB * BIT_BYTES);                      // [SRC_NG][G][3]
   uint64_t *grp_mask = (uint64_t *)(grp_rec + SRC_NG * G * 3 + (SRC_NG * G * 3) % 2);  // [SRC_NG][G][3][2]
   uint64_t *grp_union = grp_mask + SRC_NG * G * 3 * 2;                  // [SRC_NG][2]
-  __shared__ __align__(8) uint64_t bar_s1, bar_s2, bar_s3, bar_ring, bar_d2free, bar_drain0, bar_drain1, bar_drain2;
+  __shared__ __align__(8) uint64_t bar_s1, bar_s2, bar_ring, bar_d2free, bar_drain0, bar_drain1, bar_drain2;
+  __shared__ __align__(8) uint64_t bar_s3[2], bar_a3[2];  // of even and odd terms: stage 3 done, A3 handed over
   __shared__ int s3_flags[SRC_RING];  // from warpgroup 1 to the stage-3 issuer: join / no more terms
   __shared__ volatile int s_nfetch;    // terms whose block copies thread 32 has issued
-  __shared__ __align__(8) uint64_t bar_bb[SRC_NB], bar_bfree[SRC_NB];
+  __shared__ __align__(8) uint64_t bar_bb[SRC_MAX_NB], bar_bfree[SRC_MAX_NB];
   __shared__ uint32_t tmem_holder;
   __shared__ int t_src[SRC_MAX_G];
   __shared__ int s_tile, t_level, t_dap, t_dop;
   __shared__ long long t_lbase;
-  __shared__ int ring_m[SRC_RING], ring_flags[SRC_RING];
+  __shared__ int ring_flags[SRC_RING];
   __shared__ uint32_t ring_keep[SRC_RING];
   __shared__ int ring_rec[SRC_RING][SRC_MAX_G * 3];
   __shared__ volatile int abort_flag;
@@ -127,15 +133,18 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
 
   {  // zero the operand tiles once: contraction and row padding stay zero
     int4 *z = (int4 *)smem;
-    const int n16 = (9 * TILE_BYTES) / 16;
+    const int n16 = (12 * TILE_BYTES) / 16;
     for (int i = tid; i < n16; i += (int)blockDim.x) z[i] = make_int4(0, 0, 0, 0);
   }
   if (tid == 0) {
     tc::mbar_init(tc::smem_u32(&bar_s1), 1);
     tc::mbar_init(tc::smem_u32(&bar_s2), 1);
-    tc::mbar_init(tc::smem_u32(&bar_s3), 1);
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(tc::smem_u32(&bar_s3[b]), 1);
+      tc::mbar_init(tc::smem_u32(&bar_a3[b]), 1);
+    }
     tc::mbar_init(tc::smem_u32(&bar_ring), 1);
-    tc::mbar_init(tc::smem_u32(&bar_d2free), 1);
+    tc::mbar_init(tc::smem_u32(&bar_d2free), 4);  // one arrival per warp of warpgroup 1
     tc::mbar_init(tc::smem_u32(&bar_drain0), 1);
     tc::mbar_init(tc::smem_u32(&bar_drain1), 1);
     tc::mbar_init(tc::smem_u32(&bar_drain2), 1);
@@ -154,19 +163,32 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
   tc::fence_after_sync();
   const uint32_t tmem = tmem_holder;
   const uint32_t tD1 = tmem + D1_COL, tD2 = tmem + D2_COL, tD3 = tmem + D3_COL;
-  const uint32_t bs1 = tc::smem_u32(&bar_s1), bs2 = tc::smem_u32(&bar_s2), bs3 = tc::smem_u32(&bar_s3);
+  const uint32_t bs1 = tc::smem_u32(&bar_s1), bs2 = tc::smem_u32(&bar_s2);
+  auto bs3 = [&](int it) { return tc::smem_u32(&bar_s3[it & 1]); };  // barrier and phase of term it's stage 3
+  auto ba3 = [&](int it) { return tc::smem_u32(&bar_a3[it & 1]); };
+  auto ph2 = [](int it) { return (uint32_t)((it >> 1) & 1); };
   const uint32_t bring = tc::smem_u32(&bar_ring), bd2free = tc::smem_u32(&bar_d2free);
   auto idesc_n = [](int n) { return tc::idesc_bf16(128, 16 * n, 1, 0); };
-  auto adesc = [&](const unsigned char *A, int p) {
-    return tc::smem_desc(tc::smem_u32(A + p * TILE_BYTES), 128, MG_BYTES);
-  };
+  // Descriptors of a first A piece and of a term's first B block; the other pieces and buffers follow at fixed
+  // distances in the address field (16-byte units), so that an issue is a few additions and the MMAs.
+  auto adesc = [&](const unsigned char *A) { return tc::smem_desc(tc::smem_u32(A), 128, MG_BYTES); };
   auto bdesc = [&](const unsigned char *B) { return tc::smem_desc(tc::smem_u32(B), 128, 256); };
+  constexpr uint64_t A_STEP = TILE_BYTES / 16, B_STEP = BIT_BYTES / 16;
   // A piece p times B pieces 0..P-1-p (stacked along N, nb blocks per piece) into column groups
   // p..P-1; the first MMA overwrites D unless acc0
-  auto issue_stacked = [&](uint32_t d, const unsigned char *A, const unsigned char *B, int nb, uint32_t acc0) {
-    for (int p = 0; p < P; ++p)
-      tc::mma_bf16(d + (uint32_t)(16 * nb * p), adesc(A, p), bdesc(B), idesc_n(nb * (P - p)), p > 0 ? 1u : acc0);
+  auto issue_stacked = [&](uint32_t d, uint64_t A, uint64_t B, auto nbc, uint32_t acc0) {
+    constexpr int nb = decltype(nbc)::value;
+    if (P == 3) {
+      tc::mma_bf16(d, A, B, idesc_n(nb * 3), acc0);
+      tc::mma_bf16(d + 16u * nb, A + A_STEP, B, idesc_n(nb * 2), 1u);
+      tc::mma_bf16(d + 32u * nb, A + 2 * A_STEP, B, idesc_n(nb), 1u);
+    } else {
+      tc::mma_bf16(d, A, B, idesc_n(nb * 2), acc0);
+      tc::mma_bf16(d + 16u * nb, A + A_STEP, B, idesc_n(nb), 1u);
+    }
   };
+  using one_block = std::integral_constant<int, 1>;
+  using three_blocks = std::integral_constant<int, 3>;
   // store units of a thread's run: 16-byte core-matrix rows when 8 divides k, else 4-byte pairs
   constexpr int U = K % 8 == 0 ? K / 8 : K / 2;
   auto run_addrs = [&](const unsigned char *A, int mrow, int a_idx, uint32_t *addr) {
@@ -225,10 +247,8 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
 #pragma unroll
     for (int j = 0; j < K; ++j) v[j] += c[0][j];
   };
-  // warpgroup 1 hands a term (or the end) to the stage-3 issuer warp: named barrier 3, 128 + 32
-  auto wg_arrive_issuer = [&]() { asm volatile("bar.arrive 3, 160;" ::: "memory"); };
   const int mrow = quarter * 32 + lane;  // this thread's row of the tile (lane of tensor memory)
-  const int ahead = max(1, min(a.ahead, SRC_MAX_AHEAD));
+  const int ahead = max(1, min(a.ahead, SRC_NB - 2));
   // tiles of several sources join only when asked: a join depends on all the tile's records,
   // so it would make a result depend on which sources share its tile
   const int join = (G == 1 || a.join_all) ? max(1, min(a.join, SRC_MAX_JOIN)) : 1;
@@ -243,6 +263,7 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
       const int i = m1 / k2, rem = m1 - i * k2, jy = rem / K, jz = rem - jy * K;
       run_addrs(A2, i * k2 + jz * K, jy, a2_addr);
     }
+    const uint64_t da1 = adesc(A1), da2 = adesc(A2), dbx = bdesc(Bt + BX_OFF), dby = bdesc(Bt + BY_OFF);
     uint32_t p1 = 0;
     int it = 0;       // terms issued by this CTA so far (all tiles)
     int nfetch = 0;   // block copies issued (thread 32), for iterations 0 .. nfetch-1 in order
@@ -386,7 +407,6 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
         const int g = cg, m = cm;
         const bool group_end = !(cu0 | cu1);
         const int b = it % SRC_NB;
-        const unsigned char *Bb = Bt + b * BIT_BYTES;
         uint32_t keep = 0;
 #pragma unroll
         for (int i = 0; i < G; ++i)
@@ -402,7 +422,7 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
                                            &abort_flag);
           if (ok) {
             tc::fence_after_sync();
-            issue_stacked(tD1, A1, Bb + BX_OFF, 1, 0u);  // ---- stage 1: rows (i, jy, jz), contraction jx
+            issue_stacked(tD1, da1, dbx + b * B_STEP, one_block{}, 0u);  // ---- stage 1: rows (i, jy, jz), contraction jx
             tc::mma_commit(bs1);
           } else {
             abort_flag = 1;
@@ -429,22 +449,22 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
         tc::fence_before_sync();
         wg_sync(1);
         if (tid == 64) {  // ---- stage 2: rows (i, jz, ix), contraction jy
-          bool ok2 = it == 0 || tc::mbar_wait_or_abort(bd2free, (uint32_t)((it - 1) & 1), WAIT_CYCLES, &abort_flag);
-          if (ok2) {
-            const int r = it % SRC_RING;
-            ring_m[r] = m;
-            ring_keep[r] = keep;
-            ring_flags[r] = group_end ? FLAG_GROUP_END : 0;
-            if (group_end)
-              for (int e = 0; e < G * 3; ++e) ring_rec[r][e] = grp_rec[g * G * 3 + e];
-            mbar_arrive(bring);
-            ok2 = tc::mbar_wait_or_abort(tc::smem_u32(&bar_bb[b]), (uint32_t)((it / SRC_NB) & 1), WAIT_CYCLES,
-                                         &abort_flag);
-          }
+          // What warpgroup 1 needs to know goes into the ring, and the blocks are waited for, before D2 is free:
+          // from then on the MMAs are all that stands between the release of D2 and its next reading.  The slot
+          // is free: warpgroup 1 has read D2 of the term before the last, so it is done with the slots of the
+          // terms more than three back.
+          const int r = it % SRC_RING;
+          ring_keep[r] = keep;
+          ring_flags[r] = group_end ? FLAG_GROUP_END : 0;
+          if (group_end)
+            for (int e = 0; e < G * 3; ++e) ring_rec[r][e] = grp_rec[g * G * 3 + e];
+          bool ok2 = tc::mbar_wait_or_abort(tc::smem_u32(&bar_bb[b]), (uint32_t)((it / SRC_NB) & 1), WAIT_CYCLES, &abort_flag);
+          if (ok2 && it > 0) ok2 = tc::mbar_wait_or_abort(bd2free, (uint32_t)((it - 1) & 1), WAIT_CYCLES, &abort_flag);
           if (ok2) {
             tc::fence_after_sync();
-            issue_stacked(tD2, A2, Bb + BY_OFF, 1, 0u);
+            issue_stacked(tD2, da2, dby + b * B_STEP, one_block{}, 0u);
             tc::mma_commit(bs2);
+            mbar_arrive(bring);
           } else {
             abort_flag = 1;
           }
@@ -547,54 +567,67 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
     int last_handed = -1;  // the last term handed to the stage-3 issuer (plain sums)
     int joined = 0;  // terms summed in D3 since its last flush
     int it = 0;
+    const uint64_t da3 = adesc(A3), dbz = bdesc(Bt + BZ_OFF);
     for (;; ++it) {
       const int r = it % SRC_RING;
       bool ok = true;
-      if (quarter == 0) ok = tc::mbar_wait_or_abort(bring, (uint32_t)(it & 1), WAIT_CYCLES, &abort_flag);
+      if (quarter == 0) {  // one warp polls, one vote: the term's info, then (unless it is the end) its D2 and its A3
+        ok = tc::mbar_wait_or_abort(bring, (uint32_t)(it & 1), WAIT_CYCLES, &abort_flag);
+        if (ok && !(ring_flags[r] & FLAG_TERM)) {
+          ok = tc::mbar_wait_or_abort(bs2, (uint32_t)(it & 1), WAIT_CYCLES, &abort_flag);
+          if (ok && it > 1) ok = tc::mbar_wait_or_abort(bs3(it - 2), ph2(it - 2), WAIT_CYCLES, &abort_flag);
+        }
+      }
       if (wg_vote_or(2, !ok || abort_flag)) { bad = true; break; }
       const int flags = ring_flags[r];
       if (flags & FLAG_TERM) break;
-      if (quarter == 0) {
-        ok = tc::mbar_wait_or_abort(bs2, (uint32_t)(it & 1), WAIT_CYCLES, &abort_flag);
-        if (ok && it > 0) ok = tc::mbar_wait_or_abort(bs3, (uint32_t)((it - 1) & 1), WAIT_CYCLES, &abort_flag);
-      }
-      if (wg_vote_or(2, !ok || abort_flag)) { bad = true; break; }
       tc::fence_after_sync();
       const uint32_t keep = ring_keep[r];
       // D2 -> registers, then D2 is released for the next term's stage 2
       float v[K];
       load_groups(tD2, 1, v);
       tc::fence_before_sync();
-      wg_sync(2);
-      if (tid == 128) mbar_arrive(bd2free);
-      // the previous pass's D3 into the record sums and a finished group written out, unless this
-      // term's stage 3 joins it in D3 (same group, same records keeping it, room left)
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bd2free);
+      // stage-2 output -> stage-3 operand: element [jz][(i, ix, iy)], into the buffer of even or odd terms, so
+      // that neither the reading of D2 nor this waits for the previous term's stage 3
+      if (mrow < rows) {
+        const uint32_t odd = (uint32_t)(it & 1) * 3u * TILE_BYTES;
+        uint32_t addr[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) addr[u] = a3_addr[u] + odd;
+        store_units(addr, v);
+      }
+      tc::fence_proxy_async_smem();
+      // the previous passes' D3 into the record sums and a finished group written out, unless this
+      // term's stage 3 joins it in D3 (same group, same records keeping it, room left); only a flush waits
+      // for the previous term's stage 3
       const bool join_now = joined > 0 && joined < join && keep == prev_keep && !(prev_flags & FLAG_GROUP_END);
       if (it > 0 && !join_now) {
+        ok = quarter != 0 || tc::mbar_wait_or_abort(bs3(it - 1), ph2(it - 1), WAIT_CYCLES, &abort_flag);
+        if (wg_vote_or(2, !ok || abort_flag)) { bad = true; break; }
+        tc::fence_after_sync();
         flush(prev_keep);
         if (prev_flags & FLAG_GROUP_END) write_group(ring_rec[prev_slot]);
         joined = 0;
       }
-      // stage-2 output -> stage-3 operand: element [jz][(i, ix, iy)]
-      if (mrow < rows) store_units(a3_addr, v);
-      tc::fence_proxy_async_smem();
       tc::fence_before_sync();
       wg_sync(2);
-      if constexpr (PLAIN) {  // the stage-3 issuer warp takes it from here (named barrier 3)
-        if (tid == 128) s3_flags[it % SRC_RING] = join_now ? FLAG_JOIN : 0;
-        __syncwarp();
-        wg_arrive_issuer();
+      if constexpr (PLAIN) {  // the stage-3 issuer warp takes it from here
+        if (tid == 128) {
+          s3_flags[it % SRC_RING] = join_now ? FLAG_JOIN : 0;
+          mbar_arrive(ba3(it));
+        }
         last_handed = it;
       } else if (tid == 160) {  // a thread of another warp than the polling one issues stage 3
         const int b = it % SRC_NB;
-        const unsigned char *B3 = Bt + b * BIT_BYTES + BZ_OFF;
         bool okb = tc::mbar_wait_or_abort(tc::smem_u32(&bar_bb[b]), (uint32_t)((it / SRC_NB) & 1), WAIT_CYCLES,
                                           &abort_flag);
         if (okb) {
           tc::fence_after_sync();
           // ---- stage 3: rows (i, ix, iy), contraction jz, B = c_m R_{m,lz} of the window's three lz
-          issue_stacked(tD3, A3, B3, 3, join_now ? 1u : 0u);
-          tc::mma_commit(bs3);
+          issue_stacked(tD3, da3 + (it & 1) * 3 * A_STEP, dbz + b * B_STEP, three_blocks{}, join_now ? 1u : 0u);
+          tc::mma_commit(bs3(it));
           tc::mma_commit(tc::smem_u32(&bar_bfree[b]));
         } else {
           abort_flag = 1;
@@ -606,7 +639,7 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
       ++joined;
     }
     if (!bad && it > 0) {
-      bool ok = quarter != 0 || tc::mbar_wait_or_abort(bs3, (uint32_t)((it - 1) & 1), WAIT_CYCLES, &abort_flag);
+      bool ok = quarter != 0 || tc::mbar_wait_or_abort(bs3(it - 1), ph2(it - 1), WAIT_CYCLES, &abort_flag);
       if (wg_vote_or(2, !ok || abort_flag)) {
         bad = true;
       } else {
@@ -617,19 +650,11 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
     }
     if (bad) abort_flag = 1;
     if constexpr (PLAIN) {
-      // no more terms for the stage-3 issuer (also after an abort), in the slot after the last
-      // term handed over.  That term's stage 3 done means the issuer took it, so this arrival is
-      // the only one pending on barrier 3; if it never completes within the bound, the issuer has
-      // left on the abort and waits no more.
-      bool send = true;
-      if (last_handed >= 0) {
-        bool ok = quarter != 0 || tc::mbar_wait(bs3, (uint32_t)(last_handed & 1), WAIT_CYCLES);
-        send = !wg_vote_or(2, !ok);
-      }
-      if (send) {
-        if (tid == 128) s3_flags[(last_handed + 1) % SRC_RING] = FLAG_TERM;
-        __syncwarp();
-        wg_arrive_issuer();
+      // no more terms for the stage-3 issuer, in the slot after the last term handed over (that term's stage 3
+      // is done, so the issuer has taken every earlier hand-over); after an abort it leaves by the abort flag
+      if (!bad && tid == 128) {
+        s3_flags[(last_handed + 1) % SRC_RING] = FLAG_TERM;
+        mbar_arrive(ba3(last_handed + 1));
       }
     } else if (tid == 160) {
       tc::mma_commit(tc::smem_u32(&bar_drain1));
@@ -637,38 +662,38 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
     }
   } else if (PLAIN && warp == SRC_THREADS / 32) {
     // ======================================================= the stage-3 issuer (warp 8; lane 0 issues)
-    // Warpgroup 1 hands each term over on named barrier 3 (its 128 threads arrive, this warp
-    // waits: cheaper than an mbarrier round trip) and arrives once more when there are no more
-    // terms, also after an abort, so the wait always ends.  The blocks of the next term are
-    // checked as soon as their copies are known to be issued.
-    int ready = -1;  // the term whose blocks lane 0 has already seen land
-    for (int it = 0;; ++it) {
-      asm volatile("bar.sync 3, 160;" ::: "memory");
-      const int f = s3_flags[it % SRC_RING];
-      if (f & FLAG_TERM) break;
-      const int b = it % SRC_NB;
-      const unsigned char *B3 = Bt + b * BIT_BYTES + BZ_OFF;
-      if (lane == 0) {
-        bool ok = ready == it ||
-                  tc::mbar_wait_or_abort(tc::smem_u32(&bar_bb[b]), (uint32_t)((it / SRC_NB) & 1), WAIT_CYCLES, &abort_flag);
-        if (ok) {
-          tc::fence_after_sync();
-          // ---- stage 3: rows (i, ix, iy), contraction jz, B = c_m R_{m,lz} of the window's three lz
-          issue_stacked(tD3, A3, B3, 3, (f & FLAG_JOIN) ? 1u : 0u);
-          tc::mma_commit(bs3);
-          tc::mma_commit(tc::smem_u32(&bar_bfree[b]));
-          const int nx = it + 1;  // the next term's blocks, if their copies are issued
-          if (nx < s_nfetch &&
-              tc::mbar_wait_or_abort(tc::smem_u32(&bar_bb[nx % SRC_NB]), (uint32_t)((nx / SRC_NB) & 1), WAIT_CYCLES,
-                                     &abort_flag))
-            ready = nx;
-        } else {
+    // Warpgroup 1 hands each term over on the mbarrier of even or odd terms (it is at most two terms ahead: it
+    // waits for stage 3 of the term before the last) and once more when there are no more terms.  The blocks of
+    // the next term are checked as soon as their copies are known to be issued.
+    const uint64_t da3 = adesc(A3), dbz = bdesc(Bt + BZ_OFF);
+    if (lane == 0) {
+      int ready = -1;  // the term whose blocks have already been seen to land
+      for (int it = 0;; ++it) {
+        if (!tc::mbar_wait_or_abort(ba3(it), ph2(it), WAIT_CYCLES, &abort_flag)) {
           abort_flag = 1;
+          break;
         }
+        const int f = s3_flags[it % SRC_RING];
+        if (f & FLAG_TERM) break;
+        const int b = it % SRC_NB;
+        if (ready != it &&
+            !tc::mbar_wait_or_abort(tc::smem_u32(&bar_bb[b]), (uint32_t)((it / SRC_NB) & 1), WAIT_CYCLES, &abort_flag)) {
+          abort_flag = 1;
+          break;
+        }
+        tc::fence_after_sync();
+        // ---- stage 3: rows (i, ix, iy), contraction jz, B = c_m R_{m,lz} of the window's three lz
+        issue_stacked(tD3, da3 + (it & 1) * 3 * A_STEP, dbz + b * B_STEP, three_blocks{}, (f & FLAG_JOIN) ? 1u : 0u);
+        tc::mma_commit(bs3(it));
+        tc::mma_commit(tc::smem_u32(&bar_bfree[b]));
+        const int nx = it + 1;  // the next term's blocks, if their copies are issued
+        if (nx < s_nfetch &&
+            tc::mbar_wait_or_abort(tc::smem_u32(&bar_bb[nx % SRC_NB]), (uint32_t)((nx / SRC_NB) & 1), WAIT_CYCLES,
+                                   &abort_flag))
+          ready = nx;
       }
-      // one decision for the whole warp (lane 0's view), so that no lane waits alone at bar.sync
-      if (__shfl_sync(0xffffffffu, (int)abort_flag, 0)) break;
     }
+    __syncwarp();
     if (lane == 0) {
       tc::mma_commit(tc::smem_u32(&bar_drain1));
       tc::mbar_wait(tc::smem_u32(&bar_drain1), 0, WAIT_CYCLES);
@@ -888,7 +913,7 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
   a.n_rec = P;
   a.n_blocks = op.n_blocks;
   const size_t tables = (size_t)SRC_NG * G * 3 * 4 + 8 + (size_t)SRC_NG * G * 3 * 16 + (size_t)SRC_NG * 16;
-  size_t smem = (size_t)9 * TILE_BYTES + (size_t)SRC_NB * BIT_BYTES + tables;
+  size_t smem = (size_t)12 * TILE_BYTES + (size_t)src_nb(k) * BIT_BYTES + tables;
   // no more CTAs per SM than the tensor memory holds (two of 256 columns): otherwise an extra
   // CTA's allocation would wait for a resident CTA to finish
   const size_t smem_floor = (size_t)233472 / (512 / SRC_TMEM_COLS + 1) + 16;
