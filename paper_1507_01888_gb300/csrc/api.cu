@@ -178,60 +178,67 @@ static int fit_operator(Operator *op, double mu_fit, int M, double r_lo, double 
   // The grid's argmin of the max relative error over the 3000 points, the first (lowest
   // index) of equal minima.  Exact with far fewer evaluations: the maximum over 16 of the
   // points (the three at each end of the range, where the truncation of the Gaussian sum shows,
-  // and twelve spread over it) is a lower bound of each candidate's error, so candidates are
+  // and ten spread over it) is a lower bound of each candidate's error, so candidates are
   // evaluated in full in increasing order of that bound until the bound exceeds the best full
   // error found; no candidate left out can reach it.  The batches of full evaluations grow
-  // from 16 (a handful are usually enough), and a full evaluation stops once it exceeds the
-  // best error found before its batch (such a candidate can neither win nor tie).
-  const int NC = 116 * 113, NP = 3000, BATCH = 256;
+  // from 16 (a handful are usually enough).
+  const int NC = 116 * 113, NP = 3000, BATCH = 256, SUB = 16;
   std::vector<int> sub;
   for (int q = 0; q < 3; ++q) {
     sub.push_back(q);
     sub.push_back(NP - 1 - q);
   }
-  for (int q = 0; q < 12; ++q) sub.push_back((int)lround(q * (NP - 1) / 11.0));
-  std::sort(sub.begin(), sub.end());
-  sub.erase(std::unique(sub.begin(), sub.end()), sub.end());
-  double *d_err = nullptr;
+  for (int q = 1; q <= SUB - 6; ++q) sub.push_back((int)lround(q * (NP - 1) / (SUB - 5.0)));
+  double *d_err = nullptr, *d_rk = nullptr;
   int *d_cand = nullptr;
   if (pool_malloc((void **)&d_err, NC * sizeof(double), s) != cudaSuccess ||
-      pool_malloc((void **)&d_cand, (BATCH + 256) * sizeof(int), s) != cudaSuccess) {
+      pool_malloc((void **)&d_rk, fit_points_bytes(), s) != cudaSuccess ||
+      pool_malloc((void **)&d_cand, (BATCH + SUB) * sizeof(int), s) != cudaSuccess) {
     if (d_err) cudaFreeAsync(d_err, s);
+    if (d_rk) cudaFreeAsync(d_rk, s);
     cudaStreamSynchronize(s);
     return fail(MRA_ERR_CUDA, "fit search: out of device memory");
   }
   int *d_pts = d_cand + BATCH;
   std::vector<double> lower(NC), full(NC, -1.0);
-  cudaError_t e = cudaMemcpyAsync(d_pts, sub.data(), sub.size() * sizeof(int), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = launch_fit_search(mu_fit, M, r_lo, r_hi, 1, d_pts, (int)sub.size(), nullptr, NC, INFINITY, d_err, s);
+  cudaError_t e = cudaMemcpyAsync(d_pts, sub.data(), SUB * sizeof(int), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = launch_fit_lower(mu_fit, M, r_lo, r_hi, d_pts, d_rk, NC, d_err, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(lower.data(), d_err, NC * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  // a heap of the bounds, smallest first (equal ones by index): only the few that are evaluated are taken out in order.
+  // NaN bounds (never produced by the finite grid) sort last and are evaluated like the rest
   std::vector<int> order(NC);
   for (int q = 0; q < NC; ++q) order[q] = q;
-  // NaN bounds (never produced by the finite grid) sort last and are evaluated like the rest
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+  auto later = [&](int a, int b) {
     const bool na = std::isnan(lower[a]), nb = std::isnan(lower[b]);
-    return na != nb ? nb : (!na && lower[a] < lower[b]);
-  });
-  int best = -1, pos = 0, batch = 16;
-  while (e == cudaSuccess && pos < NC && (best < 0 || !(lower[order[pos]] > full[best]))) {
-    const int nb = std::min(batch, NC - pos);
+    if (na != nb) return na;
+    if (!na && lower[a] != lower[b]) return lower[a] > lower[b];
+    return a > b;
+  };
+  std::make_heap(order.begin(), order.end(), later);
+  int best = -1, batch = 16;
+  while (e == cudaSuccess && !order.empty() && (best < 0 || !(lower[order.front()] > full[best]))) {
+    const int nb = std::min(batch, (int)order.size());
     batch = std::min(2 * batch, BATCH);
+    std::vector<int> cands(nb);
+    for (int q = 0; q < nb; ++q) {
+      cands[q] = order.front();
+      std::pop_heap(order.begin(), order.end(), later);
+      order.pop_back();
+    }
     std::vector<double> part(nb);
-    e = cudaMemcpyAsync(d_cand, order.data() + pos, nb * sizeof(int), cudaMemcpyHostToDevice, s);
-    const double stop = best < 0 ? INFINITY : full[best];
-    if (e == cudaSuccess) e = launch_fit_search(mu_fit, M, r_lo, r_hi, 1, nullptr, 0, d_cand, nb, stop, d_err, s);
+    e = cudaMemcpyAsync(d_cand, cands.data(), nb * sizeof(int), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = launch_fit_full(mu_fit, M, d_cand, nb, d_rk, d_err, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(part.data(), d_err, nb * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     for (int q = 0; q < nb && e == cudaSuccess; ++q) {
-      const int c = order[pos + q];
+      const int c = cands[q];
       full[c] = part[q];
       if (best < 0 || part[q] < full[best] || (part[q] == full[best] && c < best)) best = c;
     }
-    pos += nb;
   }
   cudaFreeAsync(d_err, s);
+  cudaFreeAsync(d_rk, s);
   cudaFreeAsync(d_cand, s);
   const cudaError_t ef = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = ef;

@@ -48,14 +48,15 @@ __host__ __device__ constexpr int par_entry(int k) { return (3 * par_half(k) * k
 // maps child 0's phi_i to (-1)^i child 1's phi_i, so (phi_{0,i} +- (-1)^i phi_{1,i}) / sqrt 2 are even and odd.
 __device__ __forceinline__ double pair_sign(int c, int i, int a) { return c && ((i + a) & 1) ? -1.0 : 1.0; }
 
-// Parity table of one level: entry m holds W[comp][jj][i], comp 0: R_0, 1: E, 2: O (of l = 1), the
+// Parity table of every level (blockIdx.y): entry m holds W[comp][jj][i], comp 0: R_0, 1: E, 2: O (of l = 1), the
 // entry [i][j] of the block with j = 2 jj + (i & 1) for comp 0 and 1 and 2 jj + 1 - (i & 1) for O
 // (zero beyond k).  Non-standard operators (pairs = 1) are first turned into the basis of even and
 // odd child combinations, index 2 i + parity.
-__global__ void parity_table_kernel(int k, int D, const double *R, double *W, int pairs) {
-  const int m = blockIdx.x, h = par_half(k), nl = 2 * D + 1, hk = k / 2;
-  const double *Rm = R + (int64_t)m * nl * k * k;
-  double *Wm = W + (int64_t)m * par_entry(k);
+__global__ void parity_table_kernel(int k, int M, int min_level, const int *Dlev, const int64_t *level_off,
+                                    const double *R, double *W, int pairs) {
+  const int m = blockIdx.x, lev = min_level + blockIdx.y, D = Dlev[lev], h = par_half(k), nl = 2 * D + 1, hk = k / 2;
+  const double *Rm = R + (level_off[lev] + (int64_t)m * nl) * k * k;
+  double *Wm = W + ((int64_t)blockIdx.y * M + m) * par_entry(k);
   for (int e = threadIdx.x; e < par_entry(k); e += blockDim.x) {
     const int comp = e / (h * k), jj = (e / k) % h, i = e % k;
     const int j = 2 * jj + (comp == 2 ? 1 - (i & 1) : (i & 1));
@@ -478,11 +479,9 @@ void f64_shape(int k, int64_t n_src, int sms, int *nx_out, int *threads_out) {
 int f64_parity_build(Operator &op, cudaStream_t s) {
   const size_t we = (size_t)par_entry(op.k), levels = op.D.size();
   if (!op.d_W) MRA_CUDA_TRY(cudaMalloc((void **)&op.d_W, levels * op.M * we * sizeof(double)));
-  for (size_t li = 0; li < levels; ++li) {
-    parity_table_kernel<<<counted((unsigned)op.M), 128, 0, s>>>(op.k, op.D[li], op.d_R + op.level_off[li] * op.k * op.k,
-                                                                op.d_W + li * op.M * we, op.non_standard ? 1 : 0);
-    MRA_CUDA_TRY(cudaGetLastError());
-  }
+  parity_table_kernel<<<counted(dim3((unsigned)op.M, (unsigned)levels)), 128, 0, s>>>(
+      op.k, op.M, op.min_level, op.d_D, op.d_level_off, op.d_R, op.d_W, op.non_standard ? 1 : 0);
+  MRA_CUDA_TRY(cudaGetLastError());
   return MRA_OK;
 }
 

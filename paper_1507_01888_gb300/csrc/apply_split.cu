@@ -649,22 +649,31 @@ __global__ void group_bounds_kernel(int64_t P, const uint64_t *key2s, const int 
 // of block (m, l) sits at byte (m nl + l + D) 1536 + p 512 (block-major: the three pieces of a
 // block together), or with piece_major at (m nl 3 + p nl + l + D) 512 (all displacements of
 // one piece together, so that the pieces of consecutive displacements are consecutive).
-__global__ void split_blocks_kernel(int64_t n_blocks, int k, int nl, const double *c, const double *R,
-                                    unsigned char *out, int piece_major) {
-  int64_t blk = blockIdx.x;
-  if (blk >= n_blocks) return;
-  const double x = c ? c[blk / nl] : 1.0;
-  const int64_t m = blk / nl, l = blk - m * nl;
+// All levels and the three tables (plain and scaled block-major, scaled piece-major) in one launch, a CTA per block.
+struct SplitTables {
+  int k, n_levels;
+  int64_t off[MRA_MAX_LEVEL + 2];  // first block of each level of the operator, then their number
+  int nl[MRA_MAX_LEVEL + 1];
+  const double *c, *R;
+  unsigned char *plain, *scaled, *zpack;
+};
+__global__ void split_blocks_kernel(SplitTables a) {
+  const int64_t blk = blockIdx.x;
+  int li = 0;
+  while (li + 1 < a.n_levels && blk >= a.off[li + 1]) ++li;
+  const int64_t base = a.off[li], nl = a.nl[li], m = (blk - base) / nl, l = blk - base - m * nl;
+  const double x = a.c[m];
   for (int e = threadIdx.x; e < 256; e += blockDim.x) {
-    int i = e / 16, j = e % 16;
-    double y = (i < k && j < k) ? x * R[blk * k * k + i * k + j] : 0.0;
-    __nv_bfloat16 pc[3];
-    split3(y, pc[0], pc[1], pc[2]);
-    uint32_t off = (i / 8) * 256 + (j / 8) * 128 + (i % 8) * 16 + (j % 8) * 2;
-    for (int p = 0; p < 3; ++p) {
-      const int64_t at = piece_major ? ((m * nl * 3 + p * nl + l) * BPIECE_BYTES)
-                                     : (blk * BSTAGE_BYTES + p * BPIECE_BYTES);
-      *(__nv_bfloat16 *)(out + at + off) = pc[p];
+    const int i = e / 16, j = e % 16;
+    const double y = (i < a.k && j < a.k) ? a.R[blk * a.k * a.k + i * a.k + j] : 0.0;
+    __nv_bfloat16 p[3], q[3];
+    split3(y, p[0], p[1], p[2]);
+    split3(x * y, q[0], q[1], q[2]);
+    const uint32_t off = (i / 8) * 256 + (j / 8) * 128 + (i % 8) * 16 + (j % 8) * 2;
+    for (int pc = 0; pc < 3; ++pc) {
+      *(__nv_bfloat16 *)(a.plain + blk * BSTAGE_BYTES + pc * BPIECE_BYTES + off) = p[pc];
+      *(__nv_bfloat16 *)(a.scaled + blk * BSTAGE_BYTES + pc * BPIECE_BYTES + off) = q[pc];
+      *(__nv_bfloat16 *)(a.zpack + base * BSTAGE_BYTES + (m * nl * 3 + pc * nl + l) * BPIECE_BYTES + off) = q[pc];
     }
   }
 }
@@ -699,16 +708,21 @@ int split_blocks_build(Operator &op, cudaStream_t s, bool rebuild) {
   unsigned char *plain = (unsigned char *)op.d_Rsplit;
   unsigned char *scaled = plain + (size_t)op.n_blocks * BSTAGE_BYTES;
   unsigned char *zpack = plain + (size_t)2 * op.n_blocks * BSTAGE_BYTES;
-  for (size_t li = 0; li < op.D.size(); ++li) {
-    const int nl = 2 * op.D[li] + 1;
-    const int64_t nb = (int64_t)op.M * nl, base = op.level_off[li];
-    if (nb <= 0) continue;
-    const double *R = op.d_R + base * op.k * op.k;
-    split_blocks_kernel<<<counted((unsigned)nb), 128, 0, s>>>(nb, op.k, nl, nullptr, R, plain + base * BSTAGE_BYTES, 0);
-    split_blocks_kernel<<<counted((unsigned)nb), 128, 0, s>>>(nb, op.k, nl, op.d_c, R, scaled + base * BSTAGE_BYTES, 0);
-    split_blocks_kernel<<<counted((unsigned)nb), 128, 0, s>>>(nb, op.k, nl, op.d_c, R, zpack + base * BSTAGE_BYTES, 1);
-    MRA_CUDA_TRY(cudaGetLastError());
+  SplitTables a{};
+  a.k = op.k;
+  a.n_levels = (int)op.D.size();
+  for (int li = 0; li < a.n_levels; ++li) {
+    a.off[li] = op.level_off[li];
+    a.nl[li] = 2 * op.D[li] + 1;
   }
+  a.off[a.n_levels] = op.n_blocks;
+  a.c = op.d_c;
+  a.R = op.d_R;
+  a.plain = plain;
+  a.scaled = scaled;
+  a.zpack = zpack;
+  split_blocks_kernel<<<counted((unsigned)op.n_blocks), 128, 0, s>>>(a);
+  MRA_CUDA_TRY(cudaGetLastError());
   return MRA_OK;
 }
 

@@ -115,8 +115,13 @@ void two_scale(int k, double *U /* [2][k][k] */);  // U^(c)[i][j], Sec. 2.2
 void free_operator(Operator *op);
 
 // ---------------------------------------------------------------- launchers (setup)
-cudaError_t launch_fit_search(double mu, int M, double r_lo, double r_hi, int stride, const int *d_pts, int npts,
-                              const int *d_cands, int n_cands, double stop, double *d_err, cudaStream_t s);
+// Gaussian fit: the points' r and K (d_rk, fit_points_bytes) and every candidate's lower bound over the 16
+// points d_pts, then full errors of listed candidates.
+size_t fit_points_bytes();
+cudaError_t launch_fit_lower(double mu, int M, double r_lo, double r_hi, const int *d_pts, double *d_rk, int n_cand,
+                             double *d_err, cudaStream_t s);
+cudaError_t launch_fit_full(double mu, int M, const int *d_cands, int n_cands, const double *d_rk, double *d_err,
+                            cudaStream_t s);
 cudaError_t launch_blocks(const Operator &op, const double *d_glx, const double *d_glw,
                           cudaStream_t s);
 // Projection: 1-D factors of `entries` (factor_entry: level, dimension, coordinate), then the boxes.

@@ -30,9 +30,11 @@ namespace mra {
 namespace {
 
 // ---------------------------------------------------------------- 2k blocks
-// Blocks of one level of the non-standard operator from the level-(n+1) blocks of op.
-__global__ void ns_blocks_kernel(int k, int M, int D, const double *Rop, int64_t op_base, int Dc,
-                                 double *Rns, int64_t ns_base) {
+// Blocks of every level n (blockIdx.y) of the non-standard operator from the level-(n+1) blocks of op.
+__global__ void ns_blocks_kernel(int k, int M, int min_level, const int *Dns, const int64_t *ns_off, const int *Dop,
+                                 const int64_t *op_off, const double *Rop, double *Rns) {
+  const int n = min_level + blockIdx.y, D = Dns[n], Dc = Dop[n + 1];
+  const int64_t ns_base = ns_off[n], op_base = op_off[n + 1];
   const int nl = 2 * D + 1, nlc = 2 * Dc + 1, kk = 2 * k;
   const int q = blockIdx.x;  // m * nl + (l + D)
   if (q >= M * nl) return;
@@ -772,11 +774,10 @@ extern "C" int mra_operator_ns_create(const mra_operator *h, int max_disp, mra_o
   if (e == cudaSuccess) e = cudaMemcpyAsync(ns->d_D, Dabs.data(), 20 * sizeof(int), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ns->d_level_off, off_abs.data(), 20 * sizeof(int64_t), cudaMemcpyHostToDevice, s);
-  for (int n = ns->min_level; n <= ns->max_level && e == cudaSuccess; ++n) {
-    const int li = n - ns->min_level, lc = n + 1 - op->min_level;
-    const int D = ns->D[li];
-    ns_blocks_kernel<<<counted((unsigned)(ns->M * (2 * D + 1))), 256, 0, s>>>(op->k, ns->M, D, op->d_R, op->level_off[lc],
-                                                                       op->D[lc], ns->d_R, ns->level_off[li]);
+  if (e == cudaSuccess) {
+    const int most = 2 * *std::max_element(ns->D.begin(), ns->D.end()) + 1;
+    ns_blocks_kernel<<<counted(dim3((unsigned)(ns->M * most), (unsigned)ns->D.size())), 256, 0, s>>>(
+        op->k, ns->M, ns->min_level, ns->d_D, ns->d_level_off, op->d_D, op->d_level_off, op->d_R, ns->d_R);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {

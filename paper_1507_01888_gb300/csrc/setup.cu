@@ -32,53 +32,71 @@ __device__ __forceinline__ void legendre_phi(int k, double x01, double *out) {
 }
 
 // --------------------------------------------------------------------------- fit search
-// One CTA per candidate (h, s_lo) of the grid h = (5+i)/100, s_lo = (j-100)/4:
-// max over the log-spaced points p = 0, stride, 2 stride, ... < 3000 (or, when `pts` is given,
-// over the npts points pts[0..npts), npts <= blockDim) of
-// |sum_m c_m exp(-t_m r_p^2) - K(r_p)| / K(r_p).  Over all points this is the candidate's
-// error; over a subset it is a lower bound of it (a maximum over some of the same values).
-// `cands` lists the candidates to evaluate (NULL: every candidate, in grid order).  A CTA
-// stops early once its running maximum exceeds `stop` (a full error found already; +inf:
-// never) and then writes that partial maximum, which exceeds `stop` too; errors at or below
-// `stop` are exact.
+// A candidate (h, s_lo) of the grid h = (5+i)/100, s_lo = (j-100)/4 has the error
+// max_p |sum_m c_m exp(-t_m r_p^2) - K(r_p)| / K(r_p) over the log-spaced points p = 0 .. 2999; over a
+// subset of the points it is a lower bound of that (a maximum over some of the same values).
 constexpr int FIT_NS = 113, FIT_NP = 3000;  // s_lo values per h (116 h values), points
+constexpr int FIT_SUB = 16;                 // points of the lower bounds
 
-__global__ void fit_search_kernel(double mu, int M, double r_lo, double r_hi, int stride, const int *pts,
-                                  int npts, const int *cands, double stop, double *err) {
+// r_p and K(r_p) of every point.
+__global__ void fit_points_kernel(double mu, double r_lo, double r_hi, double *rk) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= FIT_NP) return;
+  const double r = r_lo * pow(r_hi / r_lo, (double)p / (double)(FIT_NP - 1));
+  rk[p] = r;
+  rk[FIT_NP + p] = exp(-mu * r) / r;
+}
+
+__device__ __forceinline__ void fit_term(double mu, int cand, int m, double &c, double &t) {
+  const int i = cand / FIT_NS, j = cand % FIT_NS;
+  const double h = (5.0 + i) / 100.0, s_lo = (j - 100.0) / 4.0;
+  const double two_over_sqrtpi = 2.0 / sqrt(3.14159265358979323846264338327950288);
+  const double s = s_lo + m * h;
+  c = two_over_sqrtpi * h * exp(s - mu * mu * exp(-2.0 * s) / 4.0);
+  t = exp(2.0 * s);
+}
+
+__device__ __forceinline__ double fit_error(int M, const double *c, const double *t, double r, double K) {
+  double sum = 0.0;
+  for (int m = 0; m < M; ++m) sum += c[m] * exp(-t[m] * r * r);
+  return fabs(sum - K) / K;
+}
+
+// Lower bounds of every candidate over the FIT_SUB points pts: half a warp per candidate, a lane per point
+// (one CTA per candidate used 16 of its 256 threads: 1.5 of the 2.45 ms of a fit went there).
+__global__ void fit_lower_kernel(double mu, int M, int n_cand, const int *pts, const double *rk, double *err) {
+  extern __shared__ double sh[];  // [candidates of the CTA][2][M]
+  const int half = threadIdx.x / FIT_SUB, lane = threadIdx.x % FIT_SUB;
+  const int cand = blockIdx.x * (blockDim.x / FIT_SUB) + half;
+  double *c = sh + half * 2 * M, *t = c + M;
+  if (cand < n_cand)
+    for (int m = lane; m < M; m += FIT_SUB) fit_term(mu, cand, m, c[m], t[m]);
+  __syncwarp();
+  double worst = 0.0;
+  if (cand < n_cand) {
+    const int p = pts[lane];
+    const double e = fit_error(M, c, t, rk[p], rk[FIT_NP + p]);
+    worst = e > worst ? e : worst;
+  }
+  for (int o = FIT_SUB / 2; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+  if (cand < n_cand && lane == 0) err[cand] = worst;
+}
+
+// Full errors of the listed candidates: CTA (candidate, 256 points), the maximum by atomics on the bits (the errors
+// are not negative, so their bits order as they do; err is zero before).  A candidate on one CTA kept 16 SMs busy.
+__global__ void fit_full_kernel(double mu, int M, const int *cands, const double *rk, double *err) {
   extern __shared__ double sh[];
   double *c = sh, *t = sh + M;
-  __shared__ double red[32];
-  const int cand = cands ? cands[blockIdx.x] : (int)blockIdx.x;
-  int i = cand / FIT_NS, j = cand % FIT_NS;
-  double h = (5.0 + i) / 100.0, s_lo = (j - 100.0) / 4.0;
-  const double two_over_sqrtpi = 2.0 / sqrt(3.14159265358979323846264338327950288);
-  for (int m = threadIdx.x; m < M; m += blockDim.x) {
-    double s = s_lo + m * h;
-    c[m] = two_over_sqrtpi * h * exp(s - mu * mu * exp(-2.0 * s) / 4.0);
-    t[m] = exp(2.0 * s);
-  }
+  for (int m = threadIdx.x; m < M; m += blockDim.x) fit_term(mu, cands[blockIdx.x], m, c[m], t[m]);
   __syncthreads();
+  const int p = blockIdx.y * blockDim.x + threadIdx.x;
   double worst = 0.0;
-  const int span = pts ? (int)blockDim.x : FIT_NP;
-  for (int p0 = 0; p0 < span; p0 += blockDim.x * stride) {  // block-uniform trip count
-    const int p = pts ? (threadIdx.x < npts ? pts[threadIdx.x] : FIT_NP) : p0 + threadIdx.x * stride;
-    if (p < FIT_NP) {
-      double r = r_lo * pow(r_hi / r_lo, (double)p / (double)(FIT_NP - 1));
-      double K = exp(-mu * r) / r, sum = 0.0;
-      for (int m = 0; m < M; ++m) sum += c[m] * exp(-t[m] * r * r);
-      double e = fabs(sum - K) / K;
-      worst = e > worst ? e : worst;
-    }
-    if (__syncthreads_or(worst > stop)) break;
+  if (p < FIT_NP) {
+    const double e = fit_error(M, c, t, rk[p], rk[FIT_NP + p]);
+    worst = e > worst ? e : worst;
   }
   for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = worst;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double w = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) w = fmax(w, red[q]);
-    err[blockIdx.x] = w;
-  }
+  if ((threadIdx.x & 31) == 0) atomicMax((unsigned long long *)err + blockIdx.x, (unsigned long long)__double_as_longlong(worst));
 }
 
 // --------------------------------------------------------------------------- blocks
@@ -438,11 +456,23 @@ cudaError_t upload_tables(cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_fit_search(double mu, int M, double r_lo, double r_hi, int stride, const int *d_pts, int npts,
-                              const int *d_cands, int n_cands, double stop, double *d_err, cudaStream_t s) {
-  if (d_pts && (npts < 1 || npts > 256)) return cudaErrorInvalidValue;
-  fit_search_kernel<<<counted((unsigned)n_cands), 256, 2 * M * sizeof(double), s>>>(
-      mu, M, r_lo, r_hi, stride, d_pts, npts, d_cands, stop, d_err);
+size_t fit_points_bytes() { return 2 * FIT_NP * sizeof(double); }
+
+cudaError_t launch_fit_lower(double mu, int M, double r_lo, double r_hi, const int *d_pts, double *d_rk, int n_cand,
+                             double *d_err, cudaStream_t s) {
+  fit_points_kernel<<<counted((FIT_NP + 255) / 256), 256, 0, s>>>(mu, r_lo, r_hi, d_rk);
+  const int per = 128 / FIT_SUB;
+  fit_lower_kernel<<<counted((unsigned)((n_cand + per - 1) / per)), 128, per * 2 * M * sizeof(double), s>>>(mu, M, n_cand, d_pts,
+                                                                                                          d_rk, d_err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fit_full(double mu, int M, const int *d_cands, int n_cands, const double *d_rk, double *d_err,
+                            cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(d_err, 0, n_cands * sizeof(double), s);
+  if (e != cudaSuccess) return e;
+  fit_full_kernel<<<counted(dim3((unsigned)n_cands, (FIT_NP + 255) / 256)), 256, 2 * M * sizeof(double), s>>>(mu, M, d_cands,
+                                                                                                             d_rk, d_err);
   return cudaGetLastError();
 }
 
