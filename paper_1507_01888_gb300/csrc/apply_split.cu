@@ -62,6 +62,7 @@ struct SplitArgs {
   const int *val2;               // key2-sorted -> dest-sorted position
   const int *grp_start;          // [n_groups + 1]
   const int *tile_gstart;        // [n_tiles + 1]
+  const int *tile_order;         // CTA -> tile, heaviest first (NULL: in order)
   uint64_t *out_keys;
   double *out_coeffs;
   int *err;
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wg = warp >> 2, quarter = warp & 3;
-  const int tile = blockIdx.x;
+  const int tile = a.tile_order ? MRA_IDX(a.tile_order[blockIdx.x], gridDim.x) : (int)blockIdx.x;
   const int g0 = a.tile_gstart[tile], g1 = a.tile_gstart[tile + 1];
 
   {  // zero the operand tiles once: contraction and row padding stay zero
@@ -642,6 +643,25 @@ __global__ void group_bounds_kernel(int64_t P, const uint64_t *key2s, const int 
   }
 }
 
+// Weight of a tile of G destinations: the kept terms of its records.  A warp per tile; the sort key is the
+// complement (heaviest first), capped to 16 bits so that the sort takes two passes.
+__global__ void tile_weight_kernel(int n_tiles, int G, int64_t nd, const int64_t *seg, const int *perm,
+                                   const uint64_t *rec_mask, uint32_t *key, int *val) {
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (t >= n_tiles) return;
+  const int64_t d0 = (int64_t)t * G, d1 = min(d0 + G, nd);
+  int w = 0;
+  for (int64_t r = seg[d0] + lane; r < seg[d1]; r += 32) {
+    const int64_t p = perm[r];
+    w += __popcll(rec_mask[2 * p]) + __popcll(rec_mask[2 * p + 1]);
+  }
+  for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  if (lane == 0) {
+    key[t] = 0xFFFFu - (uint32_t)min(w, 0xFFFF);
+    val[t] = t;
+  }
+}
+
 // Block pieces in the K-major core-matrix layout the MMA reads: piece p of block
 // x R (N = output index i, K = input index j), element (i, j) at
 // (i/8)*256 + (j/8)*128 + (i%8)*16 + (j%8)*2 of a 512-byte piece; zero outside k x k.  Blocks
@@ -770,6 +790,27 @@ int apply_split_run(const Operator &op, const mra_tree_view &in, const mra_apply
   group_bounds_kernel<<<counted(g), 256, 0, s>>>(P, key2s, head, gid, grp_start, tile_gstart, n_tiles);
   MRA_CUDA_TRY(cudaGetLastError());
 
+  // The tiles heaviest first, so that the last CTAs to start are short ones: a destination's terms run in
+  // series in one CTA (up to 27 M of them), and with the heavy ones last most SMs were idle at the end.
+  // Only where the CTAs do not all run at once.  key2 and key2s are free by now (n_tiles <= P entries of each).
+  int dev = 0, sms = 0;
+  MRA_CUDA_TRY(cudaGetDevice(&dev));
+  MRA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  int *tile_order = nullptr;
+  if (n_tiles > sms * (4 / tt)) {
+    uint32_t *wk0 = (uint32_t *)key2, *wk1 = wk0 + n_tiles;
+    int *wv0 = (int *)key2s, *wv1 = wv0 + n_tiles;
+    size_t need = 0;
+    MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, need, wk0, wk1, wv0, wv1, n_tiles, 0, 16, s));
+    if (need <= tmpb) {
+      tile_weight_kernel<<<counted((unsigned)((n_tiles + 7) / 8)), 256, 0, s>>>(n_tiles, G, nd, wk.seg, wk.perm, wk.rec_mask,
+                                                                                wk0, wv0);
+      MRA_CUDA_TRY(cudaGetLastError());
+      MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmpb, wk0, wk1, wv0, wv1, n_tiles, 0, 16, s));
+      tile_order = wv1;
+    }
+  }
+
   SplitArgs a{};
   a.k = k;
   a.M = op.M;
@@ -789,6 +830,7 @@ int apply_split_run(const Operator &op, const mra_tree_view &in, const mra_apply
   a.val2 = val2s;
   a.grp_start = grp_start;
   a.tile_gstart = tile_gstart;
+  a.tile_order = tile_order;
   a.out_keys = out.keys;
   a.out_coeffs = out.coeffs;
   a.err = err;
