@@ -93,6 +93,7 @@ struct SrcArgs {
   int join;                     // terms summed in D3 by the stage-3 MMAs before one flush
   int join_all;                 // 1: join in tiles of several sources too (else those flush every term)
   int compensated;              // record sums: 1 = FP32 sum + Kahan correction, 0 = plain FP32 sum
+  int parts;                    // CTAs per tile (1, 3 or 9): each takes the records of one residue of lx, or (lx, ly), mod 3
   int ahead;                    // block copies run this many terms ahead (1 .. src_nb - 2)
   int64_t n_src, n_rec, n_blocks;
 };
@@ -325,9 +326,9 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
       // ---------------------------------------------------------------- next tile
       if (tid == 0) s_tile = atomicAdd(a.tile_ctr, 1);
       wg_sync(1);
-      const int tile = s_tile;
-      if (tile >= *a.n_tiles) break;
-      if (a.inject_stall && tile == 0 && nfetch == 0) stalled = true;
+      if (s_tile >= *a.n_tiles * a.parts) break;
+      const int tile = s_tile / a.parts, part = s_tile - tile * a.parts;
+      if (a.inject_stall && s_tile == 0 && nfetch == 0) stalled = true;
       if (tid < G) t_src[tid] = a.tile_src[(int64_t)tile * G + tid];
       for (int e = tid; e < SRC_NG * G * 3; e += 128) {
         grp_rec[e] = -1;
@@ -358,6 +359,7 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
             atomicExch(a.err, 2);
             continue;
           }
+          if (a.parts > 1 && (a.parts == 3 ? lx % 3 : (lx % 3) * 3 + ly % 3) != part) continue;
           const int g = (lx * sw + ly) * SRC_NWIN + lz / 3, w = lz % 3;
           const int e = (g * G + i) * 3 + w;
           const uint64_t m0 = a.rec_mask[2 * p], m1 = a.rec_mask[2 * p + 1];
@@ -938,7 +940,12 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
   // persistent: two CTAs per SM (the tensor memory holds two of 256 columns), never more CTAs
   // than sources
   const int64_t max_tiles = G == 1 ? n_in : n_in / G + MRA_MAX_LEVEL + 1;
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)sms, max_tiles));
+  // A tile's passes run in series, so with few tiles the kernel lasts as long as one: then the (lx, ly) groups of a
+  // tile, which share nothing but the staged sources, go to three or nine CTAs.  512 boxes at k = 6 (171 tiles of
+  // 180 passes for 304 CTAs): the call 500 -> 419 us.
+  const int64_t slots = 2 * (int64_t)sms;
+  a.parts = max_tiles >= 8 * slots ? 1 : max_tiles >= slots ? 3 : 9;
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(slots, max_tiles * a.parts));
   if (((uintptr_t)partial & 15) != 0 || k3 % 4 != 0)
     return fail(MRA_ERR_ARG, "split apply: partial-sum buffer not 16-byte aligned or k^3 = %d not a multiple of 4", k3);
   if (wk.evk0) MRA_CUDA_TRY(cudaEventRecord(wk.evk0, s));

@@ -35,3 +35,22 @@ def test_split_wide_shape_is_independent_of_its_neighbours(mra, k, n_boxes):
     assert mra.compare(joined, whole)["rel_l2"] <= 4e-7
     exact, _ = mra.apply(op, tree, mra.make_opts(stencil=mra.STENCIL_NEAREST))
     assert mra.compare(whole, exact)["rel_l2"] <= 2e-7
+
+
+@pytest.mark.parametrize("k", [4, 6, 8, 10])
+def test_split_parts_of_a_tile_equal_whole_tiles(mra, k):
+    """With few tiles the source-stationary kernel gives a tile's groups to several CTAs; many copies of the
+    same function in one batch run whole tiles, and each copy has the single function's result bit for bit."""
+    import torch
+    keys, coeffs = W.random_tree_coeffs(20, k, 3, seed=k)
+    op = mra.Operator(0, 3, k, 32.0, 3, 3, max_disp=1, fit_eps=1e-4)
+    tree = mra.Tree.from_host(keys, coeffs, 32.0)
+    o = mra.make_opts(precision=mra.PREC_SPLIT_BF16, stencil=mra.STENCIL_NEAREST)
+    single, st = mra.apply(op, tree, o)
+    copies = 8 * 304 * {4: 8, 6: 3, 8: 2, 10: 1}[k] // 20 + 40
+    cat, offs = mra.concat_trees([tree] * copies)
+    out, out_offs = mra.BatchedApplier(op, cat, offs, o)(cat)
+    assert out.n == copies * single.n
+    want = single.coeffs[: single.n]
+    assert bool((out.coeffs[: out.n].reshape(copies, *want.shape) == want).all())
+    assert torch.equal(out.keys[: single.n], single.keys[: single.n])
