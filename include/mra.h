@@ -207,7 +207,7 @@ long long mra_launch_count(void);
 
 /* Device memory the library keeps for reuse: the scratch of the calls that allocate it
  * themselves (projection, norms and comparisons, reconstruction, truncation, products, the
- * non-standard applies) comes from a stream-ordered pool per device that holds on to freed
+ * non-standard applies; of the plain applies the partial sums, up to 4 GB in FP64) comes from a stream-ordered pool per device that holds on to freed
  * memory between calls.  This returns the pool's unused memory to the driver.  Memory of
  * allocations still in flight on a stream is not affected. */
 int mra_release_memory(void);

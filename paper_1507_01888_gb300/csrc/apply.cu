@@ -824,10 +824,13 @@ static bool apply_uses_f64_sym(const Operator &op, const mra_apply_opts &o) {
   return dmax <= 1;
 }
 
-size_t graph_partial_bytes(const Operator &op, const mra_apply_opts &o, int64_t P) {
+size_t graph_partial_bytes(const Operator &op, const mra_apply_opts &o, int64_t P, size_t *least) {
+  *least = 0;
   if (P <= 0) return 0;
-  if (apply_uses_src_path(op, o)) return (size_t)P * op.k * op.k * op.k * sizeof(float);
-  return apply_uses_f64_sym(op, o) ? f64_partial_bytes(op.k, P) : 0;
+  if (apply_uses_src_path(op, o)) return *least = (size_t)P * op.k * op.k * op.k * sizeof(float);
+  if (!apply_uses_f64_sym(op, o)) return 0;
+  *least = f64_partial_least(op.k, P);
+  return f64_partial_bytes(op.k, P);
 }
 
 size_t apply_workspace_bytes(const Operator &op, const mra_apply_opts &o, int64_t n_in) {

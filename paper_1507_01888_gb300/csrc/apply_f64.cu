@@ -37,6 +37,7 @@ namespace {
 
 constexpr int PT = 4;               // elements per thread (9 accumulators each)
 constexpr int F64_MAX_THREADS = 416;
+constexpr size_t F64_MAX_SMEM = 200 * 1024;  // dynamic shared memory of a CTA
 constexpr size_t F64_PARTIAL_BYTES = (size_t)4 << 30;      // most scratch of one range of records
 constexpr size_t F64_PARTIAL_BYTES_MIN = (size_t)64 << 20;  // smallest tried when memory is short
 
@@ -459,7 +460,7 @@ void f64_shape(int k, int64_t n_src, int sms, int *nx_out, int *threads_out) {
     for (int ept = PT / 2; ept >= 1; --ept) {
       const int threads = ((nx * k * k + ept - 1) / ept + 31) / 32 * 32, warps = threads / 32;
       const size_t smem = f64_smem(k, nx) + 1024;
-      if (threads > F64_MAX_THREADS || smem > 200 * 1024) continue;
+      if (threads > F64_MAX_THREADS || smem > F64_MAX_SMEM) continue;
       const int64_t ctas = n_src * ((k + 2 * nx - 1) / (2 * nx) + (k + nx - 1) / nx);
       const int64_t per_sm = (ctas + sms - 1) / sms;
       const int64_t resident = std::min<int64_t>(per_sm, std::min<int64_t>(512 / threads, (228 * 1024) / smem));
@@ -491,6 +492,11 @@ size_t f64_partial_bytes(int k, int64_t P) {
   return std::min((size_t)P * row, std::max(F64_PARTIAL_BYTES, row));
 }
 
+size_t f64_partial_least(int k, int64_t P) {
+  const size_t row = (size_t)k * k * k * sizeof(double);
+  return std::min(f64_partial_bytes(k, P), std::max(F64_PARTIAL_BYTES_MIN, row));
+}
+
 int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &out, const ApplyWork &wk, cudaStream_t s) {
   const int k = op.k, k3 = k * k * k;
   const int64_t P = wk.P, nd = wk.n_dest;
@@ -498,18 +504,20 @@ int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &ou
   int dev = 0, sms = 0;
   MRA_CUDA_TRY(cudaGetDevice(&dev));
   MRA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  size_t bytes = f64_partial_bytes(k, P);
+  size_t bytes = wk.fx ? wk.fx->partial_bytes : f64_partial_bytes(k, P);
+  const size_t least = f64_partial_least(k, P);
   double *partial = wk.fx ? (double *)wk.fx->partial : nullptr;
   if (!wk.fx) {
     // when memory is short, smaller ranges of records
     while (pool_malloc((void **)&partial, bytes, s) != cudaSuccess) {
       cudaGetLastError();
-      if (bytes <= std::max(F64_PARTIAL_BYTES_MIN, row)) return fail(MRA_ERR_CUDA, "mra_apply: out of device memory for the partial sums");
-      bytes = std::max(bytes / 2, row);
+      if (bytes <= least) return fail(MRA_ERR_CUDA, "mra_apply: out of device memory for the partial sums");
+      bytes = std::max(bytes / 2, least);
     }
   }
   if (!partial) return fail(MRA_ERR_ARG, "mra_apply: no partial-sum buffer for the recorded apply");
   const int64_t range = (int64_t)(bytes / row);
+  if (range < 1) return fail(MRA_ERR_ARG, "mra_apply: partial-sum buffer smaller than one record");
   F64Args a{};
   a.k = k;
   int threads = 32;
@@ -535,9 +543,11 @@ int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &ou
   a.n_src = in.n;
   a.n_rec = P;
   const size_t smem = f64_smem(k, a.nx), dsm = a.pairs ? row : 0;
-  cudaError_t e = cudaFuncSetAttribute(apply_f64_sym_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && dsm > 48 * 1024)
-    e = cudaFuncSetAttribute(dest_sum_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
+  // the same limit whatever the order, so that callers on several threads do not lower it for one another
+  cudaError_t e = cudaFuncSetAttribute(apply_f64_sym_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F64_MAX_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(dest_sum_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             MRA_MAX_NS_K * MRA_MAX_NS_K * MRA_MAX_NS_K * (int)sizeof(double));
   if (e == cudaSuccess && wk.ev0) e = cudaEventRecord(wk.ev0, s);
   for (int64_t p0 = 0; p0 < P && e == cudaSuccess; p0 += range) {
     a.p0 = p0;

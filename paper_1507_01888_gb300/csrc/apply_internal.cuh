@@ -14,7 +14,8 @@ struct FixedSizes {
   int64_t P = 0, nd = 0;
   int *status = nullptr;                  // device word
   const int64_t *d_in_offsets = nullptr;  // device copy of the batched input offsets (nfunc + 1)
-  void *partial = nullptr;                // the source-stationary kernels' partial sums (graph_partial_bytes)
+  void *partial = nullptr;                // the source-stationary kernels' partial sums, of partial_bytes
+  size_t partial_bytes = 0;
 };
 
 // The sorted work list handed from the screen/sort stage to an apply kernel.
@@ -65,8 +66,10 @@ bool apply_uses_src_path(const Operator &op, const mra_apply_opts &o);
 int f64_parity_build(Operator &op, cudaStream_t s);
 size_t f64_partial_bytes(int k, int64_t P);
 int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &out, const ApplyWork &wk, cudaStream_t s);
-// bytes of partial sums that a recorded apply with P records owns (0: its kernel needs none)
-size_t graph_partial_bytes(const Operator &op, const mra_apply_opts &o, int64_t P);
+// bytes of partial sums that a recorded apply with P records owns (0: its kernel needs none), and the fewest it
+// can do with
+size_t graph_partial_bytes(const Operator &op, const mra_apply_opts &o, int64_t P, size_t *least);
+size_t f64_partial_least(int k, int64_t P);
 // test hook of the failure path (one-shot), and the fixed-size mode's status from a kernel error word
 bool take_injected_stall();
 void split_fixed_err(const int *err, int *status, cudaStream_t s);

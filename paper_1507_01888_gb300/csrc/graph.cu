@@ -84,10 +84,15 @@ int mra_apply_graph_create(const mra_operator *h, int nfunc, const mra_tree_view
   g->fx.d_in_offsets = g->d_in_offsets;
   g->n_out = out->n;
   const Operator *op = reinterpret_cast<const Operator *>(h);
-  if (const size_t pb = graph_partial_bytes(*op, *o, st.pairs)) {  // the recorded apply's partial sums, owned by the graph
-    e = cudaMalloc(&g->d_partial, pb);
+  size_t least = 0;
+  if (size_t pb = graph_partial_bytes(*op, *o, st.pairs, &least)) {  // the recorded apply's partial sums, owned by the graph
+    while ((e = cudaMalloc(&g->d_partial, pb)) != cudaSuccess && pb > least) {  // memory is short: less where less will do
+      cudaGetLastError();
+      pb = pb / 2 > least ? pb / 2 : least;
+    }
     if (e != cudaSuccess) return bail(MRA_ERR_CUDA, "partial-sum buffer", e);
     g->fx.partial = g->d_partial;
+    g->fx.partial_bytes = pb;
   }
   e = cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) return bail(MRA_ERR_CUDA, "capture stream", e);

@@ -108,6 +108,9 @@ constexpr int BOX_THREADS = 512;
 // Shared memory of the transforms: U (k^2) and the buffers up (S 8 k^3, a 4 k^3) and down (7 k^3) need.
 size_t up_smem(int k) { return (size_t)(k * k + 12 * k * k * k) * 8; }
 size_t down_smem(int k) { return (size_t)(k * k + 7 * k * k * k) * 8; }
+// The kernels' dynamic shared memory limit: one value for every order, so that callers on several threads do not
+// lower it for one another (at order 16 a box takes 226 KB, beside up to 1 KB of static shared memory).
+constexpr int BOX_SMEM = 226 * 1024;
 
 // S (shared, complete, overwritten) filtered to the parent's coefficients, written to s_out.
 __device__ __forceinline__ void filter_box(int k, const double *U, double *S, double *a, double *s_out) {
@@ -586,7 +589,7 @@ __global__ void emit_kept_kernel(int64_t n_in, int64_t nc, int k3, const uint64_
                                  const uint64_t *cand, const double *pv, const int *keep, const int *pos, int64_t cap,
                                  uint64_t *okeys, double *ocoeffs) {
   const int64_t i = blockIdx.x;
-  if (!keep[i]) return;
+  if (!keep[i] || pos[n_in + nc] > cap) return;
   const bool leaf = i < n_in;
   const uint64_t key = leaf ? keys[i] : cand[i - n_in];
   const uint64_t *other = leaf ? cand : keys;
@@ -596,7 +599,6 @@ __global__ void emit_kept_kernel(int64_t n_in, int64_t nc, int k3, const uint64_
     if (other[mid] < key) lo = mid + 1; else hi = mid;
   }
   const int64_t o = leaf ? (int64_t)pos[i] + pos[n_in + lo] - pos[n_in] : (int64_t)pos[i] - pos[n_in] + pos[lo];
-  if (o >= cap) return;
   const double *v = leaf ? coeffs + i * k3 : pv + (i - n_in) * k3;
   if (threadIdx.x == 0) okeys[o] = key;
   for (int e = threadIdx.x; e < k3; e += blockDim.x) ocoeffs[o * k3 + e] = v[e];
@@ -854,8 +856,8 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
 
   // ---- compress: S^n and s^n for n = N-1 .. n0
   const size_t sh_c = up_smem(k), sh_d = down_smem(k);
-  MRA_CUDA_TRY(cudaFuncSetAttribute(compress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_c));
-  MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
+  MRA_CUDA_TRY(cudaFuncSetAttribute(compress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BOX_SMEM));
+  MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BOX_SMEM));
   double *s_all = (double *)(w + Lw.s), *S_all = (double *)(w + Lw.S);
   for (int n = N - 1; n >= n0; --n) {
     const double *fine = n == N - 1 ? in->coeffs : s_all + Lw.first[n + 1] * k3;
@@ -1117,6 +1119,8 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
                 (long long)out->cap);
   }
   NS_ALLOC(dst, int64_t, 8 * nh);
+  const uint64_t *leaf_sorted = nullptr;
+  const int *leaf_id = nullptr;
   {
     NS_ALLOC(lk, uint64_t, 8 * nh);
     NS_ALLOC(lks, uint64_t, 8 * nh);
@@ -1135,16 +1139,16 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
     MRA_CUDA_TRY(cudaStreamSynchronize(s));
     if ((int64_t)hfound != nh - boxes(n0))  // every halo box is a child of one of the level above
       return fail(MRA_ERR_NUMERIC, "mra_apply_ns_tree: a halo box lies outside the result tree");
-    leaf_places_kernel<<<counted((unsigned)((nout + 255) / 256)), 256, 0, s>>>(nout, lks, ids, dst, out->keys);
-    MRA_CUDA_TRY(cudaGetLastError());
-    for (void *p : {(void *)lk, (void *)lks, (void *)id, (void *)ids, (void *)tmp, (void *)found}) drop(p);
+    for (void *p : {(void *)lk, (void *)id, (void *)tmp, (void *)found}) drop(p);
+    leaf_sorted = lks;
+    leaf_id = ids;
   }
 
   // ---- compress, from the deepest interior level up; all levels' S and s back to back in key order
   const size_t sh_c = up_smem(k), sh_d = down_smem(k);
   const int kk3 = kk * kk * kk;
-  MRA_CUDA_TRY(cudaFuncSetAttribute(compress_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_c));
-  MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
+  MRA_CUDA_TRY(cudaFuncSetAttribute(compress_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BOX_SMEM));
+  MRA_CUDA_TRY(cudaFuncSetAttribute(sum_down_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BOX_SMEM));
   NS_ALLOC(S_all, double, n_int * kk3);
   NS_ALLOC(s_all, double, n_int * k3);
   auto first = [&](int n) { return off_int[n] - off_int[n0]; };
@@ -1159,6 +1163,9 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
   MRA_CUDA_TRY(cudaMemcpyAsync(hint, d_int, sizeof(int), cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
   if (hint[0]) return fail(MRA_ERR_ARG, "mra_apply_ns_tree: the leaves are not a complete octree");
+  // the input has been read: the result may be written (also where it shares the input's buffers)
+  leaf_places_kernel<<<counted((unsigned)((nout + 255) / 256)), 256, 0, s>>>(nout, leaf_sorted, leaf_id, dst, out->keys);
+  MRA_CUDA_TRY(cudaGetLastError());
 
   // one library apply of opx on the interior boxes [b0, b1) (their coefficients at coeffs): its rows appended
   // at okeys/ocoeffs + *nout_rows
@@ -1381,7 +1388,7 @@ extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void
   copy_tops_kernel<<<counted((unsigned)n_in), 128, 0, s>>>(n_in, 8 * ni, k3, dst, in->coeffs, out->coeffs);
   MRA_CUDA_TRY(cudaGetLastError());
   const size_t sh_d = down_smem(k);
-  MRA_CUDA_TRY(cudaFuncSetAttribute(pass_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_d));
+  MRA_CUDA_TRY(cudaFuncSetAttribute(pass_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BOX_SMEM));
   RC_ALLOC(r, double, ni * k3);
   for (int n = nmin; n < nmax; ++n) {
     const int64_t nj = info[n + 1] - info[n];
@@ -1478,7 +1485,7 @@ extern "C" int mra_truncate(const mra_tree_view *in, double thresh, mra_tree_vie
     // S stays in shared memory up to k = 12 (96 k^3 bytes); above, only the filter's pieces (56 k^3)
     const int s_smem = k <= 12 ? 1 : 0;
     const size_t sh = s_smem ? up_smem(k) : down_smem(k);
-    MRA_CUDA_TRY(cudaFuncSetAttribute(truncate_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
+    MRA_CUDA_TRY(cudaFuncSetAttribute(truncate_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BOX_SMEM));
     int64_t end = nc;
     for (int n = 19; n >= 0; --n) {
       const int64_t here = info[23 + n];
@@ -1501,8 +1508,22 @@ extern "C" int mra_truncate(const mra_tree_view *in, double thresh, mra_tree_vie
   MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp2, tsc, keep, pos, (int)(ne + 1), s));
   sum_kernel<<<counted(1), 1024, 0, s>>>(nc, d2, d2 + nc);
   MRA_CUDA_TRY(cudaGetLastError());
+  // where the result shares the input's buffers, it is put together elsewhere first
+  auto overlap = [](const void *a, size_t na, const void *b, size_t nb) {
+    return (const char *)a < (const char *)b + nb && (const char *)b < (const char *)a + na;
+  };
+  const size_t row = (size_t)k3 * sizeof(double), cap = (size_t)std::min<int64_t>(out->cap, ne);
+  const bool shared = overlap(in->keys, n_in * 8, out->keys, cap * 8) || overlap(in->coeffs, n_in * row, out->coeffs, cap * row);
+  uint64_t *okeys = out->keys;
+  double *ocoeffs = out->coeffs;
+  if (shared) {
+    TR_ALLOC(tk, uint64_t, cap);
+    TR_ALLOC(tv, double, cap * k3);
+    okeys = tk;
+    ocoeffs = tv;
+  }
   emit_kept_kernel<<<counted((unsigned)ne), 128, 0, s>>>(n_in, nc, k3, in->keys, in->coeffs, cand, pv, keep, pos, out->cap,
-                                                         out->keys, out->coeffs);
+                                                         okeys, ocoeffs);
   MRA_CUDA_TRY(cudaGetLastError());
   int nout = 0;
   double e2 = 0.0;
@@ -1512,6 +1533,11 @@ extern "C" int mra_truncate(const mra_tree_view *in, double thresh, mra_tree_vie
   out->n = nout;
   if (nout > out->cap)
     return fail(MRA_ERR_CAPACITY, "mra_truncate: %d leaves, capacity %lld", nout, (long long)out->cap);
+  if (shared) {
+    MRA_CUDA_TRY(cudaMemcpyAsync(out->keys, okeys, (size_t)nout * 8, cudaMemcpyDeviceToDevice, s));
+    MRA_CUDA_TRY(cudaMemcpyAsync(out->coeffs, ocoeffs, (size_t)nout * row, cudaMemcpyDeviceToDevice, s));
+    MRA_CUDA_TRY(cudaStreamSynchronize(s));
+  }
   if (err2) *err2 = e2;
   return MRA_OK;
 #undef TR_ALLOC

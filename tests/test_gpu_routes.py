@@ -54,3 +54,40 @@ def test_split_parts_of_a_tile_equal_whole_tiles(mra, k):
     want = single.coeffs[: single.n]
     assert bool((out.coeffs[: out.n].reshape(copies, *want.shape) == want).all())
     assert torch.equal(out.keys[: single.n], single.keys[: single.n])
+
+
+def test_truncate_into_its_own_buffers(mra):
+    """mra_truncate with the result in the input's buffers, and with too little room (which leaves them as they are)."""
+    import ctypes
+    f = W.gaussian_sum(2, 1.0, 50.0, seed=5, centre_box=5.0)
+    t = mra.project(f, 5, 16.0, thresh=1e-6)
+    ref, err2 = mra.truncate(t, 1e-3)
+    assert ref.n < t.n
+    keys, coeffs = t.keys.clone(), t.coeffs.clone()
+    vin, vout, e2 = t.view(), t.view(), ctypes.c_double()
+    vout.cap = ref.n - 1
+    assert mra.load().mra_truncate(ctypes.byref(vin), 1e-3, ctypes.byref(vout), ctypes.byref(e2),
+                                   mra._stream(None)) == mra.MRA_ERR_CAPACITY
+    assert vout.n == ref.n and bool((t.keys == keys).all()) and bool((t.coeffs == coeffs).all())
+    vout = t.view()
+    assert mra.load().mra_truncate(ctypes.byref(vin), 1e-3, ctypes.byref(vout), ctypes.byref(e2), mra._stream(None)) == 0
+    assert vout.n == ref.n and e2.value == err2
+    assert bool((t.keys[: ref.n] == ref.keys[: ref.n]).all()) and bool((t.coeffs[: ref.n] == ref.coeffs[: ref.n]).all())
+
+
+@pytest.mark.parametrize("k", [3, 10])
+def test_fp64_graph_replay_equals_plain_apply(mra, k):
+    import torch
+    keys, coeffs = W.random_tree_coeffs(60, k, 3, seed=k)
+    op = mra.Operator(0, 5, k, 32.0, 3, 3, max_disp=1, fit_eps=1e-4)
+    tree = mra.Tree.from_host(keys, coeffs, 32.0)
+    o = mra.make_opts()
+    plain, _ = mra.apply(op, tree, o)
+    g = mra.ApplyGraph(op, tree, o)
+    for scale in (1.0, -0.5):
+        tree.coeffs.mul_(scale)
+        got = g.launch()
+        g.status()
+        want, _ = mra.apply(op, tree, o)
+        assert torch.equal(got.coeffs[: got.n], want.coeffs[: want.n])
+        assert torch.equal(got.keys[: got.n], plain.keys[: plain.n])
