@@ -23,6 +23,7 @@
 #include <cub/cub.cuh>
 
 #include "apply_internal.cuh"
+#include "reconstruct.cuh"
 #include "twoscale.cuh"
 
 namespace mra {
@@ -419,37 +420,51 @@ __global__ void recon_nodes_kernel(int64_t ni, const uint64_t *ikeys, int64_t n_
   }
 }
 
+// One or two functions on the same boxes (blockIdx.y): their input, the sums on the interior boxes, the leaves.
+struct SumDownSets {
+  SumDown f[2];
+  double *r[2];
+};
+__device__ __forceinline__ const double *box_coeffs(const SumDown &f, int64_t b, int k3) {
+  if (b >= 0 && f.row) b = f.row[b];
+  return b >= 0 ? f.coeffs + b * k3 : nullptr;
+}
+
 // The tops that are leaves, copied to their places.
-__global__ void copy_tops_kernel(int64_t n_in, int64_t base, int k3, const int64_t *dst, const double *coeffs, double *out) {
+__global__ void copy_tops_kernel(int64_t n_in, int64_t base, int k3, const int64_t *dst,
+                                 const __grid_constant__ SumDownSets sets) {
   const int64_t b = blockIdx.x, t = dst[base + b];
   if (t == -1) return;
-  double *o = out + (-2 - t) * k3;
-  for (int e = threadIdx.x; e < k3; e += blockDim.x) o[e] = coeffs[b * k3 + e];
+  const SumDown f = blockIdx.y ? sets.f[1] : sets.f[0];
+  const double *c = box_coeffs(f, b, k3);
+  double *o = f.out + (-2 - t) * k3;
+  for (int e = threadIdx.x; e < k3; e += blockDim.x) o[e] = c ? c[e] : 0.0;
 }
 
 // One CTA per interior box of one level (j0 + blockIdx.x): what it was passed plus its own input coefficients,
 // to its eight children by the two-scale relation; a leaf child adds its own input coefficients.
-__global__ void pass_down_kernel(int k, int64_t j0, double *r, const int64_t *iown, const unsigned char *start,
-                                 const int64_t *dst, const int64_t *own, const double *coeffs, const double *Ub,
-                                 double *out) {
+__global__ void pass_down_kernel(int k, int64_t j0, const int64_t *iown, const unsigned char *start, const int64_t *dst,
+                                 const int64_t *own, const double *Ub, const __grid_constant__ SumDownSets sets) {
   extern __shared__ double sh[];
   __shared__ double *to[8];
   __shared__ const double *add[8];
   const int64_t p = j0 + blockIdx.x;
   const int k3 = k * k * k;
+  const SumDown f = blockIdx.y ? sets.f[1] : sets.f[0];
+  double *r = blockIdx.y ? sets.r[1] : sets.r[0];
   double *U = sh, *d = U + k * k, *a = d + k3, *b = a + 2 * k3;
-  const int64_t in = iown[p];
+  const double *in = box_coeffs(f, iown[p], k3);
   const bool first = start[p];
   for (int e = threadIdx.x; e < k * k; e += blockDim.x) U[e] = Ub[e];
   for (int e = threadIdx.x; e < k3; e += blockDim.x) {
     double v = first ? 0.0 : r[p * k3 + e];
-    if (in >= 0) v = first ? coeffs[in * k3 + e] : v + coeffs[in * k3 + e];
+    if (in) v = first ? in[e] : v + in[e];
     d[e] = v;
   }
   if (threadIdx.x < 8) {
-    const int64_t t = dst[8 * p + threadIdx.x], o = own[8 * p + threadIdx.x];
-    to[threadIdx.x] = t >= 0 ? r + t * k3 : out + (-2 - t) * k3;
-    add[threadIdx.x] = o >= 0 ? coeffs + o * k3 : nullptr;
+    const int64_t t = dst[8 * p + threadIdx.x];
+    to[threadIdx.x] = t >= 0 ? r + t * k3 : f.out + (-2 - t) * k3;
+    add[threadIdx.x] = box_coeffs(f, own[8 * p + threadIdx.x], k3);
   }
   __syncthreads();
   twoscale::down(k, U, d, a, b, [&](int I, int J, int Lq, double v) {
@@ -1264,56 +1279,48 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
 
 
 // ---------------------------------------------------------------- reconstruct (host)
-extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void *stream) {
-  if (!in || !out) return fail(MRA_ERR_ARG, "mra_reconstruct: NULL argument");
-  if (in->n < 0 || (in->n > 0 && (!in->keys || !in->coeffs))) return fail(MRA_ERR_ARG, "mra_reconstruct: bad input");
-  if (in->k < 1 || in->k > MRA_MAX_K) return fail(MRA_ERR_ARG, "mra_reconstruct: k=%d outside 1..%d", in->k, MRA_MAX_K);
-  if (in->n >= (1LL << 31)) return fail(MRA_ERR_ARG, "mra_reconstruct: more than 2^31 boxes");
-  if (out->k != in->k || out->cap < 0 || (out->cap > 0 && (!out->keys || !out->coeffs)))
-    return fail(MRA_ERR_ARG, "mra_reconstruct: bad output view");
-  out->L = in->L;
-  if (in->n == 0) {
-    out->n = 0;
-    return MRA_OK;
-  }
-  cudaStream_t s = (cudaStream_t)stream;
-  const int k = in->k, kk = 2 * k, k3 = k * k * k;
-  const int64_t n_in = in->n;
-  std::vector<void *> held;
-  struct Release {
-    std::vector<void *> &v;
-    cudaStream_t s;
-    ~Release() {
-      for (void *p : v) cudaFreeAsync(p, s);
-      cudaStreamSynchronize(s);
-    }
-  } release{held, s};
-  auto dalloc = [&](size_t bytes) -> void * {
-    void *p = nullptr;
-    if (pool_malloc(&p, bytes ? bytes : 1, s) != cudaSuccess) return nullptr;
-    held.push_back(p);
-    return p;
-  };
-  auto drop = [&](void *p) {
-    auto it = std::find(held.begin(), held.end(), p);
-    if (it != held.end()) {
-      cudaFreeAsync(p, s);
-      held.erase(it);
-    }
-  };
-#define RC_ALLOC(var, type, count)                                                              \
-  type *var = (type *)dalloc((size_t)(count) * sizeof(type));                                   \
-  if (!var) return fail(MRA_ERR_CUDA, "mra_reconstruct: out of device memory (%s)", #var);
+namespace mra {
 
+Reconstruct::~Reconstruct() {
+  for (void *p : held) cudaFreeAsync(p, s);
+}
+
+void *Reconstruct::dalloc(size_t bytes) {
+  void *p = nullptr;
+  if (pool_malloc(&p, bytes ? bytes : 1, s) != cudaSuccess) return nullptr;
+  held.push_back(p);
+  return p;
+}
+
+void Reconstruct::drop(void *p) {
+  auto it = std::find(held.begin(), held.end(), p);
+  if (it != held.end()) {
+    cudaFreeAsync(p, s);
+    held.erase(it);
+  }
+}
+
+#define RC_GET(var, type, count)                        \
+  var = (type *)dalloc((size_t)(count) * sizeof(type)); \
+  if (!var) return fail(MRA_ERR_CUDA, "mra_reconstruct: out of device memory (%s)", #var);
+#define RC_ALLOC(var, type, count) \
+  type *var = nullptr;             \
+  RC_GET(var, type, count)
+
+int Reconstruct::plan(int k_, int64_t n, const uint64_t *keys_) {
+  k = k_;
+  n_in = n;
+  keys = keys_;
+  const int kk = 2 * k;
   // order and the level ranges of the sorted input
   RC_ALLOC(d_off, int64_t, 22);
   MRA_CUDA_TRY(cudaMemsetAsync(d_off, 0, 22 * 8, s));
-  leaf_offsets_kernel<<<counted((unsigned)((n_in + 256) / 256)), 256, 0, s>>>(n_in, in->keys, d_off, d_off + 21);
+  leaf_offsets_kernel<<<counted((unsigned)((n_in + 256) / 256)), 256, 0, s>>>(n_in, keys, d_off, d_off + 21);
   MRA_CUDA_TRY(cudaGetLastError());
-  RC_ALLOC(top, int, n_in);
-  top_level_kernel<<<counted((unsigned)((n_in + 255) / 256)), 256, 0, s>>>(n_in, in->keys, top);
+  RC_GET(top, int, n_in);
+  top_level_kernel<<<counted((unsigned)((n_in + 255) / 256)), 256, 0, s>>>(n_in, keys, top);
   MRA_CUDA_TRY(cudaGetLastError());
-  RC_ALLOC(Ub, double, kk * k);
+  RC_GET(Ub, double, kk * k);
   std::vector<double> U(2 * k * k);
   two_scale(k, U.data());  // [c][i][j]: the rows (c, i) of Ubar in order
   MRA_CUDA_TRY(cudaMemcpyAsync(Ub, U.data(), U.size() * 8, cudaMemcpyHostToDevice, s));
@@ -1322,7 +1329,7 @@ extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
   if (off[21] == 2) return fail(MRA_ERR_ARG, "mra_reconstruct: level above %d", MRA_MAX_LEVEL);
   if (off[21]) return fail(MRA_ERR_ARG, "mra_reconstruct: keys must be sorted and unique");
-  int nmin = 0, nmax = MRA_MAX_LEVEL;
+  nmin = 0, nmax = MRA_MAX_LEVEL;
   while (off[nmin + 1] == 0) ++nmin;
   while (off[nmax] == n_in) --nmax;
   // The result's tree depends on the keys alone: the interior boxes of all levels (one sort), their children and
@@ -1336,7 +1343,7 @@ extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void
   RC_ALLOC(d_info, int64_t, 24);  // offsets of the interior levels, then tops, interior tops, interior boxes
   MRA_CUDA_TRY(cudaMemsetAsync(d_info, 0, 24 * 8, s));
   int64_t *d_ni = d_info + 23;
-  interior_all_kernel<<<counted((unsigned)((na + 255) / 256)), 256, 0, s>>>(n_in, in->keys, top, nmin, nlev, anc);
+  interior_all_kernel<<<counted((unsigned)((na + 255) / 256)), 256, 0, s>>>(n_in, keys, top, nmin, nlev, anc);
   MRA_CUDA_TRY(cudaGetLastError());
   {
     size_t tb = 0, t2 = 0;
@@ -1350,28 +1357,28 @@ extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void
     MRA_CUDA_TRY(cub::DeviceSelect::Unique(tmp, tt, iall, anc, d_ni, (int)na, s));
     drop(tmp);
   }
-  const uint64_t *ik = anc;  // the unique interior keys, in key order (so level by level)
+  ik = anc;  // the unique interior keys, in key order (so level by level)
   level_offsets_kernel<<<counted(1), 32, 0, s>>>(ik, d_ni, d_info);
   MRA_CUDA_TRY(cudaGetLastError());
-  count_tops_kernel<<<counted((unsigned)((n_in + 255) / 256)), 256, 0, s>>>(n_in, in->keys, top, ik, d_info + 20,
+  count_tops_kernel<<<counted((unsigned)((n_in + 255) / 256)), 256, 0, s>>>(n_in, keys, top, ik, d_info + 20,
                                                                             (unsigned long long *)(d_info + 21));
   MRA_CUDA_TRY(cudaGetLastError());
-  int64_t info[24];
   MRA_CUDA_TRY(cudaMemcpyAsync(info, d_info, 24 * 8, cudaMemcpyDeviceToHost, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
   drop(iall);
-  const int64_t ni = info[20], ntop = info[21], itop = info[22];
-  const int64_t nout = 8 * ni - (ni - itop) + (ntop - itop);
-  if (nout > out->cap) {
-    out->n = nout;
-    return fail(MRA_ERR_CAPACITY, "mra_reconstruct: %lld leaves, capacity %lld", (long long)nout, (long long)out->cap);
-  }
+  const int64_t ntop = info[21], itop = info[22];
+  ni = info[20];
+  nout = 8 * ni - (ni - itop) + (ntop - itop);
+  return MRA_OK;
+}
+
+int Reconstruct::place(uint64_t *out_keys) {
   const int64_t nn = 8 * ni + n_in;
   if (nn >= (int64_t)INT32_MAX) return fail(MRA_ERR_ARG, "mra_reconstruct: too many boxes in the result");
-  RC_ALLOC(dst, int64_t, nn);
-  RC_ALLOC(own, int64_t, 8 * ni);
-  RC_ALLOC(iown, int64_t, ni);
-  RC_ALLOC(start, unsigned char, ni);
+  RC_GET(dst, int64_t, nn);
+  RC_GET(own, int64_t, 8 * ni);
+  RC_GET(iown, int64_t, ni);
+  RC_GET(start, unsigned char, ni);
   RC_ALLOC(lk, uint64_t, nn);
   RC_ALLOC(lks, uint64_t, nn);
   RC_ALLOC(id, int, nn);
@@ -1379,28 +1386,66 @@ extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void
   size_t tb = 0;
   MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, lk, lks, id, ids, (int)nn, 0, 64, s));
   RC_ALLOC(tmp, unsigned char, tb);
-  recon_nodes_kernel<<<counted((unsigned)((nn + 255) / 256)), 256, 0, s>>>(ni, ik, n_in, in->keys, top, dst, own, iown, start,
-                                                                           lk, id);
+  recon_nodes_kernel<<<counted((unsigned)((nn + 255) / 256)), 256, 0, s>>>(ni, ik, n_in, keys, top, dst, own, iown, start, lk,
+                                                                           id);
   MRA_CUDA_TRY(cudaGetLastError());
   MRA_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp, tb, lk, lks, id, ids, (int)nn, 0, 64, s));
-  leaf_places_kernel<<<counted((unsigned)((nout + 255) / 256)), 256, 0, s>>>(nout, lks, ids, dst, out->keys);
+  leaf_places_kernel<<<counted((unsigned)((nout + 255) / 256)), 256, 0, s>>>(nout, lks, ids, dst, out_keys);
   MRA_CUDA_TRY(cudaGetLastError());
-  copy_tops_kernel<<<counted((unsigned)n_in), 128, 0, s>>>(n_in, 8 * ni, k3, dst, in->coeffs, out->coeffs);
+  return MRA_OK;
+}
+
+int Reconstruct::run(int nf, const SumDown *f) {
+  const int k3 = k * k * k;
+  SumDownSets sets{};
+  for (int i = 0; i < nf; ++i) {
+    sets.f[i] = f[i];
+    RC_GET(sets.r[i], double, ni * k3);
+  }
+  copy_tops_kernel<<<counted(dim3((unsigned)n_in, (unsigned)nf)), 128, 0, s>>>(n_in, 8 * ni, k3, dst, sets);
   MRA_CUDA_TRY(cudaGetLastError());
   const size_t sh_d = down_smem(k);
   MRA_CUDA_TRY(cudaFuncSetAttribute(pass_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BOX_SMEM));
-  RC_ALLOC(r, double, ni * k3);
   for (int n = nmin; n < nmax; ++n) {
     const int64_t nj = info[n + 1] - info[n];
     if (nj == 0) continue;
-    pass_down_kernel<<<counted((unsigned)nj), BOX_THREADS, sh_d, s>>>(k, info[n], r, iown, start, dst, own, in->coeffs, Ub,
-                                                              out->coeffs);
+    pass_down_kernel<<<counted(dim3((unsigned)nj, (unsigned)nf)), BOX_THREADS, sh_d, s>>>(k, info[n], iown, start, dst, own, Ub,
+                                                                                     sets);
     MRA_CUDA_TRY(cudaGetLastError());
   }
-  MRA_CUDA_TRY(cudaStreamSynchronize(s));
-  out->n = nout;
   return MRA_OK;
+}
 #undef RC_ALLOC
+#undef RC_GET
+
+}  // namespace mra
+
+extern "C" int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void *stream) {
+  if (!in || !out) return fail(MRA_ERR_ARG, "mra_reconstruct: NULL argument");
+  if (in->n < 0 || (in->n > 0 && (!in->keys || !in->coeffs))) return fail(MRA_ERR_ARG, "mra_reconstruct: bad input");
+  if (in->k < 1 || in->k > MRA_MAX_K) return fail(MRA_ERR_ARG, "mra_reconstruct: k=%d outside 1..%d", in->k, MRA_MAX_K);
+  if (in->n >= (1LL << 31)) return fail(MRA_ERR_ARG, "mra_reconstruct: more than 2^31 boxes");
+  if (out->k != in->k || out->cap < 0 || (out->cap > 0 && (!out->keys || !out->coeffs)))
+    return fail(MRA_ERR_ARG, "mra_reconstruct: bad output view");
+  out->L = in->L;
+  if (in->n == 0) {
+    out->n = 0;
+    return MRA_OK;
+  }
+  cudaStream_t s = (cudaStream_t)stream;
+  Reconstruct rec(s);
+  int rc = rec.plan(in->k, in->n, in->keys);
+  if (rc) return rc;
+  if (rec.leaves() > out->cap) {
+    out->n = rec.leaves();
+    return fail(MRA_ERR_CAPACITY, "mra_reconstruct: %lld leaves, capacity %lld", (long long)out->n, (long long)out->cap);
+  }
+  if ((rc = rec.place(out->keys)) != MRA_OK) return rc;
+  const SumDown f{in->coeffs, nullptr, out->coeffs};
+  if ((rc = rec.run(1, &f)) != MRA_OK) return rc;
+  MRA_CUDA_TRY(cudaStreamSynchronize(s));
+  out->n = rec.leaves();
+  return MRA_OK;
 }
 
 

@@ -91,3 +91,64 @@ def test_fp64_graph_replay_equals_plain_apply(mra, k):
         want, _ = mra.apply(op, tree, o)
         assert torch.equal(got.coeffs[: got.n], want.coeffs[: want.n])
         assert torch.equal(got.keys[: got.n], plain.keys[: plain.n])
+
+
+def _leaves(rng, k, depth, keep):
+    """Random disjoint boxes of levels 1 to `depth` (a box is divided, kept with probability `keep`, or left out)."""
+    def key(n, x, y, z):
+        return (n << 57) | (x << 38) | (y << 19) | z
+    todo, out = [(1, x, y, z) for x in (0, 1) for y in (0, 1) for z in (0, 1)], []
+    while todo:
+        n, x, y, z = todo.pop()
+        if n < depth and rng.random() < 0.3:
+            todo += [(n + 1, 2 * x + i, 2 * y + j, 2 * z + m) for i in (0, 1) for j in (0, 1) for m in (0, 1)]
+        elif rng.random() < keep:
+            out.append(key(n, x, y, z))
+    keys = np.array(sorted(out) or [key(1, 0, 1, 0)], dtype=np.uint64)
+    return keys, rng.standard_normal((len(keys), k, k, k))
+
+
+@pytest.mark.parametrize("k", [1, 5, 10])
+@pytest.mark.parametrize("form", ["any", "second finer", "first finer", "apart", "nested"])
+def test_products_use_the_sums_of_each_tree_by_itself(mra, k, form):
+    """Product and inner product on the common leaves, against each tree with zero boxes at the other's keys summed
+    down by itself: leaves at different levels on either side, one tree at or below the other's leaves, trees
+    without a common box, and a tree with boxes below one another."""
+    import torch
+    rng = np.random.default_rng(7 * k + len(form))
+    (ka, ca), (kb, cb) = _leaves(rng, k, 4, 0.8), _leaves(rng, k, 5, 0.7)
+    if form in ("second finer", "first finer"):
+        t = mra.reconstruct(mra.Tree.from_host(*_union(ka, ca, kb, cb), 8.0))
+        kb = t.keys[: t.n].cpu().numpy().view("uint64")
+        cb = rng.standard_normal((t.n, k, k, k))
+        if form == "first finer":
+            (ka, ca), (kb, cb) = (kb, cb), (ka, ca)
+    elif form == "apart":
+        left = (ka >> np.uint64(38)) & np.uint64(0x7ffff) < (np.uint64(1) << ((ka >> np.uint64(57)) - np.uint64(1)))
+        right = (kb >> np.uint64(38)) & np.uint64(0x7ffff) >= (np.uint64(1) << ((kb >> np.uint64(57)) - np.uint64(1)))
+        ka, ca, kb, cb = ka[left], ca[left], kb[right], cb[right]
+        assert len(ka) and len(kb)
+    elif form == "nested":
+        ka, ca = _union(ka, ca, *_leaves(rng, k, 4, 0.8))
+    ta, tb = mra.Tree.from_host(ka, ca, 8.0), mra.Tree.from_host(kb, cb, 8.0)
+    sa = mra.reconstruct(mra.Tree.from_host(*_union(ka, ca, kb, 0 * cb), 8.0))
+    sb = mra.reconstruct(mra.Tree.from_host(*_union(kb, cb, ka, 0 * ca), 8.0))
+    assert torch.equal(sa.keys[: sa.n], sb.keys[: sb.n])
+    got, want = mra.multiply(ta, tb), mra.multiply(sa, sb)
+    assert torch.equal(got.keys[: got.n], want.keys[: want.n])
+    assert torch.equal(got.coeffs[: got.n], want.coeffs[: want.n])
+    assert mra.inner(ta, tb) == mra.inner(sa, sb)
+    if len(ka) > 1:
+        wrong = mra.Tree.from_host(ka[::-1].copy(), ca, 8.0)
+        for pair in ((wrong, tb), (tb, wrong)):
+            with pytest.raises(mra.MraError):
+                mra.inner(*pair)
+
+
+def _union(ka, ca, kb, cb):
+    """Boxes of both, coefficients added where both have the box."""
+    keys = np.union1d(ka, kb)
+    c = np.zeros((len(keys),) + ca.shape[1:])
+    c[np.searchsorted(keys, ka)] += ca
+    c[np.searchsorted(keys, kb)] += cb
+    return keys, c
