@@ -3,11 +3,14 @@
 // Everything here is FP64 and runs once per operator or per input function;
 // none of it is on the timed apply path.  Compiled with --fmad=false so that
 // the fit search evaluates its error exactly as written.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "mra_internal.cuh"
 
 namespace mra {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -112,18 +115,23 @@ struct HalfRange {
   int npan;
 };
 
-__device__ HalfRange half_range(double T, double wa, double wb) {
+// `wide`: panels of at most 1, 1/sqrt(T) and 2/(T wmin) instead of 1/8, 1/2 and 1 of these.  Enough for the Gaussian
+// times a polynomial of degree below 16: on such a panel a polynomial of degree 24 is within 1e-23 of the
+// Gaussian's own scale there, and 20 points integrate the product of the two exactly.
+__device__ HalfRange half_range(double T, double wa, double wb, bool wide = false) {
   HalfRange r;
   double wmin = wa > 0.0 ? wa : (wb < 0.0 ? -wb : 0.0);
   r.lo = wa;
   r.hi = wb;
-  double width = 0.125;
+  wide = wide && T > 0.0;
+  double width = wide ? 1.0 : 0.125;
+  const double grow = wide ? 2.0 : 1.0;
   if (T > 0.0) {
     double W = sqrt(wmin * wmin + 46.0 / T);
     if (-W > r.lo) r.lo = -W;
     if (W < r.hi) r.hi = W;
-    width = fmin(width, 0.5 / sqrt(T));
-    if (wmin > 0.0) width = fmin(width, 1.0 / (T * wmin));
+    width = fmin(width, grow * 0.5 / sqrt(T));
+    if (wmin > 0.0) width = fmin(width, grow / (T * wmin));
   }
   if (r.hi <= r.lo) {
     r.npan = 0;
@@ -214,74 +222,100 @@ __global__ void blocks_kernel(int k, double L, int min_level, int nlev, const in
 // A factor depends on (level, dimension, coordinate) and the Gaussian only, and the boxes of a
 // refined neighbourhood share their coordinates, so the integrals are done once per distinct
 // coordinate (an "entry") and not once per box.  8 Gaussians, k = 10, 17,200 leaves: the integrals
-// 179 -> 1.5 ms, the refinement test 8.0 -> 0.7 ms with the children's assembly, the call 190 -> 3.7 ms
-// (FP64-bound exponentials and recurrences; the rest is the host's decision after every level).
+// 179 -> 0.50 ms, the refinement test 8.0 -> 0.49 ms with the children's assembly, the call 190 -> 2.4 ms
+// (FP64-bound exponentials, recurrences and products; the rest is the host's decision after every level).
 
 // A factor entry: level, dimension and coordinate.
 __host__ __device__ inline uint64_t make_entry(int level, int dim, int64_t x) {
   return ((uint64_t)level << 40) | ((uint64_t)dim << 32) | (uint64_t)x;
 }
 
-// Legendre recurrence P_{m+1} = a_m x P_m - b_m P_{m-1}, and sqrt(2i+1).
-__constant__ double c_leg_a[MRA_MAX_K], c_leg_b[MRA_MAX_K], c_leg_s[MRA_MAX_K];
+// Legendre polynomials of leading coefficient one, Q_{m+1} = x Q_m - b_m Q_{m-1}, and sqrt(2i+1) P_i / Q_i.
+__constant__ double c_leg_b[MRA_MAX_K], c_leg_s[MRA_MAX_K];
 
-// One warp per (entry, Gaussian): F[(e * ng + g) * stride + i], i < k; nz[e * ng + g] = 0 when all k are
-// zero, which needs no quadrature where the Gaussian underflows on the whole box.  Lanes stride
-// over the nodes of the panel rule over the offset w = u - uc; FP64-bound.
-__global__ void factor_kernel(int64_t n_task, int ng, const double *g, int k, double L, const uint64_t *entries,
-                              int stride, double *F, unsigned char *nz) {
-  const int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (task >= n_task) return;
-  const int64_t en = task / ng;
-  const int gi = (int)(task - en * ng);
-  const uint64_t ent = entries[en];
-  const int n = (int)(ent >> 40), d = (int)(ent >> 32) & 255;
-  const double bx = (double)(ent & 0xFFFFFFFFull);
-  const double h = 2.0 * L / (double)(1LL << n);
-  const double T = g[ng + gi] * h * h;
-  const double x = (g[(2 + d) * ng + gi] + L) / h;  // uc = x - b
-  const double wa = bx - x;                         // w at u = 0
-  const double wb = (bx + 1.0) - x;                 // w at u = 1
-  double acc[MRA_MAX_K];
+constexpr int FACTOR_THREADS = 128, FACTOR_SUB = 8;  // threads per sum over the nodes, one sum per i
+static_assert(FACTOR_SUB * MRA_MAX_K <= FACTOR_THREADS, "a group of threads for every i");
+
+// Where the factors of a set of entries go: F[(e * ng + g) * stride + i], i < k; nz[e * ng + g] = 0 when all
+// k are zero, which needs no quadrature where the Gaussian underflows on the whole box.
+struct FactorSet {
+  int stride;
+  double *F;
+  unsigned char *nz;
+};
+
+// One CTA per (entry, Gaussian), the first n_first entries into one set and the rest into the other (parents and
+// children in one launch); threads stride over the nodes of the panel rule over the offset w = u - uc
+// (the sums over the threads go through shared memory, an eighth of a shuffle reduction's additions; with it
+// and a recurrence of leading coefficient one 0.64 -> 0.50 ms).
+// A level has few tasks of up to 280 nodes, each with an exponential and a serial recurrence: with one warp per task
+// and panels of half the width latency bound (63 us a launch, two launches a level; 8 Gaussians, k = 10: 1.52 ms of
+// a projection), now the FP64 pipe does at the larger levels (42 us a level, 0.50 ms).
+__global__ void __launch_bounds__(FACTOR_THREADS) factor_kernel(int64_t n_entries, int64_t n_first, int ng, const double *g,
+                                                                int k, double L, const uint64_t *entries,
+                                                                const __grid_constant__ FactorSet first,
+                                                                const __grid_constant__ FactorSet rest) {
+  __shared__ double glx[GLQ], glw[GLQ], sum[MRA_MAX_K][FACTOR_THREADS + FACTOR_SUB];
+  if (threadIdx.x < GLQ) {
+    glx[threadIdx.x] = c_glx[threadIdx.x];
+    glw[threadIdx.x] = c_glw[threadIdx.x];
+  }
+  __syncthreads();
+  for (int64_t task = blockIdx.x; task < n_entries * ng; task += gridDim.x) {
+    const int64_t en = task / ng;
+    const int gi = (int)(task - en * ng);
+    const uint64_t ent = entries[en];
+    const int n = (int)(ent >> 40), d = (int)(ent >> 32) & 255;
+    const double bx = (double)(ent & 0xFFFFFFFFull);
+    const double h = 2.0 * L / (double)(1LL << n);
+    const double T = g[ng + gi] * h * h;
+    const double x = (g[(2 + d) * ng + gi] + L) / h;  // uc = x - b
+    const double wa = bx - x;                         // w at u = 0
+    const double wb = (bx + 1.0) - x;                 // w at u = 1
+    double acc[MRA_MAX_K];
 #pragma unroll
-  for (int i = 0; i < MRA_MAX_K; ++i) acc[i] = 0.0;
-  const double wmin = wa > 0.0 ? wa : (wb < 0.0 ? -wb : 0.0);
-  if (T * wmin * wmin < 760.0) {  // exp(-745.2) is the smallest positive double
-    const HalfRange r = half_range(T, wa, wb);
-    const int nn = r.npan * GLQ;
-    const double pw = r.npan > 0 ? (r.hi - r.lo) / r.npan : 0.0;
-    for (int node = lane; node < nn; node += 32) {
-      const int p = node / GLQ, q = node % GLQ;
-      const double w = r.lo + pw * (p + 0.5 + 0.5 * c_glx[q]);
-      const double wt = 0.5 * pw * c_glw[q] * exp(-T * w * w);
-      const double t = 2.0 * (w - wa) - 1.0;  // u = w + uc, formed from the box end
-      double p0 = 1.0, p1 = t;
-      acc[0] += wt;
+    for (int i = 0; i < MRA_MAX_K; ++i) acc[i] = 0.0;
+    const double wmin = wa > 0.0 ? wa : (wb < 0.0 ? -wb : 0.0);
+    if (T * wmin * wmin < 760.0) {  // exp(-745.2) is the smallest positive double
+      const HalfRange r = half_range(T, wa, wb, true);
+      const int nn = r.npan * GLQ;
+      const double pw = r.npan > 0 ? (r.hi - r.lo) / r.npan : 0.0;
+      for (int node = threadIdx.x; node < nn; node += FACTOR_THREADS) {
+        const int p = node / GLQ, q = node % GLQ;
+        const double w = r.lo + pw * (p + 0.5 + 0.5 * glx[q]);
+        const double wt = 0.5 * pw * glw[q] * exp(-T * w * w);
+        const double t = 2.0 * (w - wa) - 1.0;  // u = w + uc, formed from the box end
+        double p0 = 1.0, p1 = t;
+        acc[0] += wt;
 #pragma unroll
-      for (int i = 1; i < MRA_MAX_K; ++i) {
-        if (i < k) {
-          acc[i] = fma(wt, p1, acc[i]);
-          const double p2 = fma(c_leg_a[i] * t, p1, -c_leg_b[i] * p0);
-          p0 = p1;
-          p1 = p2;
+        for (int i = 1; i < MRA_MAX_K; ++i) {
+          if (i < k) {
+            acc[i] = fma(wt, p1, acc[i]);
+            const double p2 = fma(t, p1, -c_leg_b[i] * p0);
+            p0 = p1;
+            p1 = p2;
+          }
         }
       }
     }
-  }
-  const double h12 = sqrt(h);
-  bool some = false;
 #pragma unroll
-  for (int i = 0; i < MRA_MAX_K; ++i) {
+    for (int i = 0; i < MRA_MAX_K; ++i)
+      if (i < k) sum[i][threadIdx.x] = acc[i];
+    __syncthreads();
+    const int i = threadIdx.x / FACTOR_SUB, sub = threadIdx.x % FACTOR_SUB;
+    double v = 0.0;
+    if (i < k)
+      for (int q = sub; q < FACTOR_THREADS; q += FACTOR_SUB) v += sum[i][q];
+    for (int o = FACTOR_SUB / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const FactorSet to = en < n_first ? first : rest;
+    const int64_t row = (en < n_first ? en : en - n_first) * ng + gi;
     if (i < k) {
-      double v = acc[i];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      v *= c_leg_s[i] * h12;
-      some |= v != 0.0;  // NaN counts as nonzero
-      if (lane == 0) F[task * stride + i] = v;
+      v *= c_leg_s[i] * sqrt(h);
+      if (sub == 0) to.F[row * to.stride + i] = v;
     }
+    const int some = __syncthreads_or(v != 0.0);  // NaN counts as nonzero
+    if (threadIdx.x == 0) to.nz[row] = some ? 1 : 0;
   }
-  if (lane == 0) nz[task] = some ? 1 : 0;
 }
 
 // The parents' factors on their children, X' = U^{(c)} X (two-scale relation of Sec. 2.2 in one dimension),
@@ -301,23 +335,36 @@ __global__ void lift_kernel(int64_t n, int ng, int k, const double *Fp, const un
 
 constexpr int ASM_THREADS = 256, ASM_G = 16;  // Gaussians staged at a time
 
-// Sum over the Gaussians at this thread's elements (threadIdx.x + q ASM_THREADS) of one box with the
+// A thread has the elements (ix, iy, sub + q S), q < EPT, of a box: S threads per (ix, iy), so that X Y is formed
+// once for all of a thread's iz.
+struct Elements {
+  int ix, iy, sub, S;
+  bool active;
+  __device__ Elements(int k) {
+    const int k2 = k * k;
+    S = max(1, min(k, ASM_THREADS / k2));
+    const int pair = min((int)threadIdx.x / S, k2 - 1);
+    active = (int)threadIdx.x < k2 * S;
+    ix = pair / k;
+    iy = pair % k;
+    sub = (int)threadIdx.x % S;
+  }
+  // the element's place in the box's coefficients, or -1
+  __device__ int at(int k, int q) const {
+    const int iz = sub + q * S;
+    return active && iz < k ? (ix * k + iy) * k + iz : -1;
+  }
+};
+
+// Sum over the Gaussians at this thread's elements of one box with the
 // factor entries e[0..2]: own[q], and with TEST the parent's projection there, par[q].  Gaussians
 // whose product is exactly zero are left out; the others are added in order.
 template <int EPT, bool TEST>
-__device__ void sum_gaussians(int ng, int k, const double *coef, const double *F, const unsigned char *nz,
+__device__ void sum_gaussians(int ng, int k, const Elements &el, const double *coef, const double *F, const unsigned char *nz,
                               const int64_t *e, double *stage, int *list, int *count, double *own, double *par) {
-  const int k2 = k * k, k3 = k2 * k, st = TEST ? 2 * k : k;
+  const int st = TEST ? 2 * k : k;
 #pragma unroll
   for (int q = 0; q < EPT; ++q) own[q] = par[q] = 0.0;
-  int ix[EPT], iy[EPT], iz[EPT];
-#pragma unroll
-  for (int q = 0; q < EPT; ++q) {
-    const int m = min((int)threadIdx.x + q * ASM_THREADS, k3 - 1);
-    ix[q] = m / k2;
-    iy[q] = (m / k) % k;
-    iz[q] = m % k;
-  }
   for (int g0 = 0; g0 < ng;) {
     __syncthreads();  // the list and the staged factors of the previous round have been used
     if (threadIdx.x < 32) {  // the next ASM_G Gaussians that matter, in order
@@ -364,41 +411,46 @@ __device__ void sum_gaussians(int ng, int k, const double *coef, const double *F
     __syncthreads();
     for (int l = 0; l < have; ++l) {
       const double *X = stage + l * 3 * st, *Y = X + st, *Z = Y + st;
+      const double xy = X[el.ix] * Y[el.iy], pxy = TEST ? X[k + el.ix] * Y[k + el.iy] : 0.0;
 #pragma unroll
       for (int q = 0; q < EPT; ++q) {
-        own[q] = fma(X[ix[q]] * Y[iy[q]], Z[iz[q]], own[q]);
-        if (TEST) par[q] = fma(X[k + ix[q]] * Y[k + iy[q]], Z[k + iz[q]], par[q]);
+        const int iz = el.sub + q * el.S;
+        if (iz < k) {
+          own[q] = fma(xy, Z[iz], own[q]);
+          if (TEST) par[q] = fma(pxy, Z[k + iz], par[q]);
+        }
       }
     }
   }
 }
 
-// One CTA per parent: its eight children's coefficients, and ||s_children - U s_parent||_F (the
-// refinement test of Sec. 2.1), the parent's projection on a child being the sum of the lifted
-// factors' products: no k^4 transform.  pidx: the parent's entry in each dimension.
+// A cluster of eight CTAs per parent: each has one child's coefficients, together ||s_children - U s_parent||_F
+// (the refinement test of Sec. 2.1), the parent's projection on a child being the sum of the lifted factors'
+// products: no k^4 transform.  pidx: the parent's entry in each dimension.  One CTA for the eight children in
+// turn, X Y formed for every element, took 61 us a level (k = 10, 8 Gaussians, up to 376 parents), now 41.
 template <int EPT>
-__global__ void __launch_bounds__(ASM_THREADS) children_kernel(int ng, int k, const double *coef, const double *F,
-                                                               const unsigned char *nz, const int *pidx, double *out,
-                                                               double *dnorm) {
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(ASM_THREADS)
+    children_kernel(int ng, int k, const double *coef, const double *F, const unsigned char *nz, const int *pidx, double *out,
+                    double *dnorm) {
   extern __shared__ double stage[];  // [ASM_G][3][2k]
   __shared__ int list[ASM_G], count[2];
-  __shared__ double red[32];
-  const int64_t p = blockIdx.x;
+  __shared__ double red[ASM_THREADS / 32], total;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int c = (int)cluster.block_rank();
+  const int64_t p = blockIdx.x >> 3;
   const int k3 = k * k * k;
-  double part = 0.0;
-  for (int c = 0; c < 8; ++c) {
-    const int64_t e[3] = {2 * (int64_t)pidx[3 * p] + (c >> 2), 2 * (int64_t)pidx[3 * p + 1] + ((c >> 1) & 1),
-                          2 * (int64_t)pidx[3 * p + 2] + (c & 1)};
-    double own[EPT], par[EPT];
-    sum_gaussians<EPT, true>(ng, k, coef, F, nz, e, stage, list, count, own, par);
+  const Elements el(k);
+  const int64_t e[3] = {2 * (int64_t)pidx[3 * p] + (c >> 2), 2 * (int64_t)pidx[3 * p + 1] + ((c >> 1) & 1),
+                        2 * (int64_t)pidx[3 * p + 2] + (c & 1)};
+  double own[EPT], par[EPT], part = 0.0;
+  sum_gaussians<EPT, true>(ng, k, el, coef, F, nz, e, stage, list, count, own, par);
 #pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-      const int m = threadIdx.x + q * ASM_THREADS;
-      if (m < k3) {
-        out[(8 * p + c) * k3 + m] = own[q];
-        const double d = own[q] - par[q];
-        part = fma(d, d, part);
-      }
+  for (int q = 0; q < EPT; ++q) {
+    const int m = el.at(k, q);
+    if (m >= 0) {
+      out[(8 * p + c) * k3 + m] = own[q];
+      const double d = own[q] - par[q];
+      part = fma(d, d, part);
     }
   }
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
@@ -407,8 +459,15 @@ __global__ void __launch_bounds__(ASM_THREADS) children_kernel(int ng, int k, co
   if (threadIdx.x == 0) {
     double v = 0.0;
     for (int q = 0; q < ASM_THREADS / 32; ++q) v += red[q];
+    total = v;
+  }
+  cluster.sync();
+  if (c == 0 && threadIdx.x == 0) {
+    double v = 0.0;
+    for (int q = 0; q < 8; ++q) v += *cluster.map_shared_rank(&total, q);
     dnorm[p] = sqrt(v);
   }
+  cluster.sync();  // the totals have been read
 }
 
 // One CTA per box of a whole level (entry of dimension d and coordinate x: d 2^n + x).
@@ -421,13 +480,13 @@ __global__ void __launch_bounds__(ASM_THREADS) boxes_kernel(int ng, int k, const
   const uint64_t key = keys[b];
   const int64_t nb = 1LL << key_level(key);
   const int64_t e[3] = {key_x(key), nb + key_y(key), 2 * nb + key_z(key)};
-  const int k3 = k * k * k;
+  const Elements el(k);
   double own[EPT], par[EPT];
-  sum_gaussians<EPT, false>(ng, k, coef, F, nz, e, stage, list, count, own, par);
+  sum_gaussians<EPT, false>(ng, k, el, coef, F, nz, e, stage, list, count, own, par);
 #pragma unroll
   for (int q = 0; q < EPT; ++q) {
-    const int m = threadIdx.x + q * ASM_THREADS;
-    if (m < k3) out[b * k3 + m] = own[q];
+    const int m = el.at(k, q);
+    if (m >= 0) out[b * k * k * k + m] = own[q];
   }
 }
 
@@ -435,20 +494,20 @@ __global__ void __launch_bounds__(ASM_THREADS) boxes_kernel(int ng, int k, const
 // (always the same values).
 cudaError_t upload_tables(cudaStream_t s) {
   struct Tables {
-    double x[GLQ], w[GLQ], a[MRA_MAX_K], b[MRA_MAX_K], r[MRA_MAX_K];
+    double x[GLQ], w[GLQ], b[MRA_MAX_K], r[MRA_MAX_K];
     Tables() {
       gauss_legendre(GLQ, x, w);
+      double lead = 1.0;  // of P_m
       for (int m = 0; m < MRA_MAX_K; ++m) {
-        a[m] = (2.0 * m + 1.0) / (m + 1.0);
-        b[m] = m / (m + 1.0);
-        r[m] = sqrt(2.0 * m + 1.0);
+        b[m] = (double)(m * m) / (4.0 * m * m - 1.0);
+        r[m] = sqrt(2.0 * m + 1.0) * lead;
+        lead *= (2.0 * m + 1.0) / (m + 1.0);
       }
     }
   };
   static const Tables t;
   cudaError_t e = cudaMemcpyToSymbolAsync(c_glx, t.x, sizeof(t.x), 0, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_glw, t.w, sizeof(t.w), 0, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_leg_a, t.a, sizeof(t.a), 0, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_leg_b, t.b, sizeof(t.b), 0, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_leg_s, t.r, sizeof(t.r), 0, cudaMemcpyHostToDevice, s);
   return e;
@@ -490,12 +549,13 @@ cudaError_t launch_blocks(const Operator &op, const double *d_glxk, const double
   return cudaGetLastError();
 }
 
-// Factors of the entries (device array) for every Gaussian: F[(e * ng + g) * stride + i], nz[e * ng + g].
-static cudaError_t launch_factors(int64_t n_entries, int ng, const double *d_g, int k, double L, const uint64_t *d_entries,
-                                  int stride, double *F, unsigned char *nz, cudaStream_t s) {
+// Factors of the entries (device array) for every Gaussian, the first n_first into one set, the others into the rest.
+static cudaError_t launch_factors(int64_t n_entries, int64_t n_first, int ng, const double *d_g, int k, double L,
+                                  const uint64_t *d_entries, FactorSet first, FactorSet rest, cudaStream_t s) {
   const int64_t tasks = n_entries * ng;
   if (tasks <= 0) return cudaSuccess;
-  factor_kernel<<<counted((unsigned)((tasks + 3) / 4)), 128, 0, s>>>(tasks, ng, d_g, k, L, d_entries, stride, F, nz);
+  factor_kernel<<<counted((unsigned)std::min<int64_t>(tasks, 1 << 20)), FACTOR_THREADS, 0, s>>>(n_entries, n_first, ng, d_g, k, L,
+                                                                                               d_entries, first, rest);
   return cudaGetLastError();
 }
 
@@ -504,11 +564,12 @@ cudaError_t launch_project_level(int ng, const double *d_g, int k, double L, int
                                  cudaStream_t s) {
   if (nbox <= 0) return cudaSuccess;
   cudaError_t e = upload_tables(s);
-  if (e == cudaSuccess) e = launch_factors(n_entries, ng, d_g, k, L, d_entries, k, F, nz, s);
+  const FactorSet f{k, F, nz};
+  if (e == cudaSuccess) e = launch_factors(n_entries, n_entries, ng, d_g, k, L, d_entries, f, f, s);
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)ASM_G * 3 * k * sizeof(double);
   if (k <= 10)
-    boxes_kernel<4><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out);
+    boxes_kernel<5><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out);
   else
     boxes_kernel<16><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out);
   return cudaGetLastError();
@@ -520,8 +581,8 @@ cudaError_t launch_project_children(int ng, const double *d_g, int k, double L, 
                                     double *d_dnorm, cudaStream_t s) {
   if (np <= 0) return cudaSuccess;
   // the parents' entries, then their children's (2 e + c)
-  cudaError_t e = launch_factors(n_entries, ng, d_g, k, L, d_entries, k, Fp, nzp, s);
-  if (e == cudaSuccess) e = launch_factors(2 * n_entries, ng, d_g, k, L, d_entries + n_entries, 2 * k, Fc, nzc, s);
+  cudaError_t e = launch_factors(3 * n_entries, n_entries, ng, d_g, k, L, d_entries, FactorSet{k, Fp, nzp},
+                                 FactorSet{2 * k, Fc, nzc}, s);
   if (e != cudaSuccess) return e;
   if (ng > 0) {
     const int64_t nl = n_entries * 2 * ng * k;
@@ -531,9 +592,9 @@ cudaError_t launch_project_children(int ng, const double *d_g, int k, double L, 
   }
   const size_t smem = (size_t)ASM_G * 6 * k * sizeof(double);
   if (k <= 10)
-    children_kernel<4><<<counted((unsigned)np), ASM_THREADS, smem, s>>>(ng, k, d_g, Fc, nzc, d_pidx, d_out, d_dnorm);
+    children_kernel<5><<<counted((unsigned)(8 * np)), ASM_THREADS, smem, s>>>(ng, k, d_g, Fc, nzc, d_pidx, d_out, d_dnorm);
   else
-    children_kernel<16><<<counted((unsigned)np), ASM_THREADS, smem, s>>>(ng, k, d_g, Fc, nzc, d_pidx, d_out, d_dnorm);
+    children_kernel<16><<<counted((unsigned)(8 * np)), ASM_THREADS, smem, s>>>(ng, k, d_g, Fc, nzc, d_pidx, d_out, d_dnorm);
   return cudaGetLastError();
 }
 

@@ -51,3 +51,12 @@ def test_no_gaussians(mra):
     t = mra.project(f, 4, 32.0, uniform_level=1)
     assert t.n == 8 and float(t.coeffs[:8].abs().max()) == 0.0
     assert mra.project(f, 4, 32.0, thresh=1e-3).n == 64
+
+
+@pytest.mark.parametrize("k,level", [(6, 2), (8, 1), (10, 2), (12, 1), (14, 2)])
+@pytest.mark.parametrize("a_lo,a_hi", [(1e-4, 1e-1), (1e-1, 1e3), (1e3, 1e7)])
+def test_flat_to_narrow_gaussians(mra, k, level, a_lo, a_hi):
+    """From one panel for the whole box to panels of a small part of it, and each split of a box over the threads."""
+    f = W.gaussian_sum(6, a_lo, a_hi, seed=k)
+    ok, oc, _ = O.project(f, k, 32.0, uniform_level=level)
+    check(mra.project(f, k, 32.0, uniform_level=level), ok, oc)
