@@ -222,7 +222,7 @@ __global__ void blocks_kernel(int k, double L, int min_level, int nlev, const in
 // A factor depends on (level, dimension, coordinate) and the Gaussian only, and the boxes of a
 // refined neighbourhood share their coordinates, so the integrals are done once per distinct
 // coordinate (an "entry") and not once per box.  8 Gaussians, k = 10, 17,200 leaves: the integrals
-// 179 -> 0.50 ms, the refinement test 8.0 -> 0.49 ms with the children's assembly, the call 190 -> 2.4 ms
+// 179 -> 0.50 ms, the refinement test 8.0 -> 0.49 ms with the children's assembly, the call 190 -> 2.2 ms
 // (FP64-bound exponentials, recurrences and products; the rest is the host's decision after every level).
 
 // A factor entry: level, dimension and coordinate.
