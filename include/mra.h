@@ -477,8 +477,8 @@ int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void *stream);
 int mra_truncate(const mra_tree_view *in, double thresh, mra_tree_view *out, double *err2, void *stream);
 
 /* Product of two functions held on trees of disjoint leaves (keys sorted and unique; same k
- * and L).  Both are first summed down to their common refinement (each tree's leaves plus zero
- * boxes at the other's keys, through mra_reconstruct); then, per leaf, the values at the k
+ * and L).  Both are first summed down to their common refinement (each tree's leaves plus empty
+ * boxes at the other's keys); then, per leaf, the values at the k
  * Gauss-Legendre points of each dimension (the third representation of Sec. 2.1) are
  * multiplied and transformed back: s_ab = h^{-3/2} (V^T W)^{x3} [(V^{x3} s_a)(V^{x3} s_b)],
  * V[q][i] = phi_i(x_q), W = diag(w_q) -- the product interpolated at the points.  out: the
