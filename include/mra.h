@@ -505,8 +505,8 @@ int mra_scale(mra_tree_view *tree, double alpha, void *stream);
  * may change the input coefficients between replays (same in->n).  The workspace stays owned
  * by the graph until mra_apply_graph_free.  Every replay checks on the device that its record
  * and destination counts equal the recorded ones; mra_apply_graph_status synchronises the
- * stream, returns MRA_ERR_CAPACITY if any replay since the last call needed other sizes (its
- * output is then not valid: create the graph again), MRA_ERR_TIMEOUT if a tensor-core wait
+ * stream, returns MRA_ERR_CAPACITY if any replay since the last call needed other sizes (such a
+ * replay runs no apply kernel and leaves the output as it was: create the graph again), MRA_ERR_TIMEOUT if a tensor-core wait
  * gave up, and clears the record.  Statistics are not gathered by replays. */
 typedef struct mra_apply_graph mra_apply_graph; /* opaque */
 int mra_apply_graph_create(const mra_operator *op, int nfunc, const mra_tree_view *in, const int64_t *in_offsets,

@@ -431,8 +431,9 @@ __global__ void __launch_bounds__(F64_THREADS) apply_f64_kernel(
     int k, int M, const double *c, const double *R, const int *Dlev, const int64_t *level_off,
     const uint64_t *in_keys, const double *in_coeffs, const int64_t *seg, const int *perm,
     const int *rec_src, const int *rec_l, const uint64_t *rec_mask, const uint64_t *dest_key,
-    uint64_t *out_keys, double *out_coeffs, int64_t n_src, int64_t n_rec, int64_t n_blocks) {
+    uint64_t *out_keys, double *out_coeffs, int64_t n_src, int64_t n_rec, int64_t n_blocks, const int *skip) {
   extern __shared__ double sm[];
+  if (skip && *skip) return;
   int k2 = k * k, k3 = k2 * k;
   double *s = sm, *t1 = s + k3, *t2 = t1 + k3, *Rs = t2 + k3;  // Rs: 3 * k2
   int64_t dst = blockIdx.x;
@@ -650,14 +651,18 @@ __global__ void debug_selftest_kernel(int *sink) {
 
 // Fixed-size (graph) mode: the record count the screen computed against the captured one.
 __global__ void fixed_count_check_kernel(const int64_t *off, const int64_t *cnt, int64_t n_in, int64_t P,
-                                         const int *d_err, int *status) {
+                                         const int *d_err, int *status, int *skip) {
   int st = 0;
   if (off[n_in - 1] + cnt[n_in - 1] != P) st |= 1;
   if (*d_err) st |= 4;
   if (st) atomicOr(status, st);
+  *skip = st != 0;
 }
-__global__ void fixed_dest_check_kernel(const int64_t *ndest, int64_t nd, int *status) {
-  if (*ndest != nd) atomicOr(status, 2);
+__global__ void fixed_dest_check_kernel(const int64_t *ndest, int64_t nd, int *status, int *skip) {
+  if (*ndest != nd) {
+    atomicOr(status, 2);
+    *skip = 1;
+  }
 }
 
 // One CTA per level n: the sum of v over the boxes of level n (keys sorted, so the level's boxes
@@ -990,7 +995,7 @@ static int screen_run(const Operator &op, const mra_tree_view &in, const mra_app
   size_t tmpb = w.tmpb;
   MRA_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp, tmpb, w.cnt, w.off, (int)n_in, s));
   if (fx) {  // graph mode: the captured record count, checked on the device
-    fixed_count_check_kernel<<<counted(1), 1, 0, s>>>(w.off, w.cnt, n_in, fx->P, d_err, fx->status);
+    fixed_count_check_kernel<<<counted(1), 1, 0, s>>>(w.off, w.cnt, n_in, fx->P, d_err, fx->status, fx->skip);
     MRA_CUDA_TRY(cudaGetLastError());
     if (fx->P > 0) {
       screen_kernel<1><<<counted(gboxes), 32 * wpb, 0, s>>>(a);
@@ -1095,7 +1100,7 @@ int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts 
   }
   int64_t nd = 0;
   if (fx) {
-    fixed_dest_check_kernel<<<counted(1), 1, 0, s>>>(ndest, fx->nd, fx->status);
+    fixed_dest_check_kernel<<<counted(1), 1, 0, s>>>(ndest, fx->nd, fx->status, fx->skip);
     MRA_CUDA_TRY(cudaGetLastError());
     nd = fx->nd;
   } else {
@@ -1161,7 +1166,7 @@ int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts 
       MRA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<counted((unsigned)nd), F64_THREADS, smem, s>>>(
         k, op.M, op.d_c, op.d_R, op.d_D, op.d_level_off, in.keys, in.coeffs, seg, pout, rsrc, rl,
-        rmask, dkey, out.keys, out.coeffs, n_in, P, op.n_blocks);
+        rmask, dkey, out.keys, out.coeffs, n_in, P, op.n_blocks, wk.skip());
     MRA_CUDA_TRY(cudaGetLastError());
     if (ev1) MRA_CUDA_TRY(cudaEventRecord(ev1, s));
     rc = MRA_OK;

@@ -93,6 +93,7 @@ struct F64Args {
   double *partial;                // [p1 - p0][k^3]
   int64_t p0, p1;                 // records of this launch
   int64_t n_src, n_rec;
+  const int *skip;                // see FixedSizes
 };
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -136,6 +137,7 @@ __global__ void __launch_bounds__(F64_MAX_THREADS, 1) apply_f64_sym_kernel(const
   __shared__ unsigned long long all[4][2], any[4][2];  // kept-term masks by (|ly|, |lz|): AND and OR over the signs
   __shared__ int rec[2][9];                            // record of (sign of lx, ly, lz), -1 = none in range
   __shared__ int lone;                                 // some mask differs from its mirror images'
+  if (a.skip && *a.skip) return;
   const int k = a.k, k2 = k * k, k3 = k2 * k, h = par_half(k), nx = a.nx, we = par_entry(k);
   const int64_t b = blockIdx.x;
   const int ch = blockIdx.y;
@@ -387,8 +389,9 @@ __global__ void __launch_bounds__(F64_MAX_THREADS, 1) apply_f64_sym_kernel(const
 // output; last: doubled-basis sums are turned back into child coefficients.
 __global__ void dest_sum_f64_kernel(int k, const int64_t *seg, const int *perm, const double *partial, int64_t p0,
                                     int64_t p1, int first, int last, int pairs, const uint64_t *dest_key,
-                                    uint64_t *out_keys, double *out_coeffs, int64_t n_rec) {
+                                    uint64_t *out_keys, double *out_coeffs, int64_t n_rec, const int *skip) {
   extern __shared__ __align__(16) double sum[];  // k^3, doubled basis only
+  if (skip && *skip) return;
   const int64_t d = blockIdx.x;
   const int k2 = k * k, k3 = k2 * k;
   int64_t r0 = seg[d], r1 = seg[d + 1];
@@ -542,6 +545,7 @@ int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &ou
   a.partial = partial;
   a.n_src = in.n;
   a.n_rec = P;
+  a.skip = wk.skip();
   const size_t smem = f64_smem(k, a.nx), dsm = a.pairs ? row : 0;
   // the same limit whatever the order, so that callers on several threads do not lower it for one another
   cudaError_t e = cudaFuncSetAttribute(apply_f64_sym_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F64_MAX_SMEM);
@@ -556,7 +560,7 @@ int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &ou
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
     dest_sum_f64_kernel<<<counted((unsigned)nd), k3 >= 512 ? 256 : 128, dsm, s>>>(
-        k, wk.seg, wk.perm, partial, a.p0, a.p1, p0 == 0, a.p1 == P, a.pairs, wk.dest_key, out.keys, out.coeffs, P);
+        k, wk.seg, wk.perm, partial, a.p0, a.p1, p0 == 0, a.p1 == P, a.pairs, wk.dest_key, out.keys, out.coeffs, P, wk.skip());
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && wk.ev1) e = cudaEventRecord(wk.ev1, s);

@@ -9,10 +9,14 @@ namespace mra {
 // the record count P and destination count nd of an earlier run of the same input are used as
 // the sizes, and kernels compare the counts the device computes with them, OR-ing into *status:
 // 1 = record count differs, 2 = destination count differs, 4 = a box on a level the operator
-// does not cover, 8 = a tensor-core wait gave up, 16 = inconsistent split work list.
+// does not cover, 8 = a tensor-core wait gave up, 16 = inconsistent split work list.  *skip is set
+// anew by every replay: 1 = its sizes are not the recorded ones, and the apply kernels return at once.  The
+// buffers have the recorded sizes, and of a work list of another size not every index would lie in them (a
+// record beyond P has no partial sums; with fewer destinations a tile's groups are an earlier replay's).
 struct FixedSizes {
   int64_t P = 0, nd = 0;
   int *status = nullptr;                  // device word
+  int *skip = nullptr;                    // device word
   const int64_t *d_in_offsets = nullptr;  // device copy of the batched input offsets (nfunc + 1)
   void *partial = nullptr;                // the source-stationary kernels' partial sums, of partial_bytes
   size_t partial_bytes = 0;
@@ -39,6 +43,7 @@ struct ApplyWork {
   cudaEvent_t ev0, ev1;       // recorded around the apply kernel when non-null
   cudaEvent_t evk0, evk1;     // around the main kernel alone, where the apply runs more kernels
   const FixedSizes *fx;       // fixed-size (graph) mode when non-null
+  const int *skip() const { return fx ? fx->skip : nullptr; }  // of the apply kernels; null: never
 };
 
 size_t apply_workspace_bytes(const Operator &op, const mra_apply_opts &o, int64_t n_in);

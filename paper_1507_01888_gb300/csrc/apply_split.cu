@@ -67,6 +67,7 @@ struct SplitArgs {
   double *out_coeffs;
   int *err;
   int inject_stall;  // test hook: CTA 0 never issues the block copies of its first term
+  const int *skip;   // see FixedSizes
   int64_t n_src, n_rec, n_blocks;  // sizes for the index checks of the checking build
 };
 
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, minb_for(TT)) apply_split_kerne
   constexpr uint32_t NCOL = tmem_cols_for(T);
   constexpr int NB = nbuf_for(TT), AHEAD = NB - 2;  // block buffers; copies run AHEAD terms ahead
   extern __shared__ __align__(1024) unsigned char smem[];
+  if (a.skip && *a.skip) return;
   const int P = a.P;
   const int ptile = P * T * TILE_BYTES;
   unsigned char *A1 = smem;              // [P][T] tiles: stage-1 operand (sources)
@@ -839,6 +841,7 @@ int apply_split_run(const Operator &op, const mra_tree_view &in, const mra_apply
   a.out_coeffs = out.coeffs;
   a.err = err;
   a.inject_stall = take_injected_stall() ? 1 : 0;
+  a.skip = wk.skip();
   a.n_src = in.n;
   a.n_rec = P;
   a.n_blocks = op.n_blocks;

@@ -95,6 +95,7 @@ struct SrcArgs {
   int compensated;              // record sums: 1 = FP32 sum + Kahan correction, 0 = plain FP32 sum
   int parts;                    // CTAs per tile (1, 3 or 9): each takes the records of one residue of lx, or (lx, ly), mod 3
   int ahead;                    // block copies run this many terms ahead (1 .. src_nb - 2)
+  const int *skip;              // see FixedSizes
   int64_t n_src, n_rec, n_blocks;
 };
 
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(PLAIN ? SRC_THREADS + 32 : SRC_THREADS, 2) app
   constexpr int k2 = K * K, k3 = K * K * K;
   constexpr int G = src_g(K), rows = G * k2, SRC_NB = src_nb(K);
   extern __shared__ __align__(1024) unsigned char smem[];
+  if (a.skip && *a.skip) return;
   const int P = a.P;
   unsigned char *A1 = smem;                    // [P] tiles: stage-1 operand (the tile's sources)
   unsigned char *A2 = A1 + 3 * TILE_BYTES;     // [P] tiles: stage-2 operand
@@ -786,7 +788,9 @@ __device__ __forceinline__ void sum2_add(float &s, float &c, float x) {
 // path covers: each thread takes four consecutive coefficients (16-byte streaming loads, read
 // once) and four records at a time.
 __global__ void dest_sum_kernel(int64_t nd, int k3, const int64_t *seg, const int *perm, const float *partial,
-                                const uint64_t *dest_key, uint64_t *out_keys, double *out_coeffs, int64_t n_rec) {
+                                const uint64_t *dest_key, uint64_t *out_keys, double *out_coeffs, int64_t n_rec,
+                                const int *skip) {
+  if (skip && *skip) return;
   const int64_t d = blockIdx.x;
   if (d >= nd) return;
   const int64_t r0 = seg[d], r1 = seg[d + 1];
@@ -911,6 +915,7 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
   a.join_all = o.join > 0 ? 1 : 0;
   a.compensated = o.sums == MRA_SUMS_COMPENSATED ? 1 : 0;
   a.ahead = o.ahead > 0 ? o.ahead : 2;
+  a.skip = wk.skip();
   a.n_src = n_in;
   a.n_rec = P;
   a.n_blocks = op.n_blocks;
@@ -953,7 +958,7 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
   MRA_CUDA_TRY(cudaGetLastError());
   if (wk.evk1) MRA_CUDA_TRY(cudaEventRecord(wk.evk1, s));
   dest_sum_kernel<<<counted((unsigned)std::max<int64_t>(nd, 1)), 256, 0, s>>>(
-      nd, k3, wk.seg, wk.perm, partial, wk.dest_key, out.keys, out.coeffs, P);
+      nd, k3, wk.seg, wk.perm, partial, wk.dest_key, out.keys, out.coeffs, P, wk.skip());
   MRA_CUDA_TRY(cudaGetLastError());
   if (wk.ev1) MRA_CUDA_TRY(cudaEventRecord(wk.ev1, s));
   if (wk.fx) {

@@ -68,9 +68,9 @@ int mra_apply_graph_create(const mra_operator *h, int nfunc, const mra_tree_view
     destroy(g);
     return fail(code, "mra_apply_graph_create: %s: %s", what, cudaGetErrorString(e));
   };
-  cudaError_t e = cudaMalloc((void **)&g->d_status, sizeof(int));
+  cudaError_t e = cudaMalloc((void **)&g->d_status, 2 * sizeof(int));  // the status, and a replay's skip word
   if (e != cudaSuccess) return bail(MRA_ERR_CUDA, "status word", e);
-  e = cudaMemset(g->d_status, 0, sizeof(int));
+  e = cudaMemset(g->d_status, 0, 2 * sizeof(int));
   if (e != cudaSuccess) return bail(MRA_ERR_CUDA, "status word", e);
   if (nfunc > 1) {
     e = cudaMalloc((void **)&g->d_in_offsets, (nfunc + 1) * sizeof(int64_t));
@@ -81,6 +81,7 @@ int mra_apply_graph_create(const mra_operator *h, int nfunc, const mra_tree_view
   g->fx.P = st.pairs;
   g->fx.nd = out->n;
   g->fx.status = g->d_status;
+  g->fx.skip = g->d_status + 1;
   g->fx.d_in_offsets = g->d_in_offsets;
   g->n_out = out->n;
   const Operator *op = reinterpret_cast<const Operator *>(h);

@@ -102,3 +102,41 @@ def test_graph_reports_a_replay_with_other_sizes(mra):
     g.status()
     ref, _ = mra.apply(op, tree, opts)
     assert np.allclose(g.out.host()[1], ref.host()[1], rtol=0, atol=1e-12 * np.abs(ref.host()[1]).max())
+
+
+@pytest.mark.parametrize("k,kw", [(6, dict()), (6, dict(max_disp=2)), (6, dict(precision=1)), (6, dict(precision=1, sums=1)),
+                                  (6, dict(precision=1, split_kernel=1)), (12, dict(precision=1))])
+@pytest.mark.parametrize("recorded", ["few", "many"])
+def test_graph_leaves_the_output_alone_when_the_sizes_differ(mra, k, kw, recorded):
+    """A replay with more records than recorded (the partial sums have no room for them) or fewer (tiles without
+    groups), in the FP64 kernels and in both split kernels: reported, and the output is as it was."""
+    import torch
+    kw = dict(dict(precision=0, max_disp=1), **kw)
+    keys, coeffs = W.random_tree_coeffs(60, k, 3, seed=k)
+    coeffs = coeffs / np.sqrt((coeffs ** 2).reshape(len(keys), -1).sum(1))[:, None, None, None]
+    op = mra.Operator(mra.BSH, 24, k, 32.0, 3, 3, max_disp=kw["max_disp"], mu=1.0, fit_eps=1e-6)
+    tree = mra.Tree.from_host(keys, coeffs, 32.0)
+    opts = mra.make_opts(stencil=mra.STENCIL_SHELLS, screen=mra.SCREEN_NORM, tau=1e-2, **kw)
+    half = tree.coeffs[30:].clone()
+    many, many_st = mra.apply(op, tree, opts)
+    tree.coeffs[30:] *= 2.0 ** -40  # the screen keeps nothing of half of the boxes
+    few, few_st = mra.apply(op, tree, opts)
+    assert 0 < few_st["pairs"] < many_st["pairs"] and few.n < many.n
+    if recorded == "many":
+        tree.coeffs[30:] = half
+    g = mra.ApplyGraph(op, tree, opts)
+    g.launch()
+    g.status()
+    want = many if recorded == "many" else few
+    assert g.out.n == want.n and torch.equal(g.out.coeffs[: want.n], want.coeffs[: want.n])
+    tree.coeffs[30:] = half * 2.0 ** -40 if recorded == "many" else half
+    g.out.coeffs.fill_(7.0)
+    g.launch()
+    with pytest.raises(mra.MraError) as e:
+        g.status()
+    assert e.value.code == mra.MRA_ERR_CAPACITY
+    assert bool((g.out.coeffs == 7.0).all()) and torch.equal(g.out.keys[: want.n], want.keys[: want.n])
+    tree.coeffs[30:] = half if recorded == "many" else half * 2.0 ** -40
+    g.launch()
+    g.status()
+    assert torch.equal(g.out.coeffs[: want.n], want.coeffs[: want.n])
