@@ -207,8 +207,8 @@ long long mra_launch_count(void);
 
 /* Device memory the library keeps for reuse: the scratch of the calls that allocate it
  * themselves (projection, norms and comparisons, reconstruction, truncation, products, the
- * non-standard applies; of the plain applies the partial sums, up to 4 GB in FP64) comes from a stream-ordered pool per device that holds on to freed
- * memory between calls.  This returns the pool's unused memory to the driver.  Memory of
+ * non-standard applies; of the plain applies the partial sums, in FP64 up to 4 GB and less or none where
+ * memory is short) comes from a stream-ordered pool per device that holds on to freed memory between calls.  This returns the pool's unused memory to the driver.  Memory of
  * allocations still in flight on a stream is not affected. */
 int mra_release_memory(void);
 
@@ -217,6 +217,11 @@ int mra_release_memory(void);
  * run out (about two seconds each); that apply returns MRA_ERR_TIMEOUT with the device context
  * intact, and later calls run normally.  One-shot; nothing else is changed. */
 int mra_debug_inject_stall(void);
+
+/* Test hook for short memory: until it is called again with 0, requests above `bytes` that the library
+ * makes for its own scratch on the calling thread (from its pool, and a graph's partial sums) fail as
+ * they do when the device is full. */
+int mra_debug_limit_memory(size_t bytes);
 
 /* The checking build (libmra_debug.so, compiled with MRA_DEBUG): the hot kernels' gather and
  * scatter indices (records, sources, operator blocks) are checked against their ranges; an

@@ -142,7 +142,16 @@ constexpr int MAX_POOL_DEVICES = 64;
 static std::mutex g_pool_mu;
 static cudaMemPool_t g_pools[MAX_POOL_DEVICES] = {};
 
+// Test hook: the largest request of this thread that is granted (0: no limit).
+static thread_local size_t g_memory_limit = 0;
+static bool over_limit(size_t bytes) { return g_memory_limit && bytes > g_memory_limit; }
+
+cudaError_t limited_malloc(void **p, size_t bytes) {
+  return over_limit(bytes) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+}
+
 cudaError_t pool_malloc(void **p, size_t bytes, cudaStream_t s) {
+  if (over_limit(bytes)) return cudaErrorMemoryAllocation;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -288,6 +297,11 @@ int mra_release_memory(void) {
     const cudaError_t e = cudaMemPoolTrimTo(mra::g_pools[d], 0);
     if (e != cudaSuccess) return fail(MRA_ERR_CUDA, "mra_release_memory: %s", cudaGetErrorString(e));
   }
+  return MRA_OK;
+}
+
+int mra_debug_limit_memory(size_t bytes) {
+  g_memory_limit = bytes;
   return MRA_OK;
 }
 

@@ -419,7 +419,8 @@ __global__ void func_offsets_kernel(int64_t n, const int *dest_func, int nfunc, 
 }
 
 // ---------------------------------------------------------------- FP64 gather-apply
-// Records beyond |l|_inf = 1 (the others run in apply_f64.cu).  One CTA per destination box.  For each of its records (source b, l, mask)
+// For applies with records beyond |l|_inf = 1 and where memory for partial sums is short (the others run in
+// apply_f64.cu).  One CTA per destination box.  For each of its records (source b, l, mask)
 // and each kept term m:  t1 = s x_1 Rx, t2 = t1 x_2 Ry, t3 = t2 x_3 Rz,
 // acc += c_m t3 (Sec. 2.3), acc held in registers across all records.
 // PT accumulators per thread: k^3 <= 256 PT (PT = 16 up to k = 16, 32 for the non-standard
@@ -1155,9 +1156,13 @@ int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts 
   wk.fx = fx;
   if (stats)
     stats->kernel = o.precision == MRA_PREC_FP64 ? MRA_KERNEL_F64 : src_path ? MRA_KERNEL_SPLIT_SRC : MRA_KERNEL_SPLIT_DEST;
+  bool ran = false;
   if (apply_uses_f64_sym(op, o)) {
-    rc = apply_f64_run(op, in, out, wk, s);
+    rc = apply_f64_run(op, in, out, wk, s, &ran);
     if (rc != MRA_OK) return rc;
+  }
+  if (ran) {
+    rc = MRA_OK;
   } else if (o.precision == MRA_PREC_FP64) {
     if (ev0) MRA_CUDA_TRY(cudaEventRecord(ev0, s));
     size_t smem = (size_t)(3 * k3 + 3 * k * k) * sizeof(double);

@@ -26,7 +26,8 @@
 // PT x 9 accumulators.  The sums of each record are written once, as FP64 partials indexed by the
 // record, and dest_sum_f64_kernel adds the partials of every destination in the order of the sorted
 // records.  The partial buffer is bounded: larger applies run in ranges of records (an addition
-// chain per destination in the same order, so the result does not depend on the ranges).
+// chain per destination in the same order, so the result does not depend on the ranges).  Where not even
+// the smallest buffer is to be had, the apply is the gather's (apply.cu), which needs none.
 #include <algorithm>
 
 #include "apply_internal.cuh"
@@ -39,7 +40,7 @@ constexpr int PT = 4;               // elements per thread (9 accumulators each)
 constexpr int F64_MAX_THREADS = 416;
 constexpr size_t F64_MAX_SMEM = 200 * 1024;  // dynamic shared memory of a CTA
 constexpr size_t F64_PARTIAL_BYTES = (size_t)4 << 30;      // most scratch of one range of records
-constexpr size_t F64_PARTIAL_BYTES_MIN = (size_t)64 << 20;  // smallest tried when memory is short
+constexpr size_t F64_PARTIAL_BYTES_MIN = (size_t)64 << 20;  // smallest: a range fills the chip a few times over
 
 __host__ __device__ constexpr int par_half(int k) { return (k + 1) / 2; }
 // doubles of one (level, m) entry of the parity table: [3 components][half of the j][k], even
@@ -500,7 +501,9 @@ size_t f64_partial_least(int k, int64_t P) {
   return std::min(f64_partial_bytes(k, P), std::max(F64_PARTIAL_BYTES_MIN, row));
 }
 
-int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &out, const ApplyWork &wk, cudaStream_t s) {
+int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &out, const ApplyWork &wk, cudaStream_t s,
+                  bool *ran) {
+  *ran = false;
   const int k = op.k, k3 = k * k * k;
   const int64_t P = wk.P, nd = wk.n_dest;
   const size_t row = (size_t)k3 * sizeof(double);
@@ -514,11 +517,12 @@ int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &ou
     // when memory is short, smaller ranges of records
     while (pool_malloc((void **)&partial, bytes, s) != cudaSuccess) {
       cudaGetLastError();
-      if (bytes <= least) return fail(MRA_ERR_CUDA, "mra_apply: out of device memory for the partial sums");
+      if (bytes <= least) return MRA_OK;
       bytes = std::max(bytes / 2, least);
     }
   }
-  if (!partial) return fail(MRA_ERR_ARG, "mra_apply: no partial-sum buffer for the recorded apply");
+  if (!partial) return MRA_OK;
+  *ran = true;
   const int64_t range = (int64_t)(bytes / row);
   if (range < 1) return fail(MRA_ERR_ARG, "mra_apply: partial-sum buffer smaller than one record");
   F64Args a{};

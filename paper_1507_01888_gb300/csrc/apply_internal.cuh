@@ -67,12 +67,14 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
 // P k^3 floats besides the workspace)
 bool apply_uses_src_path(const Operator &op, const mra_apply_opts &o);
 // FP64 source-stationary apply of records with |l|_inf <= 1 (apply_f64.cu): its parity tables (made
-// again when the blocks change), its partial buffer, and the run
+// again when the blocks change), its partial buffer, and the run (*ran = false: no room for partial sums,
+// nothing was launched)
 int f64_parity_build(Operator &op, cudaStream_t s);
 size_t f64_partial_bytes(int k, int64_t P);
-int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &out, const ApplyWork &wk, cudaStream_t s);
-// bytes of partial sums that a recorded apply with P records owns (0: its kernel needs none), and the fewest it
-// can do with
+int apply_f64_run(const Operator &op, const mra_tree_view &in, mra_tree_view &out, const ApplyWork &wk, cudaStream_t s,
+                  bool *ran);
+// bytes of partial sums that a recorded apply with P records owns (0: its kernel needs none), and the fewest
+// worth having (in FP64 the gather takes over below that; the split kernel cannot do with less)
 size_t graph_partial_bytes(const Operator &op, const mra_apply_opts &o, int64_t P, size_t *least);
 size_t f64_partial_least(int k, int64_t P);
 // test hook of the failure path (one-shot), and the fixed-size mode's status from a kernel error word

@@ -87,11 +87,16 @@ int mra_apply_graph_create(const mra_operator *h, int nfunc, const mra_tree_view
   const Operator *op = reinterpret_cast<const Operator *>(h);
   size_t least = 0;
   if (size_t pb = graph_partial_bytes(*op, *o, st.pairs, &least)) {  // the recorded apply's partial sums, owned by the graph
-    while ((e = cudaMalloc(&g->d_partial, pb)) != cudaSuccess && pb > least) {  // memory is short: less where less will do
+    while ((e = limited_malloc(&g->d_partial, pb)) != cudaSuccess && pb > least) {  // memory is short: less where less will do
       cudaGetLastError();
       pb = pb / 2 > least ? pb / 2 : least;
     }
-    if (e != cudaSuccess) return bail(MRA_ERR_CUDA, "partial-sum buffer", e);
+    if (e != cudaSuccess && o->precision != MRA_PREC_FP64) return bail(MRA_ERR_CUDA, "partial-sum buffer", e);
+    if (e != cudaSuccess) {  // none: the gather is recorded
+      cudaGetLastError();
+      g->d_partial = nullptr;
+      pb = 0;
+    }
     g->fx.partial = g->d_partial;
     g->fx.partial_bytes = pb;
   }

@@ -39,6 +39,7 @@ inline G counted(G grid) {
 // own (one per device) that keeps freed memory for the next call instead of returning it to
 // the driver at every synchronisation, as the default pool does; mra_release_memory trims it.
 cudaError_t pool_malloc(void **p, size_t bytes, cudaStream_t s);
+cudaError_t limited_malloc(void **p, size_t bytes);  // cudaMalloc under the test hook's limit
 
 // ---------------------------------------------------------------- index checks
 // The checking build (-DMRA_DEBUG) routes indices of the hot kernels' gathers and scatters

@@ -53,7 +53,7 @@ EXPORTED = [
     "mra_apply_graph_create", "mra_apply_graph_launch", "mra_apply_graph_status", "mra_apply_graph_info",
     "mra_apply_graph_free", "mra_debug_inject_stall", "mra_debug_status", "mra_debug_selftest",
     "mra_operator_refit", "mra_operator_blocks", "mra_release_memory", "mra_apply_host",
-    "mra_measure_fp64_peak", "mra_scale",
+    "mra_measure_fp64_peak", "mra_scale", "mra_debug_limit_memory",
 ]
 NOALLOC_MAX_BOXES = 1 << 20
 
@@ -150,6 +150,7 @@ def load(build_if_stale: bool = True):
         lib.mra_abi_sizeof.argtypes = [ctypes.c_char_p]
         lib.mra_launch_count.restype = ctypes.c_longlong
         lib.mra_debug_status.argtypes = [ctypes.POINTER(ctypes.c_int), ctypes.c_void_p]
+        lib.mra_debug_limit_memory.argtypes = [ctypes.c_size_t]
         lib.mra_project.argtypes = [P(GaussSum), i, d, d, i, i, i, P(TreeView), vp]
         lib.mra_operator_create.argtypes = [i, d, i, d, d, d, i, d, i, i, i, P(vp), vp]
         lib.mra_operator_blocks.argtypes = [i, d, i, d, d, d, i, d, i, i, i, P(vp), vp]
@@ -767,6 +768,11 @@ def debug_selftest(stream=None):
 def debug_inject_stall():
     """mra_debug_inject_stall: the next split-precision apply's waits run out (MRA_ERR_TIMEOUT)."""
     _check(load().mra_debug_inject_stall())
+
+
+def debug_limit_memory(nbytes: int = 0):
+    """mra_debug_limit_memory: requests above nbytes for the library's own scratch fail on this thread (0: no limit)."""
+    _check(load().mra_debug_limit_memory(int(nbytes)))
 
 
 def scale(tree: Tree, alpha: float, stream=None) -> Tree:

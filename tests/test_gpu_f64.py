@@ -113,3 +113,34 @@ def test_term_kept_for_one_sign_only(mra, k):
             break
     if done == 0:
         pytest.skip("every pair of blocks has equal norms here")
+
+
+@pytest.mark.parametrize("k,n_boxes", [(6, 200), (9, 60)])
+def test_without_room_for_partial_sums(mra, k, n_boxes):
+    """The apply and a recorded one give the result when not even the smallest partial buffer is to be had, and a
+    batch of functions gives each function's."""
+    import torch
+    keys, coeffs = W.random_tree_coeffs(n_boxes, k, 3, seed=k)
+    op = mra.Operator(1, 12, k, 32.0, 3, 3, max_disp=1, mu=0.7, fit_eps=1e-4)
+    f = oracle_fit(op)
+    ref = O.apply(keys, coeffs, f["c"], f["t"], 32.0, stencil=0, max_disp=1, tau=1e-2)
+    o = mra.make_opts(stencil=mra.STENCIL_SHELLS, max_disp=1, screen=mra.SCREEN_NORM, tau=1e-2)
+    tree = mra.Tree.from_host(keys, coeffs, 32.0)
+    cat, offs = mra.concat_trees([tree, tree])
+    free, _ = mra.apply(op, tree, o)
+    mra.debug_limit_memory(1 << 19)  # bytes; the partial sums take more than 1 MB
+    try:
+        out, st = mra.apply(op, tree, o)
+        assert st["pairs"] * k ** 3 * 8 > 1 << 20
+        g = mra.ApplyGraph(op, tree, o)
+        g.out.coeffs.zero_()
+        g.launch()
+        g.status()
+        both, _ = mra.BatchedApplier(op, cat, offs, o)(cat)
+    finally:
+        mra.debug_limit_memory(0)
+    fp64_box_check(*free.host(), ref)
+    fp64_box_check(*out.host(), ref)
+    n = out.n
+    assert g.out.n == n and torch.equal(g.out.coeffs[:n], out.coeffs[:n])
+    assert both.n == 2 * n and all(torch.equal(both.coeffs[i * n: (i + 1) * n], out.coeffs[:n]) for i in (0, 1))
