@@ -519,16 +519,23 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
   int ng = f->n;
   const int k3 = k * k * k;
   std::vector<double> hg(5 * (size_t)std::max(ng, 1));
-  for (int g = 0; g < ng; ++g) {
-    hg[g] = f->coef[g];
-    hg[ng + g] = f->expnt[g];
-    hg[2 * ng + g] = f->cx[g];
-    hg[3 * ng + g] = f->cy[g];
-    hg[4 * ng + g] = f->cz[g];
-  }
   double *d_g = nullptr;
   MRA_CUDA_TRY(pool_malloc((void **)&d_g, hg.size() * 8, s));
-  MRA_CUDA_TRY(cudaMemcpyAsync(d_g, hg.data(), hg.size() * 8, cudaMemcpyHostToDevice, s));
+  // the Gaussians in batches of gb: [5][batch] of the batch from g0 on at 5 g0
+  auto upload = [&](int gb) {
+    for (int g0 = 0; g0 < ng; g0 += gb) {
+      const int n = std::min(gb, ng - g0);
+      double *b = hg.data() + 5 * (size_t)g0;
+      const double *field[5] = {f->coef, f->expnt, f->cx, f->cy, f->cz};
+      for (int q = 0; q < 5; ++q)
+        for (int g = 0; g < n; ++g) b[q * n + g] = field[q][g0 + g];
+    }
+    return cudaMemcpyAsync(d_g, hg.data(), hg.size() * 8, cudaMemcpyHostToDevice, s);
+  };
+  // Bound of the factor tables, which grow with the product of Gaussians and coordinates: the level's Gaussians,
+  // or the parents, are taken in batches of this size (and smaller ones where memory is short).  At k = 10 with 8
+  // Gaussians no batch is cut: 3.2 KB per coordinate, at most 24,576 coordinates.
+  const size_t FACTOR_BYTES = (size_t)256 << 20;
   out->k = k;
   out->L = L;
   if (uniform_level >= 0) {
@@ -543,16 +550,25 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
     for (int64_t b = 0; b < total; ++b) keys[b] = make_key(uniform_level, b / (nb * nb), (b / nb) % nb, b % nb);
     for (int64_t q = 0; q < 3 * nb; ++q) entries[q] = factor_entry(uniform_level, (int)(q / nb), q % nb);
     uint64_t *d_entries = nullptr;
-    double *F = nullptr;
-    unsigned char *nz = nullptr;
-    const size_t rows = (size_t)(3 * nb) * std::max(ng, 1);
+    unsigned char *table = nullptr;  // F, nz
     cudaError_t e = pool_malloc((void **)&d_entries, entries.size() * 8, s);
-    if (e == cudaSuccess) e = pool_malloc((void **)&F, rows * k * 8, s);
-    if (e == cudaSuccess) e = pool_malloc((void **)&nz, rows, s);
+    const size_t per_gaussian = (size_t)(3 * nb) * (8 * k + 1);
+    int gb = (int)std::min<size_t>(std::max(ng, 1), std::max<size_t>(FACTOR_BYTES / per_gaussian, 1));
+    while (e == cudaSuccess && (e = pool_malloc((void **)&table, gb * per_gaussian, s)) != cudaSuccess && gb > 1) {
+      cudaGetLastError();
+      gb /= 2;
+      e = cudaSuccess;
+    }
+    if (e == cudaSuccess) e = upload(gb);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out->keys, keys.data(), total * 8, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_entries, entries.data(), entries.size() * 8, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = launch_project_level(ng, d_g, k, L, 3 * nb, d_entries, F, nz, total, out->keys, out->coeffs, s);
-    for (void *p : {(void *)d_entries, (void *)F, (void *)nz, (void *)d_g})
+    for (int g0 = 0; e == cudaSuccess && (g0 == 0 || g0 < ng); g0 += gb) {
+      const int n = std::min(gb, ng - g0);
+      double *F = (double *)table;
+      unsigned char *nz = table + (size_t)(3 * nb) * n * k * 8;
+      e = launch_project_level(n, d_g + 5 * (size_t)g0, k, L, 3 * nb, d_entries, F, nz, total, out->keys, out->coeffs, g0 > 0, s);
+    }
+    for (void *p : {(void *)d_entries, (void *)table, (void *)d_g})
       if (p) cudaFreeAsync(p, s);
     const cudaError_t es = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = es;
@@ -564,6 +580,7 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
     cudaFreeAsync(d_g, s);
     return fail(MRA_ERR_ARG, "mra_project: levels init=%d max=%d invalid", init_level, max_level);
   }
+  MRA_CUDA_TRY(upload(std::max(ng, 1)));
   // ---- adaptive refinement, one level of parents at a time, in chunks
   std::vector<double> U(2 * k * k);
   two_scale(k, U.data());
@@ -576,7 +593,8 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
     int64_t nb = 1LL << pl;
     for (int64_t b = 0; b < nb * nb * nb; ++b) parents.push_back(make_key(pl, b / (nb * nb), (b / nb) % nb, b % nb));
   }
-  const int64_t CH = 8192;  // parents per chunk
+  int64_t most = 8192;  // parents per chunk
+  const size_t per_entry = (size_t)ng * (5 * 8 * k + 3);  // bytes of the factor tables
   std::vector<void *> held;
   auto grab = [&](size_t bytes) -> void * {
     void *p = nullptr;
@@ -611,14 +629,16 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
   uint64_t chunk = 0;
   while (!parents.empty() && rc == MRA_OK && e == cudaSuccess) {
     std::vector<uint64_t> next;
-    for (size_t q0 = 0; q0 < parents.size() && rc == MRA_OK && e == cudaSuccess; q0 += CH) {
-      const int64_t np = std::min<int64_t>(CH, (int64_t)parents.size() - (int64_t)q0);
+    for (size_t q0 = 0; q0 < parents.size() && rc == MRA_OK && e == cudaSuccess;) {
+      const int64_t left = std::min<int64_t>(most, (int64_t)parents.size() - (int64_t)q0);
       const uint64_t *par = parents.data() + q0;
       const int n = key_level(par[0]);
       ++chunk;
       entries.clear();
-      pidx.resize(3 * np);
-      for (int64_t p = 0; p < np; ++p) {
+      pidx.resize(3 * left);
+      int64_t np = 0;
+      for (; np < left && (np == 0 || entries.size() * per_entry < FACTOR_BYTES); ++np) {
+        const int64_t p = np;
         const int64_t xyz[3] = {key_x(par[p]), key_y(par[p]), key_z(par[p])};
         for (int d = 0; d < 3; ++d) {
           uint64_t &at = seen[d * span + xyz[d]];  // chunk << 32 | entry
@@ -629,6 +649,7 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
           pidx[3 * p + d] = (int)(at & 0xFFFFFFFFu);
         }
       }
+      pidx.resize(3 * np);
       const int64_t ne = (int64_t)entries.size();
       entries.resize(3 * ne);
       for (int64_t q = 0; q < ne; ++q)
@@ -647,6 +668,11 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
         work_bytes = work ? at[9] : 0;
       }
       if (!work) {
+        cudaGetLastError();
+        if (np > 1) {  // memory is short: fewer parents at a time
+          most = np / 2;
+          continue;
+        }
         e = cudaErrorMemoryAllocation;
         break;
       }
@@ -666,6 +692,7 @@ int mra_project(const mra_gauss_sum *f, int k, double L, double thresh, int init
       if (e == cudaSuccess) e = cudaMemcpyAsync(dn.data(), d_dn, np * 8, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) break;
+      q0 += np;
       from.clear();
       const bool forced = n + 1 >= max_level;
       for (int64_t p = 0; p < np; ++p) {

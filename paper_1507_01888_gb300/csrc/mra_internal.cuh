@@ -129,10 +129,10 @@ cudaError_t launch_blocks(const Operator &op, const double *d_glx, const double 
 // d_g [5][ng]: coef, expnt, cx, cy, cz; F, nz: n_entries * ng rows of k doubles and flags.
 uint64_t factor_entry(int level, int dim, int64_t x);
 cudaError_t project_tables(cudaStream_t s);  // once on the stream, before launch_project_children
-// every box of a level: entry d 2^n + x
+// every box of a level: entry d 2^n + x; add: to the sums that d_out holds of earlier Gaussians
 cudaError_t launch_project_level(int ng, const double *d_g, int k, double L, int64_t n_entries, const uint64_t *d_entries,
                                  double *F, unsigned char *nz, int64_t nbox, const uint64_t *d_keys, double *d_out,
-                                 cudaStream_t s);
+                                 bool add, cudaStream_t s);
 // the children of np parents and the parents' refinement norms.  d_entries: the parents' n_entries
 // entries, then their children's (2 e + c); pidx[p][d]: the parent's entry; Fp: n_entries ng k, Fc: 4 n_entries ng k
 // doubles, nzp, nzc: n_entries ng and 2 n_entries ng bytes.

@@ -357,14 +357,12 @@ struct Elements {
 };
 
 // Sum over the Gaussians at this thread's elements of one box with the
-// factor entries e[0..2]: own[q], and with TEST the parent's projection there, par[q].  Gaussians
+// factor entries e[0..2], added to own[q], and with TEST the parent's projection there, to par[q].  Gaussians
 // whose product is exactly zero are left out; the others are added in order.
 template <int EPT, bool TEST>
 __device__ void sum_gaussians(int ng, int k, const Elements &el, const double *coef, const double *F, const unsigned char *nz,
                               const int64_t *e, double *stage, int *list, int *count, double *own, double *par) {
   const int st = TEST ? 2 * k : k;
-#pragma unroll
-  for (int q = 0; q < EPT; ++q) own[q] = par[q] = 0.0;
   for (int g0 = 0; g0 < ng;) {
     __syncthreads();  // the list and the staged factors of the previous round have been used
     if (threadIdx.x < 32) {  // the next ASM_G Gaussians that matter, in order
@@ -442,7 +440,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(ASM_THREADS)
   const Elements el(k);
   const int64_t e[3] = {2 * (int64_t)pidx[3 * p] + (c >> 2), 2 * (int64_t)pidx[3 * p + 1] + ((c >> 1) & 1),
                         2 * (int64_t)pidx[3 * p + 2] + (c & 1)};
-  double own[EPT], par[EPT], part = 0.0;
+  double own[EPT] = {}, par[EPT] = {}, part = 0.0;
   sum_gaussians<EPT, true>(ng, k, el, coef, F, nz, e, stage, list, count, own, par);
 #pragma unroll
   for (int q = 0; q < EPT; ++q) {
@@ -473,7 +471,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(ASM_THREADS)
 // One CTA per box of a whole level (entry of dimension d and coordinate x: d 2^n + x).
 template <int EPT>
 __global__ void __launch_bounds__(ASM_THREADS) boxes_kernel(int ng, int k, const double *coef, const double *F,
-                                                            const unsigned char *nz, const uint64_t *keys, double *out) {
+                                                            const unsigned char *nz, const uint64_t *keys, double *out,
+                                                            int add) {
   extern __shared__ double stage[];  // [ASM_G][3][k]
   __shared__ int list[ASM_G], count[2];
   const int64_t b = blockIdx.x;
@@ -481,7 +480,14 @@ __global__ void __launch_bounds__(ASM_THREADS) boxes_kernel(int ng, int k, const
   const int64_t nb = 1LL << key_level(key);
   const int64_t e[3] = {key_x(key), nb + key_y(key), 2 * nb + key_z(key)};
   const Elements el(k);
-  double own[EPT], par[EPT];
+  double own[EPT] = {}, par[EPT];
+  if (add) {
+#pragma unroll
+    for (int q = 0; q < EPT; ++q) {
+      const int m = el.at(k, q);
+      if (m >= 0) own[q] = out[b * k * k * k + m];
+    }
+  }
   sum_gaussians<EPT, false>(ng, k, el, coef, F, nz, e, stage, list, count, own, par);
 #pragma unroll
   for (int q = 0; q < EPT; ++q) {
@@ -561,7 +567,7 @@ static cudaError_t launch_factors(int64_t n_entries, int64_t n_first, int ng, co
 
 cudaError_t launch_project_level(int ng, const double *d_g, int k, double L, int64_t n_entries, const uint64_t *d_entries,
                                  double *F, unsigned char *nz, int64_t nbox, const uint64_t *d_keys, double *d_out,
-                                 cudaStream_t s) {
+                                 bool add, cudaStream_t s) {
   if (nbox <= 0) return cudaSuccess;
   cudaError_t e = upload_tables(s);
   const FactorSet f{k, F, nz};
@@ -569,9 +575,9 @@ cudaError_t launch_project_level(int ng, const double *d_g, int k, double L, int
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)ASM_G * 3 * k * sizeof(double);
   if (k <= 10)
-    boxes_kernel<5><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out);
+    boxes_kernel<5><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out, add);
   else
-    boxes_kernel<16><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out);
+    boxes_kernel<16><<<counted((unsigned)nbox), ASM_THREADS, smem, s>>>(ng, k, d_g, F, nz, d_keys, d_out, add);
   return cudaGetLastError();
 }
 

@@ -60,3 +60,55 @@ def test_flat_to_narrow_gaussians(mra, k, level, a_lo, a_hi):
     f = W.gaussian_sum(6, a_lo, a_hi, seed=k)
     ok, oc, _ = O.project(f, k, 32.0, uniform_level=level)
     check(mra.project(f, k, 32.0, uniform_level=level), ok, oc)
+
+
+def _mixed(ng, real, a_lo, a_hi, seed):
+    """`real` Gaussians spread over ng, the others with coefficient zero: the tables have room for all, the sums are those
+    of the real ones."""
+    f, rng = W.gaussian_sum(real, a_lo, a_hi, seed=seed, centre_box=31.0), np.random.default_rng(seed)
+    at = np.sort(rng.choice(ng, real, replace=False))
+    full = {"coef": np.zeros(ng), "expnt": np.full(ng, 1e3), "cx": np.zeros(ng), "cy": np.zeros(ng), "cz": np.zeros(ng)}
+    for name in full:
+        full[name][at] = f[name]
+    return f, full
+
+
+def test_many_gaussians_in_bounded_tables(mra):
+    """Factor tables of all parents of a level would take over 1 GB: the parents are taken in parts, in 256 MB of tables, and
+    the tree is that of the Gaussians that count."""
+    import torch
+    f, full = _mixed(4000, 800, 1e6, 1e7, 3)
+    few = mra.project(f, 2, 32.0, thresh=1e-2, max_level=13)
+    torch.cuda.synchronize()
+    mra.release_memory()
+    free0 = torch.cuda.mem_get_info()[0] + torch.cuda.memory_reserved()
+    many = mra.project(full, 2, 32.0, thresh=1e-2, max_level=13)
+    used = free0 - (torch.cuda.mem_get_info()[0] + torch.cuda.memory_reserved())
+    keys = many.keys[: many.n].cpu().numpy().view("uint64")
+    lv = (keys >> np.uint64(57)).astype(int)
+    coords = max(sum(len(np.unique((keys[lv == n] >> np.uint64(s)) & np.uint64(0x7ffff) >> np.uint64(1)))
+                     for s in (38, 19, 0)) for n in np.unique(lv))
+    assert coords * 4000 * (40 * 2 + 3) > 1 << 30
+    assert used < 800 << 20, f"{used >> 20} MB"
+    assert many.n == few.n and torch.equal(many.keys[: many.n], few.keys[: few.n])
+    assert torch.equal(many.coeffs[: many.n], few.coeffs[: few.n])
+
+
+def test_short_memory_takes_smaller_batches(mra):
+    """With little memory for the tables the parents of a level, or the Gaussians of a uniform level, are taken in
+    smaller parts: the same sums."""
+    import torch
+    f, full = _mixed(500, 30, 1e3, 1e5, 9)
+    whole = mra.project(full, 2, 32.0, thresh=1e-2, max_level=9)
+    g = W.gaussian_sum(60, 0.1, 1e3, seed=4)
+    level = mra.project(g, 5, 32.0, uniform_level=3)
+    assert whole.n * 64 * 2 < 3 << 20
+    mra.debug_limit_memory(3 << 20)
+    try:
+        parts = mra.project(full, 2, 32.0, thresh=1e-2, max_level=9)
+        mra.debug_limit_memory(16 << 10)
+        batches = mra.project(g, 5, 32.0, uniform_level=3)
+    finally:
+        mra.debug_limit_memory(0)
+    for a, b in ((whole, parts), (level, batches)):
+        assert a.n == b.n and torch.equal(a.keys[: a.n], b.keys[: b.n]) and torch.equal(a.coeffs[: a.n], b.coeffs[: b.n])
