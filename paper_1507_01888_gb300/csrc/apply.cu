@@ -760,6 +760,7 @@ static Layout make_layout(int64_t n_in, int64_t P, int dmax, int64_t n_tab, bool
     return at;
   };
   int64_t nb = n_in > 0 ? n_in : 1, np = P > 0 ? P : 1;
+  const int np32 = sort_size(np);
   L.snorm = take(nb * 8);
   L.dstop = take(nb * 4);
   L.cnt = take(nb * 8);
@@ -793,9 +794,9 @@ static Layout make_layout(int64_t n_in, int64_t P, int dmax, int64_t n_tab, bool
   // CUB temporary storage: the largest of the calls below
   size_t a = 0, b = 0, c = 0;
   cub::DeviceScan::ExclusiveSum(nullptr, a, (int64_t *)nullptr, (int64_t *)nullptr, (int)nb);
-  cub::DeviceScan::InclusiveSum(nullptr, b, (int *)nullptr, (int *)nullptr, (int)np);
+  cub::DeviceScan::InclusiveSum(nullptr, b, (int *)nullptr, (int *)nullptr, np32);
   cub::DeviceRadixSort::SortPairs(nullptr, c, (uint64_t *)nullptr, (uint64_t *)nullptr,
-                                  (int *)nullptr, (int *)nullptr, (int)np);
+                                  (int *)nullptr, (int *)nullptr, np32);
   size_t t = a;
   for (size_t v : {b, c}) t = v > t ? v : t;
   L.tmp_bytes = t;
@@ -1023,6 +1024,7 @@ static int screen_run(const Operator &op, const mra_tree_view &in, const mra_app
                 "(levels %d..%d)", op.min_level, op.max_level);
   const int64_t P = h.records;
   if (P > Pmax) return fail(MRA_ERR_CAPACITY, "mra_apply: internal record bound exceeded");
+  if (P > sort_size(P)) return fail(MRA_ERR_ARG, "mra_apply: %lld records, more than 2^31 - 1", (long long)P);
   if (stats) {
     *stats = mra_apply_stats{};
     stats->n_in = n_in;

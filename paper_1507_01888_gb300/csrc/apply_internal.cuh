@@ -1,6 +1,8 @@
 // apply_internal.cuh -- declarations shared by the apply translation units.
 #pragma once
 
+#include <algorithm>
+
 #include "mra_internal.cuh"
 
 namespace mra {
@@ -46,6 +48,10 @@ struct ApplyWork {
   const int *skip() const { return fx ? fx->skip : nullptr; }  // of the apply kernels; null: never
 };
 
+// records the sorts are sized for: their indices are 32-bit, and the bound on the records (every box with every
+// displacement) may pass that where the records do not
+inline int sort_size(int64_t records) { return (int)std::min<int64_t>(records, INT32_MAX); }
+int64_t apply_max_records(const Operator &op, const mra_apply_opts &o, int64_t n_in);
 size_t apply_workspace_bytes(const Operator &op, const mra_apply_opts &o, int64_t n_in);
 int apply_run(const Operator &op, const mra_tree_view &in, const mra_apply_opts &o,
               mra_tree_view &out, void *ws, size_t ws_bytes, mra_apply_stats *stats,

@@ -714,9 +714,9 @@ size_t split_workspace_bytes(int64_t P) {
   int64_t np = P > 0 ? P : 1;
   size_t t = 0;
   cub::DeviceRadixSort::SortPairs(nullptr, t, (uint64_t *)nullptr, (uint64_t *)nullptr, (int *)nullptr,
-                                  (int *)nullptr, (int)np);
+                                  (int *)nullptr, sort_size(np));
   size_t s2 = 0;
-  cub::DeviceScan::InclusiveSum(nullptr, s2, (int *)nullptr, (int *)nullptr, (int)np);
+  cub::DeviceScan::InclusiveSum(nullptr, s2, (int *)nullptr, (int *)nullptr, sort_size(np));
   if (s2 > t) t = s2;
   auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
   return al(np * 8) * 2 + al(np * 4) * 5 + al((np + 2) * 4) * 2 + al(t) + 256;

@@ -637,6 +637,20 @@ __global__ void sum_kernel(int64_t n, const double *v, double *out) {
 inline size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 inline int64_t boxes(int n) { return 1LL << (3 * n); }
 
+// Levels whose applies run as one: from level `first` on to the returned level (exclusive), as long as the bound on
+// their records together stays below this.  Coarse levels leave most SMs idle and each apply pays its launches and
+// synchronisations; a level with more records than this fills the chip by itself, and beside the others it
+// would only add to the scratch (some 150 bytes a record, and the output rows).  Whole levels at k = 6, M = 8, bound
+// of 2^16, 2^19, 2^22 records and none: |l| <= 3, 4,096 leaves 27.6, 21.4, 21.4, 21.4 ms; |l| <= 1, 32,768 leaves 14.6,
+// 14.0, 14.0, 14.0; 262,144 leaves 79.4, 78.9, 78.1, 78.1; FP64 with |l| <= 3, 32,768 leaves 1044, 1036, 996, 996.
+constexpr int64_t NS_GROUP_RECORDS = 1 << 22;
+template <class Boxes>
+int group_end(const Operator &op, const mra_apply_opts &o, int first, int last, Boxes boxes_in) {
+  int m = first + 1;
+  while (m < last && apply_max_records(op, o, boxes_in(first, m + 1)) < NS_GROUP_RECORDS) ++m;
+  return m;
+}
+
 // Options of the per-level applies and of the coarsest level's complete apply.
 mra_apply_opts level_opts(const mra_apply_opts &o) { return o; }
 mra_apply_opts coarse_opts(const mra_apply_opts &o, int n0) {
@@ -646,11 +660,12 @@ mra_apply_opts coarse_opts(const mra_apply_opts &o, int n0) {
   return c;
 }
 
-// Workspace of mra_apply_ns: dense s^n, S^n (n0 <= n < N, back to back), r ping-pong, Y, Z (all
-// levels), Ubar, an error word, the levels' keys, the applies' outputs (keys +
+// Workspace of mra_apply_ns: dense s^n, S^n (n0 <= n < N, back to back), r ping-pong, Y, Z (of the
+// largest group of levels), Ubar, an error word, the levels' keys, the applies' outputs (keys +
 // coefficients of Y and of Z / the coarse r), and the largest apply's workspace.
 struct NsLayout {
   std::vector<int64_t> first;  // first box of level n among all levels' (n0 <= n <= N)
+  std::vector<int> group;      // the levels [n0, group[0]), [group[0], group[1]), ... up to N
   size_t s, S, rA, rB, Yd, Zd, Ub, err, keys, yk, yc, zk, zc, apply, total;
   size_t apply_bytes;
 };
@@ -668,22 +683,30 @@ NsLayout ns_layout(const Operator &op, const Operator &ns, int N, int n0, const 
   L.first.assign(N + 1, 0);
   for (int n = n0; n < N; ++n) L.first[n + 1] = L.first[n] + boxes(n);
   const int64_t nt = L.first[N];
+  int64_t ng = 0;  // boxes of the largest group
+  const mra_apply_opts lo = level_opts(o);
+  for (int a = n0; a < N;) {
+    const int b = group_end(op, lo, a, N, [&](int x, int y) { return L.first[y] - L.first[x]; });
+    L.group.push_back(b);
+    ng = std::max(ng, L.first[b] - L.first[a]);
+    a = b;
+  }
   L.s = take(nt * k3 * 8);
   L.S = take(nt * kk3 * 8);
   L.rA = take(boxes(N - 1) * k3 * 8);
   L.rB = take(boxes(N - 1) * k3 * 8);
-  L.Yd = take(nt * kk3 * 8);
-  L.Zd = take(nt * k3 * 8);
+  L.Yd = take(ng * kk3 * 8);
+  L.Zd = take(ng * k3 * 8);
   L.Ub = take((size_t)kk * k * 8);
   L.err = take(8);
   L.keys = take(nt * 8);
-  L.yk = take(nt * 8);
-  L.yc = take(nt * kk3 * 8);
-  L.zk = take(nt * 8);
-  L.zc = take(nt * k3 * 8);
+  L.yk = take(ng * 8);
+  L.yc = take(ng * kk3 * 8);
+  L.zk = take(ng * 8);
+  L.zc = take(ng * k3 * 8);
   size_t ab = apply_workspace_bytes(op, coarse_opts(o, n0), boxes(n0));
-  ab = std::max(ab, apply_workspace_bytes(op, level_opts(o), nt));
-  ab = std::max(ab, apply_workspace_bytes(ns, level_opts(o), nt));
+  ab = std::max(ab, apply_workspace_bytes(op, lo, ng));
+  ab = std::max(ab, apply_workspace_bytes(ns, lo, ng));
   L.apply_bytes = ab;
   L.apply = take(ab);
   L.total = off;
@@ -933,18 +956,21 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
   rc = levels_apply(*op, n0, n0 + 1, s_all, coarse_opts(*o, n0), zk, zc, (double *)(w + Lw.Zd), &r0);
   if (rc != MRA_OK) return rc;
   MRA_CUDA_TRY(cudaMemcpyAsync(rcur, r0, (size_t)boxes(n0) * k3 * 8, cudaMemcpyDeviceToDevice, s));
-  // ---- levels n0 .. N-1: their applies do not depend on one another, so all levels in one apply each (level by
-  // level the coarse levels left most SMs idle and every apply paid its launches and synchronisations)
-  rc = levels_apply(*ns, n0, N, S_all, level_opts(*o), yk, yc, (double *)(w + Lw.Yd), &Y);
-  if (rc != MRA_OK) return rc;
-  rc = levels_apply(*op, n0, N, s_all, level_opts(*o), zk, zc, (double *)(w + Lw.Zd), &Z);
-  if (rc != MRA_OK) return rc;
-  for (int n = n0; n < N; ++n) {
-    double *fine = n == N - 1 ? out->coeffs : rnext;
-    sum_down_kernel<<<counted((unsigned)boxes(n)), BOX_THREADS, sh_d, s>>>(k, n, rcur, Z + Lw.first[n] * k3, Y + Lw.first[n] * kk3, Ub,
-                                                                   fine);
-    MRA_CUDA_TRY(cudaGetLastError());
-    std::swap(rcur, rnext);
+  // ---- levels n0 .. N-1: their applies do not depend on one another, so the levels of a group in one apply each
+  int a = n0;
+  for (const int b : Lw.group) {
+    rc = levels_apply(*ns, a, b, S_all + Lw.first[a] * kk3, level_opts(*o), yk, yc, (double *)(w + Lw.Yd), &Y);
+    if (rc != MRA_OK) return rc;
+    rc = levels_apply(*op, a, b, s_all + Lw.first[a] * k3, level_opts(*o), zk, zc, (double *)(w + Lw.Zd), &Z);
+    if (rc != MRA_OK) return rc;
+    for (int n = a; n < b; ++n) {
+      double *fine = n == N - 1 ? out->coeffs : rnext;
+      const int64_t at = Lw.first[n] - Lw.first[a];
+      sum_down_kernel<<<counted((unsigned)boxes(n)), BOX_THREADS, sh_d, s>>>(k, n, rcur, Z + at * k3, Y + at * kk3, Ub, fine);
+      MRA_CUDA_TRY(cudaGetLastError());
+      std::swap(rcur, rnext);
+    }
+    a = b;
   }
   MRA_CUDA_TRY(cudaMemcpyAsync(out->keys, in->keys, (size_t)in->n * 8, cudaMemcpyDeviceToDevice, s));
   MRA_CUDA_TRY(cudaStreamSynchronize(s));
@@ -968,8 +994,8 @@ extern "C" int mra_apply_ns(const mra_operator *h, const mra_operator *hns, cons
 // level, are the result's leaves.  The halo keeps every later level's targets inside the
 // result: a target's parent lies in the previous level's halo.
 // The tree depends on the keys alone and the levels' applies on one another's results not at all, so
-// the structure is made first (two sorts over all levels) and then three applies run: the
-// coarsest level's, and T2k and T over the sources of all levels at once.  Level by level, each
+// the structure is made first (two sorts over all levels) and then the applies run: the
+// coarsest level's, and T2k and T over the sources of a group of levels (see group_end).  Level by level, each
 // with two applies of few boxes, the launches, their synchronisations and the idle SMs took longer than
 // the kernels' work.
 extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns, const mra_tree_view *in, int n0,
@@ -1213,12 +1239,10 @@ extern "C" int mra_apply_ns_tree(const mra_operator *h, const mra_operator *hns,
     *nout_rows += vout.n;
     return MRA_OK;
   };
-  // the applies of the levels are independent: all levels in one apply (levels in groups only where the
-  // record bound of one apply would pass 2^31)
+  // the applies of the levels are independent: the levels of a group in one apply
   auto run_levels = [&](const Operator &opx, double *coeffs, uint64_t *okeys, double *ocoeffs, int64_t *rows) -> int {
     for (int n = n0; n < Nmax;) {
-      int m = n + 1;
-      while (m < Nmax && (first(m + 1) - first(n)) * w3 < (int64_t)INT32_MAX) ++m;
+      const int m = group_end(opx, level_opts(*o), n, Nmax, [&](int x, int y) { return first(y) - first(x); });
       const int rc2 = run_apply(opx, first(n), first(m), coeffs, level_opts(*o), nh, okeys, ocoeffs, rows);
       if (rc2 != MRA_OK) return rc2;
       n = m;

@@ -200,3 +200,56 @@ def test_ns_tree_rejects_bad_trees_and_grows_its_output(mra):
     out = ap(mra.Tree.from_host(keys, coeffs, L))
     rk, rc = O.apply_ns_tree(keys, coeffs, k, L, 1, fit["c"], fit["t"], 1)
     assert out.n == len(rk) and rel(out.host()[1], rc) <= 1e-12
+
+
+# ----------------------------------------------------------------- groups of levels
+
+@pytest.mark.parametrize("k,N,n0,D", [(1, 6, 1, 3), (1, 7, 1, 1), (2, 6, 3, 3)])
+def test_ns_levels_in_several_groups(mra, k, N, n0, D):
+    """Trees whose finest level is an apply of its own beside that of the coarser levels, whole and as a tree."""
+    keys, coeffs = W.random_tree_coeffs(8 ** N, k, N, seed=N)
+    op = mra.Operator(0, 2, k, 8.0, 0, N, max_disp=2 * D + 1, fit_eps=1e-2)
+    fit = oracle_fit(op)
+    ns_op = mra.NSOperator(op, max_disp=D)
+    tree = mra.Tree.from_host(keys, coeffs, 8.0)
+    opts = mra.make_opts(stencil=mra.STENCIL_SHELLS, max_disp=D)
+    out, st = mra.apply_ns(op, ns_op, tree, n0, opts)
+    ref = O.apply_ns(coeffs, k, 8.0, N, n0, fit["c"], fit["t"], D)
+    assert (out.host()[0] == keys).all() and rel(out.host()[1], ref) <= 1e-12
+    # the T and T2k applies over every level, and the coarsest level's with every displacement
+    assert st["levels"][N - 1]["sources"] == 2 * 8 ** (N - 1) and st["levels"][n0]["sources"] == 3 * 8 ** n0
+    as_tree, _ = mra.apply_ns_tree(op, ns_op, tree, n0, opts)
+    assert (as_tree.host()[0] == keys).all() and np.array_equal(as_tree.host()[1], out.host()[1])
+
+
+def _ws(mra, op, n, k, opts, ns_op=None, n0=0):
+    """Workspace sizes for a tree of n boxes (only the counts of the view are read)."""
+    import ctypes
+    v, b = mra.TreeView(n, n, 256, 256, k, 8.0), ctypes.c_size_t()
+    if ns_op is None:
+        mra._check(mra.load().mra_apply_workspace_size(op.handle, ctypes.byref(v), ctypes.byref(opts), ctypes.byref(b)))
+    else:
+        mra._check(mra.load().mra_apply_ns_workspace_size(op.handle, ns_op.handle, ctypes.byref(v), n0, ctypes.byref(opts),
+                                                          ctypes.byref(b)))
+    return b.value
+
+
+@pytest.mark.parametrize("N,D", [(8, 2), (9, 1), (9, 2)])
+def test_ns_workspace_is_that_of_the_finest_level(mra, N, D):
+    """Beside the sources of all levels: one apply of the finest level, its output rows and its dense rows."""
+    k = 1
+    op = mra.Operator(0, 1, k, 8.0, 0, N, max_disp=2 * D + 1, fit_eps=1e-2)
+    ns_op = mra.NSOperator(op, max_disp=D)
+    opts = mra.make_opts(stencil=mra.STENCIL_SHELLS, max_disp=D)
+    fine, every = 8 ** (N - 1), sum(8 ** n for n in range(N))
+    apply = max(_ws(mra, op, fine, 1, opts), _ws(mra, ns_op, fine, 2, opts))
+    rest = every * (8 + 64 + 8) + fine * (2 * 8 + 2 * (64 + 8) + 2 * 8)
+    assert _ws(mra, op, 8 ** N, k, opts, ns_op) <= apply + rest + (1 << 20)
+
+
+@pytest.mark.parametrize("bits", [31, 32])
+def test_workspace_grows_past_32_bit_record_bounds(mra, bits):
+    op = mra.Operator(0, 1, 1, 8.0, 3, 3, max_disp=7, fit_eps=1e-2)
+    opts = mra.make_opts(stencil=mra.STENCIL_SHELLS, max_disp=7)
+    below, above = (2 ** bits - 1) // 15 ** 3, (2 ** bits - 1) // 15 ** 3 + 1
+    assert _ws(mra, op, above, 1, opts) >= _ws(mra, op, below, 1, opts)
