@@ -144,3 +144,68 @@ def test_without_room_for_partial_sums(mra, k, n_boxes):
     n = out.n
     assert g.out.n == n and torch.equal(g.out.coeffs[:n], out.coeffs[:n])
     assert both.n == 2 * n and all(torch.equal(both.coeffs[i * n: (i + 1) * n], out.coeffs[:n]) for i in (0, 1))
+
+
+def test_ranges_of_records_in_the_doubled_basis(mra):
+    """The non-standard operator's apply in several ranges of records, where the sums are turned back into the
+    children's coefficients after the last one only: bit for bit the result of one range."""
+    import torch
+    k, level = 12, 3
+    keys, coeffs = W.random_tree_coeffs(400, k, level, seed=12)
+    base = mra.Operator(0, 3, k // 2, 32.0, level, level + 1, max_disp=3, fit_eps=1e-4)
+    op = mra.NSOperator(base, max_disp=1)
+    tree = mra.Tree.from_host(keys, coeffs, 32.0)
+    whole, st = mra.apply(op, tree, mra.make_opts())
+    total = st["pairs"] * k ** 3 * 8
+    assert 65 << 20 < total < 4 << 30
+    mra.debug_limit_memory(65 << 20)  # the smallest partial buffer (64 MB) fits; below that the gather would run
+    try:
+        parts, _ = mra.apply(op, tree, mra.make_opts())
+    finally:
+        mra.debug_limit_memory(0)
+    assert parts.n == whole.n and torch.equal(parts.keys[: parts.n], whole.keys[: whole.n])
+    assert torch.equal(parts.coeffs[: parts.n], whole.coeffs[: whole.n])
+
+
+@pytest.mark.parametrize("k", [2, 3])
+def test_term_kept_for_one_sign_only_in_the_doubled_basis(mra, k):
+    """As test_term_kept_for_one_sign_only, with the non-standard operator's blocks."""
+    lo, hi = 1, 6
+    op = mra.NSOperator(mra.Operator(0, 20, k, 32.0, lo, hi + 1, max_disp=3, fit_eps=1e-4), max_disp=1)
+    c, kk = op.base.fit()["c"], 2 * k
+    s = np.random.default_rng(k).standard_normal((kk, kk, kk))
+    done = 0
+    for level in range(lo + 1, hi + 1):
+        key = np.array([(level << 57) | (1 << 38) | (1 << 19) | 1], dtype=np.uint64)
+        tree = mra.Tree.from_host(key, s[None], 32.0)
+        sn = float(mra.norm(tree)[0][0])
+        R = [{l: op.block(level, m, l) for l in (-1, 0, 1)} for m in range(20)]
+        for m in range(20):
+            up, down, mid = (abs(c[m]) * R[m][l][1] * R[m][0][1] * R[m][0][1] * sn for l in (1, -1, 0))
+            tau = max(up, down)
+            if up == down or mid < tau:
+                continue
+            out, st = mra.apply(op, tree, mra.make_opts(stencil=mra.STENCIL_SHELLS, max_disp=1, screen=mra.SCREEN_NORM, tau=tau))
+            want, n_terms, lone = {}, 0, 0
+            for l in np.ndindex(3, 3, 3):
+                l = tuple(v - 1 for v in l)
+                for q in range(20):
+                    def bound(*d):
+                        return abs(c[q]) * R[q][d[0]][1] * R[q][d[1]][1] * R[q][d[2]][1] * sn
+                    if not bound(*l) >= tau:
+                        continue
+                    n_terms += 1
+                    lone += not bound(-l[0], l[1], l[2]) >= tau
+                    d = int(key[0]) + (l[0] << 38) + (l[1] << 19) + l[2]
+                    r = want.setdefault(d, [np.zeros_like(s), 0.0])
+                    r[0] += c[q] * np.einsum("ai,bj,cl,ijl->abc", R[q][l[0]][0], R[q][l[1]][0], R[q][l[2]][0], s)
+                    r[1] += bound(*l)
+            assert lone > 0 and st["terms_kept"] == n_terms
+            gk, gc = out.host()
+            assert sorted(want) == [int(v) for v in gk]
+            for d, got in zip(gk, gc):
+                r, scale = want[int(d)]
+                assert np.linalg.norm(got - r) <= 1e-12 * max(np.linalg.norm(r), scale)
+            done += 1
+            break
+    assert done > 0, "no pair of blocks with unequal norms"

@@ -56,6 +56,26 @@ def test_split_parts_of_a_tile_equal_whole_tiles(mra, k):
     assert torch.equal(out.keys[: single.n], single.keys[: single.n])
 
 
+@pytest.mark.parametrize("k", [4, 6, 8, 10])
+def test_split_three_parts_of_a_tile_equal_nine(mra, k):
+    """Between one and eight tiles for every CTA slot a tile's groups go to three CTAs: each copy of a batch of that
+    size has the single function's result (nine CTAs a tile) bit for bit."""
+    import torch
+    keys, coeffs = W.random_tree_coeffs(20, k, 3, seed=k)
+    op = mra.Operator(0, 3, k, 32.0, 3, 3, max_disp=1, fit_eps=1e-4)
+    tree = mra.Tree.from_host(keys, coeffs, 32.0)
+    o = mra.make_opts(precision=mra.PREC_SPLIT_BF16, stencil=mra.STENCIL_NEAREST)
+    single, _ = mra.apply(op, tree, o)
+    slots, G = 2 * torch.cuda.get_device_properties(0).multi_processor_count, {4: 8, 6: 3, 8: 2, 10: 1}[k]
+    copies = 2 * slots * G // 20 + 1
+    assert slots <= 20 * copies // G and 20 * copies // G + 20 < 8 * slots
+    cat, offs = mra.concat_trees([tree] * copies)
+    out, _ = mra.BatchedApplier(op, cat, offs, o)(cat)
+    want = single.coeffs[: single.n]
+    assert out.n == copies * single.n
+    assert bool((out.coeffs[: out.n].reshape(copies, *want.shape) == want).all())
+
+
 def test_truncate_into_its_own_buffers(mra):
     """mra_truncate with the result in the input's buffers, and with too little room (which leaves them as they are)."""
     import ctypes
