@@ -39,6 +39,23 @@ import workloads as W  # noqa: E402
 SPLIT_TRAFFIC = {("bsh_m60_adaptive_k10", "apply_src_kernel"): 68.46e6 + 687.48e6}
 
 METRIC = "3D operator-apply boxes/s & % roofline, mixed vs FP64 GPU at 1e-6 rel L2"
+
+
+def fp64_roofline(parts, kernel_ms, peak, peak_source):
+    """Roofline entry of FP64 applies: parts = (algorithmic flops, widest displacement of its records) of each apply.
+    Records within |l|_inf <= 1 run in apply_f64_sym_kernel, which shares mode products between terms and uses the
+    blocks' parity: 19.5 k^4 FMAs for a source's 27 terms of one m instead of 81 k^4, and a larger share of the
+    81 k^4 where a source keeps fewer of the 27, so `achieved` is a lower bound of what it executes.  Wider ones run
+    in apply_f64_kernel, three full products per term."""
+    executed = sum(f * (19.5 / 81 if d <= 1 else 1.0) for f, d in parts) / (kernel_ms / 1e3) / 1e12
+    names = [n for n, wide in (("apply_f64_sym_kernel and dest_sum_f64_kernel", False), ("apply_f64_kernel", True))
+             if any((d > 1) == wide and f > 0 for f, d in parts)]
+    return {"bound": "alu", "achieved": executed, "peak": peak, "unit": "TFLOP/s", "frac": executed / peak,
+            "traffic": None, "kernel": ", ".join(names), "peak_source": peak_source, "kernel_ms": kernel_ms,
+            "flops": "executed; per term 6k^4+k^3 with three full products, 19.5/81 of it where products are shared",
+            "algorithmic_tflops": sum(f for f, _ in parts) / (kernel_ms / 1e3) / 1e12}
+
+
 def fixed_schedule(opts, text):
     """opts with the schedule fields given as 'field=value,...' (no tuning)."""
     from paper_1507_01888_gb300 import autotune, mra
@@ -437,12 +454,9 @@ def run_ns(args, w, rank, world):
     pk, pk_kind = peaks()
     if prec == mra.PREC_FP64:
         p64 = fp64_peak()["dfma_tflops"]
-        roof = {"bound": "alu", "achieved": achieved, "peak": p64, "unit": "TFLOP/s",
-                "frac": achieved / p64, "traffic": None, "kernel": "apply_f64_sym_kernel (all levels)",
-                "peak_source": fp64_peak_source(), "kernel_ms": kms_mean,
-                "flops": "algorithmic (6k'^4+k'^3 per term, k' = k or 2k: three full products per term; the "
-                         "kernel shares products between terms and uses the blocks' parity, so it executes about "
-                         "a quarter of these and frac exceeds 1)"}
+        # the coarsest level's complete apply, then the levels' (the operator's deepest level has room for either)
+        fl = [(t * (6 * (f * k) ** 4 + (f * k) ** 3), (1 << n0) - 1 if i == 0 else D) for i, (_, f, t) in enumerate(terms)]
+        roof = fp64_roofline(fl, kms_mean, p64, fp64_peak_source())
         dtype = "f64"
     else:
         peak = pk.get("bf16_tflops", 1856.3)
@@ -1034,13 +1048,8 @@ def main():
     achieved_tflops = terms * flops_per_term / (kms / 1e3) / 1e12
     if prec == mra.PREC_FP64:
         p64 = fp64_peak(local)["dfma_tflops"]
-        roof = {"bound": "alu", "achieved": achieved_tflops, "peak": p64, "unit": "TFLOP/s",
-                "frac": achieved_tflops / p64, "traffic": None,
-                "kernel": "apply_f64_sym_kernel with its summation kernel", "peak_source": fp64_peak_source(local),
-                "kernel_ms": kms,
-                "flops": "algorithmic (6k^4+k^3 per kept term: three full products; the kernel shares products "
-                         "between terms and uses the blocks' parity, so it executes about a quarter of these and "
-                         "frac exceeds 1)"}
+        widest = min(1 if opts.stencil == mra.STENCIL_NEAREST else opts.max_disp, (1 << op.max_level) - 1)
+        roof = fp64_roofline([(terms * flops_per_term, widest)], kms, p64, fp64_peak_source(local))
         dtype = "f64"
     else:
         peak = pk.get("bf16_tflops", 1856.3)
