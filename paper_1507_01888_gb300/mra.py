@@ -286,7 +286,7 @@ def project(gauss: dict, k: int, L: float, thresh: float = 0.0, init_level: int 
         if trim and keep < cap:
             # The copies run on torch's current stream (the large buffer goes back to that stream's pool) and are
             # complete on return, as the library's own work is: the tree may be used on any stream.
-            t.keys, t.coeffs = t.keys[:keep].clone(), t.coeffs[:keep].clone()
+            t.coeffs, t.keys = t.coeffs[:keep].clone(), t.keys[:keep].clone()  # the large one first
             torch.cuda.current_stream(t.keys.device).synchronize()
         return t
 
