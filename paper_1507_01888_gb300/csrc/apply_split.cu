@@ -795,8 +795,9 @@ int apply_split_run(const Operator &op, const mra_tree_view &in, const mra_apply
   // The tiles heaviest first, so that the last CTAs to start are short ones: a destination's terms run in
   // series in one CTA (up to 27 M of them), and with the heavy ones last most SMs were idle at the end.
   // Only where the CTAs do not all run at once, and up to 32 rounds of them: the end matters less with every
-  // round, while key order keeps the sources that neighbours gather in L2 (171,592 boxes at k = 14, 564 rounds:
-  // 635 ms in key order, 658 heaviest first; 6,586 destinations, 22 rounds: 26.0 and 25.2).  key2 and
+  // round, while key order keeps the sources that neighbours gather in L2.  In key order and heaviest first, k = 14:
+  // 5 rounds 7.8 and 6.4 ms, 12 16.0 and 14.3, 22 28.2 and 27.5, 25 30.6 and 29.9, 44 55.2 and 55.2, 57 69.2 and 69.7, 564
+  // 635 and 658 (171,592 boxes); k = 12 and 10 gain 3% at 50 rounds still (36.0 and 35.0; 34.2 and 33.0).  key2 and
   // key2s are free by now (n_tiles <= P entries of each).
   int dev = 0, sms = 0;
   MRA_CUDA_TRY(cudaGetDevice(&dev));

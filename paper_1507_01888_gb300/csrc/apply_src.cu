@@ -943,13 +943,19 @@ int apply_src_run(const Operator &op, const mra_tree_view &in, const mra_apply_o
   MRA_CUDA_TRY(cudaGetDevice(&dev));
   MRA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   // persistent: two CTAs per SM (the tensor memory holds two of 256 columns), never more CTAs
-  // than sources
+  // than parts of tiles
   const int64_t max_tiles = G == 1 ? n_in : n_in / G + MRA_MAX_LEVEL + 1;
   // A tile's passes run in series, so with few tiles the kernel lasts as long as one: then the (lx, ly) groups of a
   // tile, which share nothing but the staged sources, go to three or nine CTAs.  512 boxes at k = 6 (171 tiles of
-  // 180 passes for 304 CTAs): the call 500 -> 419 us.
-  const int64_t slots = 2 * (int64_t)sms;
-  a.parts = max_tiles >= 8 * slots ? 1 : max_tiles >= slots ? 3 : 9;
+  // 180 passes for 304 CTAs): the call 500 -> 419 us.  Every part stages the sources and scans their records again, which
+  // costs the more the fewer terms a record has (three parts of many tiles: M = 20 4%, M = 40 1.4%, M = 60 nothing; nine
+  // 24%, 12%, 5 to 8%), so with few terms the lines lie lower.  Kernel times with 1 / 3 / 9 parts, tiles in units of the 304
+  // slots: M = 20, k = 4: 0.5 238 / 188 / 160 us, 0.9 275 / 280 / 297, 1.2 506 / 373 / 414, 3.5 1014 / 977 / 1139,
+  // 6.3 1704 / 1749 / 2074; k = 6: 0.7 256 / 185 / 213, 5.3 1307 / 1305 / 1528, 7.3 1763 / 1804 / 2133.  M = 40, k = 8:
+  // 0.9 490 / 450 / 429, 4.3 2084 / 2006 / 2199, 7.3 3292 / 3286 / 3628, 12 5405 / 5478.  M = 60, k = 10: 0.9 724 / 651 / 594,
+  // 4.3 3007 / 2826 / 3011, 7.3 4933 / 4869 / 5230, 12 8012 / 8033.
+  const int64_t slots = 2 * (int64_t)sms, unit = slots * std::min(60, 20 + op.M) / 60;
+  a.parts = max_tiles >= 8 * unit ? 1 : max_tiles >= unit ? 3 : 9;
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(slots, max_tiles * a.parts));
   if (((uintptr_t)partial & 15) != 0 || k3 % 4 != 0)
     return fail(MRA_ERR_ARG, "split apply: partial-sum buffer not 16-byte aligned or k^3 = %d not a multiple of 4", k3);
