@@ -208,13 +208,14 @@ long long mra_launch_count(void);
 /* Device memory the library keeps for reuse: the scratch of the calls that allocate it
  * themselves (projection, norms and comparisons, reconstruction, truncation, products, the
  * non-standard applies; of the plain applies the partial sums, in FP64 up to 4 GB and less or none where
- * memory is short) comes from a stream-ordered pool per device that holds on to freed memory between calls.  This returns the pool's unused memory to the driver.  Memory of
- * allocations still in flight on a stream is not affected. */
+ * memory is short) comes from a stream-ordered pool per device that holds on to freed memory between
+ * calls.  This returns the pool's unused memory to the driver.  Memory of allocations still in flight
+ * on a stream is not affected. */
 int mra_release_memory(void);
 
 /* Test hook for the failure path: the next MRA_PREC_SPLIT_BF16 apply in this process has one
- * CTA (the one that takes the first tile) skip the block copies of its first term, so that the kernel's bounded waits on them
- * run out (about two seconds each); that apply returns MRA_ERR_TIMEOUT with the device context
+ * CTA (the one that takes the first tile) skip the block copies of its first term, so that the
+ * kernel's bounded waits on them run out (about two seconds each); that apply returns MRA_ERR_TIMEOUT with the device context
  * intact, and later calls run normally.  One-shot; nothing else is changed. */
 int mra_debug_inject_stall(void);
 
@@ -439,7 +440,7 @@ int mra_apply_ns_workspace_size(const mra_operator *op, const mra_operator *ns_o
  * n0..N, max_disp >= 2^n0 - 1); ns_op: mra_operator_ns_create(op, ...).  Steps: compress
  * (s^n = filter of the children tensor S^n, n = N-1 .. n0); T^{n0} s^{n0} with every
  * displacement of level n0; for n = n0 .. N-1, Y^n = T2k^n S^n and Z^n = T^n s^n with
- * opts' stencil and screen (each an mra_apply on level n's boxes, in opts' precision),
+ * opts' stencil and screen (an mra_apply on the boxes of one or several levels, in opts' precision),
  * and the children of every box b get U^{x3} (r^n_b - Z^n_b) + Y^n_b as r^{n+1}.  out:
  * the level-N result, same keys as in (cap >= in->n, else MRA_ERR_CAPACITY with out->n
  * the size needed).  opts.screen: NONE or NORM.  With every displacement the result equals
@@ -468,7 +469,7 @@ int mra_apply_ns_tree(const mra_operator *op, const mra_operator *ns_op, const m
  * level), representing f = sum_b f_b; out: disjoint leaves holding the same function, keys
  * sorted.  Every box with input boxes below it, and every box on the path down to them, passes
  * its accumulated coefficients to its eight children through the two-scale relation; the
- * others are the leaves.  k <= MRA_MAX_K / 2.  Capacity as mra_apply_ns_tree; temporaries
+ * others are the leaves.  k <= MRA_MAX_K.  Capacity as mra_apply_ns_tree; temporaries
  * stream-ordered; synchronises the stream. */
 int mra_reconstruct(const mra_tree_view *in, mra_tree_view *out, void *stream);
 
@@ -487,7 +488,7 @@ int mra_truncate(const mra_tree_view *in, double thresh, mra_tree_view *out, dou
  * Gauss-Legendre points of each dimension (the third representation of Sec. 2.1) are
  * multiplied and transformed back: s_ab = h^{-3/2} (V^T W)^{x3} [(V^{x3} s_a)(V^{x3} s_b)],
  * V[q][i] = phi_i(x_q), W = diag(w_q) -- the product interpolated at the points.  out: the
- * common leaves (capacity as mra_reconstruct).  k <= MRA_MAX_K / 2.  Synchronises. */
+ * common leaves (capacity as mra_reconstruct).  k <= MRA_MAX_K.  Synchronises. */
 int mra_multiply(const mra_tree_view *a, const mra_tree_view *b, mra_tree_view *out, void *stream);
 
 /* Inner product <a, b> = integral of a b, the coefficient dot product over the two trees'

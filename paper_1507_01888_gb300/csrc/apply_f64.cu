@@ -14,8 +14,8 @@
 // A full neighbourhood takes 19.5 k^4 FMAs per source and term instead of 81 k^4.  Measured on the
 // whole apply against the per-destination gather with full products (apply_f64_kernel, now for wider
 // displacements only): bound-state Helmholtz M = 60, k = 10, 17,200 boxes, 5.92 M kept terms 314 ->
-// 78.9 ms (0.565 T FMA/s, the FP64 pipe's rate); order 20, 1,408 leaves in non-standard form 931 ->
-// 86 ms; 64 boxes, k = 6, M = 20 1.51 -> 0.39 ms.
+// 78.6 ms (0.567 T FMA/s, 90% of two per SM and clock); order 20, 1,408 leaves in non-standard form, all levels in
+// one apply, 931 -> 71.6 ms; 64 boxes, k = 6, M = 20 1.51 -> 0.29 ms (0.39 before the apply's small kernels were joined).
 //
 // Work decomposition.  The output index ix of the first product is carried unchanged through the
 // other two, so the work of a source splits without redundancy into slices (cx, ix), cx = 0, E, O:
@@ -456,8 +456,8 @@ size_t f64_smem(int k, int nx) {
 // 16 cycles), times 8 / (resident warps) where fewer than eight warps are there to hide their own
 // latency; the least wins.  Large trees get the split with the fewest idle lanes (k = 10: 5 slices,
 // 256 threads, two elements of each half per thread), small ones more CTAs of fewer elements per thread.
-// 64 boxes, k = 6, M = 20, whole call: 1 slice and two elements in one warp 501 us, 6 slices and one
-// element in seven warps 394 us.
+// 64 boxes, k = 6, M = 20, whole call when it was chosen: 1 slice and two elements in one warp 501 us, 6 slices and
+// one element in seven warps 394 us (now 293).
 void f64_shape(int k, int64_t n_src, int sms, int *nx_out, int *threads_out) {
   double best = -1.0;
   for (int nx = 1; nx <= k; ++nx)

@@ -1,7 +1,7 @@
 // setup.cu -- set-up kernels: Gaussian-fit search, 1-D operator blocks, projection.
 //
-// Everything here is FP64 and runs once per operator or per input function;
-// none of it is on the timed apply path.  Compiled with --fmad=false so that
+// Everything here is FP64 and runs once per operator or per input function, outside the
+// applies; the fit also runs in every refit, so in every step of the bound-state solver.  Compiled with --fmad=false so that
 // the fit search evaluates its error exactly as written.
 #include <cooperative_groups.h>
 #include <math.h>
